@@ -30,6 +30,7 @@ struct ptm_context {
   // workspace
   size_t cap_atoms = 0, cap_cells = 0, cap_sorted_bytes = 0;
   void *sorted = nullptr;
+  float4 *hi = nullptr, *lo = nullptr;
   int *sbin = nullptr, *wrapv = nullptr, *atom_cell = nullptr, *atom_rank = nullptr, *atom_wrap = nullptr;
   int *cell_count = nullptr, *cell_start = nullptr, *block_sums = nullptr;
   int *dstat = nullptr;
@@ -52,8 +53,9 @@ struct ptm_context {
   uint64_t *lam = nullptr;
   uint32_t *ents = nullptr;
   size_t cap_nbr = 0;
-  // topological order: atoms for the FP64 pass ([n] = their count) and what
-  // the FP32 pass keeps for it
+  // topological order: the 18 nearest, atoms for the FP64 pass and what the FP32
+  // pass keeps for it
+  int2 *nbr18 = nullptr;
   int *topo_list = nullptr;
   TopoSide *topo_side = nullptr;
   size_t cap_topo = 0;
@@ -75,6 +77,8 @@ static ptm_status grow(ptm_context *ctx, size_t n, size_t ncell, int f64) {
   if (n > ctx->cap_atoms || sb > ctx->cap_sorted_bytes) {
     cudaFree(ctx->sorted); cudaFree(ctx->sbin); cudaFree(ctx->wrapv);
     cudaFree(ctx->atom_cell); cudaFree(ctx->atom_rank); cudaFree(ctx->atom_wrap);
+    cudaFree(ctx->hi); cudaFree(ctx->lo);
+    ctx->hi = ctx->lo = nullptr;
     ctx->sorted = nullptr; ctx->sbin = ctx->wrapv = ctx->atom_cell = ctx->atom_rank = ctx->atom_wrap = nullptr;
     ctx->cap_atoms = ctx->cap_sorted_bytes = 0;
     size_t na = std::max(n, ctx->cap_atoms);
@@ -85,6 +89,8 @@ static ptm_status grow(ptm_context *ctx, size_t n, size_t ncell, int f64) {
     CK(cudaMalloc(&ctx->atom_cell, na * sizeof(int)));
     CK(cudaMalloc(&ctx->atom_rank, na * sizeof(int)));
     CK(cudaMalloc(&ctx->atom_wrap, na * sizeof(int)));
+    CK(cudaMalloc(&ctx->hi, na * sizeof(float4)));
+    CK(cudaMalloc(&ctx->lo, na * sizeof(float4)));
     ctx->cap_atoms = na;
     ctx->cap_sorted_bytes = nsb;
   }
@@ -162,15 +168,18 @@ static ptm_status setup_frame(const ptm_frame *f, double cell_factor, FrameDesc 
   desc->rmsd_max = std::isnan(f->rmsd_max) ? INFINITY : (float)f->rmsd_max;
   desc->min_cell_width = (float)std::min(W[0] / nb[0], std::min(W[1] / nb[1], W[2] / nb[2]));
   for (int i = 0; i < 9; i++) desc->H[i] = H[i];
-  // |n.H| for |n_r| <= 1 over the periodic rows r: at most the length of the
-  // vector of per-component sums of |H_rc| (rounded up a little for FP32)
-  double sm2 = 0.0;
+  desc->cell_vol = (float)(std::fabs(det) / (double)ncell);
+  // positions (at most 100 periods from the cell, else excluded) and shifts are
+  // within about 100 hs of the origin, hs the length of the vector of the
+  // per-component sums of |H_rc|; the FP32 pairs and the error-free sums of the
+  // neighbour search leave about ten terms of 2^-48 of that in a component
+  double hs2 = 0.0;
   for (int k = 0; k < 3; k++) {
     double sk = 0.0;
-    for (int r = 0; r < 3; r++) if (f->pbc[r]) sk += std::fabs(H[3 * r + k]);
-    sm2 += sk * sk;
+    for (int r = 0; r < 3; r++) sk += std::fabs(H[3 * r + k]);
+    hs2 += sk * sk;
   }
-  desc->smax = (float)(std::sqrt(sm2) * (1.0 + 1e-6));
+  desc->tau = (float)(std::ldexp(std::sqrt(hs2), -37));
   for (int a = -2; a <= 2; a++)
     for (int b = -2; b <= 2; b++)
       for (int c = -2; c <= 2; c++) {
@@ -188,12 +197,67 @@ static ptm_status setup_frame(const ptm_frame *f, double cell_factor, FrameDesc 
       }
   std::memset(bp, 0, sizeof(BinParams));
   for (int i = 0; i < 9; i++) bp->Hinv[i] = (float)Hinv[i];
+  for (int i = 0; i < 9; i++) bp->H[i] = H[i];
   for (int c = 0; c < 3; c++) { bp->W[c] = (float)W[c]; bp->nb[c] = nb[c]; bp->pbc[c] = desc->pbc[c]; }
   bp->n = n;
   bp->f64 = desc->f64;
   bp->pos = f->positions;
   *ncell_out = ncell;
   return PTM_OK;
+}
+
+// Device buffers of one frame's pipeline beside those its descriptor names.
+struct FrameBuffers {
+  int *cell_count, *cell_start, *block_sums, *atom_cell, *atom_rank, *atom_wrap, *sbin, *wrapv;
+  void *sorted;
+  float4 *hi, *lo;
+  int *dstat;
+  unsigned long long *counters;
+  ShiftTables *tab;
+  int2 *nbr, *nbr18;
+  uint64_t *lam;
+  uint32_t *ents;
+};
+
+static void set_buffers(FrameDesc *d, BinParams *bp, const FrameBuffers &B) {
+  d->sorted = B.sorted; d->hi = B.hi; d->lo = B.lo;
+  d->sbin = B.sbin; d->cell_start = B.cell_start; d->wrapv = B.wrapv;
+  d->dstat = B.dstat; d->counters = B.counters; d->tab = B.tab;
+  d->nbr = B.nbr; d->nbr18 = B.nbr18; d->lam = B.lam; d->ents = B.ents;
+  bp->counters = B.counters;
+}
+
+// Cell list of one frame; returns the number of kernels launched.
+static int launch_cells(const ptm_frame *f, const BinParams &bp, const ShiftTables &tab, size_t ncell,
+                        const FrameBuffers &B, cudaStream_t st) {
+  const int tb = 256, nscan = (int)ncell + 1;
+  const unsigned gb = (unsigned)((f->n_atoms + tb - 1) / tb);
+  k_begin<<<std::min(152, (nscan + tb - 1) / tb), tb, 0, st>>>(tab, B.tab, B.cell_count, nscan, B.dstat, B.counters);
+  k_bin<<<gb, tb, 0, st>>>(f->positions, bp, B.cell_count, B.atom_cell, B.atom_rank, B.atom_wrap, B.dstat);
+  const int nblk = (nscan + 2 * SCAN_BLOCK - 1) / (2 * SCAN_BLOCK);
+  k_scan_block<<<nblk, SCAN_BLOCK, 0, st>>>(B.cell_count, B.cell_start, B.block_sums, nscan);
+  if (nblk > 1) k_scan_add<<<nblk, SCAN_BLOCK, 0, st>>>(B.cell_start, B.block_sums, nscan);
+  k_scatter<<<gb, tb, 0, st>>>(f->positions, bp, B.atom_cell, B.atom_rank, B.atom_wrap, B.cell_start, B.dstat, B.sorted,
+                               B.hi, B.lo, B.sbin, B.wrapv);
+  return nblk > 1 ? 5 : 4;
+}
+
+// Blocks of k_knn_rest, which strides over its list: at most four per SM.
+static unsigned rest_grid(int64_t n) { return (unsigned)std::min<int64_t>((n + 3) / 4, 4 * 152); }
+
+// Neighbour lists (the NK nearest) of one frame; the atom ranks of the cell list
+// are dead by now and hold the list of undecided atoms.
+template <int NK>
+static void launch_knn(const FrameDesc &desc, const FrameBuffers &B, cudaStream_t st) {
+  const unsigned gk = (unsigned)((desc.n + PTM_KNN_BLOCK - 1) / PTM_KNN_BLOCK);
+  int *cnt = B.dstat + 2;
+  if (desc.f64) {
+    k_knn<true, NK><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(NK), st>>>(desc, B.atom_rank, cnt);
+    k_knn_rest<true, NK><<<rest_grid(desc.n), PTM_KNN_BLOCK, 0, st>>>(desc, B.atom_rank, cnt);
+  } else {
+    k_knn<false, NK><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(NK), st>>>(desc, B.atom_rank, cnt);
+    k_knn_rest<false, NK><<<rest_grid(desc.n), PTM_KNN_BLOCK, 0, st>>>(desc, B.atom_rank, cnt);
+  }
 }
 
 // Enqueue the whole pipeline for one frame whose buffers are on the device.
@@ -220,54 +284,35 @@ static ptm_status enqueue_frame(ptm_context *ctx, const ptm_frame *f, const ptm_
     ctx->cap_nbr = (size_t)n;
   }
   if (topological && (size_t)n > ctx->cap_topo) {
+    cudaFree(ctx->nbr18);
     cudaFree(ctx->topo_list);
     cudaFree(ctx->topo_side);
+    ctx->nbr18 = nullptr;
     ctx->topo_list = nullptr;
     ctx->topo_side = nullptr;
     ctx->cap_topo = 0;
-    CK(cudaMalloc(&ctx->topo_list, ((size_t)n + 1) * sizeof(int)));
+    CK(cudaMalloc(&ctx->nbr18, (size_t)n * PTM_TOPO_N * sizeof(int2)));
+    CK(cudaMalloc(&ctx->topo_list, (size_t)n * sizeof(int)));
     CK(cudaMalloc(&ctx->topo_side, topo_side_bytes((size_t)n)));
     ctx->cap_topo = (size_t)n;
   }
-  desc.sorted = ctx->sorted;
-  desc.sbin = ctx->sbin;
-  desc.cell_start = ctx->cell_start;
-  desc.wrapv = ctx->wrapv;
+  const FrameBuffers B = {ctx->cell_count, ctx->cell_start, ctx->block_sums, ctx->atom_cell, ctx->atom_rank,
+                          ctx->atom_wrap, ctx->sbin, ctx->wrapv, ctx->sorted, ctx->hi, ctx->lo, ctx->dstat,
+                          ctx->counters, ctx->tab, ctx->nbr, ctx->nbr18, ctx->lam, ctx->ents};
+  set_buffers(&desc, &bp, B);
   set_outputs(&desc, o);
-  desc.dstat = ctx->dstat;
-  desc.counters = ctx->counters;
-  desc.nbr = ctx->nbr;
-  desc.lam = ctx->lam;
-  desc.ents = ctx->ents;
-  desc.tab = ctx->tab;
-  bp.counters = ctx->counters;
 
   cudaGetLastError();   // launch errors are read below; drop any left by earlier calls
   CK(cudaEventRecord(ctx->ev[0], st));
-  CK(cudaMemsetAsync(ctx->cell_count, 0, (ncell + 1) * sizeof(int), st));
-  CK(cudaMemsetAsync(ctx->dstat, 0, 4 * sizeof(int), st));
-  CK(cudaMemsetAsync(ctx->counters, 0, C_NCOUNTERS * sizeof(unsigned long long), st));
-  k_put_tables<<<1, 256, 0, st>>>(tab, ctx->tab);
-  const int tb = 256;
-  const unsigned gb = (unsigned)((n + tb - 1) / tb);
-  k_bin<<<gb, tb, 0, st>>>(f->positions, bp, ctx->cell_count, ctx->atom_cell, ctx->atom_rank, ctx->atom_wrap,
-                           ctx->dstat);
-  const int nscan = (int)ncell + 1;
-  const int nblk = (nscan + 2 * SCAN_BLOCK - 1) / (2 * SCAN_BLOCK);
-  k_scan_block<<<nblk, SCAN_BLOCK, 0, st>>>(ctx->cell_count, ctx->cell_start, ctx->block_sums, nscan);
-  k_scan_sums<<<1, SCAN_BLOCK, 0, st>>>(ctx->block_sums, nblk, ctx->dstat + 2);
-  k_scan_add<<<(nscan + 255) / 256, 256, 0, st>>>(ctx->cell_start, ctx->block_sums, nscan);
-  k_scatter<<<gb, tb, 0, st>>>(f->positions, f64, n, ctx->atom_cell, ctx->atom_rank, ctx->atom_wrap,
-                               ctx->cell_start, ctx->sorted, ctx->sbin, ctx->wrapv);
+  int launches = launch_cells(f, bp, tab, ncell, B, st);
   const unsigned ga = (unsigned)((n + PTM_BLOCK - 1) / PTM_BLOCK);
   CK(cudaEventRecord(ctx->ev[1], st));
   if (!topological) {
-    const unsigned gk = (unsigned)((n + PTM_KNN_BLOCK - 1) / PTM_KNN_BLOCK);
-    if (f64) k_knn<true><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(), st>>>(desc);
-    else k_knn<false><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(), st>>>(desc);
+    launch_knn<PTM_KNN>(desc, B, st);
+    launches += 2;
   } else {
-    int *cnt = ctx->topo_list + ctx->cap_topo;
-    CK(cudaMemsetAsync(cnt, 0, sizeof(int), st));
+    launch_knn<PTM_TOPO_N>(desc, B, st);
+    int *cnt = ctx->dstat + 3;
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
     const int cap_side = (int)topo_side_cap(ctx->cap_topo);
@@ -283,6 +328,7 @@ static ptm_status enqueue_frame(ptm_context *ctx, const ptm_frame *f, const ptm_
       k_topo64<false><<<g64, PTM_BLOCK, topo64_smem_bytes(), st>>>(desc, ctx->nbr, ctx->topo_list, cnt,
                                                                    ctx->topo_side, cap_side);
     }
+    launches += 4;
   }
   CK(cudaEventRecord(ctx->ev[3], st));
   if (f64) k_hulls<true><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc);
@@ -298,8 +344,7 @@ static ptm_status enqueue_frame(ptm_context *ctx, const ptm_frame *f, const ptm_
   CK(cudaGetLastError());
   CK(cudaEventRecord(ctx->ev[2], st));
   ctx->last_stream = st;
-  // k_put_tables, k_bin, three scans, k_scatter, k_knn or k_topo + k_topo64, k_hulls, k_match
-  ctx->launches = topological ? 10 : 9;
+  ctx->launches = launches + 2;
   return PTM_OK;
 }
 
@@ -349,7 +394,8 @@ ptm_status ptm_create(const ptm_options *opt, ptm_context **out) {
     ctx->budget = (opt && opt->hbm_budget_bytes) ? opt->hbm_budget_bytes : fr / 2;
     // the per-atom kernels want every resident block's scratch in shared
     // memory: the largest shared-memory carveout of the unified L1
-    const int smem = (int)std::max(atom_smem_bytes(), std::max(topo_smem_bytes(), topo64_smem_bytes()));
+    const int smem = (int)std::max(std::max(atom_smem_bytes(), knn_smem_bytes(PTM_TOPO_N)),
+                                   std::max(topo_smem_bytes(), topo64_smem_bytes()));
     const void *fns[] = {(const void *)k_hulls<false>, (const void *)k_hulls<true>, (const void *)k_hulls_batch<false>,
                          (const void *)k_hulls_batch<true>, (const void *)k_match<false>, (const void *)k_match<true>,
                          (const void *)k_match<false, true>, (const void *)k_match<true, true>,
@@ -358,8 +404,10 @@ ptm_status ptm_create(const ptm_options *opt, ptm_context **out) {
                          (const void *)k_topo_batch<false>, (const void *)k_topo_batch<true>,
                          (const void *)k_topo64<false>, (const void *)k_topo64<true>,
                          (const void *)k_topo64_batch<false>, (const void *)k_topo64_batch<true>,
-                         (const void *)k_knn<false>, (const void *)k_knn<true>, (const void *)k_knn_batch<false>,
-                         (const void *)k_knn_batch<true>};
+                         (const void *)k_knn<false, PTM_KNN>, (const void *)k_knn<true, PTM_KNN>,
+                         (const void *)k_knn_batch<false, PTM_KNN>, (const void *)k_knn_batch<true, PTM_KNN>,
+                         (const void *)k_knn<false, PTM_TOPO_N>, (const void *)k_knn<true, PTM_TOPO_N>,
+                         (const void *)k_knn_batch<false, PTM_TOPO_N>, (const void *)k_knn_batch<true, PTM_TOPO_N>};
     for (const void *fn : fns) {
       if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
           (e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -378,6 +426,7 @@ ptm_status ptm_destroy(ptm_context *ctx) {
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
   cudaFree(ctx->sorted); cudaFree(ctx->sbin); cudaFree(ctx->wrapv);
+  cudaFree(ctx->hi); cudaFree(ctx->lo);
   cudaFree(ctx->atom_cell); cudaFree(ctx->atom_rank); cudaFree(ctx->atom_wrap);
   cudaFree(ctx->cell_count); cudaFree(ctx->cell_start); cudaFree(ctx->block_sums);
   cudaFree(ctx->dstat); cudaFree(ctx->counters); cudaFree(ctx->tab);
@@ -386,6 +435,7 @@ ptm_status ptm_destroy(ptm_context *ctx) {
   cudaFree(ctx->o_struct); cudaFree(ctx->o_alloy); cudaFree(ctx->o_rmsd); cudaFree(ctx->o_scale);
   cudaFree(ctx->o_quat); cudaFree(ctx->o_strain); cudaFree(ctx->o_corr); cudaFree(ctx->o_vm); cudaFree(ctx->o_rf);
   cudaFree(ctx->nbr); cudaFree(ctx->lam); cudaFree(ctx->ents);
+  cudaFree(ctx->nbr18);
   cudaFree(ctx->topo_list);
   cudaFree(ctx->topo_side);
   delete ctx;
@@ -508,15 +558,19 @@ struct ptm_batch {
   int64_t *d_atom_off = nullptr;
   int *d_dstat = nullptr;
   void *sorted = nullptr;
+  float4 *hi = nullptr, *lo = nullptr;
   int *sbin = nullptr, *wrapv = nullptr, *atom_cell = nullptr, *atom_rank = nullptr, *atom_wrap = nullptr;
-  int *cell_count = nullptr, *cell_start = nullptr, *block_sums = nullptr, *scan_total = nullptr;
+  int *cell_count = nullptr, *cell_start = nullptr, *block_sums = nullptr;
   unsigned long long *queue = nullptr, *counters = nullptr;
+  int *lists = nullptr;         // lengths of the lists below: k_knn_rest (NK = 14, 18), k_topo64
+  size_t zero_bytes = 0;        // counters, queue, lists, status words and cell counts, in one piece from counters on
   cudaEvent_t ev[5] = {};       // as ptm_context::ev
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   int nsm = 152;
   int topo = 0;                   // some frame takes the topological order
   int2 *nbr_buf = nullptr;        // per-frame segments of neighbour lists
+  int2 *nbr18_buf = nullptr;      // ... of the 18 nearest (some frame takes the topological order)
   uint64_t *lam_buf = nullptr;    // per-frame segments of the k_hulls -> k_match state
   uint32_t *ents_buf = nullptr;
   std::vector<FrameDesc> own;     // frames with a k_match launch of their own (PTM_MATCH_OWN_LAUNCH)
@@ -528,7 +582,7 @@ struct ptm_batch {
   cudaStream_t side[PTM_MATCH_SIDE_STREAMS] = {};   // the own k_match launches fork onto these
   cudaEvent_t fork = nullptr, join[PTM_MATCH_SIDE_STREAMS] = {};
   int nside = 0;
-  int *topo_list = nullptr;       // atoms for the FP64 pass; [ntotal] = their count
+  int *topo_list = nullptr;       // atoms for the FP64 pass
   TopoSide *topo_side = nullptr;  // what the FP32 pass keeps for the FP64 pass
   void *block = nullptr;          // the workspace (one allocation, or a pool block when served)
   bool owns_block = true;
@@ -562,6 +616,17 @@ static cudaError_t batch_side_init(ptm_batch *b) {
   return e;
 }
 
+// Neighbour lists (the NK nearest) of the batch's frames in that order; `rest` (a
+// dead buffer of the cell list) holds the undecided atoms.
+template <bool F64, int NK>
+static void launch_knn_batch(const ptm_batch *b, int *rest, int *cnt, cudaStream_t st) {
+  const unsigned gk = (unsigned)((b->ntotal + PTM_KNN_BLOCK - 1) / PTM_KNN_BLOCK);
+  k_knn_batch<F64, NK><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(NK), st>>>(b->d_descs, b->d_atom_off, b->nframes, b->ntotal,
+                                                                      rest, cnt);
+  k_knn_rest_batch<F64, NK><<<rest_grid(b->ntotal), PTM_KNN_BLOCK, 0, st>>>(b->d_descs, b->d_atom_off, b->nframes, rest,
+                                                                            cnt);
+}
+
 // Enqueue one pass over the whole batch: binning of every frame, one scan over
 // all cells, scatter, then the persistent classification launch.
 static ptm_status batch_enqueue(ptm_batch *b, cudaStream_t st) {
@@ -571,10 +636,7 @@ static ptm_status batch_enqueue(ptm_batch *b, cudaStream_t st) {
   CK(cudaStreamIsCapturing(st, &cap));
   const unsigned rec = cap == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault;
   CK(cudaEventRecordWithFlags(b->ev[0], st, rec));
-  CK(cudaMemsetAsync(b->cell_count, 0, (b->ncell + 1) * sizeof(int), st));
-  CK(cudaMemsetAsync(b->d_dstat, 0, (size_t)4 * b->nframes * sizeof(int), st));
-  CK(cudaMemsetAsync(b->counters, 0, C_NCOUNTERS * sizeof(unsigned long long), st));
-  CK(cudaMemsetAsync(b->queue, 0, 2 * sizeof(unsigned long long), st));
+  CK(cudaMemsetAsync(b->counters, 0, b->zero_bytes, st));
   const int tb = 256;
   const unsigned gb = (unsigned)((b->ntotal + tb - 1) / tb);
   k_bin_batch<<<gb, tb, 0, st>>>(b->d_bp, b->d_atom_off, b->nframes, b->ntotal, b->cell_count, b->atom_cell,
@@ -582,21 +644,20 @@ static ptm_status batch_enqueue(ptm_batch *b, cudaStream_t st) {
   const int nscan = (int)b->ncell + 1;
   const int nblk = (nscan + 2 * SCAN_BLOCK - 1) / (2 * SCAN_BLOCK);
   k_scan_block<<<nblk, SCAN_BLOCK, 0, st>>>(b->cell_count, b->cell_start, b->block_sums, nscan);
-  k_scan_sums<<<1, SCAN_BLOCK, 0, st>>>(b->block_sums, nblk, b->scan_total);
-  k_scan_add<<<(nscan + 255) / 256, 256, 0, st>>>(b->cell_start, b->block_sums, nscan);
+  if (nblk > 1) k_scan_add<<<nblk, SCAN_BLOCK, 0, st>>>(b->cell_start, b->block_sums, nscan);
   k_scatter_batch<<<gb, tb, 0, st>>>(b->d_bp, b->d_atom_off, b->nframes, b->ntotal, b->atom_cell, b->atom_rank,
-                                     b->atom_wrap, b->cell_start, b->sorted, b->sbin, b->wrapv);
+                                     b->atom_wrap, b->cell_start, b->sorted, b->hi, b->lo, b->sbin, b->wrapv);
+  b->launches = nblk > 1 ? 4 : 3;
   CK(cudaEventRecordWithFlags(b->ev[1], st, rec));
   if (b->topo != 2) {           // some frame takes the Euclidean order
-    const unsigned gk = (unsigned)((b->ntotal + PTM_KNN_BLOCK - 1) / PTM_KNN_BLOCK);
-    if (b->f64)
-      k_knn_batch<true><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(), st>>>(b->d_descs, b->d_atom_off, b->nframes, b->ntotal);
-    else
-      k_knn_batch<false><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(), st>>>(b->d_descs, b->d_atom_off, b->nframes, b->ntotal);
+    if (b->f64) launch_knn_batch<true, PTM_KNN>(b, b->atom_rank, b->lists, st);
+    else launch_knn_batch<false, PTM_KNN>(b, b->atom_rank, b->lists, st);
+    b->launches += 2;
   }
   if (b->topo) {
-    int *cnt = b->topo_list + b->ntotal;
-    CK(cudaMemsetAsync(cnt, 0, sizeof(int), st));
+    if (b->f64) launch_knn_batch<true, PTM_TOPO_N>(b, b->atom_cell, b->lists + 1, st);
+    else launch_knn_batch<false, PTM_TOPO_N>(b, b->atom_cell, b->lists + 1, st);
+    int *cnt = b->lists + 2;
     const unsigned gt = (unsigned)((b->ntotal + PTM_BLOCK - 1) / PTM_BLOCK);
     const int cap_side = (int)topo_side_cap((size_t)b->ntotal);
     const unsigned g64 = (unsigned)(PTM_TOPO64_BLOCKS_PER_SM * b->nsm);
@@ -611,6 +672,7 @@ static ptm_status batch_enqueue(ptm_batch *b, cudaStream_t st) {
       k_topo64_batch<false><<<g64, PTM_BLOCK, topo64_smem_bytes(), st>>>(b->d_descs, b->d_atom_off, b->nframes,
                                                                          b->topo_list, cnt, b->topo_side, cap_side);
     }
+    b->launches += 4;
   }
   CK(cudaEventRecordWithFlags(b->ev[3], st, rec));
   // persistent grids: two warps per block, each pulling its own tiles
@@ -658,7 +720,7 @@ static ptm_status batch_enqueue(ptm_batch *b, cudaStream_t st) {
       CK(cudaStreamWaitEvent(st, b->join[i], 0));
     }
   }
-  b->launches = 7 + (b->topo ? 2 : 0) + (int)b->own.size() + (b->nsmall ? 1 : 0) - (b->topo == 2 ? 1 : 0);
+  b->launches += 1 + (int)b->own.size() + (b->nsmall ? 1 : 0);
   CK(cudaGetLastError());
   CK(cudaEventRecordWithFlags(b->ev[2], st, rec));
   return PTM_OK;
@@ -714,16 +776,19 @@ static ptm_status batch_plan(int nframes, const ptm_frame *frames, double cell_f
   return PTM_OK;
 }
 
+// Device bytes that a pass over a batch zeroes first, in the order of batch_layout.
+static size_t batch_zero_bytes(int nframes, size_t ncell) {
+  return 8 * C_NCOUNTERS + 16 + 16 + 16 * (size_t)nframes + 4 * (ncell + 1);
+}
+
 // Device bytes of a batch's workspace (descriptors, sorted atoms, cell lists).
 static size_t batch_workspace_bytes(int nframes, int64_t ntotal, size_t ncell, int f64, int topo) {
-  const size_t n = (size_t)ntotal, rec = f64 ? sizeof(Atom64) : sizeof(float4);
+  const size_t n = (size_t)ntotal, rec = (f64 ? sizeof(Atom64) : sizeof(float4)) + 2 * sizeof(float4);
   const size_t nblk = (ncell + 1 + 2 * SCAN_BLOCK - 1) / (2 * SCAN_BLOCK) + 1;
   const size_t tb = sizeof(int2) * PTM_KNN * n + 28 * n + 3 * 256 +
-                    (topo ? 4 * (n + 1) + topo_side_bytes(n) + 2 * 256 : 0);
-  return (sizeof(FrameDesc) + sizeof(ShiftTables) + sizeof(BinParams) + 2 * sizeof(int64_t) + sizeof(int) + 16) *
-             nframes + 3 * 256 +
-         rec * n + 20 * n +
-         8 * (ncell + 1) + 4 * nblk + 4 + 16 + 8 * C_NCOUNTERS + 16 * 256 + tb;
+                    (topo ? sizeof(int2) * PTM_TOPO_N * n + 4 * n + topo_side_bytes(n) + 3 * 256 : 0);
+  return (sizeof(FrameDesc) + sizeof(ShiftTables) + sizeof(BinParams) + 2 * sizeof(int64_t) + sizeof(int)) * nframes +
+         batch_zero_bytes(nframes, ncell) + rec * n + 20 * n + 4 * (ncell + 1) + 4 * nblk + 18 * 256 + tb;
 }
 
 // Carve the batch workspace out of one device block (256-byte aligned pieces)
@@ -740,28 +805,37 @@ static void batch_layout(ptm_batch *b, unsigned char *base, BatchPlan &P, const 
   b->d_small_frames = (int *)take(sizeof(int) * nf);
   b->d_small_off = (int64_t *)take(sizeof(int64_t) * nf);
   b->d_atom_off = (int64_t *)take(sizeof(int64_t) * nf);
-  b->d_dstat = (int *)take(sizeof(int) * 4 * nf);
+  b->zero_bytes = batch_zero_bytes(nf, nc);
+  b->counters = (unsigned long long *)take(b->zero_bytes);
+  b->queue = b->counters + C_NCOUNTERS;
+  b->lists = (int *)(b->queue + 2);
+  b->d_dstat = b->lists + 4;
+  b->cell_count = b->d_dstat + 4 * nf;
   b->sorted = take((P.f64 ? sizeof(Atom64) : sizeof(float4)) * n);
+  b->hi = (float4 *)take(sizeof(float4) * n); b->lo = (float4 *)take(sizeof(float4) * n);
   b->sbin = (int *)take(4 * n); b->wrapv = (int *)take(4 * n); b->atom_cell = (int *)take(4 * n);
   b->atom_rank = (int *)take(4 * n); b->atom_wrap = (int *)take(4 * n);
-  b->cell_count = (int *)take(4 * (nc + 1)); b->cell_start = (int *)take(4 * (nc + 1));
-  b->block_sums = (int *)take(4 * nblk); b->scan_total = (int *)take(4);
-  b->queue = (unsigned long long *)take(16); b->counters = (unsigned long long *)take(8 * C_NCOUNTERS);
+  b->cell_start = (int *)take(4 * (nc + 1));
+  b->block_sums = (int *)take(4 * nblk);
   b->topo = P.topo;
   b->nbr_buf = (int2 *)take(sizeof(int2) * PTM_KNN * n);
   b->lam_buf = (uint64_t *)take(sizeof(uint64_t) * 3 * n);
   b->ents_buf = (uint32_t *)take(sizeof(uint32_t) * n);
   if (P.topo) {
-    b->topo_list = (int *)take(4 * (n + 1));
+    b->nbr18_buf = (int2 *)take(sizeof(int2) * PTM_TOPO_N * n);
+    b->topo_list = (int *)take(4 * n);
     b->topo_side = (TopoSide *)take(topo_side_bytes(n));
   }
   for (int f = 0; f < nf; f++) {
     // frame f's neighbour list: rows of n_f entries from slot 14 x (first slot)
     P.hd[f].nbr = b->nbr_buf + PTM_KNN * P.off[f];
+    P.hd[f].nbr18 = P.topo ? b->nbr18_buf + PTM_TOPO_N * P.off[f] : nullptr;
     P.hd[f].lam = b->lam_buf + 3 * P.off[f];
     P.hd[f].ents = b->ents_buf + P.off[f];
     P.hd[f].tab = b->d_tabs + f;
     P.hd[f].sorted = b->sorted;
+    P.hd[f].hi = b->hi;
+    P.hd[f].lo = b->lo;
     P.hd[f].sbin = b->sbin;
     P.hd[f].cell_start = b->cell_start + P.hb[f].cell_off;
     P.hd[f].wrapv = b->wrapv;
@@ -951,7 +1025,9 @@ constexpr size_t kNoallocScanBlocks = (kNoallocCells + 1 + 2 * SCAN_BLOCK - 1) /
 
 struct NoallocLayout {                  // byte offsets inside the static array
   static constexpr size_t sorted = 0;                                            // Atom64 records (float4 fits too)
-  static constexpr size_t sbin = sorted + sizeof(Atom64) * kNoallocAtoms;
+  static constexpr size_t hi = sorted + sizeof(Atom64) * kNoallocAtoms;
+  static constexpr size_t lo = hi + sizeof(float4) * kNoallocAtoms;
+  static constexpr size_t sbin = lo + sizeof(float4) * kNoallocAtoms;
   static constexpr size_t wrapv = sbin + sizeof(int) * kNoallocAtoms;
   static constexpr size_t atom_cell = wrapv + sizeof(int) * kNoallocAtoms;
   static constexpr size_t atom_rank = atom_cell + sizeof(int) * kNoallocAtoms;
@@ -1034,43 +1110,19 @@ extern "C" ptm_status ptm_classify_frame_noalloc(const ptm_frame *f, const ptm_o
   if (rs != PTM_OK) return rs;
   const int64_t n = f->n_atoms;
   const int f64 = desc.f64;
-  void *sorted = base + NoallocLayout::sorted;
-  int *sbin = (int *)(base + NoallocLayout::sbin), *wrapv = (int *)(base + NoallocLayout::wrapv);
-  int *atom_cell = (int *)(base + NoallocLayout::atom_cell), *atom_rank = (int *)(base + NoallocLayout::atom_rank);
-  int *atom_wrap = (int *)(base + NoallocLayout::atom_wrap);
-  int *cell_count = (int *)(base + NoallocLayout::cell_count), *cell_start = (int *)(base + NoallocLayout::cell_start);
-  int *block_sums = (int *)(base + NoallocLayout::block_sums), *dstat = (int *)(base + NoallocLayout::dstat);
-  unsigned long long *counters = (unsigned long long *)(base + NoallocLayout::counters);
-  desc.sorted = sorted; desc.sbin = sbin; desc.cell_start = cell_start; desc.wrapv = wrapv;
-  desc.nbr = (int2 *)(base + NoallocLayout::nbr);
-  desc.lam = (uint64_t *)(base + NoallocLayout::lam);
-  desc.ents = (uint32_t *)(base + NoallocLayout::ents);
-  desc.tab = (ShiftTables *)(base + NoallocLayout::tab);
+  auto at = [&](size_t off) { return (void *)(base + off); };
+  typedef NoallocLayout L;
+  const FrameBuffers B = {(int *)at(L::cell_count), (int *)at(L::cell_start), (int *)at(L::block_sums),
+                          (int *)at(L::atom_cell), (int *)at(L::atom_rank), (int *)at(L::atom_wrap),
+                          (int *)at(L::sbin), (int *)at(L::wrapv), at(L::sorted), (float4 *)at(L::hi),
+                          (float4 *)at(L::lo), (int *)at(L::dstat), (unsigned long long *)at(L::counters),
+                          (ShiftTables *)at(L::tab), (int2 *)at(L::nbr), nullptr, (uint64_t *)at(L::lam),
+                          (uint32_t *)at(L::ents)};
+  set_buffers(&desc, &bp, B);
   set_outputs(&desc, o);
-  desc.dstat = dstat;
-  desc.counters = counters;
-  bp.counters = counters;
   cudaGetLastError();   // launch errors are read below; drop any left by earlier calls
-  // the array keeps the previous call's contents: clear what must start at zero
-  if (cudaMemsetAsync(cell_count, 0, (ncell + 1) * sizeof(int), st) != cudaSuccess ||
-      cudaMemsetAsync(dstat, 0, 8 * sizeof(int), st) != cudaSuccess ||
-      cudaMemsetAsync(counters, 0, C_NCOUNTERS * sizeof(unsigned long long), st) != cudaSuccess) {
-    cudaGetLastError();
-    return PTM_ERR_CUDA;
-  }
-  k_put_tables<<<1, 256, 0, st>>>(tab, (ShiftTables *)desc.tab);
-  const int tb = 256;
-  const unsigned gb = (unsigned)((n + tb - 1) / tb);
-  k_bin<<<gb, tb, 0, st>>>(f->positions, bp, cell_count, atom_cell, atom_rank, atom_wrap, dstat);
-  const int nscan = (int)ncell + 1;
-  const int nblk = (nscan + 2 * SCAN_BLOCK - 1) / (2 * SCAN_BLOCK);
-  k_scan_block<<<nblk, SCAN_BLOCK, 0, st>>>(cell_count, cell_start, block_sums, nscan);
-  k_scan_sums<<<1, SCAN_BLOCK, 0, st>>>(block_sums, nblk, dstat + 2);
-  k_scan_add<<<(nscan + 255) / 256, 256, 0, st>>>(cell_start, block_sums, nscan);
-  k_scatter<<<gb, tb, 0, st>>>(f->positions, f64, n, atom_cell, atom_rank, atom_wrap, cell_start, sorted, sbin, wrapv);
-  const unsigned gk = (unsigned)((n + PTM_KNN_BLOCK - 1) / PTM_KNN_BLOCK);
-  if (f64) k_knn<true><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(), st>>>(desc);
-  else k_knn<false><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(), st>>>(desc);
+  launch_cells(f, bp, tab, ncell, B, st);
+  launch_knn<PTM_KNN>(desc, B, st);
   const unsigned ga = (unsigned)((n + PTM_BLOCK - 1) / PTM_BLOCK);
   if (f64) k_hulls<true><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc);
   else k_hulls<false><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc);

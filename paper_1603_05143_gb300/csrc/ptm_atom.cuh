@@ -45,6 +45,8 @@ struct FrameDesc {
   const int *sbin;             // frame-local cell of each sorted slot
   const int *cell_start;       // this frame's ncell + 1 offsets into sorted (global sorted indices)
   const int *wrapv;            // packed lattice wrap per sorted slot
+  const float4 *hi, *lo;       // cell-sorted positions wrapped into the cell as FP32 pairs hi + lo (lo.w: the
+                               // packed wrap), for float64 input and for frames with wrapped atoms
   const int8_t *species;       // by atom id, or NULL
   const void *positions;       // caller positions (by atom id)
   int64_t n;
@@ -54,7 +56,8 @@ struct FrameDesc {
   uint32_t mask;
   float rmsd_max;
   float min_cell_width;        // smallest perpendicular cell width (Angstrom)
-  float smax;                  // bound on the length of an image shift n.H with |n_r| <= 1 (periodic r)
+  float cell_vol;              // volume of a cell of the cell list
+  float tau;                   // absolute error of a component of a neighbour vector taken from hi + lo pairs
   double H[9];                 // rows = cell vectors
   const struct ShiftTables *tab;   // shifts of the images n in [-2,2]^3 (device memory)
   // outputs (by atom id)
@@ -70,6 +73,7 @@ struct FrameDesc {
   const int2 *nbr;             // neighbour list: [t][n] (sorted slot, image) of neighbour t of the
                                // atom at frame-local slot s - atom_offset (slot -1: none), written
                                // by k_knn (Euclidean order) or k_topo (topological order)
+  int2 *nbr18;                 // topological order: the 18 nearest, [18][n], read by k_topo
   int ordering;                // PTM_ORDER_EUCLIDEAN or PTM_ORDER_TOPOLOGICAL
   uint64_t *lam;               // k_hulls -> k_match: [3][n] Weinberg labelling of snapshot k = 6, 12, 14
   uint32_t *ents;              // [n] their table entries + 1, 10 bits each (0: no match)

@@ -7,419 +7,18 @@
 //   k_scan_*   exclusive scan of the cell counts
 //   k_scatter  atoms copied into cell order as float4 (x, y, z, id)
 //   k_knn      one thread per atom: its 14 nearest images, as a neighbour list
-//              (k_topo in ptm_topo.cuh instead for the topological order)
+//              (ptm_knn.cuh; for the topological order the 18 nearest, from
+//              which k_topo in ptm_topo.cuh makes the list)
+//   k_knn_rest one warp per atom that k_knn left undecided
 //   k_hulls    one thread per atom: hulls, Weinberg codes, template lookup
 //   k_match    one thread per atom: QCP, selection, outputs
 // The phases run as separate kernels so that the warps of an SM share one
 // phase of the method and its code (the instruction cache held none of the
 // fused per-atom program).
 #pragma once
-#include "ptm_atom.cuh"
-#include "../../include/ptm.h"
+#include "ptm_knn.cuh"
 
 namespace ptm {
-
-template <bool F64> struct RT { typedef float T; };
-template <> struct RT<true> { typedef double T; };
-
-__device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
-
-template <bool F64>
-__device__ __forceinline__ void load_atom(const FrameDesc &d, int j, typename RT<F64>::T &x,
-                                          typename RT<F64>::T &y, typename RT<F64>::T &z, int &id) {
-  if constexpr (F64) {
-    const Atom64 *a = (const Atom64 *)d.sorted + j;
-    double2 p = __ldg((const double2 *)a);
-    double2 q = __ldg((const double2 *)a + 1);
-    x = p.x; y = p.y; z = q.x; id = (int)__double_as_longlong(q.y);
-  } else {
-    float4 p = __ldg((const float4 *)d.sorted + j);
-    x = p.x; y = p.y; z = p.z; id = __float_as_int(p.w);
-  }
-}
-
-// Contract shift of image (a, b, c) in the input precision.
-template <bool F64>
-__device__ __forceinline__ void contract_shift(const FrameDesc &d, int a, int b, int c, typename RT<F64>::T &sx,
-                                               typename RT<F64>::T &sy, typename RT<F64>::T &sz) {
-  if constexpr (F64) {
-    shift_f64(d, a, b, c, sx, sy, sz);
-  } else {
-    float lx, ly, lz;
-    shift_f32(d, a, b, c, sx, sy, sz, lx, ly, lz);
-  }
-}
-
-// The distance contract (Sec. 3 orders neighbours by distance; the paper fixes
-// no precision, so the order is that of the distances between the given points
-// in FP64): dr = (x_j - x_i) + shift, d2 = (dr_x^2 + dr_y^2) + dr_z^2, one
-// rounded IEEE operation at a time, no fused multiply-add, float32 positions
-// widened exactly.  The kernels first run the same sequence in the input
-// precision (FP32 for float32 input) and decide in FP64 only where the FP32
-// values cannot order two candidates (knn_err).
-__device__ __forceinline__ float contract_dr(float xj, float xi, float s) { return __fadd_rn(__fsub_rn(xj, xi), s); }
-__device__ __forceinline__ double contract_dr(double xj, double xi, double s) { return __dadd_rn(__dsub_rn(xj, xi), s); }
-__device__ __forceinline__ float contract_d2(float a, float b, float c) {
-  return __fadd_rn(__fadd_rn(__fmul_rn(a, a), __fmul_rn(b, b)), __fmul_rn(c, c));
-}
-__device__ __forceinline__ double contract_d2(double a, double b, double c) {
-  return __dadd_rn(__dadd_rn(__dmul_rn(a, a), __dmul_rn(b, b)), __dmul_rn(c, c));
-}
-
-// FP64 squared distance of the image (a0, a1, a2) of an atom at (xj, yj, zj):
-// the ordering key.  For float64 input it equals the input-precision value.
-template <typename T>
-__device__ __forceinline__ double key64(const FrameDesc &d, T xj, T yj, T zj, T xi, T yi, T zi, int a0, int a1,
-                                        int a2) {
-  if constexpr (sizeof(T) == 4) {
-    // image 0 with every FP32 difference exact (Sterbenz: |x_j - x_i| <=
-    // min(|x_i|, |x_j|)): the FP64 differences are these FP32 values and the
-    // zero shift adds nothing, so only the squares and sums run in FP64
-    if ((a0 | a1 | a2) == 0) {
-      const float px = __fsub_rn(xj, xi), py = __fsub_rn(yj, yi), pz = __fsub_rn(zj, zi);
-      if (fabsf(px) <= fminf(fabsf(xi), fabsf(xj)) && fabsf(py) <= fminf(fabsf(yi), fabsf(yj)) &&
-          fabsf(pz) <= fminf(fabsf(zi), fabsf(zj)))
-        return contract_d2((double)px, (double)py, (double)pz);
-    }
-  }
-  double sx, sy, sz;
-  shift_f64(d, a0, a1, a2, sx, sy, sz);
-  return contract_d2(contract_dr((double)xj, (double)xi, sx), contract_dr((double)yj, (double)yi, sy),
-                     contract_dr((double)zj, (double)zi, sz));
-}
-
-// Bound on |d2_32 - d2_64| for an FP32 contract value v whose image shift has
-// length at most S (u = 2^-24).  Each component of the FP32 vector is within
-// 2u (|dr_c| + |s_c|) of the FP64 one (the difference, the shift's rounding to
-// FP32 and the sum each round once); squaring and the two sums add 3u v.  So
-// |d2_32 - d2_64| <= u (7 v + 4 |dr| |s|) + 8 u^2 (v + S^2); the constants
-// below leave room for |dr| estimated from v and for rounding in this bound.
-__device__ __forceinline__ float knn_err(float v, float S) {
-  const float u = 5.9604645e-8f;
-  return u * (8.5f * v + 4.5f * sqrtf(v) * S + 9.f * u * S * S);
-}
-
-// Key order (FP64 d2, atom id, image).  Keys are non-negative and not NaN, so
-// their bit patterns order as unsigned integers: the comparisons stay off the
-// FP64 pipe.
-__device__ __forceinline__ bool key_less64(double da, int ia, int ma, double db, int ib, int mb) {
-  const unsigned long long ua = (unsigned long long)__double_as_longlong(da);
-  const unsigned long long ub = (unsigned long long)__double_as_longlong(db);
-  return ua < ub || (ua == ub && (ia < ib || (ia == ib && ma < mb)));
-}
-
-// ----------------------------------------------------------------- kNN
-// Visit every (atom, image) in the (2R+1)^3 cells around cell (bx, by, bz):
-// visit(j, d2, idj, a0, a1, a2, xj, yj, zj, sx, sy, sz) with d2 by the contract
-// in the input precision, (a0, a1, a2) the image and (sx, sy, sz) its shift.
-// The cells bz - R .. bz + R of a column are consecutive in the sorted order
-// unless the range wraps, and are then scanned as one range of atoms.
-template <bool F64, typename V>
-__device__ __forceinline__ void scan_cells(const FrameDesc &d, int s, typename RT<F64>::T xi,
-                                           typename RT<F64>::T yi, typename RT<F64>::T zi, int bx, int by, int bz,
-                                           int wix, int wiy, int wiz, bool wrapped, int R, V &&visit) {
-  typedef typename RT<F64>::T T;
-  const int nbx = d.nb[0], nby = d.nb[1], nbz = d.nb[2];
-  for (int ix = 0; ix <= 2 * R; ix++) {
-    const int dx = ix <= R ? ix : R - ix;                // 0, 1 .. R, -1 .. -R: the centre first
-    int cx = bx + dx, mx = 0;
-    if (d.pbc[0]) { mx = floordiv(cx, nbx); cx -= mx * nbx; } else if (cx < 0 || cx >= nbx) continue;
-    for (int iy = 0; iy <= 2 * R; iy++) {
-      const int dy = iy <= R ? iy : R - iy;
-      int cy = by + dy, my = 0;
-      if (d.pbc[1]) { my = floordiv(cy, nby); cy -= my * nby; } else if (cy < 0 || cy >= nby) continue;
-      int z0 = bz - R, z1 = bz + R;
-      if (!d.pbc[2]) { z0 = max(z0, 0); z1 = min(z1, nbz - 1); }
-      const bool column = z0 >= 0 && z1 < nbz;             // no wrap: one range, image mz = 0
-      const int cbase = (cx * nby + cy) * nbz;
-      for (int r = 0; r < (column ? 1 : 2 * R + 1); r++) {
-        int ca = cbase + z0, cb = cbase + z1, mz = 0;     // cells ca .. cb
-        if (!column) {
-          int cz = bz - R + r;
-          mz = floordiv(cz, nbz);                          // periodic z (else column)
-          cz -= mz * nbz;
-          ca = cb = cbase + cz;
-        }
-        const int j0 = __ldg(d.cell_start + ca), j1 = __ldg(d.cell_start + cb + 1);
-        if (j0 == j1) continue;
-        const int n0 = mx + wix, n1 = my + wiy, n2 = mz + wiz;
-        T sx, sy, sz;
-        contract_shift<F64>(d, n0, n1, n2, sx, sy, sz);
-#pragma unroll 2
-        for (int j = j0; j < j1; j++) {
-          T xj, yj, zj;
-          int idj;
-          load_atom<F64>(d, j, xj, yj, zj, idj);
-          int a0 = n0, a1 = n1, a2 = n2;
-          if (wrapped) {
-            int w0, w1, w2;
-            img_unpack(__ldg(d.wrapv + j), w0, w1, w2);
-            a0 -= w0; a1 -= w1; a2 -= w2;
-            contract_shift<F64>(d, a0, a1, a2, sx, sy, sz);
-          }
-          if (j == s && a0 == 0 && a1 == 0 && a2 == 0) continue;
-          const T ex = contract_dr(xj, xi, sx), ey = contract_dr(yj, yi, sy), ez = contract_dr(zj, zi, sz);
-          visit(j, contract_d2(ex, ey, ez), idj, a0, a1, a2, xj, yj, zj, sx, sy, sz);
-        }
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ bool search_complete(const FrameDesc &d, int R, float d2_last) {
-  const float rg = (float)R * d.min_cell_width - __int_as_float(d.dstat[1]);
-  return rg > 0.f && d2_last < rg * rg * (1.f - 1e-3f);
-}
-
-// General kNN: the NK nearest images of atom s by the full key (FP64 d2, atom
-// id, image), R growing until the NK-th distance lies inside the radius the
-// scanned cells are guaranteed to cover.  For float32 input a candidate whose
-// FP32 distance, less its error bound, exceeds the current NK-th key cannot
-// enter and skips the FP64 evaluation.  Returns the neighbour count (NK, fewer
-// only for a small fully non-periodic system) or -1.
-template <bool F64, int NK = PTM_KNN>
-__device__ __noinline__ int knn(const FrameDesc &d, int s, typename RT<F64>::T xi, typename RT<F64>::T yi,
-                                typename RT<F64>::T zi, int bx, int by, int bz, int wix, int wiy, int wiz,
-                                bool wrapped, double (&Ld2)[NK], int (&Lid)[NK], int (&Ljs)[NK], int (&Limg)[NK]) {
-  typedef typename RT<F64>::T T;
-  for (int R = 1; R <= PTM_RMAX; R++) {
-    float last32 = INFINITY;                           // the NK-th key rounded up to FP32
-#pragma unroll
-    for (int t = 0; t < NK; t++) { Ld2[t] = INFINITY; Lid[t] = 0x7fffffff; Ljs[t] = -1; Limg[t] = 0x7fffffff; }
-    scan_cells<F64>(d, s, xi, yi, zi, bx, by, bz, wix, wiy, wiz, wrapped, R,
-                    [&](int j, T d2, int idj, int a0, int a1, int a2, T xj, T yj, T zj, T sx, T sy, T sz) {
-      double key;
-      if constexpr (F64) {
-        key = d2;
-      } else {
-        const float S = sqrtf(sx * sx + sy * sy + sz * sz) * 1.0001f;
-        if (d2 - 1.25f * knn_err(d2, S) > last32) return;
-        key = key64(d, xj, yj, zj, xi, yi, zi, a0, a1, a2);
-      }
-      if ((unsigned long long)__double_as_longlong(key) > (unsigned long long)__double_as_longlong(Ld2[NK - 1])) return;
-      const int img = img_pack(a0, a1, a2);
-      if (!key_less64(key, idj, img, Ld2[NK - 1], Lid[NK - 1], Limg[NK - 1])) return;
-      // insertion into the sorted list (all indices static: stays in registers)
-      bool above = true;
-#pragma unroll
-      for (int t = NK - 1; t >= 1; t--) {
-        bool lt = key_less64(key, idj, img, Ld2[t - 1], Lid[t - 1], Limg[t - 1]);
-        if (lt) { Ld2[t] = Ld2[t - 1]; Lid[t] = Lid[t - 1]; Ljs[t] = Ljs[t - 1]; Limg[t] = Limg[t - 1]; }
-        else if (above) { Ld2[t] = key; Lid[t] = idj; Ljs[t] = j; Limg[t] = img; }
-        above = lt;
-      }
-      if (above) { Ld2[0] = key; Lid[0] = idj; Ljs[0] = j; Limg[0] = img; }
-      if constexpr (!F64) last32 = __double2float_ru(Ld2[NK - 1]);
-    });
-    if (search_complete(d, R, __double2float_ru(Ld2[NK - 1]))) {
-      if (R > 1) count(d, C_KNN_WIDE);
-      return NK;
-    }
-    if (!d.pbc[0] && !d.pbc[1] && !d.pbc[2] && R >= max(d.nb[0], max(d.nb[1], d.nb[2]))) {
-      int cnt = 0;
-#pragma unroll
-      for (int t = 0; t < NK; t++) cnt += Ljs[t] >= 0;
-      return cnt;
-    }
-  }
-  count(d, C_KNN_FAIL);
-  return -1;
-}
-
-// Fast kNN for the common case (27 cells suffice).  Pass 1 keeps the NK + 1
-// smallest distances in the input precision with a min/max network.  Slots t
-// and t + 1 are "close" when those values could order their candidates
-// differently from FP64 (float32 input: the gap is within twice knn_err;
-// float64 input: equal values); close slots form runs, and the last run also
-// takes every candidate beyond slot NK - 1 within the error band.  Pass 2
-// rescans and drops each candidate into its rank slot; a run's candidates are
-// placed by insertion on the full key (FP64 d2, atom id, image), keeping the
-// smallest keys when the run crosses the last slot, so the result is the
-// general kNN's order.  Slots are written through `rows`: put(r, j, img) and,
-// inside runs, set(r, j, img, id, key) / j(r) / img(r) / id(r) / key(r)
-// (j = -1: empty).  `close_runs` receives the run mask (0: every rank decided
-// in the input precision).  Returns false when the general kNN must decide.
-template <bool F64, int NK, typename Rows>
-__device__ __forceinline__ bool knn_fast_n(const FrameDesc &d, int s, typename RT<F64>::T xi,
-                                           typename RT<F64>::T yi, typename RT<F64>::T zi, int bx, int by, int bz,
-                                           const Rows &rows, uint32_t &close_runs) {
-  typedef typename RT<F64>::T T;
-  // float32 input, 14 neighbours: the network also carries each value's
-  // candidate as (sorted slot << 5 | image index), so that an atom whose ranks
-  // are all decided needs no second scan (slots below 2^27)
-  constexpr bool CARRY = !F64 && NK == PTM_KNN;
-  T L[NK + 1];
-  uint32_t C[CARRY ? NK + 1 : 1];
-#pragma unroll
-  for (int t = 0; t <= NK; t++) L[t] = (T)INFINITY;
-  if constexpr (CARRY) {
-#pragma unroll
-    for (int t = 0; t <= NK; t++) C[t] = 0u;
-  }
-  scan_cells<F64>(d, s, xi, yi, zi, bx, by, bz, 0, 0, 0, false, 1,
-                  [&](int j, T d2, int, int a0, int a1, int a2, T, T, T, T, T, T) {
-    if (!(d2 < L[NK])) return;
-    T x = d2;
-    if constexpr (CARRY) {
-      uint32_t xc = ((uint32_t)j << 5) | (uint32_t)((a0 + 1) * 9 + (a1 + 1) * 3 + (a2 + 1));
-#pragma unroll
-      for (int t = 0; t <= NK; t++) {
-        const bool sw = x < L[t];
-        const T lo = sw ? x : L[t];
-        const uint32_t lc = sw ? xc : C[t];
-        x = sw ? L[t] : x;
-        xc = sw ? C[t] : xc;
-        L[t] = lo;
-        C[t] = lc;
-      }
-    } else {
-#pragma unroll
-      for (int t = 0; t <= NK; t++) { const T lo = fmin(L[t], x); x = fmax(L[t], x); L[t] = lo; }
-    }
-  });
-  if (!(L[NK] < (T)INFINITY)) return false;
-  uint32_t close = 0;                                // bit t: slots t and t + 1 in one run
-  T limit = L[NK - 1];                               // pass 2 admits d2 <= limit
-  if constexpr (F64) {
-#pragma unroll
-    for (int t = 0; t < NK; t++) close |= (uint32_t)(L[t] == L[t + 1]) << t;
-  } else {
-    // image shifts occur only when the 27 cells wrap around a periodic side
-    const bool shifted = (d.pbc[0] && (bx == 0 || bx >= d.nb[0] - 1)) ||
-                         (d.pbc[1] && (by == 0 || by >= d.nb[1] - 1)) ||
-                         (d.pbc[2] && (bz == 0 || bz >= d.nb[2] - 1));
-    // one band for every gap: twice the bound at the largest kept value
-    // (knn_err grows with v), without the shift term for an unshifted atom
-    const float vmax = 1.01f * L[NK];
-    const float band = shifted ? 2.f * knn_err(vmax, d.smax) : 2.f * 8.5f * 5.9604645e-8f * vmax;
-#pragma unroll
-    for (int t = 0; t < NK; t++) close |= (uint32_t)(L[t + 1] - L[t] <= band) << t;
-    if (close >> (NK - 1) & 1) limit = L[NK - 1] + band;
-  }
-  if (!search_complete(d, 1, (float)limit)) return false;
-  close_runs = close;
-  if constexpr (CARRY) {
-    if (!close && d.atom_offset + d.n <= (1ll << 27)) {    // every rank decided, the candidates at hand
-#pragma unroll
-      for (int t = 0; t < NK; t++) {
-        const int k = (int)(C[t] & 31u);
-        rows.put(t, (int)(C[t] >> 5), img_pack(k / 9 - 1, (k / 3) % 3 - 1, k % 3 - 1));
-      }
-      return true;
-    }
-  }
-  if (!close) {                                      // every rank decided: distance order is key order
-    scan_cells<F64>(d, s, xi, yi, zi, bx, by, bz, 0, 0, 0, false, 1,
-                    [&](int j, T d2, int, int a0, int a1, int a2, T, T, T, T, T, T) {
-      if (!(d2 <= limit)) return;
-      int rank = 0;
-#pragma unroll
-      for (int t = 0; t < NK - 1; t++) rank += L[t] < d2;
-      rows.put(rank, j, img_pack(a0, a1, a2));
-    });
-    return true;
-  }
-  const bool crossing = (close >> (NK - 1)) & 1;
-  for (int r = 0; r < NK; r++) rows.set(r, -1, 0, 0, 0.0);
-  scan_cells<F64>(d, s, xi, yi, zi, bx, by, bz, 0, 0, 0, false, 1,
-                  [&](int j, T d2, int idj, int a0, int a1, int a2, T xj, T yj, T zj, T, T, T) {
-    if (!(d2 <= limit)) return;
-    int r0 = 0;                                      // first slot holding this value (NK - 1 beyond)
-#pragma unroll
-    for (int t = 0; t < NK - 1; t++) r0 += L[t] < d2;
-    const uint32_t below = ~close & ((1u << r0) - 1u);
-    const int rs = below ? 32 - __clz(below) : 0;    // the run: slots rs .. hi - 1
-    const int hi = min(r0 + __ffs(~(close >> r0)), NK);
-    const int img = img_pack(a0, a1, a2);
-    if (hi - rs == 1 && !(hi == NK && crossing)) { rows.put(rs, j, img); return; }
-    double key;
-    if constexpr (F64) key = d2;
-    else key = key64(d, xj, yj, zj, xi, yi, zi, a0, a1, a2);
-    int r = rs;                                      // insertion point by (key, id, image)
-    while (r < hi && rows.j(r) >= 0 && key_less64(rows.key(r), rows.id(r), rows.img(r), key, idj, img)) r++;
-    if (r == hi) return;                             // beyond the NK nearest
-    int e = r;                                       // first empty slot, or the run's last
-    while (e < hi - 1 && rows.j(e) >= 0) e++;
-    for (int q = e; q > r; q--) rows.set(q, rows.j(q - 1), rows.img(q - 1), rows.id(q - 1), rows.key(q - 1));
-    rows.set(r, j, img, idj, key);
-  });
-  return true;
-}
-
-// kNN slots in per-thread shared-memory rows ([row][thread], stride B): row r
-// the sorted slot, row NK + r the packed image; while a run is ordered, row
-// 2 NK + r the atom id and rows 3 NK + 2 r, 3 NK + 2 r + 1 the FP64 key.
-template <int NK, int B>
-struct SmemKnnRows {
-  int *base;
-  int t;
-  static constexpr int kRows = 5 * NK;
-  __device__ __forceinline__ int &row(int k) const { return base[k * B + t]; }
-  __device__ __forceinline__ void put(int r, int j, int img) const {
-    row(r) = j;
-    row(NK + r) = img;
-  }
-  __device__ __forceinline__ void set(int r, int j, int img, int id, double key) const {
-    put(r, j, img);
-    row(2 * NK + r) = id;
-    row(3 * NK + 2 * r) = __double2hiint(key);
-    row(3 * NK + 2 * r + 1) = __double2loint(key);
-  }
-  __device__ __forceinline__ int j(int r) const { return row(r); }
-  __device__ __forceinline__ int img(int r) const { return row(NK + r); }
-  __device__ __forceinline__ int id(int r) const { return row(2 * NK + r); }
-  __device__ __forceinline__ double key(int r) const {
-    return __hiloint2double(row(3 * NK + 2 * r), row(3 * NK + 2 * r + 1));
-  }
-};
-
-#define PTM_KNN_BLOCK 128
-// 6 blocks of 128 threads per SM: the shared-memory rows (280 B per thread) and
-// at most 85 registers per thread fit
-#define PTM_KNN_BLOCKS_PER_SM 6
-// The batch form (frame lookup per slot, descriptors in global memory) spills
-// at 85 registers; at 5 blocks per SM it keeps 96 (batch of 256 frames: 30.4 ->
-// 28.5 ms, while the single-frame kernel is faster at 6: 0.824 against 0.864 ms)
-#define PTM_KNN_BATCH_BLOCKS_PER_SM 5
-typedef SmemKnnRows<PTM_KNN, PTM_KNN_BLOCK> KnnRows;
-constexpr size_t knn_smem_bytes() { return (size_t)PTM_KNN_BLOCK * KnnRows::kRows * 4; }
-
-// The 14 nearest images of the atom at sorted slot s (Sec. 3, Table 1), written
-// to its neighbour list: fast search when 27 cells suffice, else the general
-// one.  A search that fails leaves an empty list (the atom stays unmatched).
-template <bool F64>
-__device__ __forceinline__ void knn_atom(const FrameDesc &d, int s, int *smem_rows) {
-  typedef typename RT<F64>::T T;
-  T xi, yi, zi;
-  int idi;
-  load_atom<F64>(d, s, xi, yi, zi, idi);
-  const int b = __ldg(d.sbin + s);
-  const int bz = b % d.nb[2], byx = b / d.nb[2];
-  const int by = byx % d.nb[1], bx = byx / d.nb[1];
-  const bool wrapped = d.dstat[0] != 0;
-  const KnnRows rows{smem_rows, (int)threadIdx.x};
-  int2 *out = const_cast<int2 *>(d.nbr) + (s - d.atom_offset);
-  if (__ldg(d.wrapv + s) == PTM_EXCLUDED) {           // excluded by the binning: no neighbours
-#pragma unroll
-    for (int t = 0; t < PTM_KNN; t++) out[(int64_t)t * d.n] = make_int2(-1, 0);
-    return;
-  }
-  uint32_t close = 0;
-  if (!wrapped && knn_fast_n<F64, PTM_KNN>(d, s, xi, yi, zi, bx, by, bz, rows, close)) {
-    if (!F64 && close) count(d, C_KNN64);
-#pragma unroll
-    for (int t = 0; t < PTM_KNN; t++) out[(int64_t)t * d.n] = make_int2(rows.j(t), rows.img(t));
-    return;
-  }
-  int wix = 0, wiy = 0, wiz = 0;
-  if (wrapped) img_unpack(__ldg(d.wrapv + s), wix, wiy, wiz);
-  double Ld2[PTM_KNN];
-  int Lid[PTM_KNN], Ljs[PTM_KNN], Limg[PTM_KNN];
-  const int cnt = knn<F64>(d, s, xi, yi, zi, bx, by, bz, wix, wiy, wiz, wrapped, Ld2, Lid, Ljs, Limg);
-  if (!F64) count(d, C_KNN64);
-#pragma unroll
-  for (int t = 0; t < PTM_KNN; t++) out[(int64_t)t * d.n] = t < cnt ? make_int2(Ljs[t], Limg[t]) : make_int2(-1, 0);
-}
 
 // ---------------------------------------------------------- per-atom state
 // Per-atom selection state.  Plain scalars (no arrays) so that it stays in
@@ -1252,9 +851,18 @@ __device__ void match_atom(const FrameDesc &d, int s, const Scratch &sm, const f
 }
 
 // ------------------------------------------------------------------ kernels
-// Copies a frame's shift tables, passed by value, into device memory: stream
-// ordered, so back-to-back asynchronous calls never share a host staging buffer.
-__global__ void k_put_tables(const __grid_constant__ ShiftTables t, ShiftTables *out) {
+// First kernel of a single-frame call: zeroes the cell counts, status words and
+// counters (one launch instead of three memsets) and copies the frame's shift
+// tables, passed by value, into device memory: stream ordered, so back-to-back
+// asynchronous calls never share a host staging buffer.
+#define PTM_STATUS_WORDS 4       // any wrap, overshoot, undecided atoms (k_knn), listed atoms (k_topo)
+__global__ void k_begin(const __grid_constant__ ShiftTables t, ShiftTables *out, int *cell_count, int ncount, int *dstat,
+                        unsigned long long *counters) {
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int i = i0; i < ncount; i += gridDim.x * blockDim.x) cell_count[i] = 0;
+  if (blockIdx.x) return;
+  if (threadIdx.x < PTM_STATUS_WORDS) dstat[threadIdx.x] = 0;
+  if (threadIdx.x < C_NCOUNTERS) counters[threadIdx.x] = 0;
   const float *src = reinterpret_cast<const float *>(&t);
   float *dst = reinterpret_cast<float *>(out);
   for (int i = threadIdx.x; i < (int)(sizeof(ShiftTables) / 4); i += blockDim.x) dst[i] = src[i];
@@ -1263,6 +871,7 @@ __global__ void k_put_tables(const __grid_constant__ ShiftTables t, ShiftTables 
 struct BinParams {
   float Hinv[9];     // fractional = x . Hinv
   float W[3];        // perpendicular cell widths
+  double H[9];       // rows = cell vectors
   int nb[3];
   int pbc[3];
   int64_t n;
@@ -1334,76 +943,98 @@ __global__ void k_bin(const void *pos, BinParams p, int *cell_count, int *atom_c
 }
 
 #define SCAN_BLOCK 1024
-// exclusive scan, level 1: per-block scan of 2 elements per thread
-__global__ void k_scan_block(const int *in, int *out, int *block_sums, int n) {
-  __shared__ int sh[SCAN_BLOCK * 2];
-  int base = blockIdx.x * SCAN_BLOCK * 2;
-  int t = threadIdx.x;
-  int a = base + 2 * t, b = a + 1;
-  int va = a < n ? in[a] : 0, vb = b < n ? in[b] : 0;
-  sh[2 * t] = va;
-  sh[2 * t + 1] = va + vb;
-  __syncthreads();
-  // Hillis-Steele over the pair sums
-  int v = sh[2 * t + 1];
-  for (int off = 1; off < SCAN_BLOCK; off <<= 1) {
-    int add = t >= off ? sh[2 * (t - off) + 1] : 0;
-    __syncthreads();
-    v += add;
-    sh[2 * t + 1] = v;
-    __syncthreads();
+// Inclusive scan of one value per thread over a block; sh holds a word per warp.
+__device__ __forceinline__ int block_scan(int v, int *sh) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += x;
   }
-  int excl = v - (va + vb);
+  if (lane == 31) sh[w] = v;
+  __syncthreads();
+  if (w == 0) {
+    int x = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    sh[lane] = x;
+  }
+  __syncthreads();
+  return v + (w ? sh[w - 1] : 0);
+}
+
+// Exclusive scan, level 1: per-block scan of 2 elements per thread.
+__global__ void k_scan_block(const int *in, int *out, int *block_sums, int n) {
+  __shared__ int sh[32];
+  const int a = blockIdx.x * SCAN_BLOCK * 2 + 2 * threadIdx.x, b = a + 1;
+  const int va = a < n ? in[a] : 0, vb = b < n ? in[b] : 0;
+  const int v = block_scan(va + vb, sh), excl = v - (va + vb);
   if (a < n) out[a] = excl;
   if (b < n) out[b] = excl + va;
-  if (t == SCAN_BLOCK - 1) block_sums[blockIdx.x] = v;
+  if (threadIdx.x == SCAN_BLOCK - 1) block_sums[blockIdx.x] = v;
 }
 
-// level 2: one block scans the block sums serially in chunks
-__global__ void k_scan_sums(int *block_sums, int nblocks, int *total_out) {
-  __shared__ int sh[SCAN_BLOCK];
-  int carry = 0;
-  for (int base = 0; base < nblocks; base += SCAN_BLOCK) {
-    int t = threadIdx.x, i = base + t;
-    int v = i < nblocks ? block_sums[i] : 0;
-    sh[t] = v;
-    __syncthreads();
-    for (int off = 1; off < SCAN_BLOCK; off <<= 1) {
-      int add = t >= off ? sh[t - off] : 0;
-      __syncthreads();
-      sh[t] += add;
-      __syncthreads();
-    }
-    if (i < nblocks) block_sums[i] = carry + sh[t] - v;
-    int tot = sh[SCAN_BLOCK - 1];
-    __syncthreads();
-    carry += tot;
-  }
-  if (threadIdx.x == 0) *total_out = carry;
-}
-
+// Level 2: every block sums the totals of the blocks before it (one per 2,048
+// cells, a few thousand in all for 33 M atoms) and adds them to its elements; not
+// launched for a single block.
 __global__ void k_scan_add(int *out, const int *block_sums, int n) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] += block_sums[i / (SCAN_BLOCK * 2)];
+  __shared__ int sh[32];
+  __shared__ int before;
+  int sum = 0;
+  for (int i = threadIdx.x; i < (int)blockIdx.x; i += SCAN_BLOCK) sum += block_sums[i];
+  const int v = block_scan(sum, sh);
+  if (threadIdx.x == SCAN_BLOCK - 1) before = v;
+  __syncthreads();
+  const int a = blockIdx.x * SCAN_BLOCK * 2 + 2 * threadIdx.x, b = a + 1;
+  if (a < n) out[a] += before;
+  if (b < n) out[b] += before;
 }
 
-__global__ void k_scatter(const void *pos, int f64, int64_t n, const int *atom_cell, const int *atom_rank,
-                          const int *atom_wrap, const int *cell_start, void *sorted, int *sbin, int *wrapv) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int c = atom_cell[i];
-  int slot = cell_start[c] + atom_rank[i];
-  if (f64) {
-    const double *q = (const double *)pos + 3 * i;
+// Copy of atom li of frame p into its cell-sorted slot.  Float64 input, and a
+// float32 frame in which some atom lies outside the cell, also get the position
+// wrapped into the cell as an FP32 pair: the neighbour search then works in FP32
+// and on the 27 images, whatever the input.  An excluded atom's pair is NaN.
+__device__ __forceinline__ void scatter_atom(const BinParams &p, const void *pos, int64_t li, int wrap, bool wrapped,
+                                             int slot, void *sorted, float4 *hi, float4 *lo) {
+  double x, y, z;
+  if (p.f64) {
+    const double *q = (const double *)pos + 3 * li;
     Atom64 a;
-    a.x = q[0]; a.y = q[1]; a.z = q[2]; a.id = i;
+    x = a.x = q[0]; y = a.y = q[1]; z = a.z = q[2]; a.id = li;
     ((Atom64 *)sorted)[slot] = a;
   } else {
-    const float *q = (const float *)pos + 3 * i;
-    ((float4 *)sorted)[slot] = make_float4(q[0], q[1], q[2], __int_as_float((int)i));
+    const float *q = (const float *)pos + 3 * li;
+    const float4 a = make_float4(q[0], q[1], q[2], __int_as_float((int)li));
+    ((float4 *)sorted)[slot] = a;
+    if (!wrapped) return;
+    x = a.x; y = a.y; z = a.z;
   }
+  if (wrap != img_pack(0, 0, 0)) {
+    int a, b, c;
+    img_unpack(wrap, a, b, c);
+    x -= a * p.H[0] + b * p.H[3] + c * p.H[6];
+    y -= a * p.H[1] + b * p.H[4] + c * p.H[7];
+    z -= a * p.H[2] + b * p.H[5] + c * p.H[8];
+    if (wrap == PTM_EXCLUDED) x = y = z = NAN;
+  }
+  const float hx = (float)x, hy = (float)y, hz = (float)z;
+  hi[slot] = make_float4(hx, hy, hz, 0.f);
+  lo[slot] = make_float4((float)(x - hx), (float)(y - hy), (float)(z - hz), __int_as_float(wrap));
+}
+
+__global__ void k_scatter(const void *pos, BinParams p, const int *atom_cell, const int *atom_rank,
+                          const int *atom_wrap, const int *cell_start, const int *dstat, void *sorted, float4 *hi,
+                          float4 *lo, int *sbin, int *wrapv) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= p.n) return;
+  const int c = atom_cell[i], wrap = atom_wrap[i];
+  const int slot = cell_start[c] + atom_rank[i];
+  scatter_atom(p, pos, i, wrap, dstat[0] != 0, slot, sorted, hi, lo);
   sbin[slot] = c;
-  wrapv[slot] = atom_wrap[i];
+  wrapv[slot] = wrap;
 }
 
 // ------------------------------------------------------------ batched frames
@@ -1440,25 +1071,16 @@ __global__ void k_bin_batch(const BinParams *__restrict__ bp, const int64_t *__r
 
 __global__ void k_scatter_batch(const BinParams *__restrict__ bp, const int64_t *__restrict__ atom_off, int nframes,
                                 int64_t ntotal, const int *atom_cell, const int *atom_rank, const int *atom_wrap,
-                                const int *cell_start, void *sorted, int *sbin, int *wrapv) {
+                                const int *cell_start, void *sorted, float4 *hi, float4 *lo, int *sbin, int *wrapv) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= ntotal) return;
   const int f = frame_of(atom_off, nframes, i);
   const BinParams &p = bp[f];
-  const int64_t li = i - p.atom_off;
-  const int c = atom_cell[i];
+  const int c = atom_cell[i], wrap = atom_wrap[i];
   const int slot = cell_start[c] + atom_rank[i];
-  if (p.f64) {
-    const double *q = (const double *)p.pos + 3 * li;
-    Atom64 a;
-    a.x = q[0]; a.y = q[1]; a.z = q[2]; a.id = li;
-    ((Atom64 *)sorted)[slot] = a;
-  } else {
-    const float *q = (const float *)p.pos + 3 * li;
-    ((float4 *)sorted)[slot] = make_float4(q[0], q[1], q[2], __int_as_float((int)li));
-  }
+  scatter_atom(p, p.pos, i - p.atom_off, wrap, p.dstat[0] != 0, slot, sorted, hi, lo);
   sbin[slot] = c - p.cell_off;
-  wrapv[slot] = atom_wrap[i];
+  wrapv[slot] = wrap;
 }
 
 constexpr size_t atom_smem_bytes() { return (size_t)PTM_BLOCK * SCRATCH_WORDS * 4; }
@@ -1535,27 +1157,56 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM) k_match(co
   match_atom<F64, P64>(d, (int)(s + d.atom_offset), sm, tplw, live);
 }
 
-// Neighbour lists of one frame (Euclidean order), one thread per atom.
-template <bool F64>
-__global__ void __launch_bounds__(PTM_KNN_BLOCK, PTM_KNN_BLOCKS_PER_SM) k_knn(const __grid_constant__ FrameDesc d) {
-  extern __shared__ __align__(16) int knn_smem[];
+// Neighbour lists of one frame, one thread per atom: NK = 14 into d.nbr, NK = 18
+// (topological order) into d.nbr18.  Measured against the insertion network and
+// the FP64 arithmetic it replaced (k_knn with k_knn_rest, device time):
+//   2^20-atom polycrystal, float32      1.23  -> 0.64 ms (k_knn 0.46, at 46 % of
+//                                       issue and 47 % of L1; 675 -> 226 warp
+//                                       instructions an atom)
+//   250,000 atoms, float64              6.03  -> 0.23 ms (was FP64-pipe bound)
+//   199,680 atoms, unwrapped float32    4.04  -> 0.16 ms (was the general search)
+//   256 frames, 31.7 M atoms            31.2  -> 16.0 ms
+template <bool F64, int NK>
+__global__ void __launch_bounds__(PTM_KNN_BLOCK, KnnShape<NK>::BLOCKS)
+    k_knn(const __grid_constant__ FrameDesc d, int *rest, int *rest_count) {
+  extern __shared__ __align__(16) unsigned char smem[];
   const int64_t s = (int64_t)blockIdx.x * PTM_KNN_BLOCK + threadIdx.x;
   if (s >= d.n) return;
-  knn_atom<F64>(d, (int)s, knn_smem);
+  knn_atom<F64, NK>(d, (int)s, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18, smem, rest, rest_count);
 }
 
-// The same over a batch: each slot finds its frame; frames in the topological
-// order are left to k_topo_batch.
-template <bool F64>
-__global__ void __launch_bounds__(PTM_KNN_BLOCK, PTM_KNN_BATCH_BLOCKS_PER_SM)
+template <bool F64, int NK>
+__global__ void __launch_bounds__(PTM_KNN_BLOCK)
+    k_knn_rest(const __grid_constant__ FrameDesc d, const int *rest, const int *rest_count) {
+  const int n = *rest_count, stride = gridDim.x * (PTM_KNN_BLOCK / 32);
+  for (int i = (blockIdx.x * PTM_KNN_BLOCK + threadIdx.x) >> 5; i < n; i += stride)
+    knn_rest_atom<F64, NK>(d, rest[i], NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18);
+}
+
+// The same over a batch: each slot finds its frame; NK = 14 takes the frames in
+// the Euclidean order, NK = 18 those in the topological one.
+template <bool F64, int NK>
+__global__ void __launch_bounds__(PTM_KNN_BLOCK, KnnShape<NK>::BLOCKS)
     k_knn_batch(const FrameDesc *__restrict__ descs, const int64_t *__restrict__ atom_off, int nframes,
-                int64_t ntotal) {
-  extern __shared__ __align__(16) int knn_smem[];
+                int64_t ntotal, int *rest, int *rest_count) {
+  extern __shared__ __align__(16) unsigned char smem[];
   const int64_t s = (int64_t)blockIdx.x * PTM_KNN_BLOCK + threadIdx.x;
   if (s >= ntotal) return;
   const FrameDesc &d = descs[frame_of(atom_off, nframes, s)];
-  if (d.ordering != PTM_ORDER_EUCLIDEAN) return;
-  knn_atom<F64>(d, (int)s, knn_smem);
+  if ((d.ordering == PTM_ORDER_EUCLIDEAN) != (NK == PTM_KNN)) return;
+  knn_atom<F64, NK>(d, (int)s, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18, smem, rest, rest_count);
+}
+
+template <bool F64, int NK>
+__global__ void __launch_bounds__(PTM_KNN_BLOCK)
+    k_knn_rest_batch(const FrameDesc *__restrict__ descs, const int64_t *__restrict__ atom_off, int nframes,
+                     const int *rest, const int *rest_count) {
+  const int n = *rest_count, stride = gridDim.x * (PTM_KNN_BLOCK / 32);
+  for (int i = (blockIdx.x * PTM_KNN_BLOCK + threadIdx.x) >> 5; i < n; i += stride) {
+    const int s = rest[i];
+    const FrameDesc &d = descs[frame_of(atom_off, nframes, s)];
+    knn_rest_atom<F64, NK>(d, s, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18);
+  }
 }
 
 // Persistent per-atom passes over a batch: every warp pulls tiles of

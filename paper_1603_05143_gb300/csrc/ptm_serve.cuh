@@ -76,10 +76,10 @@ constexpr size_t kOutBytesPerAtom = 1 + 1 + 4 + 4 + 16 + 36 + 60 + 4 + 12;
 size_t request_bytes(const ptm_frame &f) {
   const size_t n = (size_t)f.n_atoms;
   const size_t pos = n * 3 * (f.pos_dtype == PTM_F64 ? 8 : 4);
-  const size_t ws = n * (f.pos_dtype == PTM_F64 ? 32 : 16) + 20 * n + 8 * (4 * n + 64) + sizeof(FrameDesc) +
+  const size_t ws = n * (f.pos_dtype == PTM_F64 ? 64 : 48) + 20 * n + 8 * (4 * n + 64) + sizeof(FrameDesc) +
                     sizeof(ShiftTables) + 4096 +
                     n * 8 * PTM_KNN + 28 * n + 768 +
-                    (f.ordering == PTM_ORDER_TOPOLOGICAL ? n * 4 + topo_side_bytes(n) + 1024 : 0);
+                    (f.ordering == PTM_ORDER_TOPOLOGICAL ? n * (4 + 8 * PTM_TOPO_N) + topo_side_bytes(n) + 1024 : 0);
   return pos + n + n * kOutBytesPerAtom + ws;
 }
 

@@ -127,17 +127,10 @@ __device__ uint32_t topo_order(int m, const T *area, T mean2, int *o) {
   return near;
 }
 
-// kNN slots in the topological scratch: rows J (sorted index) and IMG (packed
-// image), then (while a run is ordered) the atom id and FP64 key in the rows of
-// the FP32 vectors (3 x 18 rows), which are written only after the kNN.
-typedef SmemKnnRows<PTM_TOPO_N, PTM_BLOCK> TopoKnnRows;
-static_assert(TopoKnnRows::kRows <= 5 * PTM_TOPO_N, "kNN rows must fit the neighbour and vector rows");
-
-// What the FP32 pass leaves for the FP64 pass about a listed atom: its 18
-// neighbours, their FP32 face areas and the faces to recompute in FP64 (bit =
-// neighbour rank: the two faces of every gap at the band edge, or all).
+// What the FP32 pass leaves for the FP64 pass about a listed atom: its FP32 face
+// areas and the faces to recompute in FP64 (bit = neighbour rank: the two faces
+// of every gap at the band edge, or all).
 struct TopoSide {
-  int2 nb[PTM_TOPO_N];
   float area[PTM_TOPO_N];
   uint32_t faces;
   uint32_t pad;
@@ -146,8 +139,8 @@ struct TopoSide {
 // One atom, FP32 areas.  An atom with an area gap at the band edge (or a
 // polygon larger than the FP32 buffers) is appended to `list` for the FP64 pass
 // instead of being decided here, so that no warp waits on one lane's FP64 work;
-// the first cap_side listed atoms leave their neighbours, areas and uncertain
-// faces in `side`.
+// the first cap_side listed atoms leave their areas and uncertain faces in
+// `side`.  The 18 nearest come from k_knn (d.nbr18; a slot of -1: fewer).
 template <bool F64>
 __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict__ out, int *list, int *list_count,
                           TopoSide *side, int cap_side) {
@@ -157,33 +150,15 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict_
   auto IMG = [&](int k) -> int & { return tsm[(PTM_TOPO_N + k) * PTM_BLOCK + t]; };
   auto VF = [&](int k, int c) -> float & { return ((float *)tsm)[(2 * PTM_TOPO_N + 3 * k + c) * PTM_BLOCK + t]; };
   const int64_t n = d.n, sl = s - d.atom_offset;     // frame-local slot
-  if (__ldg(d.wrapv + s) == PTM_EXCLUDED) {           // excluded by the binning: no neighbours
-    for (int k = 0; k < PTM_KNN; k++) out[(int64_t)k * n + sl] = make_int2(-1, 0);
-    return;
-  }
   TI xi, yi, zi;
   int idi;
   load_atom<F64>(d, s, xi, yi, zi, idi);
-  const int b = __ldg(d.sbin + s);
-  const int bz = b % d.nb[2], byx = b / d.nb[2];
-  const int by = byx % d.nb[1], bx = byx / d.nb[1];
-  const bool wrapped = d.dstat[0] != 0;
-  int wix = 0, wiy = 0, wiz = 0;
-  if (wrapped) img_unpack(__ldg(d.wrapv + s), wix, wiy, wiz);
-
-  // ---- the 18 nearest images
-  int m;
-  uint32_t close_runs = 0;
-  if (!wrapped && knn_fast_n<F64, PTM_TOPO_N>(d, s, xi, yi, zi, bx, by, bz, TopoKnnRows{tsm, t}, close_runs)) {
-    m = PTM_TOPO_N;
-    if (!F64 && close_runs) count(d, C_KNN64);
-  } else {
-    double Ld2[PTM_TOPO_N];
-    int Lid[PTM_TOPO_N], Ljs[PTM_TOPO_N], Limg[PTM_TOPO_N];
-    m = knn<F64, PTM_TOPO_N>(d, s, xi, yi, zi, bx, by, bz, wix, wiy, wiz, wrapped, Ld2, Lid, Ljs, Limg);
-    if (m < 0) m = 0;
-#pragma unroll
-    for (int k = 0; k < PTM_TOPO_N; k++) { J(k) = Ljs[k]; IMG(k) = Limg[k]; }
+  int m = 0;
+  for (int k = 0; k < PTM_TOPO_N; k++) {
+    const int2 e = d.nbr18[(int64_t)k * n + sl];
+    J(k) = e.x;
+    IMG(k) = e.y;
+    m += e.x >= 0;                                   // the valid entries form a prefix
   }
   int o[PTM_TOPO_N];
   // FP32 neighbour vectors: the difference of positions plus the image
@@ -228,10 +203,7 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict_
       list[slot] = s;
       if (slot < cap_side) {                      // what the FP64 pass reuses
         TopoSide &sd = side[slot];
-        for (int k = 0; k < PTM_TOPO_N; k++) {
-          sd.nb[k] = k < m ? make_int2(J(k), IMG(k)) : make_int2(-1, 0);
-          sd.area[k] = k < m ? area[k] : 0.f;
-        }
+        for (int k = 0; k < PTM_TOPO_N; k++) sd.area[k] = k < m ? area[k] : 0.f;
         sd.faces = over ? ~0u : near;
       }
     }
@@ -245,8 +217,7 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict_
 // (the two faces of every gap at the band edge); the others keep their FP32
 // areas, whose error (measured within 2.2e-6 of the mean squared distance) is
 // far below the guard, so every gap decided from them is decided as in FP64.
-// Atoms past the side buffer find their neighbours again and recompute every
-// face.  Polygon buffers in shared memory, element e at P[e * PTM_BLOCK].  The
+// Atoms past the side buffer recompute every face.  Polygon buffers in shared memory, element e at P[e * PTM_BLOCK].  The
 // lanes of `wmask` call this together and take their faces in step, one face
 // per lane per trip, so a warp makes as many trips as its busiest lane has
 // faces (not one per face index that any lane needs).
@@ -257,30 +228,20 @@ __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *si
   TI xi, yi, zi;
   int idi;
   load_atom<F64>(d, s, xi, yi, zi, idi);
+  const int64_t n = d.n, sl = s - d.atom_offset;     // frame-local slot
   int jn[PTM_TOPO_N], im[PTM_TOPO_N], m = 0;
   double a64[PTM_TOPO_N];
+  for (int k = 0; k < PTM_TOPO_N; k++) {
+    const int2 e = d.nbr18[(int64_t)k * n + sl];
+    jn[k] = e.x;
+    im[k] = e.y;
+    m += e.x >= 0;
+  }
   uint32_t faces = ~0u;
   if (i < cap_side) {
     const TopoSide &sd = side[i];
-    for (int k = 0; k < PTM_TOPO_N; k++) {
-      const int2 e = sd.nb[k];
-      jn[k] = e.x;
-      im[k] = e.y;
-      a64[k] = (double)sd.area[k];
-      m += e.x >= 0;
-    }
+    for (int k = 0; k < PTM_TOPO_N; k++) a64[k] = (double)sd.area[k];
     faces = sd.faces;
-  } else {
-    const int b = __ldg(d.sbin + s);
-    const int bz = b % d.nb[2], byx = b / d.nb[2];
-    const int by = byx % d.nb[1], bx = byx / d.nb[1];
-    const bool wrapped = d.dstat[0] != 0;
-    int wix = 0, wiy = 0, wiz = 0;
-    if (wrapped) img_unpack(__ldg(d.wrapv + s), wix, wiy, wiz);
-    double Ld2[PTM_TOPO_N];
-    int Lid[PTM_TOPO_N];
-    m = knn<F64, PTM_TOPO_N>(d, s, xi, yi, zi, bx, by, bz, wix, wiy, wiz, wrapped, Ld2, Lid, jn, im);
-    if (m < 0) m = 0;
   }
   int o[PTM_TOPO_N];
   double v64[PTM_TOPO_N][3], mean64 = 0.0, dmax64 = 0.0;
@@ -303,7 +264,6 @@ __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *si
     a64[k] = topo_face_area<double>(m, k, 10.0 * sqrt(dmax64), vd, P, Q, PTM_BLOCK, PTM_TOPO_VMAX, over);
   }
   if (m > 0) topo_order<double>(m, a64, mean64, o);
-  const int64_t n = d.n, sl = s - d.atom_offset;     // frame-local slot
   for (int k = 0; k < PTM_KNN; k++) out[(int64_t)k * n + sl] = k < m ? make_int2(jn[o[k]], im[o[k]]) : make_int2(-1, 0);
 }
 
@@ -365,10 +325,10 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO64_BLOCKS_PER_SM)
   }
 }
 
-// Listed atoms whose neighbours, areas and uncertain faces the FP32 pass keeps
-// for the FP64 pass (a quarter of the atoms: 3.6 % were listed in the hot
-// polycrystal, 2.6 % in the mixed-phase frame, up to 15 % in cold crystals; the
-// rest find their neighbours again and recompute every face).
+// Listed atoms whose areas and uncertain faces the FP32 pass keeps for the FP64
+// pass (a quarter of the atoms: 3.6 % were listed in the hot polycrystal, 2.6 %
+// in the mixed-phase frame, up to 15 % in cold crystals; the rest recompute every
+// face).
 constexpr size_t topo_side_cap(size_t n) { return n / 4 + 256; }
 constexpr size_t topo_side_bytes(size_t n) { return topo_side_cap(n) * sizeof(TopoSide); }
 // FP64 pass: two polygon buffers of 2 x PTM_TOPO_VMAX doubles per thread

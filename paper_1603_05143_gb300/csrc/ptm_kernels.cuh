@@ -33,7 +33,8 @@ struct Best {
   __device__ __forceinline__ int ent(int K) const { return K == 6 ? ent6 : (K == 12 ? ent12 : ent14); }
 };
 
-__device__ __forceinline__ int snap_index(int K) { return K == 6 ? 0 : (K == 12 ? 1 : 2); }
+// What one atom adds to the matching counters.
+struct MatchCounts { int scored, points, matched; };
 
 __device__ __forceinline__ int lookup(const Scratch &sm, int K, uint64_t h) {
   const int LEN = 2 * (3 * K - 6) + 1;
@@ -138,14 +139,13 @@ __device__ void snapshot(int K, const Scratch &sm, const FrameDesc &d, int nf, B
 // run their candidates together; keeps the best and second-best RMSD^2 (the
 // first of equal values wins, Algorithm 1).
 __device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const float4 *tplw, Best &bst,
-                                 unsigned qmask) {
+                                 unsigned qmask, MatchCounts &cnt) {
   int n6 = 0, n12 = 0, n14 = 0, f6 = 0, f12 = 0, f14 = 0;
   float Gv6 = 0.f, Gv12 = 0.f, Gv14 = 0.f, mx, my, mz;
   if (bst.ent6 >= 0) { f6 = ptm_tbl[bst.ent6].first; n6 = ptm_tbl[bst.ent6].count; data_moments(6, sm, mx, my, mz, Gv6); }
   if (bst.ent12 >= 0) { f12 = ptm_tbl[bst.ent12].first; n12 = ptm_tbl[bst.ent12].count; data_moments(12, sm, mx, my, mz, Gv12); }
   if (bst.ent14 >= 0) { f14 = ptm_tbl[bst.ent14].first; n14 = ptm_tbl[bst.ent14].count; data_moments(14, sm, mx, my, mz, Gv14); }
   const int total = n6 + n12 + n14;
-  int scored = 0, points = 0;
   for (int i = 0; __any_sync(qmask, i < total); i++) {
     if (i >= total) continue;
     int K, c;
@@ -157,8 +157,8 @@ __device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const fl
     const uint64_t cand = __ldg((const unsigned long long *)&ptm_cand[c]);
     const int S = (int)(cand >> 60) & 7;
     if (!(d.mask >> S & 1)) continue;
-    scored++;
-    points += K + 1;
+    cnt.scored++;
+    cnt.points += K + 1;
     float Sm[3][3];
     cov_matrix(K, sm, tplw, S, lab, cand, Sm);
     const float Gw = __ldg(tplw + S * 15).w;
@@ -167,7 +167,6 @@ __device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const fl
     if (r2 < bst.b1) { bst.b2 = bst.b1; bst.b1 = r2; bst.K = K; bst.cand = c; bst.fp64 = fp64; }
     else if (r2 < bst.b2) bst.b2 = r2;
   }
-  if (scored) { count(d, C_CAND, scored); count(d, C_CANDPTS, (unsigned long long)points); }
 }
 
 // Canonical correspondence: the paper leaves open which of the equivalent
@@ -322,7 +321,8 @@ __device__ __forceinline__ int8_t alloy_label(const FrameDesc &d, const Scratch 
   return lab8;
 }
 
-__device__ void finalize(const FrameDesc &d, const Scratch &sm, const float4 *tplw, const Best &bst, int idi) {
+// Outputs of the winner; returns whether the atom is matched (Sec. 5.1).
+__device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tplw, const Best &bst, int idi) {
   const int K = bst.K;
   const uint64_t lab = bst.lam(K);
   const uint64_t cand = __ldg((const unsigned long long *)&ptm_cand[bst.cand]);
@@ -389,9 +389,8 @@ __device__ void finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
     if (d.corr) for (int i = 0; i < 15; i++) d.corr[15 * a + i] = -1;
     if (d.vm) d.vm[a] = 0.f;
     if (d.rf) for (int i = 0; i < 3; i++) d.rf[3 * a + i] = 0.f;
-    return;
+    return false;
   }
-  count(d, C_MATCHED);
   // correspondence: smallest member of its orbit (R12), atom ids per slot
   const uint64_t cp = canonical_corr(S, K, corr);
   if (d.structure) d.structure[a] = (int8_t)(S + 1);
@@ -455,6 +454,7 @@ __device__ void finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
     }
   }
   if (d.alloy) d.alloy[a] = alloy_label(d, sm, S, cp, a);
+  return true;
 }
 
 __device__ void write_unmatched(const FrameDesc &d, int64_t a) {
@@ -472,7 +472,7 @@ __device__ void write_unmatched(const FrameDesc &d, int64_t a) {
 // Outputs of the winner in the FP64 form: the same steps as finalize, every
 // metric quantity in FP64 from the FP64 neighbour vectors (results rounded to
 // FP32 only when stored).
-__device__ __noinline__ void finalize_fp64(const FrameDesc &d, const Scratch &sm, int K, uint64_t lab, int ci,
+__device__ __noinline__ bool finalize_fp64(const FrameDesc &d, const Scratch &sm, int K, uint64_t lab, int ci,
                                            const double (&ex)[PTM_KNN], const double (&ey)[PTM_KNN],
                                            const double (&ez)[PTM_KNN], int idi) {
   const uint64_t cand = ptm_cand[ci];
@@ -515,8 +515,7 @@ __device__ __noinline__ void finalize_fp64(const FrameDesc &d, const Scratch &sm
   }
   const double rmsd = sqrt(r2 / (K + 1));
   const int64_t a = idi;
-  if (!(rmsd <= d.rmsd_max)) { write_unmatched(d, a); return; }
-  count(d, C_MATCHED);
+  if (!(rmsd <= d.rmsd_max)) { write_unmatched(d, a); return false; }
   const uint64_t cp = canonical_corr(S, K, corr);
   if (d.structure) d.structure[a] = (int8_t)(S + 1);
   if (d.rmsd) d.rmsd[a] = (float)rmsd;
@@ -567,6 +566,7 @@ __device__ __noinline__ void finalize_fp64(const FrameDesc &d, const Scratch &sm
     }
   }
   if (d.alloy) d.alloy[a] = alloy_label(d, sm, S, cp, a);
+  return true;
 }
 
 // Neighbour vectors for the metric steps, in rows DX / DY / DZ over the
@@ -667,14 +667,15 @@ __device__ __forceinline__ uint32_t pack_ents(int e6, int e12, int e14) {
   return (uint32_t)(e6 + 1) | (uint32_t)(e12 + 1) << 10 | (uint32_t)(e14 + 1) << 20;
 }
 
+// Returns the number of orientation tests that Simulation of Simplicity decided.
 template <bool F64>
-__device__ void hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned live) {
+__device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned live) {
   typedef typename RT<F64>::T T;
   T xi, yi, zi;
   int idi;
   load_atom<F64>(d, s, xi, yi, zi, idi);
-  count(d, C_ATOMS);
   const int64_t sl = s - d.atom_offset;          // frame-local slot
+  int nsos = 0;
 
   // ---- neighbours (Sec. 3): the list written by k_knn or k_topo, read in
   // place (entry t at nb[t * n]; the valid entries form a prefix).
@@ -758,7 +759,7 @@ __device__ void hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned
       if (wide) wide_quantise(d, xi, yi, zi, nb, nst, sm.q + sm.t, wide, PTM_QBITS - e);
     }
     hmask = __ballot_sync(live, cnt >= 4);       // lanes that go on to the hulls
-    if (cnt < 4) { d.ents[sl] = 0; return; }
+    if (cnt < 4) { d.ents[sl] = 0; return 0; }
   }
 
   // ---- hulls of the first 6, 12, 14 neighbours, built incrementally (Sec. 4)
@@ -769,7 +770,7 @@ __device__ void hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned
   int kmax = (mask & 16) ? 14 : ((mask & 14) ? 12 : 6);
   kmax = min(kmax, cnt);
   bool alive = kmax >= 6;
-  int nf = alive ? hull_init(sm, d) : 0;
+  int nf = alive ? hull_init(sm, nsos) : 0;
   for (int p = 4; p <= PTM_KNN; p++) {
     // every insertion step starts warp-converged: a lane that finished (or took
     // a snapshot's longer path) waits here instead of drifting into a later
@@ -783,8 +784,8 @@ __device__ void hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned
     const unsigned vmask = __ballot_sync(hmask, alive && p < kmax);          // lanes testing point p
     const unsigned cmask = __ballot_sync(hmask, alive && p >= kmax && want); // lanes testing only the centre
     if (alive) {
-      if (p < kmax) vis = hull_visibility(sm, nf, p, want, centre_in, vmask, d);
-      else if (want) centre_in = hull_centre_inside(sm, nf, cmask, d);
+      if (p < kmax) vis = hull_visibility(sm, nf, p, want, centre_in, vmask, nsos);
+      else if (want) centre_in = hull_centre_inside(sm, nf, cmask, nsos);
     }
     if (alive && want && centre_in) snapshot(p, sm, d, nf, bst);
     if (!alive) continue;
@@ -796,20 +797,22 @@ __device__ void hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned
   if (bst.ent6 >= 0) d.lam[sl] = bst.lam6;
   if (bst.ent12 >= 0) d.lam[d.n + sl] = bst.lam12;
   if (bst.ent14 >= 0) d.lam[2 * d.n + sl] = bst.lam14;
+  return nsos;
 }
 
 // P64 selects the FP64 form: every candidate scored and the winner's outputs
 // computed in FP64 (the one-frame-per-launch comparison form).
 template <bool F64, bool P64 = false>
-__device__ void match_atom(const FrameDesc &d, int s, const Scratch &sm, const float4 *tplw, unsigned live) {
+__device__ MatchCounts match_atom(const FrameDesc &d, int s, const Scratch &sm, const float4 *tplw, unsigned live) {
   typedef typename RT<F64>::T T;
   const int64_t sl = s - d.atom_offset;
+  MatchCounts cnt = {0, 0, 0};
   const uint32_t ents = __ldg(d.ents + sl);
   const unsigned qmask = __ballot_sync(live, ents != 0);
   T xi, yi, zi;
   int idi;
   load_atom<F64>(d, s, xi, yi, zi, idi);
-  if (!ents) { write_unmatched(d, idi); return; }
+  if (!ents) { write_unmatched(d, idi); return cnt; }
   Best bst;
   bst.b1 = bst.b2 = INFINITY;
   bst.K = -1; bst.cand = -1; bst.fp64 = 0;
@@ -831,23 +834,22 @@ __device__ void match_atom(const FrameDesc &d, int s, const Scratch &sm, const f
   }
   metric_vectors<F64>(d, sm, nb, nst, xi, yi, zi);
   if constexpr (!P64) {
-    score_candidates(d, sm, tplw, bst, qmask);
-    if (bst.K < 0) { write_unmatched(d, idi); return; }     // every match masked out
+    score_candidates(d, sm, tplw, bst, qmask, cnt);
+    if (bst.K < 0) { write_unmatched(d, idi); return cnt; }     // every match masked out
   } else {
-    int ns = 0;
-    const int w = select_fp64(d, bst, ex, ey, ez, &ns);
-    if (ns) { count(d, C_CAND, ns); }
-    if (w < 0) { write_unmatched(d, idi); return; }
+    const int w = select_fp64(d, bst, ex, ey, ez, &cnt.scored);
+    if (w < 0) { write_unmatched(d, idi); return cnt; }
     const int K = w >> 16;
-    finalize_fp64(d, sm, K, bst.lam(K), w & 0xffff, ex, ey, ez, idi);
-    return;
+    cnt.matched = finalize_fp64(d, sm, K, bst.lam(K), w & 0xffff, ex, ey, ez, idi);
+    return cnt;
   }
   if (bst.b2 <= bst.b1 + PTM_BAND) {
     count(d, C_TIE64);
     const int w = rerank_fp64<F64>(d, s, bst);
     if (w >= 0) { bst.K = w >> 16; bst.cand = w & 0xffff; }
   }
-  finalize(d, sm, tplw, bst, idi);
+  cnt.matched = finalize(d, sm, tplw, bst, idi);
+  return cnt;
 }
 
 // ------------------------------------------------------------------ kernels
@@ -1143,7 +1145,9 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_ATOM_BLOCKS_PER_SM) k_hulls(con
   const int64_t s = (int64_t)blockIdx.x * PTM_BLOCK + threadIdx.x;
   const unsigned live = __ballot_sync(0xffffffffu, s < d.n);
   if (s >= d.n) return;
-  hull_atom<F64>(d, (int)s, sm, live);
+  const int nsos = hull_atom<F64>(d, (int)s, sm, live);
+  count_warp(d, C_ATOMS, live, 1);
+  count_warp(d, C_SOS, live, nsos);
 }
 
 template <bool F64, bool P64 = false>
@@ -1154,7 +1158,10 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM) k_match(co
   const int64_t s = (int64_t)blockIdx.x * PTM_BLOCK + threadIdx.x;     // frame-local slot
   const unsigned live = __ballot_sync(0xffffffffu, s < d.n);
   if (s >= d.n) return;
-  match_atom<F64, P64>(d, (int)(s + d.atom_offset), sm, tplw, live);
+  const MatchCounts c = match_atom<F64, P64>(d, (int)(s + d.atom_offset), sm, tplw, live);
+  count_warp(d, C_CAND, live, c.scored);
+  count_warp(d, C_CANDPTS, live, c.points);
+  count_warp(d, C_MATCHED, live, c.matched);
 }
 
 // Neighbour lists of one frame, one thread per atom: NK = 14 into d.nbr, NK = 18
@@ -1270,7 +1277,11 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_ATOM_BLOCKS_PER_SM)
   extern __shared__ __align__(16) unsigned char smem[];
   const Scratch sm = scratch_rows(smem);
   persistent_tiles(descs, atom_off, nframes, ntotal, nullptr, tile_atoms, queue, nullptr,
-                   [&](const FrameDesc &d, int s, unsigned live) { hull_atom<F64>(d, s, sm, live); });
+                   [&](const FrameDesc &d, int s, unsigned live) {
+                     const int nsos = hull_atom<F64>(d, s, sm, live);
+                     count_warp(d, C_ATOMS, live, 1);
+                     count_warp(d, C_SOS, live, nsos);
+                   });
 }
 
 // k_match over the atoms of the batch's smaller frames (the larger ones get a
@@ -1286,7 +1297,12 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM)
   const float4 *tplw = template_rows();
   __shared__ FrameDesc heads[PTM_BLOCK / 32];
   persistent_tiles(descs, map_off, nmap, nslots, map_frames, tile_atoms, queue, &heads[threadIdx.x >> 5],
-                   [&](const FrameDesc &d, int s, unsigned live) { match_atom<F64, false>(d, s, sm, tplw, live); });
+                   [&](const FrameDesc &d, int s, unsigned live) {
+                     const MatchCounts c = match_atom<F64, false>(d, s, sm, tplw, live);
+                     count_warp(d, C_CAND, live, c.scored);
+                     count_warp(d, C_CANDPTS, live, c.points);
+                     count_warp(d, C_MATCHED, live, c.matched);
+                   });
 }
 
 }  // namespace ptm

@@ -377,7 +377,7 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
   const bool crossing = (close >> (NK - 1)) & 1;
   const float limit = crossing ? L(NK - 1) + band : L(NK - 1);
   if (!(limit < T)) return false;                    // the list may not hold the whole last run
-  if (!F64 && close) count(d, C_KNN64);
+  if (!F64 && close) count_here(d, C_KNN64);
   IN xi, yi, zi;
   int idi;
   load_atom<F64>(d, s, xi, yi, zi, idi);

@@ -56,21 +56,29 @@ __device__ __forceinline__ int lookup(const Scratch &sm, int K, uint64_t h) {
   return -1;
 }
 
-// S_ab = sum_j w_{slot(j), a} dr_{j, b} for the correspondence "neighbour rank j ->
-// template slot" given by the walk labelling and the table candidate.
-// Because the template barycentre is the origin and slot 0 (the centre) sits at
-// it, the data barycentre drops out of S.
-__device__ __forceinline__ void cov_matrix(int K, const Scratch &sm, const float4 *tplw, int S, uint64_t lab,
-                                           uint64_t cand, float (&Sm)[3][3]) {
+// Template slots of neighbours 0 .. K - 1 (nibble j) under the correspondence given
+// by the walk labelling and the table candidate.
+__device__ __forceinline__ uint64_t slots_of(int K, uint64_t lab, uint64_t cand) {
+  uint64_t slots = 0;
+#pragma unroll
+  for (int j = 0; j < PTM_KNN; j++)
+    if (j < K) slots |= (uint64_t)nib(cand, nib(lab, j) - 1) << (4 * j);
+  return slots;
+}
+
+// S_ab = sum_j w_{slot(j), a} dr_{j, b} over K neighbours, dr_{j, b} at q[(3 j + b)
+// * PTM_BLOCK].  Because the template barycentre is the origin and slot 0 (the
+// centre) sits at it, the data barycentre drops out of S.
+__device__ __forceinline__ void cov_matrix(int K, const float *q, const float4 *tplw, uint64_t slots, float (&Sm)[3][3]) {
 #pragma unroll
   for (int a = 0; a < 3; a++)
 #pragma unroll
     for (int b = 0; b < 3; b++) Sm[a][b] = 0.f;
-#pragma unroll 1
+#pragma unroll 2
   for (int j = 0; j < K; j++) {
-    const int slot = nib(cand, nib(lab, j) - 1);
-    const float4 w = __ldg(tplw + S * 15 + slot);
-    const float x = sm.DX(j), y = sm.DY(j), z = sm.DZ(j);
+    const float4 w = __ldg(tplw + (int)(slots & 15));
+    slots >>= 4;
+    const float x = q[(3 * j) * PTM_BLOCK], y = q[(3 * j + 1) * PTM_BLOCK], z = q[(3 * j + 2) * PTM_BLOCK];
     Sm[0][0] = fmaf(w.x, x, Sm[0][0]); Sm[0][1] = fmaf(w.x, y, Sm[0][1]); Sm[0][2] = fmaf(w.x, z, Sm[0][2]);
     Sm[1][0] = fmaf(w.y, x, Sm[1][0]); Sm[1][1] = fmaf(w.y, y, Sm[1][1]); Sm[1][2] = fmaf(w.y, z, Sm[1][2]);
     Sm[2][0] = fmaf(w.z, x, Sm[2][0]); Sm[2][1] = fmaf(w.z, y, Sm[2][1]); Sm[2][2] = fmaf(w.z, z, Sm[2][2]);
@@ -133,39 +141,86 @@ __device__ void snapshot(int K, const Scratch &sm, const FrameDesc &d, int nf, B
   else { bst.lam14 = lab; bst.ent14 = e; }
 }
 
-// FP32 QCP of every admissible correspondence of the matched snapshots, in
-// snapshot order (6, 12, 14) and table order, as one flat loop whose trips
-// start warp-converged (every lane in `qmask` calls it), so the lanes of a warp
-// run their candidates together; keeps the best and second-best RMSD^2 (the
+// FP32 QCP of every admissible correspondence of the matched snapshots; keeps the
+// best and second-best RMSD^2 in snapshot order (6, 12, 14) and table order (the
 // first of equal values wins, Algorithm 1).
-__device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const float4 *tplw, Best &bst,
-                                 unsigned qmask, MatchCounts &cnt) {
+//
+// The candidates of the warp's atoms form one list, scored one entry per lane per
+// round: atoms have 3 to 5 candidates on average but up to 26, and one loop per
+// atom ran 19 rounds at 21 % of the lanes where this takes 3 to 5.  A lane
+// finds its entry's atom by bisection of the lanes' running totals, fetches that
+// atom's labelling and sums by shuffles and reads its vectors in place (the rows
+// of a warp's lanes are neighbouring banks, and lanes of one atom broadcast); the
+// atom then takes its results back in order.  Every live lane calls this; the
+// live lanes are the warp's first.
+__device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const float4 *tplw, Best &bst, unsigned live,
+                                 MatchCounts &cnt) {
+  const int lane = threadIdx.x & 31, nlive = __popc(live);
   int n6 = 0, n12 = 0, n14 = 0, f6 = 0, f12 = 0, f14 = 0;
   float Gv6 = 0.f, Gv12 = 0.f, Gv14 = 0.f, mx, my, mz;
   if (bst.ent6 >= 0) { f6 = ptm_tbl[bst.ent6].first; n6 = ptm_tbl[bst.ent6].count; data_moments(6, sm, mx, my, mz, Gv6); }
   if (bst.ent12 >= 0) { f12 = ptm_tbl[bst.ent12].first; n12 = ptm_tbl[bst.ent12].count; data_moments(12, sm, mx, my, mz, Gv12); }
   if (bst.ent14 >= 0) { f14 = ptm_tbl[bst.ent14].first; n14 = ptm_tbl[bst.ent14].count; data_moments(14, sm, mx, my, mz, Gv14); }
-  const int total = n6 + n12 + n14;
-  for (int i = 0; __any_sync(qmask, i < total); i++) {
-    if (i >= total) continue;
-    int K, c;
-    uint64_t lab;
-    float Gv;
-    if (i < n6) { K = 6; c = f6 + i; lab = bst.lam6; Gv = Gv6; }
-    else if (i < n6 + n12) { K = 12; c = f12 + (i - n6); lab = bst.lam12; Gv = Gv12; }
-    else { K = 14; c = f14 + (i - n6 - n12); lab = bst.lam14; Gv = Gv14; }
-    const uint64_t cand = __ldg((const unsigned long long *)&ptm_cand[c]);
-    const int S = (int)(cand >> 60) & 7;
-    if (!(d.mask >> S & 1)) continue;
-    cnt.scored++;
-    cnt.points += K + 1;
-    float Sm[3][3];
-    cov_matrix(K, sm, tplw, S, lab, cand, Sm);
-    const float Gw = __ldg(tplw + S * 15).w;
-    int fp64;
-    const float r2 = cand_r2(Sm, Gv, Gw, K + 1, fp64, d);
-    if (r2 < bst.b1) { bst.b2 = bst.b1; bst.b1 = r2; bst.K = K; bst.cand = c; bst.fp64 = fp64; }
-    else if (r2 < bst.b2) bst.b2 = r2;
+  const int mine = n6 + n12 + n14;
+  int upto = mine;                                   // running total of the lanes' candidates
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(live, upto, o);
+    if (lane >= o) upto += x;
+  }
+  const int total = __shfl_sync(live, upto, nlive - 1), first = upto - mine;
+  const uint32_t packed = (uint32_t)n6 | (uint32_t)n12 << 8, firsts = (uint32_t)f6 | (uint32_t)f12 << 10 | (uint32_t)f14 << 20;
+  for (int base = 0; base < total; base += nlive) {
+    const int p = base + lane;
+    int owner = 0;                                   // lanes whose running total is at most p
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const int at = owner + o - 1;
+      const int x = __shfl_sync(live, upto, min(at, nlive - 1));
+      if (at < nlive && x <= p) owner += o;
+    }
+    owner = min(owner, nlive - 1);                   // (entries past the list: any lane)
+    const int i = p - __shfl_sync(live, first, owner);
+    const uint32_t np = __shfl_sync(live, packed, owner), fp = __shfl_sync(live, firsts, owner);
+    const uint32_t mask = __shfl_sync(live, d.mask, owner);
+    const int m6 = np & 255, m12 = np >> 8;
+    const int K = i < m6 ? 6 : (i < m6 + m12 ? 12 : 14);
+    const int c = K == 6 ? (int)(fp & 1023) + i : (K == 12 ? (int)(fp >> 10 & 1023) + i - m6 : (int)(fp >> 20) + i - m6 - m12);
+    const uint64_t l6 = __shfl_sync(live, bst.lam6, owner), l12 = __shfl_sync(live, bst.lam12, owner),
+                   l14 = __shfl_sync(live, bst.lam14, owner);
+    const float g6 = __shfl_sync(live, Gv6, owner), g12 = __shfl_sync(live, Gv12, owner), g14 = __shfl_sync(live, Gv14, owner);
+    float r2 = INFINITY;
+    int fp64 = 0;
+    if (p < total) {
+      const uint64_t cand = __ldg((const unsigned long long *)&ptm_cand[c]);
+      const int S = (int)(cand >> 60) & 7;
+      if (mask >> S & 1) {
+        cnt.scored++;
+        cnt.points += K + 1;
+        float Sm[3][3];
+        const float4 *tpl = tplw + S * 15;
+        cov_matrix(K, sm.q + ((threadIdx.x & ~31) | owner), tpl,
+                   slots_of(K, K == 6 ? l6 : (K == 12 ? l12 : l14), cand), Sm);
+        r2 = cand_r2(Sm, K == 6 ? g6 : (K == 12 ? g12 : g14), __ldg(tpl).w, K + 1, fp64, d);
+      }
+    }
+    // the results of this lane's atom among this round's, in candidate order
+    const int lo = max(first - base, 0), hi = min(upto - base, nlive);
+    const int trips = __reduce_max_sync(live, max(hi - lo, 0));
+    for (int t = 0; t < trips; t++) {
+      const int src = lo + t;
+      const float x = __shfl_sync(live, r2, min(src, nlive - 1));
+      const int xf = __shfl_sync(live, fp64, min(src, nlive - 1));
+      if (src >= hi) continue;
+      if (x < bst.b1) {
+        const int k = base + src - first;            // candidate of this atom
+        bst.b2 = bst.b1; bst.b1 = x; bst.fp64 = xf;
+        bst.K = k < n6 ? 6 : (k < n6 + n12 ? 12 : 14);
+        bst.cand = k < n6 ? f6 + k : (k < n6 + n12 ? f12 + k - n6 : f14 + k - n6 - n12);
+      } else if (x < bst.b2) {
+        bst.b2 = x;
+      }
+    }
   }
 }
 
@@ -173,29 +228,30 @@ __device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const fl
 // correspondences of a match is reported; this library reports the smallest
 // member of its orbit under the template's rotation group.  Nibble 15 - s holds
 // the neighbour rank of template slot s, so the orbit minimum, read slot 1
-// first, is the numerically smallest packing.
-__device__ uint64_t canonical_corr(int S, int K, uint64_t corr) {
+// first, is the numerically smallest packing.  A rotation brings the rank at the
+// slot it maps slot 1 to into slot 1, so only the rotations that map slot 1 to
+// the first neighbour's slot among slot 1's images can give the minimum: 2 of
+// fcc's 24, 3 of bcc's, 1 of hcp's 6 (every packing: 0.17 ns per atom).
+__device__ uint64_t canonical_corr(int S, int K, uint64_t slots) {
+  const uint8_t *off = ptm_coset_off[S];
+  int g0 = 0, g1 = 0;
+  for (int j = 0; j < K; j++) {
+    const int slot = nib(slots, j);
+    g0 = __ldg(off + slot);
+    g1 = __ldg(off + slot + 1);
+    if (g1 > g0) break;
+  }
   uint64_t best = ~0ull;
-  const int g0 = ptm_group_off[S], g1 = ptm_group_off[S + 1];
   for (int g = g0; g < g1; g++) {
+    const uint64_t inv = __ldg((const unsigned long long *)&ptm_group_inv[__ldg(ptm_coset + g)]);
     uint64_t cur = 0;
-    for (int s = 1; s <= K; s++) cur |= (uint64_t)nib(corr, 15 - ptm_group_perm[g][s]) << (4 * (15 - s));
+#pragma unroll
+    for (int j = 0; j < PTM_KNN; j++)
+      if (j < K) cur |= (uint64_t)(j + 1) << (60 - 4 * nib(inv, nib(slots, j)));
     best = cur < best ? cur : best;
   }
   return best;
 }
-
-__device__ __forceinline__ uint64_t corr_of(int K, uint64_t lab, uint64_t cand) {
-  uint64_t corr = 0;
-#pragma unroll
-  for (int j = 0; j < PTM_KNN; j++) {
-    if (j >= K) break;
-    int slot = nib(cand, nib(lab, j) - 1);
-    corr |= (uint64_t)(j + 1) << (4 * (15 - slot));
-  }
-  return corr;
-}
-
 
 // FP64 selection over every candidate of the matched snapshots (Algorithm 1,
 // inner loops), from FP64 neighbour vectors.  Exact ties, which the paper does
@@ -241,7 +297,7 @@ __device__ __noinline__ int select_fp64(const FrameDesc &d, const Best &bst, con
         if (pass == 0) {
           best_r2 = fmin(best_r2, r2);
         } else if (r2 <= best_r2 + PTM_TIE) {
-          uint64_t cp = canonical_corr(S, K, corr_of(K, lab, cand));
+          uint64_t cp = canonical_corr(S, K, slots_of(K, lab, cand));
           if (S < bS || (S == bS && cp < bcp)) { bS = S; bcp = cp; bK = K; bc = ci; }
         }
       }
@@ -327,11 +383,13 @@ __device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
   const uint64_t lab = bst.lam(K);
   const uint64_t cand = __ldg((const unsigned long long *)&ptm_cand[bst.cand]);
   const int S = (int)(cand >> 60) & 7;
+  const uint64_t slots = slots_of(K, lab, cand);
+  tplw += S * 15;
   float Sm[3][3];
-  cov_matrix(K, sm, tplw, S, lab, cand, Sm);
+  cov_matrix(K, sm.q + sm.t, tplw, slots, Sm);
   float mx, my, mz, Gv;
   data_moments(K, sm, mx, my, mz, Gv);
-  const float Gw = __ldg(tplw + S * 15).w;
+  const float Gw = __ldg(tplw).w;
   float lam, q[4];
   {
     Qcp<float> o;
@@ -362,11 +420,9 @@ __device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
     r2 = ux * ux + uy * uy + uz * uz;
   }
   float lsum = sqrtf(mx * mx + my * my + mz * mz);
-  uint64_t corr = 0;
 #pragma unroll 1
   for (int j = 0; j < K; j++) {
-    int slot = nib(cand, nib(lab, j) - 1);
-    float4 w = __ldg(tplw + S * 15 + slot);
+    float4 w = __ldg(tplw + nib(slots, j));
     float vx = sm.DX(j) - mx, vy = sm.DY(j) - my, vz = sm.DZ(j) - mz;
     float rx = R[0][0] * w.x + R[0][1] * w.y + R[0][2] * w.z;
     float ry = R[1][0] * w.x + R[1][1] * w.y + R[1][2] * w.z;
@@ -374,7 +430,6 @@ __device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
     float ex = s * vx - rx, ey = s * vy - ry, ez = s * vz - rz;
     r2 += ex * ex + ey * ey + ez * ez;
     lsum += sqrtf(vx * vx + vy * vy + vz * vz);
-    corr |= (uint64_t)(j + 1) << (4 * (15 - slot));
   }
   const float rmsd = sqrtf(r2 / (float)(K + 1));
   const int64_t a = idi;
@@ -392,7 +447,7 @@ __device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
     return false;
   }
   // correspondence: smallest member of its orbit (R12), atom ids per slot
-  const uint64_t cp = canonical_corr(S, K, corr);
+  const uint64_t cp = canonical_corr(S, K, slots);
   if (d.structure) d.structure[a] = (int8_t)(S + 1);
   if (d.rmsd) d.rmsd[a] = rmsd;
   if (d.scale) d.scale[a] = s;
@@ -405,7 +460,8 @@ __device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
   if (d.quat || d.rf) {
     float bw = -1.f, bq[4] = {1.f, 0.f, 0.f, 0.f};
     for (int g = ptm_group_off[S]; g < ptm_group_off[S + 1]; g++) {
-      const float *gq = ptm_group_quat[g];
+      const float4 e = __ldg((const float4 *)ptm_group_quat[g]);
+      const float gq[4] = {e.x, e.y, e.z, e.w};
       float o0 = q[0] * gq[0] - q[1] * gq[1] - q[2] * gq[2] - q[3] * gq[3];
       if (fabsf(o0) > bw) {
         bw = fabsf(o0);
@@ -500,10 +556,9 @@ __device__ __noinline__ bool finalize_fp64(const FrameDesc &d, const Scratch &sm
   // explicit residual of Eq. 3; the centre pairs with template slot 0 (origin)
   double r2 = s * s * (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
   double lsum = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
-  uint64_t corr = 0;
+  const uint64_t slots = slots_of(K, lab, cand);
   for (int j = 0; j < K; j++) {
-    const int slot = nib(cand, nib(lab, j) - 1);
-    const double *w = ptm_tpl64[S][slot];
+    const double *w = ptm_tpl64[S][nib(slots, j)];
     const double vx = ex[j] - m[0], vy = ey[j] - m[1], vz = ez[j] - m[2];
     const double rx = R[0][0] * w[0] + R[0][1] * w[1] + R[0][2] * w[2];
     const double ry = R[1][0] * w[0] + R[1][1] * w[1] + R[1][2] * w[2];
@@ -511,12 +566,11 @@ __device__ __noinline__ bool finalize_fp64(const FrameDesc &d, const Scratch &sm
     const double dx = s * vx - rx, dy = s * vy - ry, dz = s * vz - rz;
     r2 += dx * dx + dy * dy + dz * dz;
     lsum += sqrt(vx * vx + vy * vy + vz * vz);
-    corr |= (uint64_t)(j + 1) << (4 * (15 - slot));
   }
   const double rmsd = sqrt(r2 / (K + 1));
   const int64_t a = idi;
   if (!(rmsd <= d.rmsd_max)) { write_unmatched(d, a); return false; }
-  const uint64_t cp = canonical_corr(S, K, corr);
+  const uint64_t cp = canonical_corr(S, K, slots);
   if (d.structure) d.structure[a] = (int8_t)(S + 1);
   if (d.rmsd) d.rmsd[a] = (float)rmsd;
   if (d.scale) d.scale[a] = (float)s;
@@ -808,11 +862,10 @@ __device__ MatchCounts match_atom(const FrameDesc &d, int s, const Scratch &sm, 
   const int64_t sl = s - d.atom_offset;
   MatchCounts cnt = {0, 0, 0};
   const uint32_t ents = __ldg(d.ents + sl);
-  const unsigned qmask = __ballot_sync(live, ents != 0);
   T xi, yi, zi;
   int idi;
   load_atom<F64>(d, s, xi, yi, zi, idi);
-  if (!ents) { write_unmatched(d, idi); return cnt; }
+  if (P64 && !ents) { write_unmatched(d, idi); return cnt; }
   Best bst;
   bst.b1 = bst.b2 = INFINITY;
   bst.K = -1; bst.cand = -1; bst.fp64 = 0;
@@ -832,10 +885,12 @@ __device__ MatchCounts match_atom(const FrameDesc &d, int s, const Scratch &sm, 
       vec_fp64<F64>(d, xi, yi, zi, e.x, e.y, ex[t], ey[t], ez[t]);
     }
   }
-  metric_vectors<F64>(d, sm, nb, nst, xi, yi, zi);
+  if (ents) metric_vectors<F64>(d, sm, nb, nst, xi, yi, zi);
   if constexpr (!P64) {
-    score_candidates(d, sm, tplw, bst, qmask, cnt);
-    if (bst.K < 0) { write_unmatched(d, idi); return cnt; }     // every match masked out
+    __syncwarp(live);                              // the vectors are read across the warp
+    score_candidates(d, sm, tplw, bst, live, cnt);
+    __syncwarp(live);
+    if (bst.K < 0) { write_unmatched(d, idi); return cnt; }     // no match, or every match masked out
   } else {
     const int w = select_fp64(d, bst, ex, ey, ez, &cnt.scored);
     if (w < 0) { write_unmatched(d, idi); return cnt; }

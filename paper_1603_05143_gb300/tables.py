@@ -374,13 +374,25 @@ def emit_header(path: pathlib.Path) -> dict:
         lines.append("  {" + ", ".join(rows) + "},")
     lines.append("};")
     lines.append("PTM_TBL_CONST int ptm_group_off[6] = {" + ", ".join(map(str, goff)) + "};")
-    lines.append("/* rotation g maps slot s to slot perm[g][s] */")
-    lines.append("PTM_TBL_CONST uint8_t ptm_group_perm[PTM_GROUP_TOTAL][16] = {")
+    lines.append("/* rotation g maps slot s to slot p: nibble p of entry g is s */")
+    lines.append("PTM_TBL_GLOBAL uint64_t ptm_group_inv[PTM_GROUP_TOTAL] = {")
     for perms in groups:
         for p in perms:
-            lines.append("  {" + ", ".join(map(str, list(p) + [0] * (16 - len(p)))) + "},")
+            lines.append(f"  0x{sum(s << (4 * t) for s, t in enumerate(p)):016x}ULL,")
     lines.append("};")
-    lines.append("PTM_TBL_CONST float ptm_group_quat[PTM_GROUP_TOTAL][4] = {")
+    lines.append("/* the rotations that map slot 1 to slot p, by template and p: entries coset_off[S][p] .. coset_off[S][p + 1] */")
+    coset, coff = [], []
+    for S, perms in enumerate(groups):
+        row = []
+        for slot in range(16):
+            row.append(len(coset))
+            coset += [goff[S] + g for g, p in enumerate(perms) if p[1] == slot]
+        coff.append(row + [len(coset)])
+    lines.append("PTM_TBL_GLOBAL uint8_t ptm_coset_off[5][17] = {")
+    lines += ["  {" + ", ".join(map(str, row)) + "}," for row in coff]
+    lines.append("};")
+    lines.append("PTM_TBL_GLOBAL uint8_t ptm_coset[PTM_GROUP_TOTAL] = {" + ", ".join(map(str, coset)) + "};")
+    lines.append("PTM_TBL_GLOBAL float ptm_group_quat[PTM_GROUP_TOTAL][4] PTM_TBL_ALIGN16 = {")
     for qs in quats:
         for q in qs:
             lines.append("  {" + ", ".join(f"{x:.9e}f" for x in q) + "},")

@@ -392,7 +392,7 @@ ptm_status ptm_create(const ptm_options *opt, ptm_context **out) {
     size_t fr = 0, tot = 0;
     cudaMemGetInfo(&fr, &tot);
     ctx->budget = (opt && opt->hbm_budget_bytes) ? opt->hbm_budget_bytes : fr / 2;
-    // the per-atom kernels want every resident block's scratch in shared
+    // the other per-atom kernels want every resident block's scratch in shared
     // memory: the largest shared-memory carveout of the unified L1
     const int smem = (int)std::max(std::max(atom_smem_bytes(), knn_smem_bytes(PTM_TOPO_N)),
                                    std::max(topo_smem_bytes(), topo64_smem_bytes()));
@@ -414,6 +414,12 @@ ptm_status ptm_create(const ptm_options *opt, ptm_context **out) {
                                     (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
         break;
     }
+    // k_match: its resident blocks need 160 KB; the rest caches neighbour records
+    // (4 M atoms: 2.23 -> 2.10 ms; 65 % of the maximum drops a block: 2.21 ms)
+    const void *match[] = {(const void *)k_match<false>, (const void *)k_match<true>, (const void *)k_match_batch<false>,
+                           (const void *)k_match_batch<true>};
+    for (const void *fn : match)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 75);
     if (e != cudaSuccess) { rs = cuda_fail(ctx, e, "cudaFuncSetAttribute"); break; }
   } while (0);
   if (rs != PTM_OK) { ptm_destroy(ctx); return rs; }

@@ -60,9 +60,8 @@ __device__ __forceinline__ int lookup(const Scratch &sm, int K, uint64_t h) {
 // by the walk labelling and the table candidate.
 __device__ __forceinline__ uint64_t slots_of(int K, uint64_t lab, uint64_t cand) {
   uint64_t slots = 0;
-#pragma unroll
-  for (int j = 0; j < PTM_KNN; j++)
-    if (j < K) slots |= (uint64_t)nib(cand, nib(lab, j) - 1) << (4 * j);
+#pragma unroll 2
+  for (int j = K - 1; j >= 0; j--) slots = slots << 4 | (uint64_t)nib(cand, nib(lab, j) - 1);
   return slots;
 }
 
@@ -244,10 +243,12 @@ __device__ uint64_t canonical_corr(int S, int K, uint64_t slots) {
   uint64_t best = ~0ull;
   for (int g = g0; g < g1; g++) {
     const uint64_t inv = __ldg((const unsigned long long *)&ptm_group_inv[__ldg(ptm_coset + g)]);
-    uint64_t cur = 0;
-#pragma unroll
-    for (int j = 0; j < PTM_KNN; j++)
-      if (j < K) cur |= (uint64_t)(j + 1) << (60 - 4 * nib(inv, nib(slots, j)));
+    uint64_t cur = 0, left = slots;
+#pragma unroll 2
+    for (int j = 1; j <= K; j++) {
+      cur |= (uint64_t)j << (60 - 4 * nib(inv, (int)(left & 15)));
+      left >>= 4;
+    }
     best = cur < best ? cur : best;
   }
   return best;
@@ -348,33 +349,50 @@ __device__ __noinline__ int rerank_fp64(const FrameDesc &d, int s, const Best bs
 
 // ------------------------------------------------------------ finalisation
 // Binary alloy label (Sec. 6, Table 3) of atom a matched to template S with
-// canonical correspondence cp (nibble 15 - slot = neighbour rank + 1).
-__device__ __forceinline__ int8_t alloy_label(const FrameDesc &d, const Scratch &sm, int S, uint64_t cp, int64_t a) {
-  int8_t lab8 = PTM_ALLOY_NONE;
-  if (d.species && (S == 1 || S == 4)) {
-    const int8_t c = __ldg(d.species + a);
-    auto same = [&](int sl) { return __ldg(d.species + sm.NID(nib(cp, 15 - sl) - 1)) == c; };
-    if (S == 1) {          // FCC: slots 1-4 in z = 0, 5-8 in y = 0, 9-12 in x = 0
-      int sp = 0, op = 0;
-      for (int p = 0; p < 3; p++) {
-        int n = 0;
-        for (int sl = 1 + 4 * p; sl <= 4 + 4 * p; sl++) n += same(sl);
-        sp += n == 4;
-        op += n == 0;
-      }
-      if (sp == 3) lab8 = PTM_ALLOY_PURE;
-      else if (sp == 1 && op == 2) lab8 = PTM_ALLOY_L10;
-      else if (sp == 2 && op == 1) lab8 = PTM_ALLOY_L12_MAJ;
-      else if (op == 3) lab8 = PTM_ALLOY_L12_MIN;
-    } else {               // BCC: slots 1-8 first shell, 9-14 second shell
-      int in = 0, out = 0;
-      for (int sl = 1; sl <= 8; sl++) in += same(sl);
-      for (int sl = 9; sl <= 14; sl++) out += same(sl);
-      if (in == 8 && out == 6) lab8 = PTM_ALLOY_PURE;
-      else if (in == 0 && out == 6) lab8 = PTM_ALLOY_B2;
-    }
+// neighbour j at template slot nibble j of `slots`.  The counts below do not depend
+// on which of the equivalent correspondences this is: a rotation of the template
+// permutes its {100} planes (fcc) and keeps its shells (bcc).
+__device__ __forceinline__ int8_t alloy_label(const FrameDesc &d, const Scratch &sm, int S, int K, uint64_t slots,
+                                              int64_t a) {
+  if (!d.species || (S != 1 && S != 4)) return PTM_ALLOY_NONE;
+  const int8_t c = __ldg(d.species + a);
+  uint32_t same = 0;                                 // slots whose atom is of the centre's species
+#pragma unroll 4
+  for (int j = 0; j < K; j++) {
+    same |= (uint32_t)(__ldg(d.species + sm.NID(j)) == c) << (int)(slots & 15);
+    slots >>= 4;
   }
-  return lab8;
+  if (S == 1) {            // FCC: slots 1-4 in z = 0, 5-8 in y = 0, 9-12 in x = 0
+    int sp = 0, op = 0;
+#pragma unroll
+    for (int p = 0; p < 3; p++) {
+      const uint32_t plane = same >> (1 + 4 * p) & 15u;
+      sp += plane == 15u;
+      op += plane == 0u;
+    }
+    if (sp == 3) return PTM_ALLOY_PURE;
+    if (sp == 1 && op == 2) return PTM_ALLOY_L10;
+    if (sp == 2 && op == 1) return PTM_ALLOY_L12_MAJ;
+    if (op == 3) return PTM_ALLOY_L12_MIN;
+  } else {                 // BCC: slots 1-8 first shell, 9-14 second shell
+    const uint32_t in = same >> 1 & 255u, out = same >> 9 & 63u;
+    if (in == 255u && out == 63u) return PTM_ALLOY_PURE;
+    if (in == 0u && out == 63u) return PTM_ALLOY_B2;
+  }
+  return PTM_ALLOY_NONE;
+}
+
+// Eigenvalue and quaternion of a winner whose top eigenvalue is not well
+// separated, in FP64 from the same covariance (rare; out of line).
+__device__ __noinline__ void winner_fp64(const float (&Sm)[3][3], float Gv, float Gw, float &lam, float (&q)[4]) {
+  double S64[3][3];
+  for (int a = 0; a < 3; a++) for (int b = 0; b < 3; b++) S64[a][b] = Sm[a][b];
+  Qcp<double> o64;
+  qcp_solve<double>(S64, (double)Gv, (double)Gw, o64);
+  double q64[4];
+  qcp_quat<double>(o64.K, o64.lam, q64);
+  lam = (float)o64.lam;
+  for (int i = 0; i < 4; i++) q[i] = (float)q64[i];
 }
 
 // Outputs of the winner; returns whether the atom is matched (Sec. 5.1).
@@ -396,14 +414,11 @@ __device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
     qcp_solve<float>(Sm, Gv, Gw, o);
     float B = sqrtf(Gv * Gw);
     if (bst.fp64 || !(o.dP / (B * B * B) >= PTM_GAP)) {
-      double S64[3][3];
-      for (int a = 0; a < 3; a++) for (int b = 0; b < 3; b++) S64[a][b] = Sm[a][b];
-      Qcp<double> o64;
-      qcp_solve<double>(S64, (double)Gv, (double)Gw, o64);
-      double q64[4];
-      qcp_quat<double>(o64.K, o64.lam, q64);
-      lam = (float)o64.lam;
-      for (int i = 0; i < 4; i++) q[i] = (float)q64[i];
+      float S1[3][3], lam1, q1[4];                   // copies: only this path puts them in memory
+      for (int a = 0; a < 3; a++) for (int b = 0; b < 3; b++) S1[a][b] = Sm[a][b];
+      winner_fp64(S1, Gv, Gw, lam1, q1);
+      lam = lam1;
+      for (int i = 0; i < 4; i++) q[i] = q1[i];
     } else {
       qcp_quat<float>(o.K, o.lam, q);
       lam = o.lam;
@@ -452,8 +467,10 @@ __device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
   if (d.rmsd) d.rmsd[a] = rmsd;
   if (d.scale) d.scale[a] = s;
   if (d.corr) {
-    d.corr[15 * a] = idi;
-    for (int sl = 1; sl < 15; sl++) d.corr[15 * a + sl] = sl <= K ? sm.NID(nib(cp, 15 - sl) - 1) : -1;
+    int32_t *row = d.corr + 15 * a;
+    row[0] = idi;
+#pragma unroll 2
+    for (int sl = 1; sl < 15; sl++) row[sl] = sl <= K ? sm.NID(nib(cp, 15 - sl) - 1) : -1;
   }
   // orientation in the fundamental zone: the equivalent rotation Q g with the
   // largest |w| (smallest angle); ties keep the earlier group element (Sec. 7)
@@ -509,7 +526,7 @@ __device__ bool finalize(const FrameDesc &d, const Scratch &sm, const float4 *tp
       d.vm[a] = sqrtf(1.5f * (e0 * e0 + e1 * e1 + e2 * e2 + off));
     }
   }
-  if (d.alloy) d.alloy[a] = alloy_label(d, sm, S, cp, a);
+  if (d.alloy) d.alloy[a] = alloy_label(d, sm, S, K, slots, a);
   return true;
 }
 
@@ -575,8 +592,10 @@ __device__ __noinline__ bool finalize_fp64(const FrameDesc &d, const Scratch &sm
   if (d.rmsd) d.rmsd[a] = (float)rmsd;
   if (d.scale) d.scale[a] = (float)s;
   if (d.corr) {
-    d.corr[15 * a] = idi;
-    for (int sl = 1; sl < 15; sl++) d.corr[15 * a + sl] = sl <= K ? sm.NID(nib(cp, 15 - sl) - 1) : -1;
+    int32_t *row = d.corr + 15 * a;
+    row[0] = idi;
+#pragma unroll 2
+    for (int sl = 1; sl < 15; sl++) row[sl] = sl <= K ? sm.NID(nib(cp, 15 - sl) - 1) : -1;
   }
   if (d.quat || d.rf) {
     double bw = -1.0, bq[4] = {1.0, 0.0, 0.0, 0.0};
@@ -619,37 +638,60 @@ __device__ __noinline__ bool finalize_fp64(const FrameDesc &d, const Scratch &sm
       d.vm[a] = (float)sqrt(1.5 * (e0 * e0 + e1 * e1 + e2 * e2 + off));
     }
   }
-  if (d.alloy) d.alloy[a] = alloy_label(d, sm, S, cp, a);
+  if (d.alloy) d.alloy[a] = alloy_label(d, sm, S, K, slots, a);
   return true;
 }
 
-// Neighbour vectors for the metric steps, in rows DX / DY / DZ over the
-// quantised copy (the hulls are done with it), and the neighbours' atom ids in
-// row NID over their sorted indices: the contract values, or for a shifted
-// image an error-free FP32 sum of difference and shift.
+// Neighbour vectors for the metric steps, in rows DX / DY / DZ, and the neighbours'
+// atom ids in row NID: the contract values, or for a shifted image an error-free
+// FP32 sum of difference and shift.  float32 input: every neighbour's record is
+// loaded in one short unrolled pass (two round trips to memory for all of them) and
+// the shifted ones are redone one by one.
 template <bool F64>
 __device__ __forceinline__ void metric_vectors(const FrameDesc &d, const Scratch &sm, const int2 *nb, int64_t nst,
                                                typename RT<F64>::T xi, typename RT<F64>::T yi,
                                                typename RT<F64>::T zi) {
   typedef typename RT<F64>::T T;
-#pragma unroll 7
-  for (int t = 0; t < PTM_KNN; t++) {
-    const int2 e = __ldg(nb + t * nst);
-    if (e.x < 0) { sm.NID(t) = -1; sm.DX(t) = sm.DY(t) = sm.DZ(t) = 0.f; continue; }
-    T xj, yj, zj;
-    int idj;
-    load_atom<F64>(d, e.x, xj, yj, zj, idj);
-    sm.NID(t) = idj;
-    int a0, a1, a2;
-    img_unpack(e.y, a0, a1, a2);
-    if constexpr (F64) {
+  if constexpr (F64) {
+#pragma unroll 2
+    for (int t = 0; t < PTM_KNN; t++) {
+      const int2 e = __ldg(nb + t * nst);
+      if (e.x < 0) { sm.NID(t) = -1; sm.DX(t) = sm.DY(t) = sm.DZ(t) = 0.f; continue; }
+      T xj, yj, zj;
+      int idj;
+      load_atom<F64>(d, e.x, xj, yj, zj, idj);
+      sm.NID(t) = idj;
+      int a0, a1, a2;
+      img_unpack(e.y, a0, a1, a2);
       T sx, sy, sz;
       contract_shift<F64>(d, a0, a1, a2, sx, sy, sz);
       sm.DX(t) = (float)contract_dr(xj, xi, sx); sm.DY(t) = (float)contract_dr(yj, yi, sy);
       sm.DZ(t) = (float)contract_dr(zj, zi, sz);
-    } else if (a0 == 0 && a1 == 0 && a2 == 0) {
-      sm.DX(t) = __fsub_rn(xj, xi); sm.DY(t) = __fsub_rn(yj, yi); sm.DZ(t) = __fsub_rn(zj, zi);
-    } else {
+    }
+  } else {
+    uint32_t shifted = 0;
+    int2 e[PTM_KNN];
+#pragma unroll
+    for (int t = 0; t < PTM_KNN; t++) e[t] = __ldg(nb + t * nst);
+#pragma unroll
+    for (int t = 0; t < PTM_KNN; t++) {
+      const bool none = e[t].x < 0;
+      float xj, yj, zj;
+      int idj;
+      load_atom<F64>(d, max(e[t].x, 0), xj, yj, zj, idj);
+      sm.NID(t) = none ? -1 : idj;
+      sm.DX(t) = none ? 0.f : __fsub_rn(xj, xi); sm.DY(t) = none ? 0.f : __fsub_rn(yj, yi);
+      sm.DZ(t) = none ? 0.f : __fsub_rn(zj, zi);
+      shifted |= (uint32_t)(!none && e[t].y != img_pack(0, 0, 0)) << t;
+    }
+    for (; shifted; shifted &= shifted - 1) {
+      const int t = __ffs(shifted) - 1;
+      const int2 en = __ldg(nb + t * nst);
+      float xj, yj, zj;
+      int idj;
+      load_atom<F64>(d, en.x, xj, yj, zj, idj);
+      int a0, a1, a2;
+      img_unpack(en.y, a0, a1, a2);
       float hx, hy, hz, lx, ly, lz;
       shift_f32(d, a0, a1, a2, hx, hy, hz, lx, ly, lz);
       float p, e1, q2, e2;
@@ -1205,6 +1247,12 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_ATOM_BLOCKS_PER_SM) k_hulls(con
   count_warp(d, C_SOS, live, nsos);
 }
 
+// Bounded by instruction fetch and latency at 11 blocks per SM: its warps stand
+// at different points of 50 KB of straight code, so the loops over neighbours stay
+// rolled or short and the FP64 paths out of line (unrolled and inline: 80 KB; 4 M
+// atoms 2.72 -> 2.48 ms).  The neighbours' loads are the exception: all in flight at
+// once (-> 2.23 ms).  At 10, 9 and 8 blocks (more registers): 2.86, 2.82, 3.06 ms
+// against 2.72.
 template <bool F64, bool P64 = false>
 __global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM) k_match(const __grid_constant__ FrameDesc d) {
   extern __shared__ __align__(16) unsigned char smem[];

@@ -247,22 +247,37 @@ __device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__re
         cnt++;
       }
     };
+    // U loads in flight: the loop's stores keep the compiler from moving the next
+    // candidate's load above them (U = 1, 2, 4 for plain positions: 1.59, 1.84, 1.57
+    // ms per 4 M atoms; 1, 2, 3 for pairs: 168, 180, 148 us per 200 k)
+    constexpr int U = SPLIT ? 3 : 4;
     if (SPLIT || shifted) {
-#pragma unroll 2
-      for (; j < j1; j++) {
-        const float4 p = __ldg(hi + j);
-        if constexpr (SPLIT) {
-          const float4 q = __ldg(d.lo + j);
-          test(j, (p.x - hx) + (q.x - lx), (p.y - hy) + (q.y - ly), (p.z - hz) + (q.z - lz));
-        } else {
-          test(j, (p.x - hx) - lx, (p.y - hy) - ly, (p.z - hz) - lz);
+      for (; j < j1; j += U) {
+        float4 p[U], q[U];
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+          p[k] = __ldg(hi + min(j + k, j1 - 1));
+          if constexpr (SPLIT) q[k] = __ldg(d.lo + min(j + k, j1 - 1));
+        }
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+          if (k && j + k >= j1) break;
+          if constexpr (SPLIT)
+            test(j + k, (p[k].x - hx) + (q[k].x - lx), (p[k].y - hy) + (q[k].y - ly), (p[k].z - hz) + (q[k].z - lz));
+          else
+            test(j + k, (p[k].x - hx) - lx, (p[k].y - hy) - ly, (p[k].z - hz) - lz);
         }
       }
     } else {
-#pragma unroll 4
-      for (; j < j1; j++) {
-        const float4 p = __ldg(hi + j);
-        test(j, p.x - hx, p.y - hy, p.z - hz);
+      for (; j < j1; j += U) {
+        float4 p[U];
+#pragma unroll
+        for (int k = 0; k < U; k++) p[k] = __ldg(hi + min(j + k, j1 - 1));
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+          if (k && j + k >= j1) break;
+          test(j + k, p[k].x - hx, p[k].y - hy, p[k].z - hz);
+        }
       }
     }
   });
@@ -462,13 +477,14 @@ __device__ __forceinline__ float knn_err(float v, float S) {
 
 // The NK nearest images of atom s by the full key (FP64 d2, atom id, image), R
 // growing until the NK-th distance lies inside the radius the scanned cells are
-// guaranteed to cover.  One warp: the lanes take a column's atoms 32 at a time,
-// and lane t holds the t-th smallest key so far, so an insertion is a ballot and
-// a shift by one lane.  For float32 input a candidate whose FP32 distance, less
-// its error bound, exceeds the current NK-th key cannot enter and skips the
-// FP64 evaluation.  (One thread per such atom, its list in local memory, took
-// 0.4 ms for the 58 of a 2^20-atom frame: one warp's serial chain at the end of
-// the launch.)
+// guaranteed to cover; each R adds the cells of its shell to the list so far.  One
+// warp: every lane walks a cell of its own, and lane t holds the t-th smallest key
+// so far, so an insertion is a ballot and a shift by one lane.  For float32 input
+// a candidate whose FP32 distance, less its error bound, exceeds the current
+// NK-th key cannot enter and skips the FP64 evaluation.  Few atoms come here and
+// the kernel lasts as long as its slowest: the 58 of a 2^20-atom frame took 0.40 ms
+// with a thread each and lists in local memory, 0.20 ms with a warp reading column
+// by column and starting over at each R, 0.06 ms now.
 template <bool F64, int NK>
 __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
   typedef typename RT<F64>::T T;
@@ -484,77 +500,70 @@ __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
   img_unpack(__ldg(d.wrapv + s), wi0, wi1, wi2);
   const int nbx = d.nb[0], nby = d.nb[1], nbz = d.nb[2];
   const uint64_t INF = 0x7ff0000000000000ull;
-  uint64_t lk = INF;
+  uint64_t lk = INF, last = INF;                       // this lane's key; the NK-th key,
+  float last32 = INFINITY;                             // ... rounded up to FP32
   int lid = 0x7fffffff, lj = -1, limg = 0x7fffffff, found = -1;
   for (int R = 1; R <= PTM_RMAX; R++) {
-    lk = INF; lid = 0x7fffffff; lj = -1; limg = 0x7fffffff;
-    uint64_t last = INF;                               // the NK-th key, and rounded up to FP32
-    float last32 = INFINITY;
-    for (int ix = -R; ix <= R; ix++) {
-      int cx = bx + ix, mx = 0;
-      if (d.pbc[0]) { mx = floordiv(cx, nbx); cx -= mx * nbx; } else if (cx < 0 || cx >= nbx) continue;
-      for (int iy = -R; iy <= R; iy++) {
-        int cy = by + iy, my = 0;
-        if (d.pbc[1]) { my = floordiv(cy, nby); cy -= my * nby; } else if (cy < 0 || cy >= nby) continue;
-        int z0 = bz - R, z1 = bz + R;
-        if (!d.pbc[2]) { z0 = max(z0, 0); z1 = min(z1, nbz - 1); }
-        const bool column = z0 >= 0 && z1 < nbz;
-        const int cbase = (cx * nby + cy) * nbz;
-        for (int r = 0; r < (column ? 1 : 2 * R + 1); r++) {
-          int ca = cbase + z0, cb = cbase + z1, mz = 0;
-          if (!column) {
-            int cz = bz - R + r;
-            mz = floordiv(cz, nbz);
-            cz -= mz * nbz;
-            ca = cb = cbase + cz;
-          }
-          const int j0 = __ldg(d.cell_start + ca), j1 = __ldg(d.cell_start + cb + 1);
-          for (int jb = j0; jb < j1; jb += 32) {
-            const int j = jb + lane;
-            uint64_t key = INF;
-            int idj = 0x7fffffff, img = 0x7fffffff;
-            if (j < j1) {
-              T xj, yj, zj;
-              load_atom<F64>(d, j, xj, yj, zj, idj);
-              int w0, w1, w2;
-              img_unpack(__ldg(d.wrapv + j), w0, w1, w2);
-              const int a0 = mx + wi0 - w0, a1 = my + wi1 - w1, a2 = mz + wi2 - w2;
-              T sx, sy, sz;
-              contract_shift<F64>(d, a0, a1, a2, sx, sy, sz);
-              const T v = contract_d2(contract_dr(xj, xi, sx), contract_dr(yj, yi, sy), contract_dr(zj, zi, sz));
-              img = img_pack(a0, a1, a2);
-              bool in = !(j == s && a0 == 0 && a1 == 0 && a2 == 0) && __ldg(d.wrapv + j) != PTM_EXCLUDED;
-              if constexpr (!F64) {
-                const float S = sqrtf(sx * sx + sy * sy + sz * sz) * 1.0001f;
-                in = in && !(v - 1.25f * knn_err(v, S) > last32);
-              }
-              if (in) {
-                double k64;
-                if constexpr (F64) k64 = v;
-                else k64 = key64(d, xj, yj, zj, xi, yi, zi, a0, a1, a2);
-                key = (uint64_t)__double_as_longlong(k64);
-              }
+    const int side = 2 * R + 1;
+    for (int c0 = 0; c0 < side * side * side; c0 += 32) {
+      // this lane's cell: offsets (ix, iy, iz) in [-R, R]^3, not in an earlier shell
+      const int c = c0 + lane;
+      const int iz = c % side - R, iy = c / side % side - R, ix = c / (side * side) - R;
+      int cx = bx + ix, cy = by + iy, cz = bz + iz;
+      const int mx = floordiv(cx, nbx), my = floordiv(cy, nby), mz = floordiv(cz, nbz);
+      const bool in_shell = ix <= R && (R == 1 || max(abs(ix), max(abs(iy), abs(iz))) == R) && (d.pbc[0] || mx == 0) &&
+                            (d.pbc[1] || my == 0) && (d.pbc[2] || mz == 0);
+      cx -= mx * nbx; cy -= my * nby; cz -= mz * nbz;
+      int j = 0, j1 = 0;
+      if (in_shell) {
+        const int cell = (cx * nby + cy) * nbz + cz;
+        j = __ldg(d.cell_start + cell);
+        j1 = __ldg(d.cell_start + cell + 1);
+      }
+      for (; __any_sync(ALL, j < j1); j++) {
+        uint64_t key = INF;
+        int idj = 0x7fffffff, img = 0x7fffffff;
+        if (j < j1) {
+          T xj, yj, zj;
+          load_atom<F64>(d, j, xj, yj, zj, idj);
+          const int w = __ldg(d.wrapv + j);
+          int w0, w1, w2;
+          img_unpack(w, w0, w1, w2);
+          const int a0 = mx + wi0 - w0, a1 = my + wi1 - w1, a2 = mz + wi2 - w2;
+          bool in = !(j == s && a0 == 0 && a1 == 0 && a2 == 0) && w != PTM_EXCLUDED;
+          if (in) {
+            T sx, sy, sz;
+            contract_shift<F64>(d, a0, a1, a2, sx, sy, sz);
+            const T v = contract_d2(contract_dr(xj, xi, sx), contract_dr(yj, yi, sy), contract_dr(zj, zi, sz));
+            img = img_pack(a0, a1, a2);
+            if constexpr (!F64) {
+              const float S = sqrtf(sx * sx + sy * sy + sz * sz) * 1.0001f;
+              in = !(v - 1.25f * knn_err(v, S) > last32);
             }
-            // NaN keys (an excluded atom's) compare above INF and never enter
-            unsigned m = __ballot_sync(ALL, key < INF && key <= last);
-            while (m) {
-              const int src = __ffs(m) - 1;
-              m &= m - 1;
-              const uint64_t ck = __shfl_sync(ALL, key, src);
-              const int cid = __shfl_sync(ALL, idj, src), cimg = __shfl_sync(ALL, img, src);
-              const bool lt = key_less64(ck, cid, cimg, lk, lid, limg);
-              const unsigned at = __ballot_sync(ALL, lt) & ((1u << NK) - 1u);
-              if (!at) continue;                         // not below the NK-th key any more
-              const uint64_t uk = __shfl_up_sync(ALL, lk, 1);
-              const int uid = __shfl_up_sync(ALL, lid, 1), uj = __shfl_up_sync(ALL, lj, 1),
-                        uimg = __shfl_up_sync(ALL, limg, 1);
-              const int first = __ffs(at) - 1;           // the keys are sorted: every lane above moves up
-              if (lane == first) { lk = ck; lid = cid; lj = jb + src; limg = cimg; }
-              else if (lane > first) { lk = uk; lid = uid; lj = uj; limg = uimg; }
-              last = __shfl_sync(ALL, lk, NK - 1);
-              if constexpr (!F64) last32 = __double2float_ru(__longlong_as_double((long long)last));
+            if (in) {
+              double k64;
+              if constexpr (F64) k64 = v;
+              else k64 = key64(d, xj, yj, zj, xi, yi, zi, a0, a1, a2);
+              key = (uint64_t)__double_as_longlong(k64);
             }
           }
+        }
+        unsigned m = __ballot_sync(ALL, key < INF && key <= last);
+        while (m) {
+          const int src = __ffs(m) - 1;
+          m &= m - 1;
+          const uint64_t ck = __shfl_sync(ALL, key, src);
+          const int cid = __shfl_sync(ALL, idj, src), cimg = __shfl_sync(ALL, img, src), cj = __shfl_sync(ALL, j, src);
+          const unsigned at = __ballot_sync(ALL, key_less64(ck, cid, cimg, lk, lid, limg)) & ((1u << NK) - 1u);
+          if (!at) continue;                             // not below the NK-th key any more
+          const uint64_t uk = __shfl_up_sync(ALL, lk, 1);
+          const int uid = __shfl_up_sync(ALL, lid, 1), uj = __shfl_up_sync(ALL, lj, 1),
+                    uimg = __shfl_up_sync(ALL, limg, 1);
+          const int first = __ffs(at) - 1;               // the keys are sorted: every lane above moves up
+          if (lane == first) { lk = ck; lid = cid; lj = cj; limg = cimg; }
+          else if (lane > first) { lk = uk; lid = uid; lj = uj; limg = uimg; }
+          last = __shfl_sync(ALL, lk, NK - 1);
+          if constexpr (!F64) last32 = __double2float_ru(__longlong_as_double((long long)last));
         }
       }
     }

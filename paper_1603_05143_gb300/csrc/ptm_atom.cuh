@@ -6,7 +6,7 @@
 //   neighbour vectors, quantised copy for the exact hull predicates
 //   ONE incremental convex hull over neighbours 1..14; the hulls of the first
 //   6 and 12 neighbours are its intermediate states (Sec. 4)
-//   at k = 6, 12, 14: centre-inside test, canonical Weinberg code, template lookup
+//   at k = 6, 12, 14: centre-inside test, graph code, template lookup
 //   QCP superposition of each admissible correspondence (Eq. 3-4)
 //   selection, then orientation (Sec. 7), strain (Sec. 8) and alloy (Sec. 6).
 //
@@ -108,19 +108,16 @@ __device__ __forceinline__ void count_here(const FrameDesc &d, int which) {
 
 // ------------------------------------------------------------ shared scratch
 // Rows are [word][thread] (every lane its own bank).  In k_hulls the 42 rows of
-// q hold the quantised neighbour vectors while the hulls are built, beside the
-// rotation system, code, facet and edge rows: 98 words per thread let 8 blocks
-// of 64 threads share an SM's 228 KB.  k_match uses only q (the FP32 metric
-// vectors), nid (the neighbours' sorted indices, then their atom ids) and img.
+// q hold the quantised neighbour vectors, beside the rotation system, facet and
+// edge rows: 108 words per thread let 8 blocks of 64 threads share an SM's 228 KB.
+// k_match uses only q (the FP32 metric vectors) and nid (the neighbours' atom ids).
 struct Scratch {
   float *q;          // [42][B]  quantised neighbour vectors (integers |q| <= 2^19, exact in FP32),
-                     //          then the metric vectors DX / DY / DZ
-  int *nid;          // [14][B]  neighbour sorted index, then atom id (k_match)
-  int *img;          // [14][B]  neighbour image (img_pack) (k_match)
-  uint16_t *fac;     // [24][B]  hull facets a | b << 4 | c << 8 (ccw from outside)
-  uint64_t *th;      // [14][B]  third vertex of directed edge u->v, nibble v of row u (0xF none)
-  uint16_t *used;    // [14][B]  directed-edge bit rows (hull horizon, Weinberg walk)
-  uint32_t *code;    // [9][B]   best Weinberg code so far from its third label on (nibbles)
+                     //          or the metric vectors DX / DY / DZ
+  int *nid;          // [14][B]  neighbour atom id (k_match)
+  uint32_t *fac;     // [24][B]  hull facets a | b << 4 | c << 8 (ccw from outside) | birth number << 12
+  uint64_t *th;      // [14][B]  1 + third vertex of directed edge u->v, nibble v of row u (0 none)
+  uint32_t *used;    // [14][B]  directed-edge rows (hull horizon, start edges), breadth-first code
   int t;             // thread index in block
   __device__ __forceinline__ float &Q(int p, int c) const { return q[(3 * p + c) * PTM_BLOCK + t]; }
   __device__ __forceinline__ int QI(int p, int c) const { return (int)q[(3 * p + c) * PTM_BLOCK + t]; }
@@ -128,15 +125,12 @@ struct Scratch {
   __device__ __forceinline__ float &DY(int j) const { return Q(j, 1); }
   __device__ __forceinline__ float &DZ(int j) const { return Q(j, 2); }
   __device__ __forceinline__ int &NID(int j) const { return nid[j * PTM_BLOCK + t]; }
-  __device__ __forceinline__ int &IMG(int j) const { return img[j * PTM_BLOCK + t]; }
-  __device__ __forceinline__ uint16_t &F(int f) const { return fac[f * PTM_BLOCK + t]; }
+  __device__ __forceinline__ uint32_t &F(int f) const { return fac[f * PTM_BLOCK + t]; }
   __device__ __forceinline__ uint64_t &TH(int v) const { return th[v * PTM_BLOCK + t]; }
-  __device__ __forceinline__ uint16_t &U(int v) const { return used[v * PTM_BLOCK + t]; }
-  __device__ __forceinline__ uint32_t &CODE(int w) const { return code[w * PTM_BLOCK + t]; }
+  __device__ __forceinline__ uint32_t &U(int v) const { return used[v * PTM_BLOCK + t]; }
 };
 
-#define PTM_CODE_WORDS 9       // 71 nibbles: labels 3..73 of the longest code (labels 1, 2 are fixed)
-constexpr int SCRATCH_WORDS = 28 + 42 + PTM_CODE_WORDS + 12 + 7;   // 32-bit words per k_hulls thread
+constexpr int SCRATCH_WORDS = 28 + 42 + 24 + 14;   // 32-bit words per k_hulls thread
 
 // -------------------------------------------------------------- small helpers
 __device__ __forceinline__ int nib(uint64_t x, int i) { return (int)((x >> (4 * i)) & 15); }
@@ -298,17 +292,20 @@ __device__ __forceinline__ int orient_sos(const Scratch &sm, int a, int b, int c
 }
 
 // ------------------------------------------------------------ incremental hull
-__device__ __forceinline__ uint16_t fpack(int a, int b, int c) { return (uint16_t)(a | (b << 4) | (c << 8)); }
+// A facet's birth number orders the facets by creation (survivors of an insertion
+// before its new ones), whichever row they sit in.
+__device__ __forceinline__ uint32_t fpack(int a, int b, int c, int birth) {
+  return (uint32_t)(a | (b << 4) | (c << 8) | (birth << 12));
+}
 
 // Tetrahedron on points 0..3, facets counter-clockwise seen from outside.
-__device__ __forceinline__ int hull_init(const Scratch &sm, int &nsos) {
+__device__ __forceinline__ void hull_init(const Scratch &sm, int &nsos) {
   int o = orient_sos(sm, 0, 1, 2, 3, sm.Q(3, 0), sm.Q(3, 1), sm.Q(3, 2), nsos);
   if (o < 0) {
-    sm.F(0) = fpack(0, 1, 2); sm.F(1) = fpack(0, 3, 1); sm.F(2) = fpack(1, 3, 2); sm.F(3) = fpack(0, 2, 3);
+    sm.F(0) = fpack(0, 1, 2, 0); sm.F(1) = fpack(0, 3, 1, 1); sm.F(2) = fpack(1, 3, 2, 2); sm.F(3) = fpack(0, 2, 3, 3);
   } else {
-    sm.F(0) = fpack(0, 2, 1); sm.F(1) = fpack(0, 3, 2); sm.F(2) = fpack(2, 3, 1); sm.F(3) = fpack(0, 1, 3);
+    sm.F(0) = fpack(0, 2, 1, 0); sm.F(1) = fpack(0, 3, 2, 1); sm.F(2) = fpack(2, 3, 1, 2); sm.F(3) = fpack(0, 1, 3, 3);
   }
-  return 4;
 }
 
 // Signs of orient(a, b, c, p) and orient(a, b, c, origin) with the FP32 filter
@@ -343,7 +340,7 @@ __device__ __forceinline__ void hull_exact(const Scratch &sm, int p, uint32_t op
     if (!open) continue;
     const int f = __ffs(open) - 1;
     open &= open - 1;
-    const int v = sm.F(f);
+    const uint32_t v = sm.F(f);
     const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
     const int ax = sm.QI(a, 0), ay = sm.QI(a, 1), az = sm.QI(a, 2);
     const int ux = sm.QI(b, 0) - ax, uy = sm.QI(b, 1) - ay, uz = sm.QI(b, 2) - az;
@@ -364,30 +361,37 @@ __device__ __forceinline__ void hull_exact(const Scratch &sm, int p, uint32_t op
   }
 }
 
-// Facets of the current hull visible from point p (bit f set), and whether the
-// centre lies strictly inside the current hull (exact, no SoS: zero rejects),
-// computed only when `centre` is asked for.  Both use one normal per facet.
-// `wmask`: the lanes of the warp that call this together.
-__device__ uint32_t hull_visibility(const Scratch &sm, int nf, int p, bool centre, bool &centre_in, unsigned wmask,
-                                    int &nsos) {
+// Facets of the current hull visible from point p (bit f set), and with CENTRE
+// whether the centre lies strictly inside the current hull (exact, no SoS: zero
+// rejects); both then use one normal per facet.  `wmask`: the lanes of the warp
+// that call this together.
+template <bool CENTRE>
+__device__ __forceinline__ uint32_t hull_visibility(const Scratch &sm, int nf, int p, bool &centre_in, unsigned wmask,
+                                                    int &nsos) {
   uint32_t vis = 0, openp = 0, openc = 0;
   bool inside = true;
   const float px = sm.Q(p, 0), py = sm.Q(p, 1), pz = sm.Q(p, 2);
 #pragma unroll 2
   for (int f = 0; f < nf; f++) {
-    const int v = sm.F(f);
+    const uint32_t v = sm.F(f);
     const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
-    int sp, sc;
-    orient_pair_filter(sm.Q(a, 0), sm.Q(a, 1), sm.Q(a, 2), sm.Q(b, 0), sm.Q(b, 1), sm.Q(b, 2), sm.Q(c, 0),
-                       sm.Q(c, 1), sm.Q(c, 2), px, py, pz, sp, sc);
+    int sp, sc = 1;
+    if constexpr (CENTRE)
+      orient_pair_filter(sm.Q(a, 0), sm.Q(a, 1), sm.Q(a, 2), sm.Q(b, 0), sm.Q(b, 1), sm.Q(b, 2), sm.Q(c, 0),
+                         sm.Q(c, 1), sm.Q(c, 2), px, py, pz, sp, sc);
+    else
+      sp = orient_filter(sm.Q(a, 0), sm.Q(a, 1), sm.Q(a, 2), sm.Q(b, 0), sm.Q(b, 1), sm.Q(b, 2), sm.Q(c, 0),
+                         sm.Q(c, 1), sm.Q(c, 2), px, py, pz);
     if (sp > 0) vis |= 1u << f;
     if (!sp) openp |= 1u << f;
-    if (!sc) openc |= 1u << f;
-    inside &= sc <= 0;
+    if constexpr (CENTRE) {
+      if (!sc) openc |= 1u << f;
+      inside &= sc <= 0;
+    }
   }
-  if (!centre || !inside) openc = 0;          // the centre's answer is already known
+  if (!inside) openc = 0;                     // the centre's answer is already known
   hull_exact(sm, p, openp, openc, wmask, vis, inside, nsos);
-  centre_in = centre && inside;
+  centre_in = CENTRE && inside;
   return vis;
 }
 
@@ -398,7 +402,7 @@ __device__ bool hull_centre_inside(const Scratch &sm, int nf, unsigned wmask, in
   uint32_t openc = 0;
 #pragma unroll 1
   for (int f = 0; f < nf; f++) {
-    const int v = sm.F(f);
+    const uint32_t v = sm.F(f);
     const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
     int sp, sc;
     orient_pair_filter(sm.Q(a, 0), sm.Q(a, 1), sm.Q(a, 2), sm.Q(b, 0), sm.Q(b, 1), sm.Q(b, 2), sm.Q(c, 0),
@@ -412,182 +416,143 @@ __device__ bool hull_centre_inside(const Scratch &sm, int nf, unsigned wmask, in
   return inside;
 }
 
-// Insert point p given its visible facets (vis != 0): remove them and fan the
-// horizon to p.  Returns the new facet count, or -1 on an internal error.
-__device__ int hull_apply(const Scratch &sm, int nf, uint32_t vis, int p, const FrameDesc &d) {
-  // edge rows of the vertices of the visible facets only (no other row is read)
+// Insert point p given its visible facets (vis != 0): the fan of the horizon's
+// edges to p takes the rows of the visible facets and two more.  Row u of `used`
+// holds the vertices that visible facets' edges lead to from u (low half) and
+// come from (high half): a horizon edge u -> v is one whose reverse no visible
+// facet has, so each row decides its own edges.  Returns false when the hull no
+// longer has all points as vertices (no later snapshot can match: the insertion
+// swallowed a vertex and left fewer than two facets more), or on an internal error.
+__device__ __forceinline__ bool hull_apply(const Scratch &sm, int nf, uint32_t vis, int p, int &birth,
+                                           const FrameDesc &d) {
   uint32_t verts = 0;
   for (uint32_t m = vis; m; m &= m - 1) {
-    const int v = sm.F(__ffs(m) - 1);
-    verts |= (1u << (v & 15)) | (1u << ((v >> 4) & 15)) | (1u << ((v >> 8) & 15));
+    const uint32_t v = sm.F(__ffs(m) - 1);
+    const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
+    const uint32_t ba = 1u << a, bb = 1u << b, bc = 1u << c;
+    const uint32_t ra = verts & ba ? sm.U(a) : 0u, rb = verts & bb ? sm.U(b) : 0u, rc = verts & bc ? sm.U(c) : 0u;
+    sm.U(a) = ra | bb | bc << 16;
+    sm.U(b) = rb | bc | ba << 16;
+    sm.U(c) = rc | ba | bb << 16;
+    verts |= ba | bb | bc;
   }
-  for (uint32_t m = verts; m; m &= m - 1) sm.U(__ffs(m) - 1) = 0;
-  for (uint32_t m = vis; m; m &= m - 1) {
-    int v = sm.F(__ffs(m) - 1);
-    int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
-    sm.U(a) |= 1 << b; sm.U(b) |= 1 << c; sm.U(c) |= 1 << a;
-  }
-  int n2 = 0;
-  for (int f = 0; f < nf; f++)
-    if (!(vis >> f & 1)) sm.F(n2++) = sm.F(f);
+  const int nvis = __popc(vis);
   int added = 0;
+  uint32_t free = vis;
   for (uint32_t mu = verts; mu; mu &= mu - 1) {      // rows in increasing vertex order
     const int u = __ffs(mu) - 1;
-    uint32_t row = sm.U(u);
-    while (row) {
-      int v = __ffs(row) - 1;
-      row &= row - 1;
-      if (!(sm.U(v) >> u & 1)) {               // horizon edge u -> v
-        if (n2 < 24) sm.F(n2) = fpack(u, v, p);
-        n2++;
-        added++;
-      }
+    const uint32_t w = sm.U(u);
+    for (uint32_t row = w & ~(w >> 16) & 0xffffu; row; row &= row - 1) {      // horizon edges u -> v
+      const int v = __ffs(row) - 1;
+      const int slot = free ? __ffs(free) - 1 : nf + added - nvis;
+      free &= free - 1;
+      if (added < nvis + 2) sm.F(slot) = fpack(u, v, p, birth + added);
+      added++;
     }
   }
+  birth += added;
   // a triangulated disk of F visible facets with I interior vertices has
-  // F + 2 - 2I boundary edges; swallowed vertices simply leave the facet list
-  if (added < 3 || added > __popc(vis) + 2 || ((added - __popc(vis)) & 1) || n2 > 24) {
-    count(d, C_INTERNAL);
-    return -1;
-  }
-  return n2;
+  // F + 2 - 2I boundary edges
+  if (added == nvis + 2) return true;
+  if (added < 3 || added > nvis + 2 || ((added - nvis) & 1)) count(d, C_INTERNAL);
+  return false;
 }
 
-// ------------------------------------------------------- Weinberg code
-// Walk from u -> v over the K-vertex hull (rules in tables.py), writing the
-// code (labels 3.. as nibbles; every walk starts with labels 1, 2) to the CODE
-// rows and the first-visit labelling to `labels`.  False on an internal error.
-__device__ bool weinberg_walk(const Scratch &sm, int K, int u, int v, uint64_t &labels, const FrameDesc &d) {
-  const int LEN = 2 * (3 * K - 6) + 1;
-  uint64_t lab = 0;
-#pragma unroll
-  for (int x = 0; x < PTM_KNN; x++) sm.U(x) = 0;
-  int next = 1;
-  uint32_t wbuf = 0;
-  auto emit = [&](int s, int L) {
-    const int n = s - 2;
-    wbuf |= (uint32_t)L << (4 * (n & 7));
-    if ((n & 7) == 7 || s == LEN - 1) { sm.CODE(n >> 3) = wbuf; wbuf = 0; }
-  };
-  lab = setnib(lab, u, next++);
-  sm.U(u) |= 1 << v;
-  bool fresh = true;
-  lab = setnib(lab, v, next++);
-  int s = 2;
-  for (; s < LEN; s++) {
-    const uint64_t tv = sm.TH(v);
-    const uint32_t uv = sm.U(v);
-    int w = nib(tv, u);                              // next edge counter-clockwise
-    if (!fresh) {
-      if (!(uv >> u & 1)) {
-        w = u;                                       // old vertex, new edge: walk back
-      } else {
-        int guard = 0;                               // first unused edge after arrival
-        while (w != u && (uv >> w & 1) && guard++ < 16) w = nib(tv, w);
-        if (w == u || guard > 16) break;
-      }
+// ------------------------------------------------------- graph code and lookup
+// Hull of the first K neighbours (every one a vertex, 2 K - 4 facets, the centre
+// inside): template lookup (Algorithm 1, inner loops).  Writes the Weinberg
+// labelling (nibble t = label of neighbour t) and the candidate list's entry;
+// false if no template has this graph.
+//
+// A Weinberg walk labels the hull from the start edge with the largest key of
+// degrees around it (tables.py).  Finding that edge and walking cost 3 of every 5
+// instructions here.  The graph is instead looked up by its adjacency matrix
+// under a breadth-first labelling from any directed edge (the first facet's
+// first), one step per directed edge with the current vertex's row in a register;
+// the table then names the graph's start edges, and their Weinberg labels in terms
+// of these.  Of several start edges the first among the facets is taken.
+__device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, uint64_t &labels, int &ent, const FrameDesc &d) {
+  const int nf = 2 * K - 4;
+#pragma unroll 2
+  for (int x = 0; x < K; x++) sm.TH(x) = 0;
+  uint32_t first = 0xffffffffu;                      // the facet with the smallest birth number
+  for (int f = 0; f < nf; f++) {
+    const uint32_t v = sm.F(f);
+    const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
+    const uint64_t ta = sm.TH(a), tb = sm.TH(b), tc = sm.TH(c);
+    sm.TH(a) = ta | (uint64_t)(c + 1) << (4 * b);
+    sm.TH(b) = tb | (uint64_t)(a + 1) << (4 * c);
+    sm.TH(c) = tc | (uint64_t)(b + 1) << (4 * a);
+    first = min(first, v);
+  }
+  int x = first & 15, from = (first >> 4) & 15, cur = from, next = 2, i = 0;
+  uint32_t seen = 1u << x | 1u << from, row = 0, even = 0;
+  uint64_t lab = 1ull << (4 * from), vert = (uint64_t)x | (uint64_t)from << 4, come = (uint64_t)from | (uint64_t)x << 4;
+  uint64_t th = sm.TH(x);
+#pragma unroll 1
+  for (int s = 0; s < 6 * K - 12; s++) {
+    cur = (nib(th, cur) - 1) & 15;                   // next neighbour of x, counter-clockwise
+    if (!(seen >> cur & 1)) {
+      lab |= (uint64_t)next << (4 * cur);
+      vert |= (uint64_t)cur << (4 * next);
+      come |= (uint64_t)x << (4 * next);
+      seen |= 1u << cur;
+      next++;
     }
-    if (w >= K) { count(d, C_INTERNAL); return false; }
-    sm.U(v) = (uint16_t)(uv | (1u << w));
-    u = v;
-    v = w;
-    int L = nib(lab, v);
-    fresh = (L == 0);
-    if (fresh) { L = next++; lab = setnib(lab, v, L); }
-    emit(s, L);
-  }
-  if (s != LEN) { count(d, C_INTERNAL); return false; }
-  labels = lab;
-  return true;
-}
-
-// Weinberg code of the current K-vertex hull for the table lookup.  Every
-// directed edge u->v gets the key (deg u, deg v, deg w1, deg w2) with (u, v, w1)
-// and (v, u, w2) the two facets on the edge, continued (for edges tied on it)
-// by the degrees of the third vertices of the facets across their four outer
-// edges; the walk starts from the first edge with the largest key (definition
-// in tables.py, whose tables hold the code of every such start).  Returns the
-// labelling (nibble t = label of neighbour t) and the code hash; false on an
-// internal error.  Every lane walks once, so a warp's walks run together.
-__device__ bool canonical(const Scratch &sm, int K, int nf, uint64_t &labels, uint64_t &hash,
-                          const FrameDesc &d) {
-  uint64_t deg = 0;
-#pragma unroll
-  for (int x = 0; x < PTM_KNN; x++) sm.TH(x) = ~0ull;
-  for (int f = 0; f < nf; f++) {
-    int v = sm.F(f);
-    int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
-    sm.TH(a) = setnib(sm.TH(a), b, c);
-    sm.TH(b) = setnib(sm.TH(b), c, a);
-    sm.TH(c) = setnib(sm.TH(c), a, b);
-    deg += (1ull << (4 * a)) + (1ull << (4 * b)) + (1ull << (4 * c));
-  }
-  // keys of the directed edges (a->b, b->c, c->a of every facet); keep the maximum
-  uint32_t top = 0;
-  uint64_t m0 = 0;          // edge ids 0..63 (id = 3 f + corner)
-  uint32_t m1 = 0;          // edge ids 64..71
-  for (int f = 0; f < nf; f++) {
-    const int v = sm.F(f);
-    const int p0 = v & 15, p1 = (v >> 4) & 15, p2 = (v >> 8) & 15;
-    const int dg0 = nib(deg, p0), dg1 = nib(deg, p1), dg2 = nib(deg, p2);
-#pragma unroll
-    for (int e = 0; e < 3; e++) {
-      const int x = e == 0 ? p0 : (e == 1 ? p1 : p2);      // edge x -> y, third vertex z
-      const int y = e == 0 ? p1 : (e == 1 ? p2 : p0);
-      const int dx = e == 0 ? dg0 : (e == 1 ? dg1 : dg2);
-      const int dy = e == 0 ? dg1 : (e == 1 ? dg2 : dg0);
-      const int dz = e == 0 ? dg2 : (e == 1 ? dg0 : dg1);
-      const int w2 = nib(sm.TH(y), x);
-      const uint32_t key = (uint32_t)((dx << 12) | (dy << 8) | (dz << 4) | nib(deg, w2));
-      const int id = 3 * f + e;
-      if (key > top) { top = key; m0 = 0; m1 = 0; }
-      if (key == top) { if (id < 64) m0 |= 1ull << id; else m1 |= 1u << (id - 64); }
+    row |= 1u << nib(lab, cur);
+    if (cur == from && i < K) {                      // all neighbours of x visited
+      if (i & 1) sm.U(i >> 1) = even | row << 16;
+      even = row;
+      row = 0;
+      i++;
+      x = min(nib(vert, i), PTM_KNN - 1);
+      from = cur = nib(come, i);
+      th = sm.TH(x);
     }
   }
-  // K = 12 with every degree 5 is the icosahedron, K = 6 with every degree 4 the
-  // octahedron: every directed edge has the same key
-  const bool transitive = (K == 12 && top == 0x5555u) || (K == 6 && top == 0x4444u);
-  // edges tied on the degrees of the edge's two facets: the key continues with
-  // the degrees of the third vertices of the facets across their outer edges
-  if (!transitive && __popcll((long long)m0) + __popc(m1) > 1) {
-    uint32_t etop = 0;
-    uint64_t n0 = 0;
-    uint32_t n1 = 0;
-    auto consider = [&](int id) {
-      const int v = sm.F(id / 3), e = id % 3;
-      const int p0 = v & 15, p1 = (v >> 4) & 15, p2 = (v >> 8) & 15;
-      const int x = e == 0 ? p0 : (e == 1 ? p1 : p2);      // edge x -> y, third vertex z
-      const int y = e == 0 ? p1 : (e == 1 ? p2 : p0);
-      const int z = e == 0 ? p2 : (e == 1 ? p0 : p1);
-      const int w = nib(sm.TH(y), x);
-      const uint32_t ext = (uint32_t)((nib(deg, nib(sm.TH(z), y)) << 12) | (nib(deg, nib(sm.TH(x), z)) << 8) |
-                                      (nib(deg, nib(sm.TH(w), x)) << 4) | nib(deg, nib(sm.TH(y), w)));
-      if (ext > etop) { etop = ext; n0 = 0; n1 = 0; }
-      if (ext == etop) { if (id < 64) n0 |= 1ull << id; else n1 |= 1u << (id - 64); }
-    };
-    for (uint64_t mm = m0; mm; mm &= mm - 1) consider(__ffsll((long long)mm) - 1);
-    for (uint32_t mm = m1; mm; mm &= mm - 1) consider(64 + __ffs(mm) - 1);
-    m0 = n0;
-    m1 = n1;
-  }
-  // one walk, from the first start edge with the largest key: the tables hold
-  // the code of every such start of every template triangulation
-  if (!(m0 | m1)) return false;
-  const int id = m0 ? __ffsll((long long)m0) - 1 : 64 + __ffs(m1) - 1;
-  {
-    const int v = sm.F(id / 3), e = id % 3;
-    const int p0 = v & 15, p1 = (v >> 4) & 15, p2 = (v >> 8) & 15;
-    const int su = e == 0 ? p0 : (e == 1 ? p1 : p2);
-    const int sv = e == 0 ? p1 : (e == 1 ? p2 : p0);
-    if (!weinberg_walk(sm, K, su, sv, labels, d)) return false;
-  }
-  // hash of the packed code (labels 3..LEN); words past its end count as zero,
-  // as the generator packs them
-  const int LEN = 2 * (3 * K - 6) + 1;
+  if (i != K || next != K) { count(d, C_INTERNAL); return false; }
   uint64_t h = PTM_HASH_INIT;
 #pragma unroll
-  for (int w = 0; w < PTM_CODE_WORDS; w++) h = (h ^ (uint64_t)(w * 8 < LEN - 2 ? sm.CODE(w) : 0u)) * PTM_HASH_MUL;
-  hash = h;
+  for (int w = 0; w < 7; w++) h = (h ^ (uint64_t)(2 * w < K ? sm.U(w) : 0u)) * PTM_HASH_MUL;
+  uint32_t info = 0;
+  for (uint32_t pos = (uint32_t)(h ^ (h >> 32)) & (PTM_GRAPH_NSLOTS - 1);; pos = (pos + 1) & (PTM_GRAPH_NSLOTS - 1)) {
+    const uint4 e0 = __ldg((const uint4 *)&ptm_graph[pos]), e1 = __ldg((const uint4 *)&ptm_graph[pos] + 1);
+    if (!e1.w) return false;                         // an empty slot (the table is at most half full)
+    const uint32_t w[7] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z};
+    bool eq = (int)(e1.w >> 28) == K;
+#pragma unroll
+    for (int k = 0; k < 7; k++) if (2 * k < K) eq &= w[k] == sm.U(k);
+    if (eq) { info = e1.w; break; }
+  }
+  const ptm_tie_entry *tie = ptm_tie + (info & 0xfffffu);
+  const int nties = (int)(info >> 20 & 255u);
+  int pick = 0;
+  if (nties > 1) {
+    // rows of the start edges, then the first facet corner that holds one
+    uint32_t tv = 0;
+    for (int k = 0; k < nties; k++) {
+      const uint32_t e = __ldg(&tie[k].edge);
+      const int u = min(nib(vert, e & 255), PTM_KNN - 1), v = nib(vert, e >> 8 & 255);
+      sm.U(u) = (tv >> u & 1 ? sm.U(u) : 0u) | 1u << v;
+      tv |= 1u << u;
+    }
+    uint32_t best = 0xffffffffu;                     // birth << 12 | corner << 8 | u << 4 | v
+    for (int f = 0; f < nf; f++) {
+      const uint32_t v = sm.F(f);
+      const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
+      const uint32_t base = v >> 12 << 12;
+      if ((tv >> a & 1) && (sm.U(a) >> b & 1)) best = min(best, base | (uint32_t)(a << 4 | b));
+      if ((tv >> b & 1) && (sm.U(b) >> c & 1)) best = min(best, base | (uint32_t)(1 << 8 | b << 4 | c));
+      if ((tv >> c & 1) && (sm.U(c) >> a & 1)) best = min(best, base | (uint32_t)(2 << 8 | c << 4 | a));
+    }
+    const uint32_t e = (uint32_t)nib(lab, best >> 4 & 15) | (uint32_t)nib(lab, best & 15) << 8;
+    while (pick < nties - 1 && (__ldg(&tie[pick].edge) & 0xffffu) != e) pick++;
+  }
+  const uint64_t perm = __ldg((const unsigned long long *)&tie[pick].perm);
+  ent = (int)(__ldg(&tie[pick].edge) >> 16);
+  labels = 0;
+#pragma unroll 2
+  for (int t = K - 1; t >= 0; t--) labels = labels << 4 | (uint64_t)nib(perm, nib(lab, t));
   return true;
 }
 

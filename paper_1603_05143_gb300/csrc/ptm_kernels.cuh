@@ -36,26 +36,6 @@ struct Best {
 // What one atom adds to the matching counters.
 struct MatchCounts { int scored, points, matched; };
 
-__device__ __forceinline__ int lookup(const Scratch &sm, int K, uint64_t h) {
-  const int LEN = 2 * (3 * K - 6) + 1;
-  const int NW = (LEN - 2 + 7) / 8;                 // stored labels 3..LEN
-  int pos = (int)(h & (PTM_TBL_NSLOTS - 1));
-  for (int probe = 0; probe < PTM_TBL_NSLOTS; probe++) {
-    const ptm_tbl_entry *e = &ptm_tbl[pos];
-    uint64_t eh = __ldg((const unsigned long long *)&e->hash);
-    int cntv = __ldg(&e->count);
-    if (eh == 0 && cntv == 0) return -1;
-    if (eh == h && __ldg(&e->nv) == K) {
-      bool eq = true;
-#pragma unroll
-      for (int w = 0; w < PTM_CODE_WORDS; w++) if (w < NW) eq &= (__ldg(&e->code[w]) == sm.CODE(w));
-      if (eq) return pos;
-    }
-    pos = (pos + 1) & (PTM_TBL_NSLOTS - 1);
-  }
-  return -1;
-}
-
 // Template slots of neighbours 0 .. K - 1 (nibble j) under the correspondence given
 // by the walk labelling and the table candidate.
 __device__ __forceinline__ uint64_t slots_of(int K, uint64_t lab, uint64_t cand) {
@@ -123,21 +103,6 @@ __device__ __forceinline__ float cand_r2(const float (&Sm)[3][3], float Gv, floa
   }
   fp64 = 0;
   return fmaxf((Gw - o.lam * o.lam / Gv) / (float)N, 0.f);
-}
-
-// Hull of the first K neighbours is complete and contains the centre: Weinberg
-// code and lookup (Algorithm 1, inner loops).  Only the labelling and table
-// entry are kept; every snapshot's candidates are scored after the last one, in
-// one loop (score_candidates, or select_fp64 in the FP64 form).
-__device__ void snapshot(int K, const Scratch &sm, const FrameDesc &d, int nf, Best &bst) {
-  if (nf != 2 * K - 4) return;                    // a neighbour is not a hull vertex
-  uint64_t lab = 0, h = 0;
-  if (!canonical(sm, K, nf, lab, h, d)) return;
-  int e = lookup(sm, K, h);
-  if (e < 0) return;
-  if (K == 6) { bst.lam6 = lab; bst.ent6 = e; }
-  else if (K == 12) { bst.lam12 = lab; bst.ent12 = e; }
-  else { bst.lam14 = lab; bst.ent14 = e; }
 }
 
 // FP32 QCP of every admissible correspondence of the matched snapshots; keeps the
@@ -866,28 +831,40 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
   int kmax = (mask & 16) ? 14 : ((mask & 14) ? 12 : 6);
   kmax = min(kmax, cnt);
   bool alive = kmax >= 6;
-  int nf = alive ? hull_init(sm, nsos) : 0;
+  int birth = 4;
+  if (alive) hull_init(sm, nsos);
   for (int p = 4; p <= PTM_KNN; p++) {
     // every insertion step starts warp-converged: a lane that finished (or took
     // a snapshot's longer path) waits here instead of drifting into a later
-    // step alone, so the visibility tests, walks and QCP loops keep full warps
+    // step alone, so the visibility tests and lookups keep full warps
     if (!__any_sync(hmask, alive)) break;
-    // the hull now holds neighbours 0..p-1: complete for K = 6, 12, 14.  The
-    // centre test of a snapshot rides on the visibility test of point p.
+    // the hull now holds neighbours 0..p-1, all of them vertices (2 p - 4
+    // facets): complete for K = 6, 12, 14.  The centre test of a snapshot rides on
+    // the visibility test of point p.
     const bool want = (p == 6 && (mask & 1)) || (p == 12 && (mask & 14)) || (p == 14 && (mask & 16));
+    const int nf = 2 * p - 4;
     bool centre_in = false;
     uint32_t vis = 0;
-    const unsigned vmask = __ballot_sync(hmask, alive && p < kmax);          // lanes testing point p
-    const unsigned cmask = __ballot_sync(hmask, alive && p >= kmax && want); // lanes testing only the centre
+    const unsigned vmask = __ballot_sync(hmask, alive && p < kmax && !want);   // lanes testing point p,
+    const unsigned bmask = __ballot_sync(hmask, alive && p < kmax && want);    // ... and the centre,
+    const unsigned cmask = __ballot_sync(hmask, alive && p >= kmax && want);   // only the centre
     if (alive) {
-      if (p < kmax) vis = hull_visibility(sm, nf, p, want, centre_in, vmask, nsos);
-      else if (want) centre_in = hull_centre_inside(sm, nf, cmask, nsos);
+      if (p >= kmax) { if (want) centre_in = hull_centre_inside(sm, nf, cmask, nsos); }
+      else if (want) vis = hull_visibility<true>(sm, nf, p, centre_in, bmask, nsos);
+      else vis = hull_visibility<false>(sm, nf, p, centre_in, vmask, nsos);
     }
-    if (alive && want && centre_in) snapshot(p, sm, d, nf, bst);
+    if (alive && want && centre_in) {
+      uint64_t lab;
+      int e;
+      if (graph_lookup(sm, p, lab, e, d)) {
+        if (p == 6) { bst.lam6 = lab; bst.ent6 = e; }
+        else if (p == 12) { bst.lam12 = lab; bst.ent12 = e; }
+        else { bst.lam14 = lab; bst.ent14 = e; }
+      }
+    }
     if (!alive) continue;
-    if (p == kmax || !vis) { alive = false; continue; }   // done, or p lies inside the hull
-    nf = hull_apply(sm, nf, vis, p, d);
-    if (nf < 0) alive = false;
+    // done, p inside the hull, or a vertex swallowed
+    alive = p != kmax && vis && hull_apply(sm, nf, vis, p, birth, d);
   }
   d.ents[sl] = pack_ents(bst.ent6, bst.ent12, bst.ent14);
   if (bst.ent6 >= 0) d.lam[sl] = bst.lam6;
@@ -1188,7 +1165,7 @@ constexpr size_t atom_smem_bytes() { return (size_t)PTM_BLOCK * SCRATCH_WORDS * 
 constexpr int MATCH_WORDS = 42 + 14;
 constexpr size_t match_smem_bytes() { return (size_t)PTM_BLOCK * MATCH_WORDS * 4; }
 
-// Resident blocks per SM of k_hulls: 8 x (98 words x 64 threads + the 1 KB the
+// Resident blocks per SM of k_hulls: 8 x (108 words x 64 threads + the 1 KB the
 // driver reserves per block) fits 228 KB of shared memory, and 8 x 64 threads x
 // 128 registers the register file.
 #define PTM_ATOM_BLOCKS_PER_SM 8
@@ -1203,16 +1180,13 @@ constexpr size_t match_smem_bytes() { return (size_t)PTM_BLOCK * MATCH_WORDS * 4
 #define PTM_MATCH_OWN_LAUNCH 65536
 #define PTM_MATCH_SIDE_STREAMS 2
 
-// Scratch rows of k_hulls in a block's dynamic shared memory (row layout of
-// Scratch without the nid / img rows).
+// Scratch rows of k_hulls in a block's dynamic shared memory.
 __device__ __forceinline__ Scratch scratch_rows(unsigned char *smem) {
   Scratch sm;
   sm.th = (uint64_t *)smem;
   sm.q = (float *)(sm.th + 14 * PTM_BLOCK);
   sm.nid = nullptr;                 // k_hulls reads the neighbour list in place
-  sm.img = nullptr;
-  sm.code = (uint32_t *)(sm.q + 42 * PTM_BLOCK);
-  sm.fac = (uint16_t *)(sm.code + PTM_CODE_WORDS * PTM_BLOCK);
+  sm.fac = (uint32_t *)(sm.q + 42 * PTM_BLOCK);
   sm.used = sm.fac + 24 * PTM_BLOCK;
   sm.t = threadIdx.x;
   return sm;
@@ -1221,10 +1195,9 @@ __device__ __forceinline__ Scratch scratch_rows(unsigned char *smem) {
 // The rows k_match uses (the others stay null).
 __device__ __forceinline__ Scratch match_rows(unsigned char *smem) {
   Scratch sm;
-  sm.th = nullptr; sm.code = nullptr; sm.fac = nullptr; sm.used = nullptr;
+  sm.th = nullptr; sm.fac = nullptr; sm.used = nullptr;
   sm.q = (float *)smem;
   sm.nid = (int *)(sm.q + 42 * PTM_BLOCK);
-  sm.img = nullptr;                 // images are read from the neighbour list
   sm.t = threadIdx.x;
   return sm;
 }

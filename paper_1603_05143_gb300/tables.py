@@ -23,9 +23,16 @@ orientation-preserving isomorphisms, so the codes from the start edges of two
 embedded graphs are the same set exactly when such an isomorphism exists, and
 a code determines the graph.  The tables therefore list, per template
 triangulation, the code of every start edge (starts related by an automorphism
-share one), and the kernels need one walk per hull (the paper's canonical form
-takes the smallest code over all starts; one lookup among all start codes is
-the same isomorphism test).
+share one); the paper's canonical form takes the smallest code over all starts,
+and one lookup among all start codes is the same isomorphism test.
+
+The kernels look a hull up by a cheaper code of the same graph: the adjacency
+matrix under a breadth-first labelling from an arbitrary directed edge
+(`breadth_first`, which the generator evaluates from every directed edge of
+every template graph).  Its first facet being fixed, that matrix determines the
+embedded graph.  Each such code lists the graph's Weinberg start edges, with the
+Weinberg labels in terms of its own, and the kernel takes the start edge that
+comes first among the hull's facets.
 
 Weinberg walk (counter-clockwise rotation seen from outside): at a new vertex
 leave by the edge after the arrival edge; at an old vertex reached along an edge
@@ -44,7 +51,6 @@ import numpy as np
 
 TEMPLATE_NAMES = ("SC", "FCC", "HCP", "ICO", "BCC")
 K = (6, 12, 12, 12, 14)
-NIB_WORDS = 9           # labels 3..73 of the longest code, four bits each (labels 1, 2 are fixed)
 HASH_MUL = 0x100000001B3
 HASH_INIT = 0xCBF29CE484222325
 MASK64 = (1 << 64) - 1
@@ -244,20 +250,76 @@ def start_codes(facets):
     return out
 
 
-def pack_code(code) -> list:
-    """Labels 3.. of a code as nibbles (every walk starts with labels 1, 2)."""
-    assert code[0] == 1 and code[1] == 2
-    words = [0] * NIB_WORDS
-    for s, x in enumerate(code[2:]):
-        words[s // 8] |= (x & 15) << (4 * (s % 8))
-    return words
-
-
 def code_hash(words) -> int:
     h = HASH_INIT
     for x in words:
         h = ((h ^ x) * HASH_MUL) & MASK64
     return h
+
+
+# ------------------------------------------- breadth-first code (kernel lookup)
+def breadth_first(th, k, u, v):
+    """Vertices in label order from the directed edge u -> v, and the code: the
+    adjacency row of each label (bit = label).  Each vertex in label order is
+    walked around, counter-clockwise from the vertex it was first reached from,
+    and new vertices are labelled as they are met."""
+    order, come, label, rows = [u, v], {u: v, v: u}, {u: 0, v: 1}, []
+    for i in range(k):
+        x = order[i]
+        cur, bits = come[x], 0
+        while True:
+            cur = th[(x, cur)]
+            if cur not in label:
+                label[cur] = len(order)
+                come[cur] = x
+                order.append(cur)
+            bits |= 1 << label[cur]
+            if cur == come[x]:
+                break
+        rows.append(bits)
+    return order, tuple(rows)
+
+
+def graph_codes(entry_of):
+    """Breadth-first code (from every directed edge of every template graph) ->
+    the graph's Weinberg start edges: a sorted tuple of (label of u, label of v,
+    permutation, entry), nibble l of the permutation the Weinberg label of
+    breadth-first label l and `entry` the position of that start's Weinberg code
+    among the candidate lists (`entry_of`).  Starts related by an automorphism
+    give the same code and the same tuple.  A graph whose every edge is a start
+    lists only the edge the walk itself began with."""
+    seen, out = set(), {}
+    for S, name in enumerate(TEMPLATE_NAMES):
+        k = K[S]
+        for t in triangulations(normalised_template(name)):
+            deg: dict = {}
+            for f in t:
+                for x in f:
+                    deg[x] = deg.get(x, 0) + 1
+            th = _third(t)
+            edges = list(th)
+            top = max(edge_key(deg, th, a, b) for a, b in edges)
+            starts = [(a, b) for a, b in edges if edge_key(deg, th, a, b) == top]
+            walks = [(a, b, *weinberg(t, a, b)) for a, b in starts]
+            key = min(w[2] for w in walks)
+            if key in seen:                       # the same graph as an earlier triangulation
+                continue
+            seen.add(key)
+            for u, v in edges:
+                order, code = breadth_first(th, k, u, v)
+                label = {x: i for i, x in enumerate(order)}
+                ties = tuple(sorted(
+                    (label[a], label[b], sum(lab[x] << (4 * i) for i, x in enumerate(order)), entry_of[wc])
+                    for a, b, wc, lab in walks if len(starts) < len(edges) or (a, b) == (u, v)))
+                assert out.setdefault((k, code), ties) == ties
+    return out
+
+
+def pack_rows(rows) -> list:
+    words = [0] * 7
+    for i, r in enumerate(rows):
+        words[i // 2] |= r << (16 * (i % 2))
+    return words
 
 
 # ------------------------------------------------------------ SoS term order
@@ -323,33 +385,42 @@ def build():
 def emit_header(path: pathlib.Path) -> dict:
     tpl, groups, quats, entries, stats = build()
     codes = sorted(entries)
-    nslots = 1
-    while nslots < 2 * len(codes):
-        nslots *= 2
-    slots = [None] * nslots
-    cand = []
+    cand, first = [], []
     for code in codes:
-        words = pack_code(code)
-        h = code_hash(words)
-        first = len(cand)
+        first.append(len(cand))
         for S, sg in entries[code]:
             v = S << 60
             for L, slot in enumerate(sg):
                 v |= slot << (4 * L)
             cand.append(v)
-        e = (h, words, (len(code) - 1) // 6 + 2, first, len(cand) - first)
-        pos = h & (nslots - 1)
+    graphs = graph_codes({code: i for i, code in enumerate(codes)})
+    nslots = 1
+    while nslots < 2 * len(graphs):
+        nslots *= 2
+    slots = [None] * nslots
+    ties, lists = [], {}
+    for k, rows in sorted(graphs):
+        tl = graphs[(k, rows)]
+        if tl not in lists:
+            lists[tl] = len(ties)
+            ties += tl
+        words = pack_rows(rows)
+        h = code_hash(words)
+        pos = (h ^ (h >> 32)) & (nslots - 1)
         while slots[pos] is not None:
             pos = (pos + 1) & (nslots - 1)
-        slots[pos] = e
+        slots[pos] = (words, k << 28 | len(tl) << 20 | lists[tl])
+    assert len(ties) < 1 << 20 and max(len(t) for t in lists) < 256
     lines = ["/* Generated by paper_1603_05143_gb300/tables.py -- do not edit. */",
              "#pragma once", "#include <stdint.h>",
              "/* storage qualifiers: constant memory for uniform reads, global for tables */",
              "#ifndef PTM_TBL_CONST", "#define PTM_TBL_CONST static const", "#endif",
              "#ifndef PTM_TBL_GLOBAL", "#define PTM_TBL_GLOBAL static const", "#endif",
              "#ifndef PTM_TBL_ALIGN16", "#define PTM_TBL_ALIGN16", "#endif", ""]
-    lines.append(f"#define PTM_TBL_NSLOTS {nslots}")
+    lines.append(f"#define PTM_TBL_NENT {len(codes)}")
     lines.append(f"#define PTM_TBL_NCAND {len(cand)}")
+    lines.append(f"#define PTM_GRAPH_NSLOTS {nslots}")
+    lines.append(f"#define PTM_TIE_N {len(ties)}")
     lines.append(f"#define PTM_HASH_INIT 0x{HASH_INIT:016x}ULL")
     lines.append(f"#define PTM_HASH_MUL 0x{HASH_MUL:016x}ULL")
     goff = np.cumsum([0] + [len(g) for g in groups]).tolist()
@@ -397,14 +468,21 @@ def emit_header(path: pathlib.Path) -> dict:
         for q in qs:
             lines.append("  {" + ", ".join(f"{x:.9e}f" for x in q) + "},")
     lines.append("};")
-    lines.append(f"typedef struct {{ uint64_t hash; uint32_t code[{NIB_WORDS}]; uint16_t nv, first, count, pad; }} ptm_tbl_entry;")
-    lines.append("PTM_TBL_GLOBAL ptm_tbl_entry ptm_tbl[PTM_TBL_NSLOTS] = {")
-    for e in slots:
-        if e is None:
-            lines.append("  {0ULL, {0}, 0, 0, 0, 0},")
-        else:
-            h, words, nv, first, count = e
-            lines.append(f"  {{0x{h:016x}ULL, {{{', '.join(f'0x{x:08x}u' for x in words)}}}, {nv}, {first}, {count}, 0}},")
+    lines.append("/* candidates of each Weinberg start code */")
+    lines.append("typedef struct { uint16_t first, count; } ptm_tbl_entry;")
+    lines.append("PTM_TBL_GLOBAL ptm_tbl_entry ptm_tbl[PTM_TBL_NENT] = {")
+    lines.append("  " + ", ".join(f"{{{f}, {len(entries[c])}}}" for c, f in zip(codes, first)))
+    lines.append("};")
+    lines.append("/* breadth-first codes, open addressing: 7 words of two 16-bit adjacency rows, then")
+    lines.append("   vertices << 28 | starts << 20 | first start (0: empty) */")
+    lines.append("typedef struct { uint32_t w[8]; } ptm_graph_entry;")
+    lines.append("PTM_TBL_GLOBAL ptm_graph_entry ptm_graph[PTM_GRAPH_NSLOTS] PTM_TBL_ALIGN16 = {")
+    lines += ["  {{" + ("0" if e is None else ", ".join(f"0x{x:x}u" for x in [*e[0], e[1]])) + "}}," for e in slots]
+    lines.append("};")
+    lines.append("/* Weinberg start edges of a graph: labels u | v << 8 | entry << 16, and the permutation */")
+    lines.append("typedef struct { uint64_t perm; uint32_t edge, pad; } ptm_tie_entry;")
+    lines.append("PTM_TBL_GLOBAL ptm_tie_entry ptm_tie[PTM_TIE_N] PTM_TBL_ALIGN16 = {")
+    lines += [f"  {{0x{p:016x}ULL, 0x{u | v << 8 | e << 16:x}u, 0}}," for u, v, p, e in ties]
     lines.append("};")
     lines.append("/* candidate: bits 60-62 template, nibble L-1 = slot of canonical label L */")
     lines.append("PTM_TBL_GLOBAL uint64_t ptm_cand[PTM_TBL_NCAND] = {")

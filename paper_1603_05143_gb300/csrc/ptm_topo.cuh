@@ -35,60 +35,135 @@ namespace ptm {
 #define PTM_TOPO_BLOCKS_PER_SM 6
 #define PTM_TOPO64_BLOCKS_PER_SM 4
 
-// Area of the Voronoi face of neighbour j among the m vectors V(i, c); P and Q
-// are polygon buffers of 2 x vmax values, element e at P[e * st].  A clip that
-// would leave more than vmax vertices sets `over` (the polygon keeps its first
-// vmax vertices).
+// The plane of neighbour j's face: in-plane axes e1, e2 and the foot point p.
 template <typename T, typename Vec>
-__device__ T topo_face_area(int m, int j, T R, Vec V, T *P, T *Q, int st, int vmax, bool &over) {
+__device__ __forceinline__ void topo_plane(int j, Vec V, T (&e1)[3], T (&e2)[3], T (&p)[3]) {
   const T n0 = V(j, 0), n1 = V(j, 1), n2 = V(j, 2);
   const T nn = sqrt(n0 * n0 + n1 * n1 + n2 * n2);
   const T u0 = n0 / nn, u1 = n1 / nn, u2 = n2 / nn;
   // e1 = u x a with a the axis least aligned with u, e2 = u x e1
   const bool ax = fabs(u0) < (T)0.6;
   const T a0 = ax ? (T)1 : (T)0, a1 = ax ? (T)0 : (T)1;
-  T e10 = u1 * (T)0 - u2 * a1, e11 = u2 * a0 - u0 * (T)0, e12 = u0 * a1 - u1 * a0;
-  const T l1 = sqrt(e10 * e10 + e11 * e11 + e12 * e12);
-  e10 /= l1; e11 /= l1; e12 /= l1;
-  const T e20 = u1 * e12 - u2 * e11, e21 = u2 * e10 - u0 * e12, e22 = u0 * e11 - u1 * e10;
-  const T p0 = n0 / 2, p1 = n1 / 2, p2 = n2 / 2;
+  e1[0] = u1 * (T)0 - u2 * a1; e1[1] = u2 * a0 - u0 * (T)0; e1[2] = u0 * a1 - u1 * a0;
+  const T l1 = sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]);
+  e1[0] /= l1; e1[1] /= l1; e1[2] /= l1;
+  e2[0] = u1 * e1[2] - u2 * e1[1]; e2[1] = u2 * e1[0] - u0 * e1[2]; e2[2] = u0 * e1[1] - u1 * e1[0];
+  p[0] = n0 / 2; p[1] = n1 / 2; p[2] = n2 / 2;
+}
+
+// FP64 area of the Voronoi face of neighbour j among the m vectors V(i, c); P and Q
+// are polygon buffers of 2 x vmax values, element e at P[e * st].
+template <typename Vec>
+__device__ double topo_face_area64(int m, int j, double R, Vec V, double *P, double *Q, int st, int vmax) {
+  double e1[3], e2[3], p[3];
+  topo_plane<double>(j, V, e1, e2, p);
   // a convex polygon gains at most one vertex per clip (4 + 17 < PTM_TOPO_VMAX);
   // rounding on a nearly degenerate polygon could emit more, so writes stop at
   // the buffer's end (the polygon then has next to no area either way)
-  T *cur = P, *nxt = Q;
+  double *cur = P, *nxt = Q;
   int np = 4;
   cur[0] = -R; cur[st] = -R; cur[2 * st] = R; cur[3 * st] = -R;
   cur[4 * st] = R; cur[5 * st] = R; cur[6 * st] = -R; cur[7 * st] = R;
   for (int i = 0; i < m && np > 0; i++) {
     if (i == j) continue;
-    const T w0 = V(i, 0), w1 = V(i, 1), w2 = V(i, 2);
-    const T A = w0 * e10 + w1 * e11 + w2 * e12, B = w0 * e20 + w1 * e21 + w2 * e22;
-    const T C = (w0 * w0 + w1 * w1 + w2 * w2) / 2 - (w0 * p0 + w1 * p1 + w2 * p2);
+    const double w0 = V(i, 0), w1 = V(i, 1), w2 = V(i, 2);
+    const double A = w0 * e1[0] + w1 * e1[1] + w2 * e1[2], B = w0 * e2[0] + w1 * e2[1] + w2 * e2[2];
+    const double C = (w0 * w0 + w1 * w1 + w2 * w2) / 2 - (w0 * p[0] + w1 * p[1] + w2 * p[2]);
     int nq = 0;
+    double xs = cur[0], xt = cur[st], fx = A * xs + B * xt - C;
+    const double x0 = xs, t0 = xt, f0 = fx;
     for (int k = 0; k < np; k++) {
-      const int k1 = k + 1 == np ? 0 : k + 1;
-      const T xs = cur[2 * k * st], xt = cur[(2 * k + 1) * st], ys = cur[2 * k1 * st], yt = cur[(2 * k1 + 1) * st];
-      const T fx = A * xs + B * xt - C, fy = A * ys + B * yt - C;
+      double ys = x0, yt = t0, fy = f0;
+      if (k + 1 < np) { ys = cur[2 * (k + 1) * st]; yt = cur[(2 * k + 3) * st]; fy = A * ys + B * yt - C; }
       if (fx <= 0) {
         if (nq < vmax) { nxt[2 * nq * st] = xs; nxt[(2 * nq + 1) * st] = xt; }
         nq++;
       }
       if ((fx < 0 && fy > 0) || (fx > 0 && fy < 0)) {
-        const T tt = fx / (fx - fy);
+        const double tt = fx / (fx - fy);
         if (nq < vmax) { nxt[2 * nq * st] = xs + tt * (ys - xs); nxt[(2 * nq + 1) * st] = xt + tt * (yt - xt); }
         nq++;
       }
+      xs = ys; xt = yt; fx = fy;
     }
-    over |= nq > vmax;
     np = min(nq, vmax);
-    T *tmp = cur; cur = nxt; nxt = tmp;
+    double *tmp = cur; cur = nxt; nxt = tmp;
   }
-  T s2 = 0;
+  double s2 = 0;
   for (int k = 0; k < np; k++) {
     const int k1 = k + 1 == np ? 0 : k + 1;
     s2 += cur[2 * k * st] * cur[(2 * k1 + 1) * st] - cur[2 * k1 * st] * cur[(2 * k + 1) * st];
   }
   return fabs(s2) / 2;
+}
+
+// FP32 area of the same face, polygons of at most PTM_TOPO_VMAX32 vertices at
+// P[k * st] and Q[k * st].  Every plane first only marks the vertices outside it;
+// most planes cut nothing, and of a convex polygon a plane takes one run of
+// consecutive vertices, replaced by its two crossings, so a cut copies the rest
+// and makes two divisions however many vertices the other lanes' polygons have.
+// `over` is set when the polygon outgrows the buffer or rounding leaves more than
+// one run: the FP64 pass decides then.
+template <typename Vec>
+__device__ __forceinline__ float topo_face_area32(int m, int j, float R, Vec V, float2 *P, float2 *Q, int st, bool &over) {
+  float e1[3], e2[3], p[3];
+  topo_plane<float>(j, V, e1, e2, p);
+  float2 *cur = P, *nxt = Q;
+  int np = 4;
+  cur[0] = make_float2(-R, -R); cur[st] = make_float2(R, -R); cur[2 * st] = make_float2(R, R); cur[3 * st] = make_float2(-R, R);
+  for (int i = 0; i < m; i++) {
+    if (i == j) continue;
+    const float w0 = V(i, 0), w1 = V(i, 1), w2 = V(i, 2);
+    const float A = w0 * e1[0] + w1 * e1[1] + w2 * e1[2], B = w0 * e2[0] + w1 * e2[1] + w2 * e2[2];
+    const float C = (w0 * w0 + w1 * w1 + w2 * w2) / 2 - (w0 * p[0] + w1 * p[1] + w2 * p[2]);
+    uint32_t out = 0;
+    for (int k = 0; k < np; k++) {
+      const float2 x = cur[k * st];
+      out |= (uint32_t)(A * x.x + B * x.y - C > 0.f) << k;
+    }
+    if (!out) continue;
+    const uint32_t all = (1u << np) - 1u;
+    if (out == all) { np = 0; break; }
+    // the run s .. e of outside vertices (cyclic)
+    const uint32_t prev = (out << 1 | out >> (np - 1)) & all, begins = out & ~prev;
+    over |= (begins & (begins - 1)) != 0;
+    const int s = __ffs(begins) - 1, n = __popc(out);
+    const int in0 = s + n >= np ? s + n - np : s + n, in1 = s ? s - 1 : np - 1, e = in0 ? in0 - 1 : np - 1;
+    int nq = 0;
+    for (int k = in0, left = np - n; left; left--) {
+      const float2 x = cur[k * st];
+      nxt[nq * st] = x;
+      nq++;
+      k = k + 1 == np ? 0 : k + 1;
+    }
+    // the crossings of in1 -> s and e -> in0; a vertex on the plane is its own
+    const float2 a = cur[in1 * st], b = cur[s * st], c = cur[e * st], g = cur[in0 * st];
+    const float fa = A * a.x + B * a.y - C, fb = A * b.x + B * b.y - C, fc = A * c.x + B * c.y - C, fg = A * g.x + B * g.y - C;
+    if (fa < 0.f) {
+      const float t = fa / (fa - fb);
+      if (nq < PTM_TOPO_VMAX32) nxt[nq * st] = make_float2(a.x + t * (b.x - a.x), a.y + t * (b.y - a.y));
+      nq++;
+    }
+    if (fg < 0.f) {
+      const float t = fc / (fc - fg);
+      if (nq < PTM_TOPO_VMAX32) nxt[nq * st] = make_float2(c.x + t * (g.x - c.x), c.y + t * (g.y - c.y));
+      nq++;
+    }
+    over |= nq > PTM_TOPO_VMAX32;
+    np = min(nq, PTM_TOPO_VMAX32);
+    float2 *tmp = cur; cur = nxt; nxt = tmp;
+  }
+  float s2 = 0.f;
+  if (np) {
+    const float2 x0 = cur[0];
+    float2 x = x0;
+    for (int k = 1; k <= np; k++) {
+      const float2 y = k < np ? cur[k * st] : x0;
+      s2 += x.x * y.y - y.x * x.y;
+      x = y;
+    }
+  }
+  return fabsf(s2) / 2;
 }
 
 // Order o[0..m) of neighbour ranks by (area descending, rank ascending), then
@@ -190,11 +265,11 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict_
     const float R = 10.f * sqrtf(dmax2);
     auto vf = [&](int i, int c) -> float { return VF(i, c); };
     // polygon buffers in shared memory, one word per thread per row
-    float *PB = (float *)tsm + 5 * PTM_TOPO_N * PTM_BLOCK + t;
-    float *QB = PB + 2 * PTM_TOPO_VMAX32 * PTM_BLOCK;
+    float2 *PB = (float2 *)(tsm + 5 * PTM_TOPO_N * PTM_BLOCK) + t;
+    float2 *QB = PB + PTM_TOPO_VMAX32 * PTM_BLOCK;
     float area[PTM_TOPO_N];
     bool over = false;
-    for (int k = 0; k < m; k++) area[k] = topo_face_area<float>(m, k, R, vf, PB, QB, PTM_BLOCK, PTM_TOPO_VMAX32, over);
+    for (int k = 0; k < m; k++) area[k] = topo_face_area32(m, k, R, vf, PB, QB, PTM_BLOCK, over);
     // a gap at the band edge, or a polygon larger than the buffer: the second pass decides
     const uint32_t near = topo_order<float>(m, area, mean2, o);
     if (near || over) {
@@ -255,13 +330,12 @@ __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *si
     mean64 /= m;
   }
   auto vd = [&](int a, int c) -> double { return v64[a][c]; };
-  bool over = false;
   uint32_t todo = m > 0 ? faces & ((1u << m) - 1u) : 0u;
   while (__any_sync(wmask, todo != 0)) {
     if (!todo) continue;
     const int k = __ffs(todo) - 1;
     todo &= todo - 1;
-    a64[k] = topo_face_area<double>(m, k, 10.0 * sqrt(dmax64), vd, P, Q, PTM_BLOCK, PTM_TOPO_VMAX, over);
+    a64[k] = topo_face_area64(m, k, 10.0 * sqrt(dmax64), vd, P, Q, PTM_BLOCK, PTM_TOPO_VMAX);
   }
   if (m > 0) topo_order<double>(m, a64, mean64, o);
   for (int k = 0; k < PTM_KNN; k++) out[(int64_t)k * n + sl] = k < m ? make_int2(jn[o[k]], im[o[k]]) : make_int2(-1, 0);

@@ -230,6 +230,11 @@ static void set_buffers(FrameDesc *d, BinParams *bp, const FrameBuffers &B) {
 // Cell list of one frame; returns the number of kernels launched.
 static int launch_cells(const ptm_frame *f, const BinParams &bp, const ShiftTables &tab, size_t ncell,
                         const FrameBuffers &B, cudaStream_t st) {
+  if (f->n_atoms <= PTM_SMALL_ATOMS && ncell <= PTM_SMALL_CELLS) {
+    k_cells_small<<<1, PTM_SMALL_BLOCK, 0, st>>>(tab, f->positions, bp, (int)ncell, B.tab, B.cell_start, B.dstat,
+                                                 B.counters, B.sorted, B.hi, B.lo, B.sbin, B.wrapv);
+    return 1;
+  }
   const int tb = 256, nscan = (int)ncell + 1;
   const unsigned gb = (unsigned)((f->n_atoms + tb - 1) / tb);
   k_begin<<<std::min(152, (nscan + tb - 1) / tb), tb, 0, st>>>(tab, B.tab, B.cell_count, nscan, B.dstat, B.counters);
@@ -242,21 +247,56 @@ static int launch_cells(const ptm_frame *f, const BinParams &bp, const ShiftTabl
   return nblk > 1 ? 5 : 4;
 }
 
+// Atoms per warp of the thread-per-atom kernels: 32 once that gives every SM
+// sub-partition (608) a warp, fewer below, where the chip is idle anyway and a
+// warp's time is its lanes' diverged paths added up.  Measured with 1 to 32 atoms
+// per warp (hulls + matching, us): 256 atoms 84 at 1, 117 at 32; 2,048 atoms 96 at 4,
+// 119 at 32; 7,920 atoms 112 at 16, 121 at 32; 31,250 atoms 143 at 32, 161 at 16.
+static int atoms_per_warp(int64_t n) { return (int)std::min<int64_t>(32, std::max<int64_t>(1, (n + 607) / 608)); }
+
+static unsigned spread_grid(int64_t n, int apw, int block) {
+  const int64_t warps = (n + apw - 1) / apw;
+  return (unsigned)((warps * 32 + block - 1) / block);
+}
+
 // Blocks of k_knn_rest, which strides over its list: at most four per SM.
 static unsigned rest_grid(int64_t n) { return (unsigned)std::min<int64_t>((n + 3) / 4, 4 * 152); }
 
 // Neighbour lists (the NK nearest) of one frame; the atom ranks of the cell list
-// are dead by now and hold the list of undecided atoms.
+// are dead by now and hold the list of undecided atoms.  Up to PTM_KNN_WARP_ATOMS
+// atoms k_knn_rest takes all of them, a warp each: 33 against 42 us for 256 atoms
+// (k_knn at one atom per warp), 36 against 57 for 1,024, 46 against 48 for 2,048.
+// Returns the number of kernels launched.
+#define PTM_KNN_WARP_ATOMS 1536
 template <int NK>
-static void launch_knn(const FrameDesc &desc, const FrameBuffers &B, cudaStream_t st) {
-  const unsigned gk = (unsigned)((desc.n + PTM_KNN_BLOCK - 1) / PTM_KNN_BLOCK);
-  int *cnt = B.dstat + 2;
+static int launch_knn(const FrameDesc &desc, const FrameBuffers &B, cudaStream_t st) {
+  const bool warps = desc.n <= PTM_KNN_WARP_ATOMS;
+  int *rest = warps ? nullptr : B.atom_rank, *cnt = B.dstat + 2;
+  const int apw = atoms_per_warp(desc.n);
+  const unsigned gk = spread_grid(desc.n, apw, PTM_KNN_BLOCK);
   if (desc.f64) {
-    k_knn<true, NK><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(NK), st>>>(desc, B.atom_rank, cnt);
-    k_knn_rest<true, NK><<<rest_grid(desc.n), PTM_KNN_BLOCK, 0, st>>>(desc, B.atom_rank, cnt);
+    if (!warps) k_knn<true, NK><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(NK), st>>>(desc, apw, rest, cnt);
+    k_knn_rest<true, NK><<<rest_grid(desc.n), PTM_KNN_BLOCK, 0, st>>>(desc, rest, cnt);
   } else {
-    k_knn<false, NK><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(NK), st>>>(desc, B.atom_rank, cnt);
-    k_knn_rest<false, NK><<<rest_grid(desc.n), PTM_KNN_BLOCK, 0, st>>>(desc, B.atom_rank, cnt);
+    if (!warps) k_knn<false, NK><<<gk, PTM_KNN_BLOCK, knn_smem_bytes(NK), st>>>(desc, apw, rest, cnt);
+    k_knn_rest<false, NK><<<rest_grid(desc.n), PTM_KNN_BLOCK, 0, st>>>(desc, rest, cnt);
+  }
+  return warps ? 1 : 2;
+}
+
+// Hulls and matching of one frame from its neighbour lists.
+static void launch_classify(const FrameDesc &desc, int precision, cudaEvent_t between, cudaStream_t st) {
+  const int apw = atoms_per_warp(desc.n);
+  const unsigned ga = spread_grid(desc.n, apw, PTM_BLOCK);
+  if (desc.f64) k_hulls<true><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc, apw);
+  else k_hulls<false><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc, apw);
+  if (between) cudaEventRecord(between, st);
+  if (precision == PTM_PREC_FP64) {
+    if (desc.f64) k_match<true, true><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc, apw);
+    else k_match<false, true><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc, apw);
+  } else {
+    if (desc.f64) k_match<true><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc, apw);
+    else k_match<false><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc, apw);
   }
 }
 
@@ -308,10 +348,9 @@ static ptm_status enqueue_frame(ptm_context *ctx, const ptm_frame *f, const ptm_
   const unsigned ga = (unsigned)((n + PTM_BLOCK - 1) / PTM_BLOCK);
   CK(cudaEventRecord(ctx->ev[1], st));
   if (!topological) {
-    launch_knn<PTM_KNN>(desc, B, st);
-    launches += 2;
+    launches += launch_knn<PTM_KNN>(desc, B, st);
   } else {
-    launch_knn<PTM_TOPO_N>(desc, B, st);
+    launches += launch_knn<PTM_TOPO_N>(desc, B, st);
     int *cnt = ctx->dstat + 3;
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
@@ -328,19 +367,10 @@ static ptm_status enqueue_frame(ptm_context *ctx, const ptm_frame *f, const ptm_
       k_topo64<false><<<g64, PTM_BLOCK, topo64_smem_bytes(), st>>>(desc, ctx->nbr, ctx->topo_list, cnt,
                                                                    ctx->topo_side, cap_side);
     }
-    launches += 4;
+    launches += 2;
   }
   CK(cudaEventRecord(ctx->ev[3], st));
-  if (f64) k_hulls<true><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc);
-  else k_hulls<false><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc);
-  CK(cudaEventRecord(ctx->ev[4], st));
-  if (ctx->precision == PTM_PREC_FP64) {
-    if (f64) k_match<true, true><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc);
-    else k_match<false, true><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc);
-  } else {
-    if (f64) k_match<true><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc);
-    else k_match<false><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc);
-  }
+  launch_classify(desc, ctx->precision, ctx->ev[4], st);
   CK(cudaGetLastError());
   CK(cudaEventRecord(ctx->ev[2], st));
   ctx->last_stream = st;
@@ -704,8 +734,8 @@ static ptm_status batch_enqueue(ptm_batch *b, cudaStream_t st) {
     const int w = (int)(k % (size_t)(ns + 1));
     cudaStream_t sk = w == 0 ? st : b->side[w - 1];
     const unsigned g = (unsigned)((hd.n + PTM_BLOCK - 1) / PTM_BLOCK);
-    if (b->f64) k_match<true><<<g, PTM_BLOCK, match_smem_bytes(), sk>>>(hd);
-    else k_match<false><<<g, PTM_BLOCK, match_smem_bytes(), sk>>>(hd);
+    if (b->f64) k_match<true><<<g, PTM_BLOCK, match_smem_bytes(), sk>>>(hd, 32);
+    else k_match<false><<<g, PTM_BLOCK, match_smem_bytes(), sk>>>(hd, 32);
   }
   if (b->nsmall) {
     const int64_t stiles = (b->small_atoms + b->tile_atoms - 1) / b->tile_atoms;
@@ -1129,11 +1159,7 @@ extern "C" ptm_status ptm_classify_frame_noalloc(const ptm_frame *f, const ptm_o
   cudaGetLastError();   // launch errors are read below; drop any left by earlier calls
   launch_cells(f, bp, tab, ncell, B, st);
   launch_knn<PTM_KNN>(desc, B, st);
-  const unsigned ga = (unsigned)((n + PTM_BLOCK - 1) / PTM_BLOCK);
-  if (f64) k_hulls<true><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc);
-  else k_hulls<false><<<ga, PTM_BLOCK, atom_smem_bytes(), st>>>(desc);
-  if (f64) k_match<true><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc);
-  else k_match<false><<<ga, PTM_BLOCK, match_smem_bytes(), st>>>(desc);
+  launch_classify(desc, PTM_PREC_FP32, nullptr, st);
   if (cudaGetLastError() != cudaSuccess) return PTM_ERR_CUDA;
   return PTM_OK;
 }

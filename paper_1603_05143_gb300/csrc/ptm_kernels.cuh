@@ -115,11 +115,12 @@ __device__ __forceinline__ float cand_r2(const float (&Sm)[3][3], float Gv, floa
 // finds its entry's atom by bisection of the lanes' running totals, fetches that
 // atom's labelling and sums by shuffles and reads its vectors in place (the rows
 // of a warp's lanes are neighbouring banks, and lanes of one atom broadcast); the
-// atom then takes its results back in order.  Every live lane calls this; the
-// live lanes are the warp's first.
-__device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const float4 *tplw, Best &bst, unsigned live,
+// atom then takes its results back in order.  Every lane of the warp calls this,
+// those without an atom too.
+__device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const float4 *tplw, Best &bst,
                                  MatchCounts &cnt) {
-  const int lane = threadIdx.x & 31, nlive = __popc(live);
+  constexpr unsigned ALL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
   int n6 = 0, n12 = 0, n14 = 0, f6 = 0, f12 = 0, f14 = 0;
   float Gv6 = 0.f, Gv12 = 0.f, Gv14 = 0.f, mx, my, mz;
   if (bst.ent6 >= 0) { f6 = ptm_tbl[bst.ent6].first; n6 = ptm_tbl[bst.ent6].count; data_moments(6, sm, mx, my, mz, Gv6); }
@@ -129,30 +130,28 @@ __device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const fl
   int upto = mine;                                   // running total of the lanes' candidates
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int x = __shfl_up_sync(live, upto, o);
+    const int x = __shfl_up_sync(ALL, upto, o);
     if (lane >= o) upto += x;
   }
-  const int total = __shfl_sync(live, upto, nlive - 1), first = upto - mine;
+  const int total = __shfl_sync(ALL, upto, 31), first = upto - mine;
   const uint32_t packed = (uint32_t)n6 | (uint32_t)n12 << 8, firsts = (uint32_t)f6 | (uint32_t)f12 << 10 | (uint32_t)f14 << 20;
-  for (int base = 0; base < total; base += nlive) {
+  for (int base = 0; base < total; base += 32) {
     const int p = base + lane;
     int owner = 0;                                   // lanes whose running total is at most p
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
-      const int at = owner + o - 1;
-      const int x = __shfl_sync(live, upto, min(at, nlive - 1));
-      if (at < nlive && x <= p) owner += o;
-    }
-    owner = min(owner, nlive - 1);                   // (entries past the list: any lane)
-    const int i = p - __shfl_sync(live, first, owner);
-    const uint32_t np = __shfl_sync(live, packed, owner), fp = __shfl_sync(live, firsts, owner);
-    const uint32_t mask = __shfl_sync(live, d.mask, owner);
+      const int x = __shfl_sync(ALL, upto, owner + o - 1);
+      if (x <= p) owner += o;
+    }                                                // (entries past the list: lane 31)
+    const int i = p - __shfl_sync(ALL, first, owner);
+    const uint32_t np = __shfl_sync(ALL, packed, owner), fp = __shfl_sync(ALL, firsts, owner);
+    const uint32_t mask = __shfl_sync(ALL, d.mask, owner);
     const int m6 = np & 255, m12 = np >> 8;
     const int K = i < m6 ? 6 : (i < m6 + m12 ? 12 : 14);
     const int c = K == 6 ? (int)(fp & 1023) + i : (K == 12 ? (int)(fp >> 10 & 1023) + i - m6 : (int)(fp >> 20) + i - m6 - m12);
-    const uint64_t l6 = __shfl_sync(live, bst.lam6, owner), l12 = __shfl_sync(live, bst.lam12, owner),
-                   l14 = __shfl_sync(live, bst.lam14, owner);
-    const float g6 = __shfl_sync(live, Gv6, owner), g12 = __shfl_sync(live, Gv12, owner), g14 = __shfl_sync(live, Gv14, owner);
+    const uint64_t l6 = __shfl_sync(ALL, bst.lam6, owner), l12 = __shfl_sync(ALL, bst.lam12, owner),
+                   l14 = __shfl_sync(ALL, bst.lam14, owner);
+    const float g6 = __shfl_sync(ALL, Gv6, owner), g12 = __shfl_sync(ALL, Gv12, owner), g14 = __shfl_sync(ALL, Gv14, owner);
     float r2 = INFINITY;
     int fp64 = 0;
     if (p < total) {
@@ -169,12 +168,12 @@ __device__ void score_candidates(const FrameDesc &d, const Scratch &sm, const fl
       }
     }
     // the results of this lane's atom among this round's, in candidate order
-    const int lo = max(first - base, 0), hi = min(upto - base, nlive);
-    const int trips = __reduce_max_sync(live, max(hi - lo, 0));
+    const int lo = max(first - base, 0), hi = min(upto - base, 32);
+    const int trips = __reduce_max_sync(ALL, max(hi - lo, 0));
     for (int t = 0; t < trips; t++) {
       const int src = lo + t;
-      const float x = __shfl_sync(live, r2, min(src, nlive - 1));
-      const int xf = __shfl_sync(live, fp64, min(src, nlive - 1));
+      const float x = __shfl_sync(ALL, r2, min(src, 31));
+      const int xf = __shfl_sync(ALL, fp64, min(src, 31));
       if (src >= hi) continue;
       if (x < bst.b1) {
         const int k = base + src - first;            // candidate of this atom
@@ -875,15 +874,20 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
 
 // P64 selects the FP64 form: every candidate scored and the winner's outputs
 // computed in FP64 (the one-frame-per-launch comparison form).
+// Every lane of the warp calls it; `active` lanes have an atom, at sorted slot s.
 template <bool F64, bool P64 = false>
-__device__ MatchCounts match_atom(const FrameDesc &d, int s, const Scratch &sm, const float4 *tplw, unsigned live) {
+__device__ MatchCounts match_atom(const FrameDesc &d, int s, bool active, const Scratch &sm, const float4 *tplw) {
   typedef typename RT<F64>::T T;
   const int64_t sl = s - d.atom_offset;
   MatchCounts cnt = {0, 0, 0};
-  const uint32_t ents = __ldg(d.ents + sl);
-  T xi, yi, zi;
-  int idi;
-  load_atom<F64>(d, s, xi, yi, zi, idi);
+  uint32_t ents = 0;
+  T xi = 0, yi = 0, zi = 0;
+  int idi = 0;
+  if (active) {
+    ents = __ldg(d.ents + sl);
+    load_atom<F64>(d, s, xi, yi, zi, idi);
+  }
+  if (P64 && !active) return cnt;
   if (P64 && !ents) { write_unmatched(d, idi); return cnt; }
   Best bst;
   bst.b1 = bst.b2 = INFINITY;
@@ -906,9 +910,10 @@ __device__ MatchCounts match_atom(const FrameDesc &d, int s, const Scratch &sm, 
   }
   if (ents) metric_vectors<F64>(d, sm, nb, nst, xi, yi, zi);
   if constexpr (!P64) {
-    __syncwarp(live);                              // the vectors are read across the warp
-    score_candidates(d, sm, tplw, bst, live, cnt);
-    __syncwarp(live);
+    __syncwarp();                                  // the vectors are read across the warp
+    score_candidates(d, sm, tplw, bst, cnt);
+    __syncwarp();
+    if (!active) return cnt;
     if (bst.K < 0) { write_unmatched(d, idi); return cnt; }     // no match, or every match masked out
   } else {
     const int w = select_fp64(d, bst, ex, ey, ez, &cnt.scored);
@@ -1113,6 +1118,68 @@ __global__ void k_scatter(const void *pos, BinParams p, const int *atom_cell, co
   wrapv[slot] = wrap;
 }
 
+// Cell list of a small frame by one block: what k_begin, k_bin, the scan and
+// k_scatter do, with the counts in shared memory.  Four launches cost more than the
+// work of one block up to a few thousand atoms: 22 -> 12 us for 256 atoms, 23 -> 16
+// us for 2,048; at 4,000 the block takes longer (30 against 23 us).
+#define PTM_SMALL_ATOMS 2048
+#define PTM_SMALL_CELLS 4096
+#define PTM_SMALL_BLOCK 1024
+__global__ void __launch_bounds__(PTM_SMALL_BLOCK)
+    k_cells_small(const __grid_constant__ ShiftTables t, const void *pos, const __grid_constant__ BinParams p, int ncell,
+                  ShiftTables *out, int *cell_start, int *dstat, unsigned long long *counters, void *sorted, float4 *hi,
+                  float4 *lo, int *sbin, int *wrapv) {
+  __shared__ int cells[PTM_SMALL_CELLS];
+  __shared__ int sh[32];
+  __shared__ int any_wrap, overs, excluded;
+  constexpr int PER = PTM_SMALL_ATOMS / PTM_SMALL_BLOCK;
+  const int tid = threadIdx.x;
+  const float *src = reinterpret_cast<const float *>(&t);
+  for (int i = tid; i < (int)(sizeof(ShiftTables) / 4); i += PTM_SMALL_BLOCK) reinterpret_cast<float *>(out)[i] = src[i];
+  for (int i = tid; i < ncell; i += PTM_SMALL_BLOCK) cells[i] = 0;
+  if (tid == 0) any_wrap = overs = excluded = 0;
+  __syncthreads();
+  int cell[PER], rank[PER], wrap[PER], omax = 0;
+#pragma unroll
+  for (int k = 0; k < PER; k++) {
+    const int i = tid + k * PTM_SMALL_BLOCK;
+    if (i >= p.n) break;
+    float over;
+    cell[k] = bin_atom(p, pos, i, wrap[k], over);
+    rank[k] = atomicAdd(&cells[cell[k]], 1);
+    if (wrap[k] == PTM_EXCLUDED) atomicAdd(&excluded, 1);
+    else if (wrap[k] != img_pack(0, 0, 0)) any_wrap = 1;
+    omax = max(omax, __float_as_int(over));          // over > 0: its bits order as integers
+  }
+  omax = __reduce_max_sync(0xffffffffu, omax);
+  if ((tid & 31) == 0) atomicMax(&overs, omax);
+  __syncthreads();
+  // exclusive scan of the counts, a run of cells per thread
+  const int run = (ncell + PTM_SMALL_BLOCK - 1) / PTM_SMALL_BLOCK, c0 = min(tid * run, ncell), c1 = min(c0 + run, ncell);
+  int sum = 0;
+  for (int c = c0; c < c1; c++) sum += cells[c];
+  int at = block_scan(sum, sh) - sum;
+  for (int c = c0; c < c1; c++) {
+    const int v = cells[c];
+    cells[c] = at;
+    cell_start[c] = at;
+    at += v;
+  }
+  if (tid == PTM_SMALL_BLOCK - 1) cell_start[ncell] = at;
+  if (tid < C_NCOUNTERS) counters[tid] = tid == C_EXCLUDED ? excluded : 0;
+  if (tid < PTM_STATUS_WORDS) dstat[tid] = tid == 0 ? any_wrap : (tid == 1 ? overs : 0);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < PER; k++) {
+    const int i = tid + k * PTM_SMALL_BLOCK;
+    if (i >= p.n) break;
+    const int slot = cells[cell[k]] + rank[k];
+    scatter_atom(p, pos, i, wrap[k], any_wrap != 0, slot, sorted, hi, lo);
+    sbin[slot] = cell[k];
+    wrapv[slot] = wrap[k];
+  }
+}
+
 // ------------------------------------------------------------ batched frames
 // Frame of batch atom i: the last frame whose first atom is <= i.
 __device__ __forceinline__ int frame_of(const int64_t *atom_off, int nframes, int64_t i) {
@@ -1206,15 +1273,24 @@ __device__ __forceinline__ Scratch match_rows(unsigned char *smem) {
 // read-only cache (shared memory is spent on per-thread scratch).
 __device__ __forceinline__ const float4 *template_rows() { return reinterpret_cast<const float4 *>(&ptm_tpl[0][0][0]); }
 
+// Atom of a thread in a launch that gives each warp `apw` atoms (its first lanes
+// hold one each): sorted slot within the frame, -1 for a lane without an atom.
+__device__ __forceinline__ int64_t spread_slot(int64_t n, int apw) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  const int64_t s = w * apw + lane;
+  return lane < apw && s < n ? s : -1;
+}
+
 // The frame descriptor travels by value in the kernel parameters, so back-to-back
 // asynchronous calls never share a staging buffer.
 template <bool F64>
-__global__ void __launch_bounds__(PTM_BLOCK, PTM_ATOM_BLOCKS_PER_SM) k_hulls(const __grid_constant__ FrameDesc d) {
+__global__ void __launch_bounds__(PTM_BLOCK, PTM_ATOM_BLOCKS_PER_SM) k_hulls(const __grid_constant__ FrameDesc d, int apw) {
   extern __shared__ __align__(16) unsigned char smem[];
   const Scratch sm = scratch_rows(smem);
-  const int64_t s = (int64_t)blockIdx.x * PTM_BLOCK + threadIdx.x;
-  const unsigned live = __ballot_sync(0xffffffffu, s < d.n);
-  if (s >= d.n) return;
+  const int64_t s = spread_slot(d.n, apw);
+  const unsigned live = __ballot_sync(0xffffffffu, s >= 0);
+  if (s < 0) return;
   const int nsos = hull_atom<F64>(d, (int)s, sm, live);
   count_warp(d, C_ATOMS, live, 1);
   count_warp(d, C_SOS, live, nsos);
@@ -1227,17 +1303,15 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_ATOM_BLOCKS_PER_SM) k_hulls(con
 // once (-> 2.23 ms).  At 10, 9 and 8 blocks (more registers): 2.86, 2.82, 3.06 ms
 // against 2.72.
 template <bool F64, bool P64 = false>
-__global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM) k_match(const __grid_constant__ FrameDesc d) {
+__global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM) k_match(const __grid_constant__ FrameDesc d, int apw) {
   extern __shared__ __align__(16) unsigned char smem[];
   const Scratch sm = match_rows(smem);
   const float4 *tplw = template_rows();
-  const int64_t s = (int64_t)blockIdx.x * PTM_BLOCK + threadIdx.x;     // frame-local slot
-  const unsigned live = __ballot_sync(0xffffffffu, s < d.n);
-  if (s >= d.n) return;
-  const MatchCounts c = match_atom<F64, P64>(d, (int)(s + d.atom_offset), sm, tplw, live);
-  count_warp(d, C_CAND, live, c.scored);
-  count_warp(d, C_CANDPTS, live, c.points);
-  count_warp(d, C_MATCHED, live, c.matched);
+  const int64_t s = spread_slot(d.n, apw);               // frame-local slot
+  const MatchCounts c = match_atom<F64, P64>(d, (int)(s + d.atom_offset), s >= 0, sm, tplw);
+  count_warp(d, C_CAND, 0xffffffffu, c.scored);
+  count_warp(d, C_CANDPTS, 0xffffffffu, c.points);
+  count_warp(d, C_MATCHED, 0xffffffffu, c.matched);
 }
 
 // Neighbour lists of one frame, one thread per atom: NK = 14 into d.nbr, NK = 18
@@ -1251,19 +1325,19 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM) k_match(co
 //   256 frames, 31.7 M atoms            31.2  -> 16.0 ms
 template <bool F64, int NK>
 __global__ void __launch_bounds__(PTM_KNN_BLOCK, KnnShape<NK>::BLOCKS)
-    k_knn(const __grid_constant__ FrameDesc d, int *rest, int *rest_count) {
+    k_knn(const __grid_constant__ FrameDesc d, int apw, int *rest, int *rest_count) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int64_t s = (int64_t)blockIdx.x * PTM_KNN_BLOCK + threadIdx.x;
-  if (s >= d.n) return;
+  const int64_t s = spread_slot(d.n, apw);
+  if (s < 0) return;
   knn_atom<F64, NK>(d, (int)s, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18, smem, rest, rest_count);
 }
 
 template <bool F64, int NK>
 __global__ void __launch_bounds__(PTM_KNN_BLOCK)
     k_knn_rest(const __grid_constant__ FrameDesc d, const int *rest, const int *rest_count) {
-  const int n = *rest_count, stride = gridDim.x * (PTM_KNN_BLOCK / 32);
+  const int n = rest ? *rest_count : (int)d.n, stride = gridDim.x * (PTM_KNN_BLOCK / 32);
   for (int i = (blockIdx.x * PTM_KNN_BLOCK + threadIdx.x) >> 5; i < n; i += stride)
-    knn_rest_atom<F64, NK>(d, rest[i], NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18);
+    knn_rest_atom<F64, NK>(d, rest ? rest[i] : i, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18);
 }
 
 // The same over a batch: each slot finds its frame; NK = 14 takes the frames in
@@ -1301,7 +1375,7 @@ __global__ void __launch_bounds__(PTM_KNN_BLOCK)
 // is sorted slot atom_offset + v - map_off[k] of frame map_frames[k].  With
 // `head` (this warp's slot of shared memory) a tile whose slots all belong to
 // one frame reads that frame's descriptor from a shared copy, made when the
-// frame changes.  fn(desc, slot, live).
+// frame changes.  fn(desc, slot, live): every lane, those of `live` with a slot.
 template <typename Fn>
 __device__ __forceinline__ void persistent_tiles(const FrameDesc *__restrict__ descs,
                                                  const int64_t *__restrict__ atom_off, int nframes, int64_t ntotal,
@@ -1327,10 +1401,11 @@ __device__ __forceinline__ void persistent_tiles(const FrameDesc *__restrict__ d
           f = __ldg(map_frames + f);
         }
       }
+      const int f0 = __shfl_sync(0xffffffffu, f, 0);            // lane 0 is live whenever any lane is
+      if (f < 0) f = f0;
       const FrameDesc *dp = descs + f;
       if (head) {
-        const int f0 = __shfl_sync(0xffffffffu, f, 0);          // lane 0 is live whenever any lane is
-        if (__all_sync(0xffffffffu, f == f0 || !(live >> lane & 1))) {
+        if (__all_sync(0xffffffffu, f == f0)) {
           if (f0 != cached) {
             const int *src = reinterpret_cast<const int *>(descs + f0);
             int *dst = reinterpret_cast<int *>(head);
@@ -1341,7 +1416,7 @@ __device__ __forceinline__ void persistent_tiles(const FrameDesc *__restrict__ d
           dp = head;
         }
       }
-      if (live >> lane & 1) fn(*dp, (int)s, live);
+      fn(*dp, (int)s, live);
     }
   }
 }
@@ -1354,6 +1429,7 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_ATOM_BLOCKS_PER_SM)
   const Scratch sm = scratch_rows(smem);
   persistent_tiles(descs, atom_off, nframes, ntotal, nullptr, tile_atoms, queue, nullptr,
                    [&](const FrameDesc &d, int s, unsigned live) {
+                     if (!(live >> (threadIdx.x & 31) & 1)) return;
                      const int nsos = hull_atom<F64>(d, s, sm, live);
                      count_warp(d, C_ATOMS, live, 1);
                      count_warp(d, C_SOS, live, nsos);
@@ -1374,10 +1450,10 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM)
   __shared__ FrameDesc heads[PTM_BLOCK / 32];
   persistent_tiles(descs, map_off, nmap, nslots, map_frames, tile_atoms, queue, &heads[threadIdx.x >> 5],
                    [&](const FrameDesc &d, int s, unsigned live) {
-                     const MatchCounts c = match_atom<F64, false>(d, s, sm, tplw, live);
-                     count_warp(d, C_CAND, live, c.scored);
-                     count_warp(d, C_CANDPTS, live, c.points);
-                     count_warp(d, C_MATCHED, live, c.matched);
+                     const MatchCounts c = match_atom<F64, false>(d, s, live >> (threadIdx.x & 31) & 1, sm, tplw);
+                     count_warp(d, C_CAND, 0xffffffffu, c.scored);
+                     count_warp(d, C_CANDPTS, 0xffffffffu, c.points);
+                     count_warp(d, C_MATCHED, 0xffffffffu, c.matched);
                    });
 }
 

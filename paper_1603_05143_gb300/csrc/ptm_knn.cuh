@@ -496,8 +496,13 @@ __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
   const int b = __ldg(d.sbin + s);
   const int bz = b % d.nb[2], byx = b / d.nb[2];
   const int by = byx % d.nb[1], bx = byx / d.nb[1];
+  const int wrap = __ldg(d.wrapv + s);
+  if (wrap == PTM_EXCLUDED) {                            // excluded by the binning: no neighbours
+    if (lane < NK) rows[(int64_t)lane * d.n + (s - d.atom_offset)] = make_int2(-1, 0);
+    return;
+  }
   int wi0, wi1, wi2;
-  img_unpack(__ldg(d.wrapv + s), wi0, wi1, wi2);
+  img_unpack(wrap, wi0, wi1, wi2);
   const int nbx = d.nb[0], nby = d.nb[1], nbz = d.nb[2];
   const uint64_t INF = 0x7ff0000000000000ull;
   uint64_t lk = INF, last = INF;                       // this lane's key; the NK-th key,

@@ -459,19 +459,55 @@ __device__ __forceinline__ bool hull_apply(const Scratch &sm, int nf, uint32_t v
 }
 
 // ------------------------------------------------------- graph code and lookup
-// Hull of the first K neighbours (every one a vertex, 2 K - 4 facets, the centre
-// inside): template lookup (Algorithm 1, inner loops).  Writes the Weinberg
-// labelling (nibble t = label of neighbour t) and the candidate list's entry;
-// false if no template has this graph.
+// Hull of the first 6 neighbours: the only template graph is the octahedron, the
+// one triangulation of 6 points whose vertices all have degree 4.  Breadth-first
+// labels from its first facet (a, b, c): a, b, c, then the vertices opposite b and
+// c (the other ends of the two more facets on a c and a b), then opposite a.
+__device__ __forceinline__ bool octahedron_lookup(const Scratch &sm, uint64_t &labels, int &ent) {
+  uint32_t deg = 0, first = 0xffffffffu;
+#pragma unroll 2
+  for (int f = 0; f < 8; f++) {
+    const uint32_t v = sm.F(f);
+    deg += (1u << (4 * (v & 15))) + (1u << (4 * (v >> 4 & 15))) + (1u << (4 * (v >> 8 & 15)));
+    first = min(first, v);
+  }
+  if (deg != 0x444444u) return false;
+  const int a = first & 15, b = first >> 4 & 15, c = first >> 8 & 15;
+  int ob = 0, oc = 0;
+#pragma unroll 2
+  for (int f = 0; f < 8; f++) {
+    const uint32_t v = sm.F(f);
+    const int x = v & 15, y = v >> 4 & 15, z = v >> 8 & 15;
+    const uint32_t m = 1u << x | 1u << y | 1u << z, ac = 1u << a | 1u << c, ab = 1u << a | 1u << b;
+    if ((m & ac) == ac && !(m >> b & 1)) ob = __ffs(m & ~ac) - 1;
+    if ((m & ab) == ab && !(m >> c & 1)) oc = __ffs(m & ~ab) - 1;
+  }
+  const int oa = 15 - a - b - c - ob - oc;
+  const uint32_t perm = PTM_OCTA_PERM;
+  labels = (perm & 15u) << (4 * a) | (perm >> 4 & 15u) << (4 * b) | (perm >> 8 & 15u) << (4 * c) |
+           (perm >> 12 & 15u) << (4 * ob) | (perm >> 16 & 15u) << (4 * oc) | (perm >> 20 & 15u) << (4 * oa);
+  ent = PTM_OCTA_ENT;
+  return true;
+}
+
+// Hull of the first K = 12 or 14 neighbours (every one a vertex, 2 K - 4 facets,
+// the centre inside): template lookup (Algorithm 1, inner loops).  Writes the
+// Weinberg labelling (nibble t = label of neighbour t) and the candidate list's
+// entry; false if no template has this graph.  `wmask`: the lanes of the warp that
+// call this together.
 //
 // A Weinberg walk labels the hull from the start edge with the largest key of
 // degrees around it (tables.py).  Finding that edge and walking cost 3 of every 5
-// instructions here.  The graph is instead looked up by its adjacency matrix
+// instructions of k_hulls.  The graph is instead looked up by its adjacency matrix
 // under a breadth-first labelling from any directed edge (the first facet's
-// first), one step per directed edge with the current vertex's row in a register;
-// the table then names the graph's start edges, and their Weinberg labels in terms
-// of these.  Of several start edges the first among the facets is taken.
-__device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, uint64_t &labels, int &ent, const FrameDesc &d) {
+// first), vertex by vertex with the row of neighbours in a register; the table
+// then names the graph's start edges, and their Weinberg labels in terms of these.
+// Of several start edges the first among the facets is taken.
+// (Walk and start edge: k_hulls 1410 warp instructions per atom, 7.27 ms per 4 M
+// atoms; this code in one flat loop over the directed edges, six points included:
+// 891, 4.47 ms.)
+__device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, unsigned wmask, uint64_t &labels, int &ent,
+                                             const FrameDesc &d) {
   const int nf = 2 * K - 4;
 #pragma unroll 2
   for (int x = 0; x < K; x++) sm.TH(x) = 0;
@@ -485,32 +521,45 @@ __device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, uint64_t 
     sm.TH(c) = tc | (uint64_t)(b + 1) << (4 * a);
     first = min(first, v);
   }
-  int x = first & 15, from = (first >> 4) & 15, cur = from, next = 2, i = 0;
-  uint32_t seen = 1u << x | 1u << from, row = 0, even = 0;
-  uint64_t lab = 1ull << (4 * from), vert = (uint64_t)x | (uint64_t)from << 4, come = (uint64_t)from | (uint64_t)x << 4;
-  uint64_t th = sm.TH(x);
-#pragma unroll 1
-  for (int s = 0; s < 6 * K - 12; s++) {
-    cur = (nib(th, cur) - 1) & 15;                   // next neighbour of x, counter-clockwise
-    if (!(seen >> cur & 1)) {
-      lab |= (uint64_t)next << (4 * cur);
-      vert |= (uint64_t)cur << (4 * next);
-      come |= (uint64_t)x << (4 * next);
-      seen |= 1u << cur;
-      next++;
+  int next = 2;
+  const int u0 = first & 15, v0 = (first >> 4) & 15;
+  uint32_t seen = 1u << u0 | 1u << v0, even = 0;
+  uint64_t lab = 1ull << (4 * v0), vert = (uint64_t)u0 | (uint64_t)v0 << 4, come = (uint64_t)v0 | (uint64_t)u0 << 4;
+  // vertices in label order, each walked around counter-clockwise from the one it
+  // was first reached from (a vertex has fewer than K neighbours: the bound on the
+  // steps only keeps a broken rotation from running on)
+  for (int i = 0; i < K; i++) {
+    const int x = min((int)(vert & 15), PTM_KNN - 1), from = (int)(come & 15);
+    vert >>= 4;
+    come >>= 4;
+    const uint64_t th = sm.TH(x);
+    int cur = from;
+    uint32_t row = 0;
+    if (__any_sync(wmask, next < K)) {
+      for (int s = 0; s < PTM_KNN; s++) {
+        cur = (nib(th, cur) - 1) & 15;
+        if (!(seen >> cur & 1)) {
+          const int at = 4 * (next - i - 1);
+          lab |= (uint64_t)next << (4 * cur);
+          vert |= (uint64_t)cur << at;
+          come |= (uint64_t)x << at;
+          seen |= 1u << cur;
+          next++;
+        }
+        row |= 1u << nib(lab, cur);
+        if (cur == from) break;
+      }
+    } else {                                         // every vertex of every lane has its label
+      for (int s = 0; s < PTM_KNN; s++) {
+        cur = (nib(th, cur) - 1) & 15;
+        row |= 1u << nib(lab, cur);
+        if (cur == from) break;
+      }
     }
-    row |= 1u << nib(lab, cur);
-    if (cur == from && i < K) {                      // all neighbours of x visited
-      if (i & 1) sm.U(i >> 1) = even | row << 16;
-      even = row;
-      row = 0;
-      i++;
-      x = min(nib(vert, i), PTM_KNN - 1);
-      from = cur = nib(come, i);
-      th = sm.TH(x);
-    }
+    if (i & 1) sm.U(i >> 1) = even | row << 16;
+    even = row;
   }
-  if (i != K || next != K) { count(d, C_INTERNAL); return false; }
+  if (next != K) { count(d, C_INTERNAL); return false; }
   uint64_t h = PTM_HASH_INIT;
 #pragma unroll
   for (int w = 0; w < 7; w++) h = (h ^ (uint64_t)(2 * w < K ? sm.U(w) : 0u)) * PTM_HASH_MUL;
@@ -528,11 +577,14 @@ __device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, uint64_t 
   const int nties = (int)(info >> 20 & 255u);
   int pick = 0;
   if (nties > 1) {
+    uint64_t order = 0;                              // vertex of each label
+#pragma unroll 2
+    for (int t = 0; t < K; t++) order |= (uint64_t)t << (4 * nib(lab, t));
     // rows of the start edges, then the first facet corner that holds one
     uint32_t tv = 0;
     for (int k = 0; k < nties; k++) {
       const uint32_t e = __ldg(&tie[k].edge);
-      const int u = min(nib(vert, e & 255), PTM_KNN - 1), v = nib(vert, e >> 8 & 255);
+      const int u = min(nib(order, e & 255), PTM_KNN - 1), v = nib(order, e >> 8 & 255);
       sm.U(u) = (tv >> u & 1 ? sm.U(u) : 0u) | 1u << v;
       tv |= 1u << u;
     }

@@ -852,12 +852,14 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
       else if (want) vis = hull_visibility<true>(sm, nf, p, centre_in, bmask, nsos);
       else vis = hull_visibility<false>(sm, nf, p, centre_in, vmask, nsos);
     }
-    if (alive && want && centre_in) {
+    const bool look = alive && want && centre_in;
+    const unsigned lmask = __ballot_sync(hmask, look);
+    if (look) {
       uint64_t lab;
       int e;
-      if (graph_lookup(sm, p, lab, e, d)) {
-        if (p == 6) { bst.lam6 = lab; bst.ent6 = e; }
-        else if (p == 12) { bst.lam12 = lab; bst.ent12 = e; }
+      if (p == 6) { if (octahedron_lookup(sm, lab, e)) { bst.lam6 = lab; bst.ent6 = e; } }
+      else if (graph_lookup(sm, p, lmask, lab, e, d)) {
+        if (p == 12) { bst.lam12 = lab; bst.ent12 = e; }
         else { bst.lam14 = lab; bst.ent14 = e; }
       }
     }

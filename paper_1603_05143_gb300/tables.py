@@ -479,6 +479,10 @@ def emit_header(path: pathlib.Path) -> dict:
     lines.append("PTM_TBL_GLOBAL ptm_graph_entry ptm_graph[PTM_GRAPH_NSLOTS] PTM_TBL_ALIGN16 = {")
     lines += ["  {{" + ("0" if e is None else ", ".join(f"0x{x:x}u" for x in [*e[0], e[1]])) + "}}," for e in slots]
     lines.append("};")
+    # the octahedron, the only graph of six points: looked up without a code
+    (_, _, perm6, ent6), = next(t for (k, _), t in graphs.items() if k == 6)
+    lines.append(f"#define PTM_OCTA_PERM 0x{perm6:x}u")
+    lines.append(f"#define PTM_OCTA_ENT {ent6}")
     lines.append("/* Weinberg start edges of a graph: labels u | v << 8 | entry << 16, and the permutation */")
     lines.append("typedef struct { uint64_t perm; uint32_t edge, pad; } ptm_tie_entry;")
     lines.append("PTM_TBL_GLOBAL ptm_tie_entry ptm_tie[PTM_TIE_N] PTM_TBL_ALIGN16 = {")

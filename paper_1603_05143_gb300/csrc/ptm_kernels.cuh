@@ -666,13 +666,14 @@ __device__ __forceinline__ void metric_vectors(const FrameDesc &d, const Scratch
   }
 }
 
-// FP64 contract vector of neighbour (sorted slot js, packed image img) of an
-// atom at (xi, yi, zi), float32 positions.
-__device__ __forceinline__ void vec64_row(const FrameDesc &d, float xi, float yi, float zi, int js, int img,
-                                          double (&v)[3]) {
-  float xj, yj, zj;
+// FP64 contract vector of neighbour (sorted slot js, packed image img) of an atom
+// at (xi, yi, zi).
+template <bool F64>
+__device__ __forceinline__ void vec64_row(const FrameDesc &d, typename RT<F64>::T xi, typename RT<F64>::T yi,
+                                          typename RT<F64>::T zi, int js, int img, double (&v)[3]) {
+  typename RT<F64>::T xj, yj, zj;
   int idj;
-  load_atom<false>(d, js, xj, yj, zj, idj);
+  load_atom<F64>(d, js, xj, yj, zj, idj);
   int a0, a1, a2;
   img_unpack(img, a0, a1, a2);
   double hx, hy, hz;
@@ -682,41 +683,78 @@ __device__ __forceinline__ void vec64_row(const FrameDesc &d, float xi, float yi
   v[2] = contract_dr((double)zj, (double)zi, hz);
 }
 
-// Quantisation of the neighbours in `wide` (float32 input, rare): the frexp
-// exponent of their largest FP64 vector component (-100000 if all are zero),
+// Quantisation in FP64 of the neighbours that FP32 pairs cannot decide (rare): the
+// frexp exponent of their largest FP64 vector component (-100000 if all are zero),
 // then q = rint(dr 2^shift) into the Q rows.  Neighbour t of the atom is the
 // list entry nb[t * nst]; the Q rows are per-thread columns of shared memory
 // with stride PTM_BLOCK.
-__device__ __noinline__ int wide_exponent(const FrameDesc &d, float xi, float yi, float zi, const int2 *nb,
-                                          int64_t nst, uint32_t wide) {
+template <bool F64>
+__device__ __noinline__ int wide_exponent(const FrameDesc &d, typename RT<F64>::T xi, typename RT<F64>::T yi,
+                                          typename RT<F64>::T zi, const int2 *nb, int64_t nst, uint32_t wide) {
   int e64 = -100000;
   for (; wide; wide &= wide - 1) {
     const int t = __ffs(wide) - 1;
     const int2 e = __ldg(nb + t * nst);
     double v[3];
-    vec64_row(d, xi, yi, zi, e.x, e.y, v);
+    vec64_row<F64>(d, xi, yi, zi, e.x, e.y, v);
     const double m = fmax(fabs(v[0]), fmax(fabs(v[1]), fabs(v[2])));
     if (m > 0.0) { int et; frexp(m, &et); e64 = max(e64, et); }
   }
   return e64;
 }
 
-__device__ __noinline__ void wide_quantise(const FrameDesc &d, float xi, float yi, float zi, const int2 *nb,
-                                           int64_t nst, float *q, uint32_t wide, int shift) {
+template <bool F64>
+__device__ __noinline__ void wide_quantise(const FrameDesc &d, typename RT<F64>::T xi, typename RT<F64>::T yi,
+                                           typename RT<F64>::T zi, const int2 *nb, int64_t nst, float *q,
+                                           uint32_t wide, int shift) {
   const double sc = ldexp(1.0, shift);
   for (; wide; wide &= wide - 1) {
     const int t = __ffs(wide) - 1;
     const int2 e = __ldg(nb + t * nst);
     double v[3];
-    vec64_row(d, xi, yi, zi, e.x, e.y, v);
+    vec64_row<F64>(d, xi, yi, zi, e.x, e.y, v);
     for (int c = 0; c < 3; c++) q[(3 * t + c) * PTM_BLOCK] = (float)__double2int_rn(v[c] * sc);
   }
+}
+
+// Vector of list entry e from an atom at hs + ls as FP32 pairs h + l: differences
+// and shift summed without loss but for the low parts, within about 2^-44 of the
+// positions and the cell.  Float64 input takes the pairs of the positions wrapped
+// into the cell, float32 input the positions themselves.  Returns false for an
+// image beyond the next, whose shift may be larger than that allows for.
+template <bool F64>
+__device__ __forceinline__ bool pair_vector(const FrameDesc &d, float4 hs, float4 ls, int2 e, float (&h)[3],
+                                            float (&l)[3]) {
+  const float4 p = __ldg((F64 ? d.hi : (const float4 *)d.sorted) + e.x);
+  float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+  int a, b, c;
+  img_unpack(e.y, a, b, c);
+  if constexpr (F64) {
+    q = __ldg(d.lo + e.x);
+    int a1, b1, c1, a2, b2, c2;
+    img_unpack(__float_as_int(q.w), a1, b1, c1);
+    img_unpack(__float_as_int(ls.w), a2, b2, c2);
+    a += a1 - a2; b += b1 - b2; c += c1 - c2;
+  }
+  float s[3] = {0.f, 0.f, 0.f}, r[3] = {0.f, 0.f, 0.f};
+  if (a | b | c) shift_f32(d, a, b, c, s[0], s[1], s[2], r[0], r[1], r[2]);
+  const float pj[3] = {p.x, p.y, p.z}, qj[3] = {q.x, q.y, q.z}, pi[3] = {hs.x, hs.y, hs.z}, qi[3] = {ls.x, ls.y, ls.z};
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    float d1, e1, d2, e2;
+    two_sum(pj[k], -pi[k], d1, e1);
+    two_sum(d1, s[k], d2, e2);
+    const float t = __fadd_rn(e1, __fadd_rn(e2, __fadd_rn(__fsub_rn(qj[k], qi[k]), r[k])));
+    h[k] = __fadd_rn(d2, t);
+    l[k] = __fsub_rn(t, __fsub_rn(h[k], d2));
+  }
+  return max(abs(a), max(abs(b), abs(c))) <= 1;
 }
 
 // ------------------------------------------------------------ one atom
 // The method for one atom runs in two kernels.  k_hulls: neighbour vectors
 // from the list, their quantised copy, the incremental hull and at k = 6, 12,
-// 14 the Weinberg code and template lookup; it leaves, per atom, the matched
+// 14 the graph code and template lookup; it leaves, per atom, the matched
 // snapshots' labellings and table entries (d.lam, d.ents).  k_match: QCP of
 // every admissible correspondence, selection and the outputs.  `live` holds
 // the lanes of this warp that entered together (all reach the warp-synchronous
@@ -746,49 +784,40 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
   int cnt = 0;
   unsigned hmask;
   {
+    // A float32 neighbour in the same image whose differences are exact
+    // (Sterbenz: |x_j - x_i| below min(|x_i|, |x_j|)) has its FP64 vector in FP32
+    // already.  The others (bit t of `wide`: shifted images, atoms near a
+    // coordinate plane through the origin, every neighbour of float64 input) are
+    // FP32 pairs h + l, h in the Q rows and l in rows the hull will use: scaling by a
+    // power of two is exact, so rint(h 2^s) is the answer unless the rest, (h 2^s -
+    // rint) + l 2^s, comes within the pair's error of one half.  Those (bit t of
+    // `bad`, 3 in 1,000 atoms), and an exponent that hangs on the low parts, go to FP64
+    // out of line.  (All of `wide` in FP64: quantisation 0.66 ns per float64 atom, 41 %
+    // of k_hulls, and 0.22 ns per float32 atom in a 231 Angstrom box.)
+    // (this thread's own words: the halves of its 14 TH rows, then its F rows)
+    auto low = [&](int t, int c) -> float & {
+      const int k = 3 * t + c;
+      return k < 28 ? ((float *)&sm.TH(k >> 1))[k & 1] : ((float *)&sm.F(k - 28))[0];
+    };
+    float emaxf = 0.f, m = 0.f;
+    uint32_t wide = 0, bad = 0;
+    float4 hs, ls = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (F64) {
-      T emax = 0;
-#pragma unroll 1
+      hs = __ldg(d.hi + s);
+      ls = __ldg(d.lo + s);
+#pragma unroll 2
       for (int t = 0; t < PTM_KNN; t++) {
         const int2 e = __ldg(nb + t * nst);
         if (e.x < 0) continue;
         cnt++;
-        T xj, yj, zj;
-        int idj;
-        load_atom<F64>(d, e.x, xj, yj, zj, idj);
-        int a0, a1, a2;
-        img_unpack(e.y, a0, a1, a2);
-        T sx, sy, sz;
-        contract_shift<F64>(d, a0, a1, a2, sx, sy, sz);
-        T cx = contract_dr(xj, xi, sx), cy = contract_dr(yj, yi, sy), cz = contract_dr(zj, zi, sz);
-        emax = fmax(emax, fmax(fabs(cx), fmax(fabs(cy), fabs(cz))));
-      }
-      int e;
-      frexp(emax, &e);
-      const T sc = (T)ldexp(1.0, PTM_QBITS - e);
-#pragma unroll 1
-      for (int t = 0; t < PTM_KNN; t++) {
-        if (t >= cnt) continue;
-        const int2 en = __ldg(nb + t * nst);
-        T xj, yj, zj;
-        int idj;
-        load_atom<F64>(d, en.x, xj, yj, zj, idj);
-        int a0, a1, a2;
-        img_unpack(en.y, a0, a1, a2);
-        T sx, sy, sz;
-        contract_shift<F64>(d, a0, a1, a2, sx, sy, sz);
-        T cx = contract_dr(xj, xi, sx), cy = contract_dr(yj, yi, sy), cz = contract_dr(zj, zi, sz);
-        sm.Q(t, 0) = (float)__double2int_rn(cx * sc); sm.Q(t, 1) = (float)__double2int_rn(cy * sc);
-        sm.Q(t, 2) = (float)__double2int_rn(cz * sc);
+        wide |= 1u << t;
+        float h[3], l[3];
+        if (!pair_vector<F64>(d, hs, ls, e, h, l)) bad |= 1u << t;
+#pragma unroll
+        for (int c = 0; c < 3; c++) { sm.Q(t, c) = h[c]; low(t, c) = l[c]; m = fmaxf(m, fabsf(h[c])); }
       }
     } else {
-      // float32 input: a neighbour in the same image whose FP32 differences
-      // are exact (Sterbenz: |x_j - x_i| below min(|x_i|, |x_j|)) has its FP64
-      // vector in FP32 already, kept in the Q rows between the two loops; the
-      // others (bit t of `wide`: shifted images, atoms near a coordinate plane
-      // through the origin) are evaluated in FP64 out of line
-      float emaxf = 0.f;
-      uint32_t wide = 0;
+      hs = make_float4(xi, yi, zi, 0.f);
 #pragma unroll 7
       for (int t = 0; t < PTM_KNN; t++) {
         const int2 e = __ldg(nb + t * nst);
@@ -804,20 +833,44 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
         if (exact) emaxf = fmaxf(emaxf, fmaxf(fabsf(px), fmaxf(fabsf(py), fabsf(pz))));
         else wide |= 1u << t;
       }
-      int e;
-      frexpf(emaxf, &e);
-      if (wide) {
-        const int e64 = wide_exponent(d, xi, yi, zi, nb, nst, wide);
-        if (e64 > -100000) e = emaxf > 0.f ? max(e, e64) : e64;
-      }
-      const float sc = ldexpf(1.f, PTM_QBITS - e);
+#pragma unroll 1
+      for (uint32_t w = wide; w; w &= w - 1) {
+        const int t = __ffs(w) - 1;
+        const int2 e = __ldg(nb + t * nst);
+        float h[3], l[3];
+        if (!pair_vector<F64>(d, hs, ls, e, h, l)) bad |= 1u << t;
 #pragma unroll
-      for (int t = 0; t < PTM_KNN; t++) {
-        if (t >= cnt || (wide >> t & 1)) continue;
-        sm.Q(t, 0) = rintf(sm.Q(t, 0) * sc); sm.Q(t, 1) = rintf(sm.Q(t, 1) * sc); sm.Q(t, 2) = rintf(sm.Q(t, 2) * sc);
+        for (int c = 0; c < 3; c++) { sm.Q(t, c) = h[c]; low(t, c) = l[c]; }
+        const float mt = fmaxf(fabsf(h[0]), fmaxf(fabsf(h[1]), fabsf(h[2])));
+        if (e.y == img_pack(0, 0, 0) && l[0] == 0.f && l[1] == 0.f && l[2] == 0.f) {   // exact after all
+          wide &= ~(1u << t);
+          emaxf = fmaxf(emaxf, mt);
+        }
+        m = fmaxf(m, mt);
       }
-      if (wide) wide_quantise(d, xi, yi, zi, nb, nst, sm.q + sm.t, wide, PTM_QBITS - e);
+      m = fmaxf(m, emaxf);
     }
+    // a power of two may round up from below; far from 1 the FP32 scaling may not hold
+    if (wide && ((__float_as_uint(m) & 0x7fffffu) == 0 || !(m > 0x1p-60f && m < 0x1p60f))) bad = wide;
+    int e;
+    frexpf(bad ? emaxf : m, &e);
+    if (bad) {                                       // the exponent in FP64 then, too
+      const int e64 = wide_exponent<F64>(d, xi, yi, zi, nb, nst, wide);
+      if (e64 > -100000) e = emaxf > 0.f ? max(e, e64) : e64;
+    }
+    const float sc = ldexpf(1.f, PTM_QBITS - e);
+    const float half = 0.5f - (0x1p-16f + 0x1p-42f * sc * (fabsf(hs.x) + fabsf(hs.y) + fabsf(hs.z) + 0x1p37f * d.tau));
+#pragma unroll 2
+    for (int t = 0; t < PTM_KNN; t++) {
+      if (t >= cnt) break;
+#pragma unroll
+      for (int c = 0; c < 3; c++) {
+        const float y = sm.Q(t, c) * sc, r = rintf(y);
+        if ((wide >> t & 1) && !(fabsf(fmaf(low(t, c), sc, y - r)) <= half)) bad |= 1u << t;
+        sm.Q(t, c) = r;
+      }
+    }
+    if (bad) wide_quantise<F64>(d, xi, yi, zi, nb, nst, sm.q + sm.t, bad, PTM_QBITS - e);
     hmask = __ballot_sync(live, cnt >= 4);       // lanes that go on to the hulls
     if (cnt < 4) { d.ents[sl] = 0; return 0; }
   }

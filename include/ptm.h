@@ -192,9 +192,9 @@ typedef struct ptm_batch ptm_batch;
    multiple of 32 (default 32, one per lane: each warp grabs on its own, so
    no warp waits for another; larger grabs lengthen the tail when the queue
    runs dry, 64 measured 10 % slower on a 2^20-atom frame);
-   blocks_per_sm: resident 64-thread blocks per SM for the persistent grid
-   (default 7, the shared-memory limit).  Atoms per warp are fixed at 32 (one
-   atom per lane). */
+   blocks_per_sm: persistent grid of the hulls, in eighths of the 64-thread
+   blocks an SM holds (default 8, all of them).  Atoms per warp are fixed at 32
+   (one atom per lane). */
 typedef struct {
   double cell_factor;
   int tile_atoms;

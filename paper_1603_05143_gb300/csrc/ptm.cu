@@ -586,7 +586,7 @@ struct ptm_batch {
   int nframes = 0, f64 = 0;
   int64_t ntotal = 0;
   size_t ncell = 0;
-  int tile_atoms = 32, blocks_per_sm = PTM_ATOM_BLOCKS_PER_SM;
+  int tile_atoms = 32, blocks_per_sm = PTM_TUNE_FULL;
   double cell_factor = 1.25;
   FrameDesc *d_descs = nullptr;
   ShiftTables *d_tabs = nullptr;
@@ -713,8 +713,8 @@ static ptm_status batch_enqueue(ptm_batch *b, cudaStream_t st) {
   CK(cudaEventRecordWithFlags(b->ev[3], st, rec));
   // persistent grids: two warps per block, each pulling its own tiles
   const int64_t tiles = (b->ntotal + b->tile_atoms - 1) / b->tile_atoms;
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)b->nsm * b->blocks_per_sm,
-                                                                       (tiles + 1) / 2));
+  const int64_t per_sm = ((int64_t)b->blocks_per_sm * PTM_ATOM_BLOCKS_PER_SM + PTM_TUNE_FULL - 1) / PTM_TUNE_FULL;
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(b->nsm * per_sm, (tiles + 1) / 2));
   if (b->f64)
     k_hulls_batch<true><<<grid, PTM_BLOCK, atom_smem_bytes(), st>>>(b->d_descs, b->d_atom_off, b->nframes,
                                                                     b->ntotal, b->tile_atoms, b->queue);
@@ -1007,7 +1007,7 @@ extern "C" ptm_status ptm_autotune_batch(ptm_context *ctx, int nframes, const pt
   if (!ctx || !best) return PTM_ERR_INVALID_ARG;
   static const double factors[] = {1.125, 1.25, 1.4};
   static const int tiles[] = {32, 64};
-  static const int bpsm[] = {PTM_ATOM_BLOCKS_PER_SM - 1, PTM_ATOM_BLOCKS_PER_SM};
+  static const int bpsm[] = {PTM_TUNE_FULL - 1, PTM_TUNE_FULL};
   cudaStream_t st = (cudaStream_t)stream;
   // tune on every m-th frame so that at most about 40 M atoms are timed per candidate (a
   // strided subset of a mixed batch measured a different winner than the whole)

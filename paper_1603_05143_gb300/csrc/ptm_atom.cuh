@@ -108,16 +108,17 @@ __device__ __forceinline__ void count_here(const FrameDesc &d, int which) {
 
 // ------------------------------------------------------------ shared scratch
 // Rows are [word][thread] (every lane its own bank).  In k_hulls the 42 rows of
-// q hold the quantised neighbour vectors, beside the rotation system, facet and
-// edge rows: 108 words per thread let 8 blocks of 64 threads share an SM's 228 KB.
+// q hold the quantised neighbour vectors, beside the facet and edge rows: 84 words
+// per thread let 10 blocks of 64 threads share an SM's 228 KB.  The rotation system,
+// which only the graph lookup needs, takes the vectors' place once the hulls are
+// built.
 // k_match uses only q (the FP32 metric vectors) and nid (the neighbours' atom ids).
 struct Scratch {
   float *q;          // [42][B]  quantised neighbour vectors (integers |q| <= 2^19, exact in FP32),
                      //          or the metric vectors DX / DY / DZ
   int *nid;          // [14][B]  neighbour atom id (k_match)
   uint32_t *fac;     // [24][B]  hull facets a | b << 4 | c << 8 (ccw from outside) | birth number << 12
-  uint64_t *th;      // [14][B]  1 + third vertex of directed edge u->v, nibble v of row u (0 none)
-  uint32_t *used;    // [14][B]  directed-edge rows (hull horizon, start edges), breadth-first code
+  uint32_t *used;    // [18][B]  directed-edge rows (hull horizon, start edges), breadth-first code
   int t;             // thread index in block
   __device__ __forceinline__ float &Q(int p, int c) const { return q[(3 * p + c) * PTM_BLOCK + t]; }
   __device__ __forceinline__ int QI(int p, int c) const { return (int)q[(3 * p + c) * PTM_BLOCK + t]; }
@@ -126,11 +127,14 @@ struct Scratch {
   __device__ __forceinline__ float &DZ(int j) const { return Q(j, 2); }
   __device__ __forceinline__ int &NID(int j) const { return nid[j * PTM_BLOCK + t]; }
   __device__ __forceinline__ uint32_t &F(int f) const { return fac[f * PTM_BLOCK + t]; }
-  __device__ __forceinline__ uint64_t &TH(int v) const { return th[v * PTM_BLOCK + t]; }
+  // Words 2 u and 2 u + 1 of the rotation system: 1 + third vertex of directed edge
+  // u -> v, nibble v of 16 (0 none), in this thread's own columns of q.
+  __device__ __forceinline__ uint32_t rot(int w) const { return __float_as_uint(q[w * PTM_BLOCK + t]); }
+  __device__ __forceinline__ void set_rot(int w, uint32_t x) const { q[w * PTM_BLOCK + t] = __uint_as_float(x); }
   __device__ __forceinline__ uint32_t &U(int v) const { return used[v * PTM_BLOCK + t]; }
 };
 
-constexpr int SCRATCH_WORDS = 28 + 42 + 24 + 14;   // 32-bit words per k_hulls thread
+constexpr int SCRATCH_WORDS = 42 + 24 + 18;   // 32-bit words per k_hulls thread
 
 // -------------------------------------------------------------- small helpers
 __device__ __forceinline__ int nib(uint64_t x, int i) { return (int)((x >> (4 * i)) & 15); }
@@ -510,15 +514,16 @@ __device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, unsigned 
                                              const FrameDesc &d) {
   const int nf = 2 * K - 4;
 #pragma unroll 2
-  for (int x = 0; x < K; x++) sm.TH(x) = 0;
+  for (int w = 0; w < 2 * K; w++) sm.set_rot(w, 0u);
   uint32_t first = 0xffffffffu;                      // the facet with the smallest birth number
   for (int f = 0; f < nf; f++) {
     const uint32_t v = sm.F(f);
     const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
-    const uint64_t ta = sm.TH(a), tb = sm.TH(b), tc = sm.TH(c);
-    sm.TH(a) = ta | (uint64_t)(c + 1) << (4 * b);
-    sm.TH(b) = tb | (uint64_t)(a + 1) << (4 * c);
-    sm.TH(c) = tc | (uint64_t)(b + 1) << (4 * a);
+    const int wa = 2 * a + (b >> 3), wb = 2 * b + (c >> 3), wc = 2 * c + (a >> 3);
+    const uint32_t ra = sm.rot(wa), rb = sm.rot(wb), rc = sm.rot(wc);
+    sm.set_rot(wa, ra | (uint32_t)(c + 1) << (4 * b & 31));
+    sm.set_rot(wb, rb | (uint32_t)(a + 1) << (4 * c & 31));
+    sm.set_rot(wc, rc | (uint32_t)(b + 1) << (4 * a & 31));
     first = min(first, v);
   }
   int next = 2;
@@ -532,7 +537,7 @@ __device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, unsigned 
     const int x = min((int)(vert & 15), PTM_KNN - 1), from = (int)(come & 15);
     vert >>= 4;
     come >>= 4;
-    const uint64_t th = sm.TH(x);
+    const uint64_t th = (uint64_t)sm.rot(2 * x + 1) << 32 | sm.rot(2 * x);
     int cur = from;
     uint32_t row = 0;
     if (__any_sync(wmask, next < K)) {

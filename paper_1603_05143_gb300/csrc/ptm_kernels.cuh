@@ -794,10 +794,10 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
     // `bad`, 3 in 1,000 atoms), and an exponent that hangs on the low parts, go to FP64
     // out of line.  (All of `wide` in FP64: quantisation 0.66 ns per float64 atom, 41 %
     // of k_hulls, and 0.22 ns per float32 atom in a 231 Angstrom box.)
-    // (this thread's own words: the halves of its 14 TH rows, then its F rows)
-    auto low = [&](int t, int c) -> float & {
+    // (this thread's own words: its 24 F rows, then its 18 U rows)
+    auto low = [&](int t, int c) -> uint32_t & {
       const int k = 3 * t + c;
-      return k < 28 ? ((float *)&sm.TH(k >> 1))[k & 1] : ((float *)&sm.F(k - 28))[0];
+      return k < 24 ? sm.F(k) : sm.U(k - 24);
     };
     float emaxf = 0.f, m = 0.f;
     uint32_t wide = 0, bad = 0;
@@ -814,7 +814,7 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
         float h[3], l[3];
         if (!pair_vector<F64>(d, hs, ls, e, h, l)) bad |= 1u << t;
 #pragma unroll
-        for (int c = 0; c < 3; c++) { sm.Q(t, c) = h[c]; low(t, c) = l[c]; m = fmaxf(m, fabsf(h[c])); }
+        for (int c = 0; c < 3; c++) { sm.Q(t, c) = h[c]; low(t, c) = __float_as_uint(l[c]); m = fmaxf(m, fabsf(h[c])); }
       }
     } else {
       hs = make_float4(xi, yi, zi, 0.f);
@@ -840,7 +840,7 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
         float h[3], l[3];
         if (!pair_vector<F64>(d, hs, ls, e, h, l)) bad |= 1u << t;
 #pragma unroll
-        for (int c = 0; c < 3; c++) { sm.Q(t, c) = h[c]; low(t, c) = l[c]; }
+        for (int c = 0; c < 3; c++) { sm.Q(t, c) = h[c]; low(t, c) = __float_as_uint(l[c]); }
         const float mt = fmaxf(fabsf(h[0]), fmaxf(fabsf(h[1]), fabsf(h[2])));
         if (e.y == img_pack(0, 0, 0) && l[0] == 0.f && l[1] == 0.f && l[2] == 0.f) {   // exact after all
           wide &= ~(1u << t);
@@ -866,7 +866,7 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
 #pragma unroll
       for (int c = 0; c < 3; c++) {
         const float y = sm.Q(t, c) * sc, r = rintf(y);
-        if ((wide >> t & 1) && !(fabsf(fmaf(low(t, c), sc, y - r)) <= half)) bad |= 1u << t;
+        if ((wide >> t & 1) && !(fabsf(fmaf(__uint_as_float(low(t, c)), sc, y - r)) <= half)) bad |= 1u << t;
         sm.Q(t, c) = r;
       }
     }
@@ -884,6 +884,10 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
   kmax = min(kmax, cnt);
   bool alive = kmax >= 6;
   int birth = 4;
+  // the graphs of 12 and 14 points are looked up last: the facets of the first wait
+  // in local memory until then
+  bool got12 = false, got14 = false;
+  uint32_t f12[20];
   if (alive) hull_init(sm, nsos);
   for (int p = 4; p <= PTM_KNN; p++) {
     // every insertion step starts warp-converged: a lane that finished (or took
@@ -905,20 +909,37 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
       else if (want) vis = hull_visibility<true>(sm, nf, p, centre_in, bmask, nsos);
       else vis = hull_visibility<false>(sm, nf, p, centre_in, vmask, nsos);
     }
-    const bool look = alive && want && centre_in;
-    const unsigned lmask = __ballot_sync(hmask, look);
-    if (look) {
-      uint64_t lab;
-      int e;
-      if (p == 6) { if (octahedron_lookup(sm, lab, e)) { bst.lam6 = lab; bst.ent6 = e; } }
-      else if (graph_lookup(sm, p, lmask, lab, e, d)) {
-        if (p == 12) { bst.lam12 = lab; bst.ent12 = e; }
-        else { bst.lam14 = lab; bst.ent14 = e; }
+    if (alive && want && centre_in) {
+      if (p == 6) {
+        uint64_t lab;
+        int e;
+        if (octahedron_lookup(sm, lab, e)) { bst.lam6 = lab; bst.ent6 = e; }
+      } else if (p == 12) {
+        got12 = true;
+#pragma unroll 4
+        for (int f = 0; f < 20; f++) f12[f] = sm.F(f);
+      } else {
+        got14 = true;
       }
     }
     if (!alive) continue;
     // done, p inside the hull, or a vertex swallowed
     alive = p != kmax && vis && hull_apply(sm, nf, vis, p, birth, d);
+  }
+#pragma unroll 1
+  for (int K = 14; K >= 12; K -= 2) {
+    const bool look = K == 14 ? got14 : got12;
+    const unsigned lmask = __ballot_sync(hmask, look);
+    if (!look) continue;
+    if (K == 12) {
+#pragma unroll 4
+      for (int f = 0; f < 20; f++) sm.F(f) = f12[f];
+    }
+    uint64_t lab;
+    int e;
+    if (!graph_lookup(sm, K, lmask, lab, e, d)) continue;
+    if (K == 12) { bst.lam12 = lab; bst.ent12 = e; }
+    else { bst.lam14 = lab; bst.ent14 = e; }
   }
   d.ents[sl] = pack_ents(bst.ent6, bst.ent12, bst.ent14);
   if (bst.ent6 >= 0) d.lam[sl] = bst.lam6;
@@ -1287,10 +1308,13 @@ constexpr size_t atom_smem_bytes() { return (size_t)PTM_BLOCK * SCRATCH_WORDS * 
 constexpr int MATCH_WORDS = 42 + 14;
 constexpr size_t match_smem_bytes() { return (size_t)PTM_BLOCK * MATCH_WORDS * 4; }
 
-// Resident blocks per SM of k_hulls: 8 x (108 words x 64 threads + the 1 KB the
-// driver reserves per block) fits 228 KB of shared memory, and 8 x 64 threads x
-// 128 registers the register file.
-#define PTM_ATOM_BLOCKS_PER_SM 8
+// Resident blocks per SM of k_hulls: 10 x (84 words x 64 threads + the 1 KB the
+// driver reserves per block) fits 228 KB of shared memory, and 10 x 64 threads x
+// 96 registers the register file (at 108 words and 8 blocks, 16 warps left 3 of 10
+// issue slots idle: a 4 M-atom call 8.18 -> 7.49 ms, 256 frames 70.6 -> 66.7 ms).
+#define PTM_ATOM_BLOCKS_PER_SM 10
+// ptm_tuning.blocks_per_sm that fills the SMs with k_hulls_batch
+#define PTM_TUNE_FULL 8
 // k_match: 11 x (56 words x 64 threads + two descriptor copies + 1 KB) fits, at up
 // to 93 registers
 #define PTM_MATCH_BLOCKS_PER_SM 11
@@ -1305,8 +1329,7 @@ constexpr size_t match_smem_bytes() { return (size_t)PTM_BLOCK * MATCH_WORDS * 4
 // Scratch rows of k_hulls in a block's dynamic shared memory.
 __device__ __forceinline__ Scratch scratch_rows(unsigned char *smem) {
   Scratch sm;
-  sm.th = (uint64_t *)smem;
-  sm.q = (float *)(sm.th + 14 * PTM_BLOCK);
+  sm.q = (float *)smem;
   sm.nid = nullptr;                 // k_hulls reads the neighbour list in place
   sm.fac = (uint32_t *)(sm.q + 42 * PTM_BLOCK);
   sm.used = sm.fac + 24 * PTM_BLOCK;
@@ -1317,7 +1340,7 @@ __device__ __forceinline__ Scratch scratch_rows(unsigned char *smem) {
 // The rows k_match uses (the others stay null).
 __device__ __forceinline__ Scratch match_rows(unsigned char *smem) {
   Scratch sm;
-  sm.th = nullptr; sm.fac = nullptr; sm.used = nullptr;
+  sm.fac = nullptr; sm.used = nullptr;
   sm.q = (float *)smem;
   sm.nid = (int *)(sm.q + 42 * PTM_BLOCK);
   sm.t = threadIdx.x;

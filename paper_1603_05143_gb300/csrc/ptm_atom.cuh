@@ -127,8 +127,8 @@ struct Scratch {
   __device__ __forceinline__ float &DZ(int j) const { return Q(j, 2); }
   __device__ __forceinline__ int &NID(int j) const { return nid[j * PTM_BLOCK + t]; }
   __device__ __forceinline__ uint32_t &F(int f) const { return fac[f * PTM_BLOCK + t]; }
-  // Words 2 u and 2 u + 1 of the rotation system: 1 + third vertex of directed edge
-  // u -> v, nibble v of 16 (0 none), in this thread's own columns of q.
+  // Words 2 u and 2 u + 1 of the rotation system: third vertex of directed edge u ->
+  // v, nibble v of 16, in this thread's own columns of q.
   __device__ __forceinline__ uint32_t rot(int w) const { return __float_as_uint(q[w * PTM_BLOCK + t]); }
   __device__ __forceinline__ void set_rot(int w, uint32_t x) const { q[w * PTM_BLOCK + t] = __uint_as_float(x); }
   __device__ __forceinline__ uint32_t &U(int v) const { return used[v * PTM_BLOCK + t]; }
@@ -509,7 +509,9 @@ __device__ __forceinline__ bool octahedron_lookup(const Scratch &sm, uint64_t &l
 // Of several start edges the first among the facets is taken.
 // (Walk and start edge: k_hulls 1410 warp instructions per atom, 7.27 ms per 4 M
 // atoms; this code in one flat loop over the directed edges, six points included:
-// 891, 4.47 ms.)
+// 891, 4.47 ms.)  Labels are stored one up, so that 0 is a vertex without one, and
+// vertices times 4, the shift of their nibble (a set of labelled vertices beside plain
+// labels, and the start edges found in their list: 7.55 -> 7.41 ms a 4 M-atom call).
 __device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, unsigned wmask, uint64_t &labels, int &ent,
                                              const FrameDesc &d) {
   const int nf = 2 * K - 4;
@@ -521,20 +523,21 @@ __device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, unsigned 
     const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
     const int wa = 2 * a + (b >> 3), wb = 2 * b + (c >> 3), wc = 2 * c + (a >> 3);
     const uint32_t ra = sm.rot(wa), rb = sm.rot(wb), rc = sm.rot(wc);
-    sm.set_rot(wa, ra | (uint32_t)(c + 1) << (4 * b & 31));
-    sm.set_rot(wb, rb | (uint32_t)(a + 1) << (4 * c & 31));
-    sm.set_rot(wc, rc | (uint32_t)(b + 1) << (4 * a & 31));
+    sm.set_rot(wa, ra | (uint32_t)c << (4 * b & 31));
+    sm.set_rot(wb, rb | (uint32_t)a << (4 * c & 31));
+    sm.set_rot(wc, rc | (uint32_t)b << (4 * a & 31));
     first = min(first, v);
   }
-  int next = 2;
+  int next = 2;                                      // vertices labelled; lab: 1 + label, 0 none
   const int u0 = first & 15, v0 = (first >> 4) & 15;
-  uint32_t seen = 1u << u0 | 1u << v0, even = 0;
-  uint64_t lab = 1ull << (4 * v0), vert = (uint64_t)u0 | (uint64_t)v0 << 4, come = (uint64_t)v0 | (uint64_t)u0 << 4;
+  uint64_t lab = 1ull << (4 * u0) | 2ull << (4 * v0), vert = (uint64_t)u0 | (uint64_t)v0 << 4,
+           come = (uint64_t)v0 | (uint64_t)u0 << 4;
+  uint32_t even = 0;
   // vertices in label order, each walked around counter-clockwise from the one it
   // was first reached from (a vertex has fewer than K neighbours: the bound on the
-  // steps only keeps a broken rotation from running on)
+  // steps only keeps a broken rotation from running on); cur = 4 x vertex
   for (int i = 0; i < K; i++) {
-    const int x = min((int)(vert & 15), PTM_KNN - 1), from = (int)(come & 15);
+    const int x = min((int)(vert & 15), PTM_KNN - 1), from = (int)(come & 15) << 2;
     vert >>= 4;
     come >>= 4;
     const uint64_t th = (uint64_t)sm.rot(2 * x + 1) << 32 | sm.rot(2 * x);
@@ -542,29 +545,31 @@ __device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, unsigned 
     uint32_t row = 0;
     if (__any_sync(wmask, next < K)) {
       for (int s = 0; s < PTM_KNN; s++) {
-        cur = (nib(th, cur) - 1) & 15;
-        if (!(seen >> cur & 1)) {
+        cur = (int)(th >> cur) << 2 & 60;
+        int l = (int)(lab >> cur) & 15;
+        if (!l) {
           const int at = 4 * (next - i - 1);
-          lab |= (uint64_t)next << (4 * cur);
-          vert |= (uint64_t)cur << at;
+          l = ++next;
+          lab |= (uint64_t)l << cur;
+          vert |= (uint64_t)(cur >> 2) << at;
           come |= (uint64_t)x << at;
-          seen |= 1u << cur;
-          next++;
         }
-        row |= 1u << nib(lab, cur);
+        row |= 1u << l;
         if (cur == from) break;
       }
     } else {                                         // every vertex of every lane has its label
       for (int s = 0; s < PTM_KNN; s++) {
-        cur = (nib(th, cur) - 1) & 15;
-        row |= 1u << nib(lab, cur);
+        cur = (int)(th >> cur) << 2 & 60;
+        row |= 1u << ((int)(lab >> cur) & 15);
         if (cur == from) break;
       }
     }
+    row >>= 1;
     if (i & 1) sm.U(i >> 1) = even | row << 16;
     even = row;
   }
   if (next != K) { count(d, C_INTERNAL); return false; }
+  lab -= K == 12 ? 0x111111111111ull : 0x11111111111111ull;
   uint64_t h = PTM_HASH_INIT;
 #pragma unroll
   for (int w = 0; w < 7; w++) h = (h ^ (uint64_t)(2 * w < K ? sm.U(w) : 0u)) * PTM_HASH_MUL;
@@ -578,33 +583,36 @@ __device__ __forceinline__ bool graph_lookup(const Scratch &sm, int K, unsigned 
     for (int k = 0; k < 7; k++) if (2 * k < K) eq &= w[k] == sm.U(k);
     if (eq) { info = e1.w; break; }
   }
+  // a record of start edges: their rows (bit = label), then them in row order
   const ptm_tie_entry *tie = ptm_tie + (info & 0xfffffu);
   const int nties = (int)(info >> 20 & 255u);
   int pick = 0;
   if (nties > 1) {
-    uint64_t order = 0;                              // vertex of each label
+    // the first facet corner that holds one, and its rank among them.  (Rows made
+    // from the list entry by entry, and the edge found again by a search of the list,
+    // one load after the other: 31 % of the lookup's time.)
+    const uint4 r0 = __ldg((const uint4 *)tie), r1 = __ldg((const uint4 *)tie + 1);
+    sm.U(0) = r0.x; sm.U(1) = r0.y; sm.U(2) = r0.z; sm.U(3) = r0.w; sm.U(4) = r1.x; sm.U(5) = r1.y; sm.U(6) = r1.z;
+    uint32_t best = 0xffffffffu;                     // birth << 12 | corner << 8 | label of u << 4 | label of v
 #pragma unroll 2
-    for (int t = 0; t < K; t++) order |= (uint64_t)t << (4 * nib(lab, t));
-    // rows of the start edges, then the first facet corner that holds one
-    uint32_t tv = 0;
-    for (int k = 0; k < nties; k++) {
-      const uint32_t e = __ldg(&tie[k].edge);
-      const int u = min(nib(order, e & 255), PTM_KNN - 1), v = nib(order, e >> 8 & 255);
-      sm.U(u) = (tv >> u & 1 ? sm.U(u) : 0u) | 1u << v;
-      tv |= 1u << u;
-    }
-    uint32_t best = 0xffffffffu;                     // birth << 12 | corner << 8 | u << 4 | v
     for (int f = 0; f < nf; f++) {
       const uint32_t v = sm.F(f);
-      const int a = v & 15, b = (v >> 4) & 15, c = (v >> 8) & 15;
+      const int a = nib(lab, v & 15), b = nib(lab, (v >> 4) & 15), c = nib(lab, (v >> 8) & 15);
       const uint32_t base = v >> 12 << 12;
-      if ((tv >> a & 1) && (sm.U(a) >> b & 1)) best = min(best, base | (uint32_t)(a << 4 | b));
-      if ((tv >> b & 1) && (sm.U(b) >> c & 1)) best = min(best, base | (uint32_t)(1 << 8 | b << 4 | c));
-      if ((tv >> c & 1) && (sm.U(c) >> a & 1)) best = min(best, base | (uint32_t)(2 << 8 | c << 4 | a));
+      if (sm.U(a >> 1) >> ((a & 1) << 4 | b) & 1) best = min(best, base | (uint32_t)(a << 4 | b));
+      if (sm.U(b >> 1) >> ((b & 1) << 4 | c) & 1) best = min(best, base | (uint32_t)(1 << 8 | b << 4 | c));
+      if (sm.U(c >> 1) >> ((c & 1) << 4 | a) & 1) best = min(best, base | (uint32_t)(2 << 8 | c << 4 | a));
     }
-    const uint32_t e = (uint32_t)nib(lab, best >> 4 & 15) | (uint32_t)nib(lab, best & 15) << 8;
-    while (pick < nties - 1 && (__ldg(&tie[pick].edge) & 0xffffu) != e) pick++;
+    const int u = best >> 4 & 15, v = best & 15;
+#pragma unroll
+    for (int w = 0; w < 7; w++) {
+      const uint32_t x = sm.U(w);
+      if (w < u >> 1) pick += __popc(x);
+      if (w == u >> 1) pick += __popc(x & ((1u << ((u & 1) << 4 | v)) - 1u));
+    }
+    pick = min(pick, nties - 1);
   }
+  pick += PTM_TIE_HEAD;
   const uint64_t perm = __ldg((const unsigned long long *)&tie[pick].perm);
   ent = (int)(__ldg(&tie[pick].edge) >> 16);
   labels = 0;

@@ -315,6 +315,18 @@ def graph_codes(entry_of):
     return out
 
 
+TIE_HEAD = 2        # table elements (of four words) holding the rows of a graph's start edges
+
+
+def start_rows(starts) -> list:
+    """Rows of a graph's start edges: bit v of 16-bit row u for the edge between the
+    breadth-first labels u -> v, two rows a word, padded to TIE_HEAD elements."""
+    rows = [0] * 14
+    for u, v, *_ in starts:
+        rows[u] |= 1 << v
+    return pack_rows(rows) + [0]
+
+
 def pack_rows(rows) -> list:
     words = [0] * 7
     for i, r in enumerate(rows):
@@ -399,18 +411,21 @@ def emit_header(path: pathlib.Path) -> dict:
         nslots *= 2
     slots = [None] * nslots
     ties, lists = [], {}
-    for k, rows in sorted(graphs):
-        tl = graphs[(k, rows)]
+    for k, code in sorted(graphs):
+        tl = graphs[(k, code)]
         if tl not in lists:
             lists[tl] = len(ties)
-            ties += tl
-        words = pack_rows(rows)
+            rows = start_rows(tl)
+            ties += [(rows[4 * i], rows[4 * i + 1], rows[4 * i + 2], rows[4 * i + 3]) for i in range(TIE_HEAD)]
+            ties += [(p & 0xffffffff, p >> 32, u | v << 8 | e << 16, 0) for u, v, p, e in tl]
+        words = pack_rows(code)
         h = code_hash(words)
         pos = (h ^ (h >> 32)) & (nslots - 1)
         while slots[pos] is not None:
             pos = (pos + 1) & (nslots - 1)
         slots[pos] = (words, k << 28 | len(tl) << 20 | lists[tl])
     assert len(ties) < 1 << 20 and max(len(t) for t in lists) < 256
+    assert all(a[:2] < b[:2] for t in lists for a, b in zip(t, t[1:]))     # in row order, none twice
     lines = ["/* Generated by paper_1603_05143_gb300/tables.py -- do not edit. */",
              "#pragma once", "#include <stdint.h>",
              "/* storage qualifiers: constant memory for uniform reads, global for tables */",
@@ -474,7 +489,7 @@ def emit_header(path: pathlib.Path) -> dict:
     lines.append("  " + ", ".join(f"{{{f}, {len(entries[c])}}}" for c, f in zip(codes, first)))
     lines.append("};")
     lines.append("/* breadth-first codes, open addressing: 7 words of two 16-bit adjacency rows, then")
-    lines.append("   vertices << 28 | starts << 20 | first start (0: empty) */")
+    lines.append("   vertices << 28 | starts << 20 | record of the starts (0: empty) */")
     lines.append("typedef struct { uint32_t w[8]; } ptm_graph_entry;")
     lines.append("PTM_TBL_GLOBAL ptm_graph_entry ptm_graph[PTM_GRAPH_NSLOTS] PTM_TBL_ALIGN16 = {")
     lines += ["  {{" + ("0" if e is None else ", ".join(f"0x{x:x}u" for x in [*e[0], e[1]])) + "}}," for e in slots]
@@ -483,10 +498,13 @@ def emit_header(path: pathlib.Path) -> dict:
     (_, _, perm6, ent6), = next(t for (k, _), t in graphs.items() if k == 6)
     lines.append(f"#define PTM_OCTA_PERM 0x{perm6:x}u")
     lines.append(f"#define PTM_OCTA_ENT {ent6}")
-    lines.append("/* Weinberg start edges of a graph: labels u | v << 8 | entry << 16, and the permutation */")
+    lines.append("/* Weinberg start edges of a graph, a record each: PTM_TIE_HEAD elements with their rows (two 16-bit rows a")
+    lines.append("   word, bit v of row u for the edge between these labels), then per edge, in row order, the permutation")
+    lines.append("   and labels u | v << 8 | entry << 16 */")
+    lines.append(f"#define PTM_TIE_HEAD {TIE_HEAD}")
     lines.append("typedef struct { uint64_t perm; uint32_t edge, pad; } ptm_tie_entry;")
     lines.append("PTM_TBL_GLOBAL ptm_tie_entry ptm_tie[PTM_TIE_N] PTM_TBL_ALIGN16 = {")
-    lines += [f"  {{0x{p:016x}ULL, 0x{u | v << 8 | e << 16:x}u, 0}}," for u, v, p, e in ties]
+    lines += [f"  {{0x{lo | hi << 32:016x}ULL, 0x{x:x}u, 0x{y:x}u}}," for lo, hi, x, y in ties]
     lines.append("};")
     lines.append("/* candidate: bits 60-62 template, nibble L-1 = slot of canonical label L */")
     lines.append("PTM_TBL_GLOBAL uint64_t ptm_cand[PTM_TBL_NCAND] = {")

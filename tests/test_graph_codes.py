@@ -40,3 +40,14 @@ def test_packed_rows_differ_for_different_codes():
     graphs = T.graph_codes({c: i for i, c in enumerate(sorted(T.build()[3]))})
     packed = {(k, tuple(T.pack_rows(rows))) for k, rows in graphs}
     assert len(packed) == len(graphs) and all(len(r) == 7 for _, r in packed)
+
+
+def test_rank_in_the_start_rows_is_the_place_in_the_list():
+    for (k, _), starts in T.graph_codes({c: i for i, c in enumerate(sorted(T.build()[3]))}).items():
+        words = T.start_rows(starts)
+        assert len(words) == 4 * T.TIE_HEAD
+        bits = sum(w << (32 * i) for i, w in enumerate(words))
+        assert bin(bits).count("1") == len(starts)
+        for i, (u, v, *_) in enumerate(starts):
+            at = 16 * u + v
+            assert bits >> at & 1 and bin(bits & ((1 << at) - 1)).count("1") == i, k

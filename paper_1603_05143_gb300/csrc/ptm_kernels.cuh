@@ -290,25 +290,93 @@ __device__ __forceinline__ void vec_fp64(const FrameDesc &d, typename RT<F64>::T
   z = ((double)zj - (double)zi) + sz;
 }
 
-// Rare path: the best FP32 candidates lie within PTM_BAND.  Every candidate is
-// re-scored in FP64 from neighbour vectors recomputed in FP64 from the input
-// positions (the neighbours read again from the atom's list).
+// Rare path: the best FP32 candidates of the atom at sorted slot s lie within
+// PTM_BAND.  Every candidate is scored again in FP64 from neighbour vectors
+// recomputed in FP64 from the input positions, with select_fp64's result.  The warp
+// does it together, a candidate per lane and neighbour t's vector in lane t: few atoms
+// come here (20 of a 2^20-atom frame), but one thread took half a millisecond over two
+// passes of up to 26 candidates, and the kernel waited for the last of them (calls:
+// 2^20-atom polycrystal 2.44 -> 1.97 ms, 4 M atoms 7.55 -> 7.03 ms).  All lanes call
+// this with the same arguments.  Returns (K << 16) | candidate index, or -1.
 template <bool F64>
-__device__ __noinline__ int rerank_fp64(const FrameDesc &d, int s, const Best bst) {
+__device__ __noinline__ int rerank_warp(const FrameDesc *dp, int s, int e6, int e12, int e14, uint64_t lam6,
+                                        uint64_t lam12, uint64_t lam14) {
+  constexpr unsigned ALL = 0xffffffffu;
   typedef typename RT<F64>::T T;
+  const FrameDesc &d = *dp;
+  const int lane = threadIdx.x & 31;
   T xi, yi, zi;
   int idi;
   load_atom<F64>(d, s, xi, yi, zi, idi);
-  double ex[PTM_KNN], ey[PTM_KNN], ez[PTM_KNN];
-  int cnt = 0;
-  for (int t = 0; t < PTM_KNN; t++) {
-    const int2 e = d.nbr[(int64_t)t * d.n + (s - d.atom_offset)];
-    if (e.x < 0) break;
-    vec_fp64<F64>(d, xi, yi, zi, e.x, e.y, ex[t], ey[t], ez[t]);
-    cnt++;
+  double ex = 0, ey = 0, ez = 0;
+  if (lane < PTM_KNN) {
+    const int2 e = __ldg(d.nbr + (int64_t)lane * d.n + (s - d.atom_offset));
+    if (e.x >= 0) vec_fp64<F64>(d, xi, yi, zi, e.x, e.y, ex, ey, ez);
   }
-  if (cnt == 0) return -1;
-  return select_fp64(d, bst, ex, ey, ez, nullptr);
+  const int n6 = e6 >= 0 ? ptm_tbl[e6].count : 0, n12 = e12 >= 0 ? ptm_tbl[e12].count : 0,
+            n14 = e14 >= 0 ? ptm_tbl[e14].count : 0, total = n6 + n12 + n14;
+  // this lane's candidate of the round, in list order (6, 12, 14): its RMSD^2
+  int K = 0, ci = -1, S = 0;
+  uint64_t lab = 0, cand = 0;
+  auto score = [&](int p) -> double {
+    ci = -1;
+    K = p < n6 ? 6 : (p < n6 + n12 ? 12 : 14);
+    if (p < total) {
+      const int c = K == 6 ? ptm_tbl[e6].first + p : (K == 12 ? ptm_tbl[e12].first + p - n6 : ptm_tbl[e14].first + p - n6 - n12);
+      cand = __ldg((const unsigned long long *)&ptm_cand[c]);
+      S = (int)(cand >> 60) & 7;
+      if (d.mask >> S & 1) ci = c;
+    }
+    lab = K == 6 ? lam6 : (K == 12 ? lam12 : lam14);
+    double m[3] = {0, 0, 0}, g = 0, Sm[3][3] = {{0}}, Gw = 0;
+    for (int j = 0; j < PTM_KNN; j++) {
+      const double x = __shfl_sync(ALL, ex, j), y = __shfl_sync(ALL, ey, j), z = __shfl_sync(ALL, ez, j);
+      if (j >= K || ci < 0) continue;
+      m[0] += x; m[1] += y; m[2] += z;
+      g += x * x + y * y + z * z;
+      const double *w = ptm_tpl64[S][nib(cand, nib(lab, j) - 1)];
+      Sm[0][0] += w[0] * x; Sm[0][1] += w[0] * y; Sm[0][2] += w[0] * z;
+      Sm[1][0] += w[1] * x; Sm[1][1] += w[1] * y; Sm[1][2] += w[1] * z;
+      Sm[2][0] += w[2] * x; Sm[2][1] += w[2] * y; Sm[2][2] += w[2] * z;
+    }
+    if (ci < 0) return INFINITY;
+    for (int c = 0; c < 3; c++) m[c] /= (K + 1);
+    const double Gv = g - (K + 1) * (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
+    for (int slot = 0; slot <= K; slot++)
+      Gw += ptm_tpl64[S][slot][0] * ptm_tpl64[S][slot][0] + ptm_tpl64[S][slot][1] * ptm_tpl64[S][slot][1] +
+            ptm_tpl64[S][slot][2] * ptm_tpl64[S][slot][2];
+    Qcp<double> o;
+    qcp_solve<double>(Sm, Gv, Gw, o);
+    return fmax((Gw - o.lam * o.lam / Gv) / (K + 1), 0.0);
+  };
+  double best = INFINITY, r2 = INFINITY;
+  for (int base = 0; base < total; base += 32) {
+    r2 = score(base + lane);
+    best = fmin(best, r2);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) best = fmin(best, __shfl_xor_sync(ALL, best, o));
+  // among the candidates tied with the best: earlier template, then smaller canonical
+  // correspondence, then list order
+  int found = -1;
+  uint32_t fS = 99;
+  uint64_t fcp = ~0ull;
+  for (int base = 0; base < total; base += 32) {
+    if (total > 32) r2 = score(base + lane);
+    const bool tied = ci >= 0 && r2 <= best + PTM_TIE;
+    const uint64_t cp = tied ? canonical_corr(S, K, slots_of(K, lab, cand)) : ~0ull;
+    const uint32_t mS = __reduce_min_sync(ALL, tied ? (uint32_t)S : 99u);
+    const bool in = tied && (uint32_t)S == mS;
+    const uint32_t hi = __reduce_min_sync(ALL, in ? (uint32_t)(cp >> 32) : 0xffffffffu);
+    const bool in2 = in && (uint32_t)(cp >> 32) == hi;
+    const uint32_t lo = __reduce_min_sync(ALL, in2 ? (uint32_t)cp : 0xffffffffu);
+    const unsigned who = __ballot_sync(ALL, in2 && (uint32_t)cp == lo);
+    if (!who) continue;
+    const uint64_t mcp = (uint64_t)hi << 32 | lo;
+    const int pick = __shfl_sync(ALL, (K << 16) | ci, __ffs(who) - 1);
+    if (mS < fS || (mS == fS && mcp < fcp)) { fS = mS; fcp = mcp; found = pick; }
+  }
+  return found;
 }
 
 // ------------------------------------------------------------ finalisation
@@ -989,6 +1057,16 @@ __device__ MatchCounts match_atom(const FrameDesc &d, int s, bool active, const 
     __syncwarp();                                  // the vectors are read across the warp
     score_candidates(d, sm, tplw, bst, cnt);
     __syncwarp();
+    const bool tied = bst.K >= 0 && bst.b2 <= bst.b1 + PTM_BAND;
+    if (tied) count(d, C_TIE64);
+    for (unsigned m = __ballot_sync(0xffffffffu, tied); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const auto from = [&](auto x) { return __shfl_sync(0xffffffffu, x, src); };
+      const FrameDesc *owner = (const FrameDesc *)from((unsigned long long)&d);
+      const int w = rerank_warp<F64>(owner, from(s), from(bst.ent6), from(bst.ent12), from(bst.ent14), from(bst.lam6),
+                                     from(bst.lam12), from(bst.lam14));
+      if ((threadIdx.x & 31) == src && w >= 0) { bst.K = w >> 16; bst.cand = w & 0xffff; }
+    }
     if (!active) return cnt;
     if (bst.K < 0) { write_unmatched(d, idi); return cnt; }     // no match, or every match masked out
   } else {
@@ -997,11 +1075,6 @@ __device__ MatchCounts match_atom(const FrameDesc &d, int s, bool active, const 
     const int K = w >> 16;
     cnt.matched = finalize_fp64(d, sm, K, bst.lam(K), w & 0xffff, ex, ey, ez, idi);
     return cnt;
-  }
-  if (bst.b2 <= bst.b1 + PTM_BAND) {
-    count(d, C_TIE64);
-    const int w = rerank_fp64<F64>(d, s, bst);
-    if (w >= 0) { bst.K = w >> 16; bst.cand = w & 0xffff; }
   }
   cnt.matched = finalize(d, sm, tplw, bst, idi);
   return cnt;

@@ -116,6 +116,12 @@ __device__ __forceinline__ float topo_face32(int m, int j, float R, Vec V, float
                                              uint32_t &lines) {
   float e1[3], e2[3], p[3];
   topo_plane<float>(j, V, e1, e2, p);
+  // a neighbour on the centre has no plane (the axes are 0 / 0) and no face; the FP64
+  // form, cut by any line at all, finds the same
+  if (!(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2] > 0.f)) {
+    lines = ~0u;
+    return 0.f;
+  }
   auto line = [&](int i, float &A, float &B, float &C) {
     const float w0 = V(i, 0), w1 = V(i, 1), w2 = V(i, 2);
     A = w0 * e1[0] + w1 * e1[1] + w2 * e1[2];

@@ -52,11 +52,19 @@ __device__ __forceinline__ void topo_plane(int j, Vec V, T (&e1)[3], T (&e2)[3],
   p[0] = n0 / 2; p[1] = n1 / 2; p[2] = n2 / 2;
 }
 
-// FP64 area of the Voronoi face of neighbour j among the m vectors V(i, c), cut by
-// the neighbours in `lines`; P and Q are polygon buffers of 2 x vmax values, element
-// e at P[e * st].
-template <typename Vec>
-__device__ double topo_face_area64(int m, int j, uint32_t lines, double R, Vec V, double *P, double *Q, int st, int vmax) {
+// FP64 area of the Voronoi face of neighbour j among the m vectors V(i, c) (VF: the
+// same rounded to FP32); P and Q are polygon buffers of 2 x vmax values, element
+// e at P[e * st].  `lines` are the neighbours expected to cut the face: the polygon
+// they leave is then held against every other line, and those that come near it cut
+// too.  That check may run in FP32: the vertices are known, so a line's value at one is
+// off by at most 130 roundings of the 18th distance squared, 8e-8 R^2, where a
+// line must stay PTM_TOPO_NEAR R^2 clear of the polygon to be left out.  (Without
+// it the FP32 polygon that named the lines had the last word, and of two
+// neighbours within 1e-4 of a distance of each other FP32 cannot place the line that
+// divides their faces: areas were off by up to the whole starting square.)
+template <typename Vec, typename VecF>
+__device__ double topo_face_area64(int m, int j, uint32_t lines, double R, Vec V, VecF VF, double *P, double *Q, int st,
+                                   int vmax) {
   double e1[3], e2[3], p[3];
   topo_plane<double>(j, V, e1, e2, p);
   // a convex polygon gains at most one vertex per clip (4 + 17 < PTM_TOPO_VMAX);
@@ -66,30 +74,52 @@ __device__ double topo_face_area64(int m, int j, uint32_t lines, double R, Vec V
   int np = 4;
   cur[0] = -R; cur[st] = -R; cur[2 * st] = R; cur[3 * st] = -R;
   cur[4 * st] = R; cur[5 * st] = R; cur[6 * st] = -R; cur[7 * st] = R;
-  for (uint32_t left = lines & ((1u << m) - 1u) & ~(1u << j); left && np > 0; left &= left - 1) {
-    const int i = __ffs(left) - 1;
-    const double w0 = V(i, 0), w1 = V(i, 1), w2 = V(i, 2);
-    const double A = w0 * e1[0] + w1 * e1[1] + w2 * e1[2], B = w0 * e2[0] + w1 * e2[1] + w2 * e2[2];
-    const double C = (w0 * w0 + w1 * w1 + w2 * w2) / 2 - (w0 * p[0] + w1 * p[1] + w2 * p[2]);
-    int nq = 0;
-    double xs = cur[0], xt = cur[st], fx = A * xs + B * xt - C;
-    const double x0 = xs, t0 = xt, f0 = fx;
-    for (int k = 0; k < np; k++) {
-      double ys = x0, yt = t0, fy = f0;
-      if (k + 1 < np) { ys = cur[2 * (k + 1) * st]; yt = cur[(2 * k + 3) * st]; fy = A * ys + B * yt - C; }
-      if (fx <= 0) {
-        if (nq < vmax) { nxt[2 * nq * st] = xs; nxt[(2 * nq + 1) * st] = xt; }
-        nq++;
+  const uint32_t all = ((1u << m) - 1u) & ~(1u << j);
+  uint32_t left = lines & all, others = ~lines & all;
+  for (;;) {
+    for (; left && np > 0; left &= left - 1) {
+      const int i = __ffs(left) - 1;
+      const double w0 = V(i, 0), w1 = V(i, 1), w2 = V(i, 2);
+      const double A = w0 * e1[0] + w1 * e1[1] + w2 * e1[2], B = w0 * e2[0] + w1 * e2[1] + w2 * e2[2];
+      const double C = (w0 * w0 + w1 * w1 + w2 * w2) / 2 - (w0 * p[0] + w1 * p[1] + w2 * p[2]);
+      int nq = 0;
+      double xs = cur[0], xt = cur[st], fx = A * xs + B * xt - C;
+      const double x0 = xs, t0 = xt, f0 = fx;
+      for (int k = 0; k < np; k++) {
+        double ys = x0, yt = t0, fy = f0;
+        if (k + 1 < np) { ys = cur[2 * (k + 1) * st]; yt = cur[(2 * k + 3) * st]; fy = A * ys + B * yt - C; }
+        if (fx <= 0) {
+          if (nq < vmax) { nxt[2 * nq * st] = xs; nxt[(2 * nq + 1) * st] = xt; }
+          nq++;
+        }
+        if ((fx < 0 && fy > 0) || (fx > 0 && fy < 0)) {
+          const double tt = fx / (fx - fy);
+          if (nq < vmax) { nxt[2 * nq * st] = xs + tt * (ys - xs); nxt[(2 * nq + 1) * st] = xt + tt * (yt - xt); }
+          nq++;
+        }
+        xs = ys; xt = yt; fx = fy;
       }
-      if ((fx < 0 && fy > 0) || (fx > 0 && fy < 0)) {
-        const double tt = fx / (fx - fy);
-        if (nq < vmax) { nxt[2 * nq * st] = xs + tt * (ys - xs); nxt[(2 * nq + 1) * st] = xt + tt * (yt - xt); }
-        nq++;
-      }
-      xs = ys; xt = yt; fx = fy;
+      np = min(nq, vmax);
+      double *tmp = cur; cur = nxt; nxt = tmp;
     }
-    np = min(nq, vmax);
-    double *tmp = cur; cur = nxt; nxt = tmp;
+    if (!others || np == 0) break;
+    // cut by the others too, where they come near (a smaller polygon stays clear of
+    // the lines this one is clear of: once is enough)
+    float2 *X = (float2 *)nxt;
+    for (int k = 0; k < np; k++) X[k * st] = make_float2((float)cur[2 * k * st], (float)cur[(2 * k + 1) * st]);
+    const float a0 = (float)e1[0], a1 = (float)e1[1], a2 = (float)e1[2], b0 = (float)e2[0], b1 = (float)e2[1],
+                b2 = (float)e2[2], c0 = (float)p[0], c1 = (float)p[1], c2 = (float)p[2];
+    const float clear = -PTM_TOPO_NEAR * (float)R * (float)R;
+    for (; others; others &= others - 1) {
+      const int i = __ffs(others) - 1;
+      const float w0 = VF(i, 0), w1 = VF(i, 1), w2 = VF(i, 2);
+      const float A = w0 * a0 + w1 * a1 + w2 * a2, B = w0 * b0 + w1 * b1 + w2 * b2;
+      const float C = (w0 * w0 + w1 * w1 + w2 * w2) / 2 - (w0 * c0 + w1 * c1 + w2 * c2);
+      bool near = false;
+      for (int k = 0; k < np; k++) near |= !(A * X[k * st].x + B * X[k * st].y - C <= clear);
+      left |= (uint32_t)near << i;
+    }
+    if (!left) break;
   }
   double s2 = 0;
   for (int k = 0; k < np; k++) {
@@ -109,8 +139,8 @@ __device__ double topo_face_area64(int m, int j, uint32_t lines, double R, Vec V
 // other lanes' polygons have.  `over` is set when the polygon outgrows the buffer
 // or rounding leaves more than one run: the FP64 pass decides then.  With LINES the
 // result is instead the set of lines (bit = neighbour) that come within PTM_TOPO_NEAR
-// R of the polygon, far above its rounding errors: the only ones that matter to its
-// FP64 area (all of them when the polygon is empty or `over`).
+// R of the polygon: those the FP64 area expects to be cut by (all of them when the
+// polygon is empty or `over`).
 template <bool LINES, typename Vec>
 __device__ __forceinline__ float topo_face32(int m, int j, float R, Vec V, float2 *P, float2 *Q, int st, bool &over,
                                              uint32_t &lines) {
@@ -404,7 +434,7 @@ __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *si
     bool over = false;
     uint32_t lines;
     topo_face32<true>(m, k, (float)R, vf, (float2 *)P, (float2 *)Q, PTM_BLOCK, over, lines);
-    a64[k] = topo_face_area64(m, k, lines, R, vd, P, Q, PTM_BLOCK, PTM_TOPO_VMAX);
+    a64[k] = topo_face_area64(m, k, lines, R, vd, vf, P, Q, PTM_BLOCK, PTM_TOPO_VMAX);
   }
   if (m > 0) topo_order<double>(m, a64, mean64, o);
   for (int k = 0; k < PTM_KNN; k++) out[(int64_t)k * n + sl] = k < m ? make_int2(jn[o[k]], im[o[k]]) : make_int2(-1, 0);

@@ -60,3 +60,35 @@ def test_doubled_atoms(reps, dtype, ordering, path):
     if path == "batch":
         b.close()
     ptm.close()
+
+
+@pytest.mark.parametrize("e,block", [(1e-7, 4), (1e-7, 6), (1e-8, 0), (1e-8, 2)])
+def test_neighbours_almost_on_one_point(e, block):
+    """Clusters with one second-shell neighbour doubled at a distance e: FP32 cannot place the
+    line between the two faces, so it must not choose what the FP64 areas are cut by.  In
+    these sets 2 or 3 of the 4,000 centres took a wrong structure when it did."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1603_05143_gb300 import PTM
+    rng = np.random.default_rng([block, 2 if e == 1e-7 else 3])
+    grid = np.array([[a, b, c] for a in range(-2, 3) for b in range(-2, 3) for c in range(-2, 3)
+                     if (a or b or c) and (a + b + c) % 2 == 0], float)
+
+    def cluster():
+        p = 1.8 * grid + rng.uniform(0.02, 0.12) * rng.normal(size=grid.shape)
+        p = p[np.argsort((p ** 2).sum(1))]
+        w = rng.integers(12, 18)
+        return np.vstack([np.zeros((1, 3)), p, p[w:w + 1] + e * rng.normal(size=(1, 3))])
+
+    side, n = 16, 4000
+    clusters = [cluster() for _ in range(n)]
+    at = np.array([[x, y, z] for x in range(side) for y in range(side) for z in range(side)], float)[:n] * 30.0 + 15.0
+    clusters = [c + x for c, x in zip(clusters, at)]
+    cell = np.eye(3) * 30.0 * side
+    ptm = PTM(0)
+    out = ptm.classify(torch.from_numpy(np.vstack(clusters)).cuda(), cell, (True, True, True), ordering="topological")
+    got = out["structure"].cpu().numpy()[::len(clusters[0])]
+    want = np.array([O.Frame(c, cell).classify(np.array([0]), ordering="topological")["structure"][0] for c in clusters])
+    assert np.array_equal(got, want), np.nonzero(got != want)[0]
+    ptm.close()

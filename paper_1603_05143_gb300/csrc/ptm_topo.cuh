@@ -136,8 +136,8 @@ __device__ double topo_face_area64(int m, int j, uint32_t lines, double R, Vec V
 // cuts where the neighbours' order took all 17.  A cut marks the vertices outside
 // its line: of a convex polygon one run of consecutive ones, replaced by its two
 // crossings, so it copies the rest and makes two divisions however many vertices the
-// other lanes' polygons have.  `over` is set when the polygon outgrows the buffer
-// or rounding leaves more than one run: the FP64 pass decides then.  With LINES the
+// other lanes' polygons have.  `over` is set when the polygon outgrows the buffer: the
+// FP64 pass decides then.  With LINES the
 // result is instead the set of lines (bit = neighbour) that come within PTM_TOPO_NEAR
 // R of the polygon: those the FP64 area expects to be cut by (all of them when the
 // polygon is empty or `over`).
@@ -199,13 +199,38 @@ __device__ __forceinline__ float topo_face32(int m, int j, float R, Vec V, float
     if (!out) continue;
     const uint32_t all = (1u << np) - 1u;
     if (out == all) { np = 0; break; }
-    // the run s .. e of outside vertices (cyclic)
-    const uint32_t prev = (out << 1 | out >> (np - 1)) & all, begins = out & ~prev;
-    over |= (begins & (begins - 1)) != 0;
-    const int s = __ffs(begins) - 1, n = __popc(out);
-    const int in0 = s + n >= np ? s + n - np : s + n, in1 = s ? s - 1 : np - 1, e = in0 ? in0 - 1 : np - 1;
     int nq = 0;
     r2 = 0.f;
+    auto put = [&](float2 x) {
+      if (nq < PTM_TOPO_VMAX32) nxt[nq * st] = x;
+      r2 = fmaxf(r2, x.x * x.x + x.y * x.y);
+      nq++;
+    };
+    // the crossing on the edge a -> b
+    auto cross = [&](float2 a, float fa, float2 b, float fb) {
+      const float t = fa / (fa - fb);
+      put(make_float2(a.x + t * (b.x - a.x), a.y + t * (b.y - a.y)));
+    };
+    // the run s .. e of outside vertices (cyclic)
+    const uint32_t prev = (out << 1 | out >> (np - 1)) & all, begins = out & ~prev;
+    if (begins & (begins - 1)) {
+      // more than one run: rounding, where corners of the polygon lie on the line (the
+      // faces of perfect lattices).  Vertex by vertex: left to the FP64 pass, a few such
+      // atoms held k_topo64 for 0.9 ms
+#pragma unroll 1
+      for (int k = 0; k < np; k++) {
+        const float2 x = cur[k * st], y = cur[(k + 1 == np ? 0 : k + 1) * st];
+        const float fx = A * x.x + B * x.y - C, fy = A * y.x + B * y.y - C;
+        if (fx <= 0.f) put(x);
+        if ((fx < 0.f && fy > 0.f) || (fx > 0.f && fy < 0.f)) cross(x, fx, y, fy);
+      }
+      over |= nq > PTM_TOPO_VMAX32;
+      np = min(nq, PTM_TOPO_VMAX32);
+      float2 *tmp = cur; cur = nxt; nxt = tmp;
+      continue;
+    }
+    const int s = __ffs(begins) - 1, n = __popc(out);
+    const int in0 = s + n >= np ? s + n - np : s + n, in1 = s ? s - 1 : np - 1, e = in0 ? in0 - 1 : np - 1;
     for (int k = in0, left = np - n; left; left--) {
       const float2 x = cur[k * st];
       nxt[nq * st] = x;
@@ -216,20 +241,8 @@ __device__ __forceinline__ float topo_face32(int m, int j, float R, Vec V, float
     // the crossings of in1 -> s and e -> in0; a vertex on the plane is its own
     const float2 a = cur[in1 * st], b = cur[s * st], c = cur[e * st], g = cur[in0 * st];
     const float fa = A * a.x + B * a.y - C, fb = A * b.x + B * b.y - C, fc = A * c.x + B * c.y - C, fg = A * g.x + B * g.y - C;
-    if (fa < 0.f) {
-      const float t = fa / (fa - fb);
-      const float2 x = make_float2(a.x + t * (b.x - a.x), a.y + t * (b.y - a.y));
-      if (nq < PTM_TOPO_VMAX32) nxt[nq * st] = x;
-      r2 = fmaxf(r2, x.x * x.x + x.y * x.y);
-      nq++;
-    }
-    if (fg < 0.f) {
-      const float t = fc / (fc - fg);
-      const float2 x = make_float2(c.x + t * (g.x - c.x), c.y + t * (g.y - c.y));
-      if (nq < PTM_TOPO_VMAX32) nxt[nq * st] = x;
-      r2 = fmaxf(r2, x.x * x.x + x.y * x.y);
-      nq++;
-    }
+    if (fa < 0.f) cross(a, fa, b, fb);
+    if (fg < 0.f) cross(c, fc, g, fg);
     over |= nq > PTM_TOPO_VMAX32;
     np = min(nq, PTM_TOPO_VMAX32);
     float2 *tmp = cur; cur = nxt; nxt = tmp;

@@ -206,7 +206,11 @@ __device__ __forceinline__ float topo_face32(int m, int j, float R, Vec V, float
       r2 = fmaxf(r2, x.x * x.x + x.y * x.y);
       nq++;
     };
-    // the crossing on the edge a -> b
+    // the crossing from an inside vertex a to an outside one b, seen from the inside: the
+    // outside one may be as far as the starting square, with its rounding.  (Largest error
+    // of an area of noisy fcc, bcc and sc, of the mean squared distance: 3.1e-6; seen along
+    // the edge either way 3.6e-6, cut in the neighbours' order 3.0e-6.  Faces of free
+    // surfaces past the guard: 2,441 of 360,000 against 3,128 and 2,722.)
     auto cross = [&](float2 a, float fa, float2 b, float fb) {
       const float t = fa / (fa - fb);
       put(make_float2(a.x + t * (b.x - a.x), a.y + t * (b.y - a.y)));
@@ -222,7 +226,8 @@ __device__ __forceinline__ float topo_face32(int m, int j, float R, Vec V, float
         const float2 x = cur[k * st], y = cur[(k + 1 == np ? 0 : k + 1) * st];
         const float fx = A * x.x + B * x.y - C, fy = A * y.x + B * y.y - C;
         if (fx <= 0.f) put(x);
-        if ((fx < 0.f && fy > 0.f) || (fx > 0.f && fy < 0.f)) cross(x, fx, y, fy);
+        if (fx < 0.f && fy > 0.f) cross(x, fx, y, fy);
+        if (fx > 0.f && fy < 0.f) cross(y, fy, x, fx);
       }
       over |= nq > PTM_TOPO_VMAX32;
       np = min(nq, PTM_TOPO_VMAX32);
@@ -242,7 +247,7 @@ __device__ __forceinline__ float topo_face32(int m, int j, float R, Vec V, float
     const float2 a = cur[in1 * st], b = cur[s * st], c = cur[e * st], g = cur[in0 * st];
     const float fa = A * a.x + B * a.y - C, fb = A * b.x + B * b.y - C, fc = A * c.x + B * c.y - C, fg = A * g.x + B * g.y - C;
     if (fa < 0.f) cross(a, fa, b, fb);
-    if (fg < 0.f) cross(c, fc, g, fg);
+    if (fg < 0.f) cross(g, fg, c, fc);
     over |= nq > PTM_TOPO_VMAX32;
     np = min(nq, PTM_TOPO_VMAX32);
     float2 *tmp = cur; cur = nxt; nxt = tmp;
@@ -393,7 +398,7 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict_
 // FP64 pass for listed atom i (= list position), one thread: FP64 neighbour
 // vectors, and in FP64 the areas of the faces the FP32 pass could not decide
 // (the two faces of every gap at the band edge); the others keep their FP32
-// areas, whose error (measured within 2.2e-6 of the mean squared distance) is
+// areas, whose error (measured within 3.1e-6 of the mean squared distance) is
 // far below the guard, so every gap decided from them is decided as in FP64.
 // Atoms past the side buffer recompute every face.  Polygon buffers in shared memory, element e at P[e * PTM_BLOCK].  The
 // lanes of `wmask` call this together and take their faces in step, one face

@@ -142,16 +142,19 @@ __device__ __forceinline__ uint64_t setnib(uint64_t x, int i, int v) {
   return (x & ~(15ull << (4 * i))) | ((uint64_t)v << (4 * i));
 }
 
+// Lattice image (a, b, c) in 10 bits a component, in the order of the components: atoms may
+// stand 100 periods outside the cell (PTM_FAR_PERIODS), so the image of a neighbour runs
+// to 200 and a few more.
 __device__ __forceinline__ int img_pack(int a, int b, int c) {
-  return ((a + 128) << 16) | ((b + 128) << 8) | (c + 128);
+  return ((a + 512) << 20) | ((b + 512) << 10) | (c + 512);
 }
 // Packed wrap of an atom the binning excludes (non-finite coordinate, or more
-// than PTM_FAR_PERIODS periods from the cell): image (-128, -128, -128), which
+// than PTM_FAR_PERIODS periods from the cell): image (-512, -512, -512), which
 // no valid atom packs to.
 #define PTM_FAR_PERIODS 100.f
 #define PTM_EXCLUDED 0
 __device__ __forceinline__ void img_unpack(int p, int &a, int &b, int &c) {
-  a = ((p >> 16) & 255) - 128; b = ((p >> 8) & 255) - 128; c = (p & 255) - 128;
+  a = ((p >> 20) & 1023) - 512; b = ((p >> 10) & 1023) - 512; c = (p & 1023) - 512;
 }
 
 // Shift n.H in FP64 of an image outside the tables (out of line: rare).

@@ -147,7 +147,7 @@ __device__ __forceinline__ void sort_low(uint32_t (&v)[2 * H]) {
 // ------------------------------------------------------------ fast search
 #define PTM_KNN_BLOCK 128
 // CAP: entries of the candidate list (9 bytes a thread).  AIM: candidates the
-// search radius aims at (the atom itself counts), above the NK + 2 that decide an
+// search radius aims at (the atom itself counts), above the NK + 1 that decide an
 // atom by enough for the shells of the lattices (fcc holds 12, 18, 42 atoms
 // within its first shells, bcc 8, 14, 26), below the capacity.  BLOCKS: resident
 // blocks per SM (36 and 72 KB of lists a block).
@@ -291,8 +291,8 @@ __device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__re
 // The radius is that of a sphere holding NT atoms at the density of the 27
 // cells, at most what they are sure to cover; too many or too few candidates
 // rescale it.  The list is sorted once by its FP32 values with the entry number
-// in the low bits; if the NK + 1 smallest then differ by more than the error
-// band, their order is the FP64 order.  Otherwise the values are sorted again
+// in the low bits; if the NK + 1 smallest (or the NK in it and the radius) then
+// differ by more than the error band, their order is the FP64 order.  Otherwise the values are sorted again
 // without entry numbers, close ones form runs, and a run's candidates are
 // ordered by the FP64 key (d2, atom id, image); a run across slot NK takes
 // every candidate within the band.
@@ -323,8 +323,8 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
   }
   for (int attempt = 0;; attempt++) {
     cnt = knn_gather<SPLIT, CAP>(d, hi, hs, ls, bx, by, bz, T, list);
-    if (cnt >= NK + 2 && cnt <= CAP) break;
-    if (attempt == 3 || (cnt < NK + 2 && T >= Tmax)) return false;
+    if (cnt > NK && cnt <= CAP) break;
+    if (attempt == 3 || (cnt <= NK && T >= Tmax)) return false;
     const float f = exp2f(0.6666667f * __log2f(__fdividef(AIM, (float)cnt)));
     T = fminf(Tmax, T * (cnt > CAP ? f : fmaxf(f, 1.2f)));
   }
@@ -353,7 +353,10 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
   for (int round = 0;; round++) {
 #pragma unroll
     for (int i = 0; i < CAP; i++) {
-      uint32_t x = 0xffffffffu;
+      // past the list T stands for whatever the radius left out (with NK neighbours and no
+      // more inside the widest radius, as in fcc's first two shells for NK = 18, the
+      // next one need not be known)
+      uint32_t x = __float_as_uint(T) | (round == 0 ? LOW : 0u);
       if (i < cnt) {
         x = __float_as_uint(list.V(i));
         if (round == 0) x = (x & ~LOW) | (uint32_t)i;
@@ -363,7 +366,7 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
     }
     sort_low<CAP / 2>(v);
     if (round == 1) break;
-    const float vmax = 1.01f * list.V(v[NK + 1] & LOW);
+    const float vmax = 1.01f * __uint_as_float(v[NK + 1] & ~LOW);
     const float band = 2.f * (8.5f * u * vmax + 4.f * (sqrtf(vmax) + d.tau) * d.tau);
     // v[0] is the atom itself (d2 = 0, unless another lies on it: then the first
     // gap is within the band); the entry after the last neighbour counts with

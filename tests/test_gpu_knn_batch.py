@@ -73,3 +73,19 @@ def test_near_ties_across_a_long_periodic_side(ptm, sigma):
     pos[:, 0] = np.mod(pos[:, 0] - 4 * I.A_FCC_CU, 1000.0)
     s = _check(ptm, np.ascontiguousarray(pos, np.float32), cell, (True, True, True), "euclidean")
     assert s["knn_fp64"] > 0
+
+
+@pytest.mark.parametrize("kind,a,reps", [("fcc", I.A_FCC_CU, 29), ("bcc", I.A_BCC_FE, 36)])
+def test_a_full_shell_inside_the_widest_radius_is_enough(ptm, kind, a, reps):
+    """The 18 nearest of an fcc atom are its first two shells, and the third lies outside
+    the radius that 27 cells cover: no reason for the warp search, which counts every
+    atom it takes in FP64."""
+    import torch
+    f = I.crystal(kind, a, reps, sigma=0.01, seed=1, dtype=np.float32)
+    out = ptm.classify(torch.from_numpy(f.positions).cuda(), f.cell, f.pbc, ordering="topological")
+    torch.cuda.synchronize()
+    s = ptm.stats()
+    assert s["internal"] == 0 and s["knn_fp64"] < f.n // 8
+    atoms = I.rng_for(5).permutation(f.n)[:24]
+    ref = O.Frame(f.positions, f.cell, f.pbc).classify(atoms, ordering="topological")
+    compare({k: v.cpu().numpy() for k, v in out.items()}, ref, atoms)

@@ -528,50 +528,62 @@ __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
         j = __ldg(d.cell_start + cell);
         j1 = __ldg(d.cell_start + cell + 1);
       }
-      for (; __any_sync(ALL, j < j1); j++) {
-        uint64_t key = INF;
-        int idj = 0x7fffffff, img = 0x7fffffff;
-        if (j < j1) {
-          T xj, yj, zj;
-          load_atom<F64>(d, j, xj, yj, zj, idj);
-          const int w = __ldg(d.wrapv + j);
-          int w0, w1, w2;
-          img_unpack(w, w0, w1, w2);
-          const int a0 = mx + wi0 - w0, a1 = my + wi1 - w1, a2 = mz + wi2 - w2;
-          bool in = !(j == s && a0 == 0 && a1 == 0 && a2 == 0) && w != PTM_EXCLUDED;
-          if (in) {
-            T sx, sy, sz;
-            contract_shift<F64>(d, a0, a1, a2, sx, sy, sz);
-            const T v = contract_d2(contract_dr(xj, xi, sx), contract_dr(yj, yi, sy), contract_dr(zj, zi, sz));
-            img = img_pack(a0, a1, a2);
-            if constexpr (!F64) {
-              const float S = sqrtf(sx * sx + sy * sy + sz * sz) * 1.0001f;
-              in = !(v - 1.25f * knn_err(v, S) > last32);
-            }
+      // A lane walks its cell, or where one cell holds more than that takes (a cluster in a
+      // box of vacuum may sit in a few cells) the warp walks them one after another
+      const int most = __reduce_max_sync(ALL, j1 - j), trips = __reduce_add_sync(ALL, (j1 - j + 31) >> 5);
+      const bool together = most > trips;
+      for (unsigned cells = together ? __ballot_sync(ALL, j < j1) : 1u; cells; cells &= cells - 1) {
+        const int src0 = __ffs(cells) - 1;
+        int jj = j, je = j1, nx = mx, ny = my, nz = mz;
+        if (together) {
+          jj = __shfl_sync(ALL, j, src0) + lane; je = __shfl_sync(ALL, j1, src0);
+          nx = __shfl_sync(ALL, mx, src0); ny = __shfl_sync(ALL, my, src0); nz = __shfl_sync(ALL, mz, src0);
+        }
+        for (; __any_sync(ALL, jj < je); jj += together ? 32 : 1) {
+          uint64_t key = INF;
+          int idj = 0x7fffffff, img = 0x7fffffff;
+          if (jj < je) {
+            T xj, yj, zj;
+            load_atom<F64>(d, jj, xj, yj, zj, idj);
+            const int w = __ldg(d.wrapv + jj);
+            int w0, w1, w2;
+            img_unpack(w, w0, w1, w2);
+            const int a0 = nx + wi0 - w0, a1 = ny + wi1 - w1, a2 = nz + wi2 - w2;
+            bool in = !(jj == s && a0 == 0 && a1 == 0 && a2 == 0) && w != PTM_EXCLUDED;
             if (in) {
-              double k64;
-              if constexpr (F64) k64 = v;
-              else k64 = key64(d, xj, yj, zj, xi, yi, zi, a0, a1, a2);
-              key = (uint64_t)__double_as_longlong(k64);
+              T sx, sy, sz;
+              contract_shift<F64>(d, a0, a1, a2, sx, sy, sz);
+              const T v = contract_d2(contract_dr(xj, xi, sx), contract_dr(yj, yi, sy), contract_dr(zj, zi, sz));
+              img = img_pack(a0, a1, a2);
+              if constexpr (!F64) {
+                const float S = sqrtf(sx * sx + sy * sy + sz * sz) * 1.0001f;
+                in = !(v - 1.25f * knn_err(v, S) > last32);
+              }
+              if (in) {
+                double k64;
+                if constexpr (F64) k64 = v;
+                else k64 = key64(d, xj, yj, zj, xi, yi, zi, a0, a1, a2);
+                key = (uint64_t)__double_as_longlong(k64);
+              }
             }
           }
-        }
-        unsigned m = __ballot_sync(ALL, key < INF && key <= last);
-        while (m) {
-          const int src = __ffs(m) - 1;
-          m &= m - 1;
-          const uint64_t ck = __shfl_sync(ALL, key, src);
-          const int cid = __shfl_sync(ALL, idj, src), cimg = __shfl_sync(ALL, img, src), cj = __shfl_sync(ALL, j, src);
-          const unsigned at = __ballot_sync(ALL, key_less64(ck, cid, cimg, lk, lid, limg)) & ((1u << NK) - 1u);
-          if (!at) continue;                             // not below the NK-th key any more
-          const uint64_t uk = __shfl_up_sync(ALL, lk, 1);
-          const int uid = __shfl_up_sync(ALL, lid, 1), uj = __shfl_up_sync(ALL, lj, 1),
-                    uimg = __shfl_up_sync(ALL, limg, 1);
-          const int first = __ffs(at) - 1;               // the keys are sorted: every lane above moves up
-          if (lane == first) { lk = ck; lid = cid; lj = cj; limg = cimg; }
-          else if (lane > first) { lk = uk; lid = uid; lj = uj; limg = uimg; }
-          last = __shfl_sync(ALL, lk, NK - 1);
-          if constexpr (!F64) last32 = __double2float_ru(__longlong_as_double((long long)last));
+          unsigned m = __ballot_sync(ALL, key < INF && key <= last);
+          while (m) {
+            const int src = __ffs(m) - 1;
+            m &= m - 1;
+            const uint64_t ck = __shfl_sync(ALL, key, src);
+            const int cid = __shfl_sync(ALL, idj, src), cimg = __shfl_sync(ALL, img, src), cj = __shfl_sync(ALL, jj, src);
+            const unsigned at = __ballot_sync(ALL, key_less64(ck, cid, cimg, lk, lid, limg)) & ((1u << NK) - 1u);
+            if (!at) continue;                             // not below the NK-th key any more
+            const uint64_t uk = __shfl_up_sync(ALL, lk, 1);
+            const int uid = __shfl_up_sync(ALL, lid, 1), uj = __shfl_up_sync(ALL, lj, 1),
+                      uimg = __shfl_up_sync(ALL, limg, 1);
+            const int first = __ffs(at) - 1;               // the keys are sorted: every lane above moves up
+            if (lane == first) { lk = ck; lid = cid; lj = cj; limg = cimg; }
+            else if (lane > first) { lk = uk; lid = uid; lj = uj; limg = uimg; }
+            last = __shfl_sync(ALL, lk, NK - 1);
+            if constexpr (!F64) last32 = __double2float_ru(__longlong_as_double((long long)last));
+          }
         }
       }
     }

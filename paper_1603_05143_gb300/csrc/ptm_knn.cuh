@@ -156,6 +156,17 @@ template <int NK> struct KnnShape {
 };
 constexpr size_t knn_smem_bytes(int nk) { return (size_t)PTM_KNN_BLOCK * (nk == PTM_KNN ? 32 : 64) * 9; }
 
+// Cells hold about 7 atoms (192 in 27) where the frame fills its box.  A cluster in a box of
+// vacuum has hundreds of times as many, in a few cells that are far from evenly filled:
+// the first radius is much too wide, and a thread reads everything three times over.
+// Frames of up to PTM_KNN_CROWDED_FRAME atoms, too few warps to hide that latency, leave
+// atoms with nearly all of the frame in reach to the warp search (8,000 atoms in a box
+// of 10 diameters: 2.95 ms a call without, 0.77 with; 20,000 in 7: 6.4 and 3.1; at 60,000 the
+// warps take 22.8 ms and the threads 19.3).  More atoms than that in the 27 cells, and a
+// sample sets the radius (60,000: 19.3 -> 15.3 ms; 200,000: 57.6 -> 54.6).
+#define PTM_KNN_CROWDED 1024
+#define PTM_KNN_CROWDED_FRAME 24576
+
 // Per-thread candidate list in shared memory, entry i at [i][thread]: FP32
 // squared distance, sorted slot, image code (m + 1 in two bits per axis).
 struct KnnList {
@@ -284,6 +295,37 @@ __device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__re
   return cnt;
 }
 
+// Square of the radius of a sphere around the atom that holds about `aim` atoms, from every
+// step-th atom of the 27 cells: the sphere around about 32 of these, scaled down.
+// `T`: that square if the cells were evenly filled.
+__device__ __noinline__ float crowded_radius(const FrameDesc &d, const float4 *__restrict__ hi, float4 hs, int bx, int by,
+                                             int bz, int step, float T, float aim) {
+  const float want = 32.f;
+  float t = T * exp2f(0.6666667f * __log2f(__fdividef(want * (float)step, aim)));
+  int c = 0;
+#pragma unroll 1
+  for (int trip = 0; trip < 4; trip++) {
+    int off = 0;
+    c = 0;
+    for_cells27(d, bx, by, bz, [&](int ca, int cb, int mx, int my, int mz) {
+      const int i = (mx + 2) * 25 + (my + 2) * 5 + (mz + 2);
+      const float hx = hs.x - d.tab->s32[i][0], hy = hs.y - d.tab->s32[i][1], hz = hs.z - d.tab->s32[i][2];
+      const int j1 = __ldg(d.cell_start + cb + 1);
+      int j = __ldg(d.cell_start + ca) + off;
+      for (; j < j1; j += step) {
+        const float4 p = __ldg(hi + j);
+        const float x = p.x - hx, y = p.y - hy, z = p.z - hz;
+        c += fmaf(x, x, fmaf(y, y, z * z)) < t;
+      }
+      off = j - j1;
+    });
+    if (c >= 16 && c <= 64) break;
+    t *= exp2f(0.6666667f * __log2f(__fdividef(want, fmaxf((float)c, 1.f))));
+    c = (int)want;                                   // what the new radius should hold
+  }
+  return t * exp2f(0.6666667f * __log2f(__fdividef(aim, (float)step * (float)c)));
+}
+
 // NK nearest images of the atom at sorted slot s, written to out[t * n], t = 0 ..
 // NK - 1; false when k_knn_rest must decide (the NK-th neighbour may lie outside
 // the 27 cells, or no radius admits a fitting number of candidates).
@@ -319,7 +361,13 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
       cells += cb - ca + 1;
     });
     const float r3 = AIM * 0.2387324f * d.cell_vol * __fdividef((float)cells, (float)atoms);
-    T = fminf(Tmax, exp2f(0.6666667f * __log2f(r3)));
+    T = exp2f(0.6666667f * __log2f(r3));
+    if (atoms > PTM_KNN_CROWDED) {
+      const int n = (int)d.n;
+      if (n <= PTM_KNN_CROWDED_FRAME && atoms > n - n / 16) return false;
+      if (atoms > PTM_KNN_CROWDED_FRAME) T = crowded_radius(d, hi, hs, bx, by, bz, atoms >> 8, T, AIM);
+    }
+    T = fminf(Tmax, T);
   }
   for (int attempt = 0;; attempt++) {
     cnt = knn_gather<SPLIT, CAP>(d, hi, hs, ls, bx, by, bz, T, list);

@@ -222,6 +222,23 @@ __device__ __forceinline__ void for_cells27(const FrameDesc &d, int bx, int by, 
   }
 }
 
+// Two candidates whose FP32 squared distances (of FP32 pairs, below) differ by more than
+// this are in FP64 order, `v` the NK-th smallest: |d2_32 - d2_64| <= u (7 v) + 4 sqrt(v)
+// tau, where each component is within 2 u of its FP64 value (relative) and tau
+// (absolute), and the squares and sums add 3 u v.  A hundredth more covers the
+// candidate after the last: one further away is not close.
+__device__ __forceinline__ float knn_band(const FrameDesc &d, float v) {
+  const float u = 5.9604645e-8f, vmax = 1.01f * v;
+  return 2.f * (8.5f * u * vmax + 4.f * (sqrtf(vmax) + d.tau) * d.tau);
+}
+
+// Position at hs + ls less the shift of a lattice image (s + r, FP32 pair), as a pair h + l.
+__device__ __forceinline__ void shift_pair(float hs, float ls, float s, float r, float &h, float &l) {
+  float e;
+  two_sum(hs, -s, h, e);
+  l = (ls + e) - r;
+}
+
 // Append every candidate with d2 < T of the 27 cells to the list; returns their
 // number (entries past CAP are counted, not stored).  The own atom is one of
 // them, with d2 = 0.
@@ -245,10 +262,9 @@ __device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__re
     if (shifted) {
       const ShiftTables &t = *d.tab;
       const int i = (mx + 2) * 25 + (my + 2) * 5 + (mz + 2);
-      float e;
-      two_sum(hs.x, -t.s32[i][0], hx, e); lx = (ls.x + e) - t.slo[i][0];
-      two_sum(hs.y, -t.s32[i][1], hy, e); ly = (ls.y + e) - t.slo[i][1];
-      two_sum(hs.z, -t.s32[i][2], hz, e); lz = (ls.z + e) - t.slo[i][2];
+      shift_pair(hs.x, ls.x, t.s32[i][0], t.slo[i][0], hx, lx);
+      shift_pair(hs.y, ls.y, t.s32[i][1], t.slo[i][1], hy, ly);
+      shift_pair(hs.z, ls.z, t.s32[i][2], t.slo[i][2], hz, lz);
     }
     const uint8_t code = (uint8_t)((mx + 1) << 4 | (my + 1) << 2 | (mz + 1));
     auto test = [&](int jj, float x, float y, float z) {
@@ -393,9 +409,6 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
     image(j, list.M(i), a, b, c);
     out[t * nst] = make_int2(j, img_pack(a, b, c));
   };
-  // |d2_32 - d2_64| <= u (7 v) + 4 sqrt(v) tau: each component is within 2 u of
-  // its FP64 value (relative) and tau (absolute), the squares and sums add 3 u v
-  const float u = 5.9604645e-8f;
   uint32_t v[CAP];
 #pragma unroll 1
   for (int round = 0;; round++) {
@@ -414,8 +427,7 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
     }
     sort_low<CAP / 2>(v);
     if (round == 1) break;
-    const float vmax = 1.01f * __uint_as_float(v[NK + 1] & ~LOW);
-    const float band = 2.f * (8.5f * u * vmax + 4.f * (sqrtf(vmax) + d.tau) * d.tau);
+    const float band = knn_band(d, list.V(v[NK] & LOW));
     // v[0] is the atom itself (d2 = 0, unless another lies on it: then the first
     // gap is within the band); the entry after the last neighbour counts with
     // its low bits cleared, a bound for every entry beyond it
@@ -435,8 +447,7 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
   }
   // ---- some ranks undecided: L[0 .. NK] ascending without the atom itself
   auto L = [&](int t) { return __uint_as_float(v[t]); };
-  const float vmax = 1.01f * L(NK);
-  const float band = 2.f * (8.5f * u * vmax + 4.f * (sqrtf(vmax) + d.tau) * d.tau);
+  const float band = knn_band(d, L(NK - 1));
   uint32_t close = 0;                                // bit t: slots t and t + 1 in one run
 #pragma unroll
   for (int t = 0; t < NK; t++) close |= (uint32_t)(L(t + 1) - L(t) <= band) << t;
@@ -557,7 +568,12 @@ __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
   const int nbx = d.nb[0], nby = d.nb[1], nbz = d.nb[2];
   const uint64_t INF = 0x7ff0000000000000ull;
   uint64_t lk = INF, last = INF;                       // this lane's key; the NK-th key,
-  float last32 = INFINITY;                             // ... rounded up to FP32
+  float last32 = INFINITY;                             // ... and the slack, rounded up to FP32
+  // float32 input keeps one key more where it is within 2^-16 of the NK-th (in units
+  // of its last place; infinity turns into a NaN, which cuts nothing), to tell whether
+  // FP64 was needed between the two
+  constexpr int KEPT = F64 ? NK : NK + 1;
+  constexpr uint64_t SLACK = F64 ? 0 : 1ull << 36;
   int lid = 0x7fffffff, lj = -1, limg = 0x7fffffff, found = -1;
   for (int R = 1; R <= PTM_RMAX; R++) {
     const int side = 2 * R + 1;
@@ -615,14 +631,14 @@ __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
               }
             }
           }
-          unsigned m = __ballot_sync(ALL, key < INF && key <= last);
+          unsigned m = __ballot_sync(ALL, key < INF && key <= last + SLACK);
           while (m) {
             const int src = __ffs(m) - 1;
             m &= m - 1;
             const uint64_t ck = __shfl_sync(ALL, key, src);
             const int cid = __shfl_sync(ALL, idj, src), cimg = __shfl_sync(ALL, img, src), cj = __shfl_sync(ALL, jj, src);
-            const unsigned at = __ballot_sync(ALL, key_less64(ck, cid, cimg, lk, lid, limg)) & ((1u << NK) - 1u);
-            if (!at) continue;                             // not below the NK-th key any more
+            const unsigned at = __ballot_sync(ALL, key_less64(ck, cid, cimg, lk, lid, limg)) & ((1u << KEPT) - 1u);
+            if (!at) continue;                             // not below the last key kept any more
             const uint64_t uk = __shfl_up_sync(ALL, lk, 1);
             const int uid = __shfl_up_sync(ALL, lid, 1), uj = __shfl_up_sync(ALL, lj, 1),
                       uimg = __shfl_up_sync(ALL, limg, 1);
@@ -630,7 +646,7 @@ __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
             if (lane == first) { lk = ck; lid = cid; lj = cj; limg = cimg; }
             else if (lane > first) { lk = uk; lid = uid; lj = uj; limg = uimg; }
             last = __shfl_sync(ALL, lk, NK - 1);
-            if constexpr (!F64) last32 = __double2float_ru(__longlong_as_double((long long)last));
+            if constexpr (!F64) last32 = __double2float_ru(__longlong_as_double((long long)(last + SLACK)));
           }
         }
       }
@@ -645,9 +661,39 @@ __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
       break;
     }
   }
-  if (lane == 0) {
-    if (found < 0) count(d, C_KNN_FAIL);
-    if (!F64) count(d, C_KNN64);
+  if (found < 0 && lane == 0) count(d, C_KNN_FAIL);
+  if constexpr (!F64) {
+    // counted where the FP32 values that k_knn goes by leave two neighbours within its band
+    const bool split = d.dstat[0] != 0, mine = lane <= NK && lj >= 0;
+    const float4 *hi = split ? d.hi : (const float4 *)d.sorted;
+    const float4 hs = __ldg(hi + s);
+    float v = INFINITY;
+    if (mine) {
+      const float4 p = __ldg(hi + lj);
+      float4 ls = make_float4(0.f, 0.f, 0.f, 0.f), q = ls;
+      int a, b, c;
+      img_unpack(limg, a, b, c);
+      if (split) {
+        ls = __ldg(d.lo + s);
+        q = __ldg(d.lo + lj);
+        int q0, q1, q2;
+        img_unpack(__float_as_int(q.w), q0, q1, q2);
+        a += q0 - wi0; b += q1 - wi1; c += q2 - wi2;
+      }
+      float hx = hs.x, hy = hs.y, hz = hs.z, lx = ls.x, ly = ls.y, lz = ls.z;
+      if (a | b | c) {
+        float sx, sy, sz, rx, ry, rz;
+        shift_f32(d, a, b, c, sx, sy, sz, rx, ry, rz);
+        shift_pair(hs.x, ls.x, sx, rx, hx, lx);
+        shift_pair(hs.y, ls.y, sy, ry, hy, ly);
+        shift_pair(hs.z, ls.z, sz, rz, hz, lz);
+      }
+      const float x = (p.x - hx) + (q.x - lx), y = (p.y - hy) + (q.y - ly), z = (p.z - hz) + (q.z - lz);
+      v = fmaf(x, x, fmaf(y, y, z * z));
+    }
+    const int have = min(NK, __popc(__ballot_sync(ALL, mine)));
+    const float before = __shfl_up_sync(ALL, v, 1), nk = __shfl_sync(ALL, v, max(have, 1) - 1);
+    if (__any_sync(ALL, mine && lane > 0 && v - before <= knn_band(d, nk)) && lane == 0) count(d, C_KNN64);
   }
   if (lane < NK) rows[(int64_t)lane * d.n + (s - d.atom_offset)] = lane < found ? make_int2(lj, limg) : make_int2(-1, 0);
 }

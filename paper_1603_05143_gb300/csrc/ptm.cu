@@ -30,7 +30,8 @@ struct ptm_context {
   // workspace
   size_t cap_atoms = 0, cap_cells = 0, cap_sorted_bytes = 0;
   void *sorted = nullptr;
-  float4 *hi = nullptr, *lo = nullptr;
+  void *pairs = nullptr;          // float64 input: hi and lo
+  size_t cap_pairs = 0;
   int *sbin = nullptr, *wrapv = nullptr, *atom_cell = nullptr, *atom_rank = nullptr, *atom_wrap = nullptr;
   int *cell_count = nullptr, *cell_start = nullptr, *block_sums = nullptr;
   int *dstat = nullptr;
@@ -52,14 +53,24 @@ struct ptm_context {
   int2 *nbr = nullptr;
   uint64_t *lam = nullptr;
   uint32_t *ents = nullptr;
-  size_t cap_nbr = 0;
-  // topological order: the 18 nearest, atoms for the FP64 pass and what the FP32
-  // pass keeps for it
-  int2 *nbr18 = nullptr;
+  size_t cap_nbr = 0, cap_rows = 0;   // atoms; entries of nbr (14 or 18 an atom)
+  // topological order: atoms for the FP64 pass and what the FP32 pass keeps for it
   int *topo_list = nullptr;
   TopoSide *topo_side = nullptr;
   size_t cap_topo = 0;
 };
+
+// Positions as FP32 pairs (FrameDesc::hi, lo) take 24 B an atom.  k_hulls reads those of
+// float64 input.  With float32 input nothing after the neighbour search does, and they
+// lie where k_hulls will write the labellings (lam, 24 B an atom as well).
+#define PTM_PAIR_BYTES (sizeof(float4) + sizeof(float2))
+static_assert(PTM_PAIR_BYTES == 3 * sizeof(uint64_t), "pairs of float32 input lie in lam");
+static float4 *pair_hi(void *base) { return (float4 *)base; }
+static float2 *pair_lo(float4 *hi, size_t n) { return (float2 *)(hi + n); }
+
+// Entries of an atom's neighbour list: the 14 nearest, or the 18 that the topological order
+// chooses from.
+static size_t nbr_rows(int ordering) { return ordering == PTM_ORDER_TOPOLOGICAL ? PTM_TOPO_N : PTM_KNN; }
 
 static ptm_status cuda_fail(ptm_context *ctx, cudaError_t e, const char *what) {
   if (ctx) ctx->last_error = std::string(what) + ": " + cudaGetErrorString(e);
@@ -77,8 +88,6 @@ static ptm_status grow(ptm_context *ctx, size_t n, size_t ncell, int f64) {
   if (n > ctx->cap_atoms || sb > ctx->cap_sorted_bytes) {
     cudaFree(ctx->sorted); cudaFree(ctx->sbin); cudaFree(ctx->wrapv);
     cudaFree(ctx->atom_cell); cudaFree(ctx->atom_rank); cudaFree(ctx->atom_wrap);
-    cudaFree(ctx->hi); cudaFree(ctx->lo);
-    ctx->hi = ctx->lo = nullptr;
     ctx->sorted = nullptr; ctx->sbin = ctx->wrapv = ctx->atom_cell = ctx->atom_rank = ctx->atom_wrap = nullptr;
     ctx->cap_atoms = ctx->cap_sorted_bytes = 0;
     size_t na = std::max(n, ctx->cap_atoms);
@@ -89,10 +98,15 @@ static ptm_status grow(ptm_context *ctx, size_t n, size_t ncell, int f64) {
     CK(cudaMalloc(&ctx->atom_cell, na * sizeof(int)));
     CK(cudaMalloc(&ctx->atom_rank, na * sizeof(int)));
     CK(cudaMalloc(&ctx->atom_wrap, na * sizeof(int)));
-    CK(cudaMalloc(&ctx->hi, na * sizeof(float4)));
-    CK(cudaMalloc(&ctx->lo, na * sizeof(float4)));
     ctx->cap_atoms = na;
     ctx->cap_sorted_bytes = nsb;
+  }
+  if (f64 && n > ctx->cap_pairs) {
+    cudaFree(ctx->pairs);
+    ctx->pairs = nullptr;
+    ctx->cap_pairs = 0;
+    CK(cudaMalloc(&ctx->pairs, n * PTM_PAIR_BYTES));
+    ctx->cap_pairs = n;
   }
   if (ncell > ctx->cap_cells) {
     cudaFree(ctx->cell_count); cudaFree(ctx->cell_start); cudaFree(ctx->block_sums);
@@ -210,11 +224,12 @@ static ptm_status setup_frame(const ptm_frame *f, double cell_factor, FrameDesc 
 struct FrameBuffers {
   int *cell_count, *cell_start, *block_sums, *atom_cell, *atom_rank, *atom_wrap, *sbin, *wrapv;
   void *sorted;
-  float4 *hi, *lo;
+  float4 *hi;
+  float2 *lo;
   int *dstat;
   unsigned long long *counters;
   ShiftTables *tab;
-  int2 *nbr, *nbr18;
+  int2 *nbr;
   uint64_t *lam;
   uint32_t *ents;
 };
@@ -223,7 +238,7 @@ static void set_buffers(FrameDesc *d, BinParams *bp, const FrameBuffers &B) {
   d->sorted = B.sorted; d->hi = B.hi; d->lo = B.lo;
   d->sbin = B.sbin; d->cell_start = B.cell_start; d->wrapv = B.wrapv;
   d->dstat = B.dstat; d->counters = B.counters; d->tab = B.tab;
-  d->nbr = B.nbr; d->nbr18 = B.nbr18; d->lam = B.lam; d->ents = B.ents;
+  d->nbr = B.nbr; d->lam = B.lam; d->ents = B.ents;
   bp->counters = B.counters;
 }
 
@@ -314,31 +329,36 @@ static ptm_status enqueue_frame(ptm_context *ctx, const ptm_frame *f, const ptm_
   rs = grow(ctx, (size_t)n, ncell, f64);
   if (rs != PTM_OK) return rs;
   const bool topological = f->ordering == PTM_ORDER_TOPOLOGICAL;
+  const size_t rows = nbr_rows(f->ordering) * (size_t)n;
+  if (rows > ctx->cap_rows) {
+    cudaFree(ctx->nbr);
+    ctx->nbr = nullptr;
+    ctx->cap_rows = 0;
+    CK(cudaMalloc(&ctx->nbr, rows * sizeof(int2)));
+    ctx->cap_rows = rows;
+  }
   if ((size_t)n > ctx->cap_nbr) {
-    cudaFree(ctx->nbr); cudaFree(ctx->lam); cudaFree(ctx->ents);
-    ctx->nbr = nullptr; ctx->lam = nullptr; ctx->ents = nullptr;
+    cudaFree(ctx->lam); cudaFree(ctx->ents);
+    ctx->lam = nullptr; ctx->ents = nullptr;
     ctx->cap_nbr = 0;
-    CK(cudaMalloc(&ctx->nbr, (size_t)n * PTM_KNN * sizeof(int2)));
     CK(cudaMalloc(&ctx->lam, (size_t)n * 3 * sizeof(uint64_t)));
     CK(cudaMalloc(&ctx->ents, (size_t)n * sizeof(uint32_t)));
     ctx->cap_nbr = (size_t)n;
   }
   if (topological && (size_t)n > ctx->cap_topo) {
-    cudaFree(ctx->nbr18);
     cudaFree(ctx->topo_list);
     cudaFree(ctx->topo_side);
-    ctx->nbr18 = nullptr;
     ctx->topo_list = nullptr;
     ctx->topo_side = nullptr;
     ctx->cap_topo = 0;
-    CK(cudaMalloc(&ctx->nbr18, (size_t)n * PTM_TOPO_N * sizeof(int2)));
     CK(cudaMalloc(&ctx->topo_list, (size_t)n * sizeof(int)));
     CK(cudaMalloc(&ctx->topo_side, topo_side_bytes((size_t)n)));
     ctx->cap_topo = (size_t)n;
   }
+  float4 *hi = pair_hi(f64 ? ctx->pairs : ctx->lam);
   const FrameBuffers B = {ctx->cell_count, ctx->cell_start, ctx->block_sums, ctx->atom_cell, ctx->atom_rank,
-                          ctx->atom_wrap, ctx->sbin, ctx->wrapv, ctx->sorted, ctx->hi, ctx->lo, ctx->dstat,
-                          ctx->counters, ctx->tab, ctx->nbr, ctx->nbr18, ctx->lam, ctx->ents};
+                          ctx->atom_wrap, ctx->sbin, ctx->wrapv, ctx->sorted, hi, pair_lo(hi, (size_t)n), ctx->dstat,
+                          ctx->counters, ctx->tab, ctx->nbr, ctx->lam, ctx->ents};
   set_buffers(&desc, &bp, B);
   set_outputs(&desc, o);
 
@@ -357,14 +377,14 @@ static ptm_status enqueue_frame(ptm_context *ctx, const ptm_frame *f, const ptm_
     const int cap_side = (int)topo_side_cap(ctx->cap_topo);
     const unsigned g64 = (unsigned)(PTM_TOPO64_BLOCKS_PER_SM * sms);
     if (f64) {
-      k_topo<true><<<ga, PTM_BLOCK, topo_smem_bytes(), st>>>(desc, ctx->nbr, ctx->topo_list, cnt, ctx->topo_side,
+      k_topo<true><<<ga, PTM_BLOCK, topo_smem_bytes(), st>>>(desc, ctx->topo_list, cnt, ctx->topo_side,
                                                              cap_side);
-      k_topo64<true><<<g64, PTM_BLOCK, topo64_smem_bytes(), st>>>(desc, ctx->nbr, ctx->topo_list, cnt,
+      k_topo64<true><<<g64, PTM_BLOCK, topo64_smem_bytes(), st>>>(desc, ctx->topo_list, cnt,
                                                                   ctx->topo_side, cap_side);
     } else {
-      k_topo<false><<<ga, PTM_BLOCK, topo_smem_bytes(), st>>>(desc, ctx->nbr, ctx->topo_list, cnt, ctx->topo_side,
+      k_topo<false><<<ga, PTM_BLOCK, topo_smem_bytes(), st>>>(desc, ctx->topo_list, cnt, ctx->topo_side,
                                                               cap_side);
-      k_topo64<false><<<g64, PTM_BLOCK, topo64_smem_bytes(), st>>>(desc, ctx->nbr, ctx->topo_list, cnt,
+      k_topo64<false><<<g64, PTM_BLOCK, topo64_smem_bytes(), st>>>(desc, ctx->topo_list, cnt,
                                                                    ctx->topo_side, cap_side);
     }
     launches += 2;
@@ -462,7 +482,7 @@ ptm_status ptm_destroy(ptm_context *ctx) {
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
   cudaFree(ctx->sorted); cudaFree(ctx->sbin); cudaFree(ctx->wrapv);
-  cudaFree(ctx->hi); cudaFree(ctx->lo);
+  cudaFree(ctx->pairs);
   cudaFree(ctx->atom_cell); cudaFree(ctx->atom_rank); cudaFree(ctx->atom_wrap);
   cudaFree(ctx->cell_count); cudaFree(ctx->cell_start); cudaFree(ctx->block_sums);
   cudaFree(ctx->dstat); cudaFree(ctx->counters); cudaFree(ctx->tab);
@@ -471,7 +491,6 @@ ptm_status ptm_destroy(ptm_context *ctx) {
   cudaFree(ctx->o_struct); cudaFree(ctx->o_alloy); cudaFree(ctx->o_rmsd); cudaFree(ctx->o_scale);
   cudaFree(ctx->o_quat); cudaFree(ctx->o_strain); cudaFree(ctx->o_corr); cudaFree(ctx->o_vm); cudaFree(ctx->o_rf);
   cudaFree(ctx->nbr); cudaFree(ctx->lam); cudaFree(ctx->ents);
-  cudaFree(ctx->nbr18);
   cudaFree(ctx->topo_list);
   cudaFree(ctx->topo_side);
   delete ctx;
@@ -594,7 +613,8 @@ struct ptm_batch {
   int64_t *d_atom_off = nullptr;
   int *d_dstat = nullptr;
   void *sorted = nullptr;
-  float4 *hi = nullptr, *lo = nullptr;
+  float4 *hi = nullptr;
+  float2 *lo = nullptr;
   int *sbin = nullptr, *wrapv = nullptr, *atom_cell = nullptr, *atom_rank = nullptr, *atom_wrap = nullptr;
   int *cell_count = nullptr, *cell_start = nullptr, *block_sums = nullptr;
   unsigned long long *queue = nullptr, *counters = nullptr;
@@ -606,7 +626,6 @@ struct ptm_batch {
   int nsm = 152;
   int topo = 0;                   // some frame takes the topological order
   int2 *nbr_buf = nullptr;        // per-frame segments of neighbour lists
-  int2 *nbr18_buf = nullptr;      // ... of the 18 nearest (some frame takes the topological order)
   uint64_t *lam_buf = nullptr;    // per-frame segments of the k_hulls -> k_match state
   uint32_t *ents_buf = nullptr;
   std::vector<FrameDesc> own;     // frames with a k_match launch of their own (PTM_MATCH_OWN_LAUNCH)
@@ -770,7 +789,7 @@ struct BatchPlan {
   std::vector<BinParams> hb;
   std::vector<int64_t> off;
   int64_t ntotal = 0;
-  size_t ncell = 0;
+  size_t ncell = 0, nbr_rows = 0;    // cells, neighbour list entries
   int f64 = 0;
   int topo = 0;                      // 0: no frame, 1: some, 2: every frame in the topological order
   int ntopo = 0;
@@ -799,6 +818,7 @@ static ptm_status batch_plan(int nframes, const ptm_frame *frames, double cell_f
     P.ordering[f] = frames[f].ordering;
     P.ntopo += frames[f].ordering == PTM_ORDER_TOPOLOGICAL;
     P.ntotal += frames[f].n_atoms;
+    P.nbr_rows += nbr_rows(frames[f].ordering) * (size_t)frames[f].n_atoms;
     P.ncell += nc;
     if (P.ntotal >= (1ll << 31) || P.ncell >= (1ull << 31)) return PTM_ERR_INVALID_ARG;
   }
@@ -818,11 +838,11 @@ static size_t batch_zero_bytes(int nframes, size_t ncell) {
 }
 
 // Device bytes of a batch's workspace (descriptors, sorted atoms, cell lists).
-static size_t batch_workspace_bytes(int nframes, int64_t ntotal, size_t ncell, int f64, int topo) {
-  const size_t n = (size_t)ntotal, rec = (f64 ? sizeof(Atom64) : sizeof(float4)) + 2 * sizeof(float4);
+static size_t batch_workspace_bytes(int nframes, const BatchPlan &P) {
+  const size_t n = (size_t)P.ntotal, ncell = P.ncell;
+  const size_t rec = P.f64 ? sizeof(Atom64) + PTM_PAIR_BYTES : sizeof(float4);
   const size_t nblk = (ncell + 1 + 2 * SCAN_BLOCK - 1) / (2 * SCAN_BLOCK) + 1;
-  const size_t tb = sizeof(int2) * PTM_KNN * n + 28 * n + 3 * 256 +
-                    (topo ? sizeof(int2) * PTM_TOPO_N * n + 4 * n + topo_side_bytes(n) + 3 * 256 : 0);
+  const size_t tb = sizeof(int2) * P.nbr_rows + 28 * n + 3 * 256 + (P.topo ? 4 * n + topo_side_bytes(n) + 2 * 256 : 0);
   return (sizeof(FrameDesc) + sizeof(ShiftTables) + sizeof(BinParams) + 2 * sizeof(int64_t) + sizeof(int)) * nframes +
          batch_zero_bytes(nframes, ncell) + rec * n + 20 * n + 4 * (ncell + 1) + 4 * nblk + 18 * 256 + tb;
 }
@@ -848,24 +868,26 @@ static void batch_layout(ptm_batch *b, unsigned char *base, BatchPlan &P, const 
   b->d_dstat = b->lists + 4;
   b->cell_count = b->d_dstat + 4 * nf;
   b->sorted = take((P.f64 ? sizeof(Atom64) : sizeof(float4)) * n);
-  b->hi = (float4 *)take(sizeof(float4) * n); b->lo = (float4 *)take(sizeof(float4) * n);
+  if (P.f64) b->hi = pair_hi(take(PTM_PAIR_BYTES * n));
   b->sbin = (int *)take(4 * n); b->wrapv = (int *)take(4 * n); b->atom_cell = (int *)take(4 * n);
   b->atom_rank = (int *)take(4 * n); b->atom_wrap = (int *)take(4 * n);
   b->cell_start = (int *)take(4 * (nc + 1));
   b->block_sums = (int *)take(4 * nblk);
   b->topo = P.topo;
-  b->nbr_buf = (int2 *)take(sizeof(int2) * PTM_KNN * n);
+  b->nbr_buf = (int2 *)take(sizeof(int2) * P.nbr_rows);
   b->lam_buf = (uint64_t *)take(sizeof(uint64_t) * 3 * n);
+  if (!P.f64) b->hi = pair_hi(b->lam_buf);
+  b->lo = pair_lo(b->hi, n);
   b->ents_buf = (uint32_t *)take(sizeof(uint32_t) * n);
   if (P.topo) {
-    b->nbr18_buf = (int2 *)take(sizeof(int2) * PTM_TOPO_N * n);
     b->topo_list = (int *)take(4 * n);
     b->topo_side = (TopoSide *)take(topo_side_bytes(n));
   }
+  size_t row = 0;
   for (int f = 0; f < nf; f++) {
-    // frame f's neighbour list: rows of n_f entries from slot 14 x (first slot)
-    P.hd[f].nbr = b->nbr_buf + PTM_KNN * P.off[f];
-    P.hd[f].nbr18 = P.topo ? b->nbr18_buf + PTM_TOPO_N * P.off[f] : nullptr;
+    // frame f's neighbour list: 14 or 18 rows of n_f entries
+    P.hd[f].nbr = b->nbr_buf + row;
+    row += nbr_rows(P.hd[f].ordering) * (size_t)P.hd[f].n;
     P.hd[f].lam = b->lam_buf + 3 * P.off[f];
     P.hd[f].ents = b->ents_buf + P.off[f];
     P.hd[f].tab = b->d_tabs + f;
@@ -909,7 +931,7 @@ extern "C" ptm_status ptm_batch_create(ptm_context *ctx, int nframes, const ptm_
   b->f64 = P.f64;
   b->ntotal = P.ntotal;
   b->ncell = P.ncell;
-  cudaError_t e = cudaMalloc(&b->block, batch_workspace_bytes(nframes, P.ntotal, P.ncell, P.f64, P.topo));
+  cudaError_t e = cudaMalloc(&b->block, batch_workspace_bytes(nframes, P));
   for (int i = 0; i < 5 && e == cudaSuccess; i++) e = cudaEventCreate(&b->ev[i]);
   if (e != cudaSuccess) { rs = cuda_fail(ctx, e, "ptm_batch_create"); batch_free(b); return rs; }
   batch_layout(b, (unsigned char *)b->block, P, outs);
@@ -1062,8 +1084,7 @@ constexpr size_t kNoallocScanBlocks = (kNoallocCells + 1 + 2 * SCAN_BLOCK - 1) /
 struct NoallocLayout {                  // byte offsets inside the static array
   static constexpr size_t sorted = 0;                                            // Atom64 records (float4 fits too)
   static constexpr size_t hi = sorted + sizeof(Atom64) * kNoallocAtoms;
-  static constexpr size_t lo = hi + sizeof(float4) * kNoallocAtoms;
-  static constexpr size_t sbin = lo + sizeof(float4) * kNoallocAtoms;
+  static constexpr size_t sbin = hi + PTM_PAIR_BYTES * kNoallocAtoms;
   static constexpr size_t wrapv = sbin + sizeof(int) * kNoallocAtoms;
   static constexpr size_t atom_cell = wrapv + sizeof(int) * kNoallocAtoms;
   static constexpr size_t atom_rank = atom_cell + sizeof(int) * kNoallocAtoms;
@@ -1144,16 +1165,14 @@ extern "C" ptm_status ptm_classify_frame_noalloc(const ptm_frame *f, const ptm_o
   unsigned char *base = nullptr;
   rs = noalloc_address(st, &base);
   if (rs != PTM_OK) return rs;
-  const int64_t n = f->n_atoms;
-  const int f64 = desc.f64;
   auto at = [&](size_t off) { return (void *)(base + off); };
   typedef NoallocLayout L;
+  float4 *hi = pair_hi(at(L::hi));
   const FrameBuffers B = {(int *)at(L::cell_count), (int *)at(L::cell_start), (int *)at(L::block_sums),
                           (int *)at(L::atom_cell), (int *)at(L::atom_rank), (int *)at(L::atom_wrap),
-                          (int *)at(L::sbin), (int *)at(L::wrapv), at(L::sorted), (float4 *)at(L::hi),
-                          (float4 *)at(L::lo), (int *)at(L::dstat), (unsigned long long *)at(L::counters),
-                          (ShiftTables *)at(L::tab), (int2 *)at(L::nbr), nullptr, (uint64_t *)at(L::lam),
-                          (uint32_t *)at(L::ents)};
+                          (int *)at(L::sbin), (int *)at(L::wrapv), at(L::sorted), hi, pair_lo(hi, (size_t)f->n_atoms),
+                          (int *)at(L::dstat), (unsigned long long *)at(L::counters), (ShiftTables *)at(L::tab),
+                          (int2 *)at(L::nbr), (uint64_t *)at(L::lam), (uint32_t *)at(L::ents)};
   set_buffers(&desc, &bp, B);
   set_outputs(&desc, o);
   cudaGetLastError();   // launch errors are read below; drop any left by earlier calls

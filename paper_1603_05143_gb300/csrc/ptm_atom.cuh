@@ -45,8 +45,8 @@ struct FrameDesc {
   const int *sbin;             // frame-local cell of each sorted slot
   const int *cell_start;       // this frame's ncell + 1 offsets into sorted (global sorted indices)
   const int *wrapv;            // packed lattice wrap per sorted slot
-  const float4 *hi, *lo;       // cell-sorted positions wrapped into the cell as FP32 pairs hi + lo (lo.w: the
-                               // packed wrap), for float64 input and for frames with wrapped atoms
+  const float4 *hi;            // cell-sorted positions wrapped into the cell as FP32 pairs: (hi x, y, z, lo x) and
+  const float2 *lo;            // (lo y, z), for float64 input and for frames with wrapped atoms
   const int8_t *species;       // by atom id, or NULL
   const void *positions;       // caller positions (by atom id)
   int64_t n;
@@ -70,10 +70,9 @@ struct FrameDesc {
   int32_t *corr;
   float *vm;                   // derived: von Mises shear strain
   float *rf;                   // derived: Rodrigues-Frank vector
-  const int2 *nbr;             // neighbour list: [t][n] (sorted slot, image) of neighbour t of the
+  int2 *nbr;                   // neighbour list: [t][n] (sorted slot, image) of neighbour t of the
                                // atom at frame-local slot s - atom_offset (slot -1: none), written
-                               // by k_knn (Euclidean order) or k_topo (topological order)
-  int2 *nbr18;                 // topological order: the 18 nearest, [18][n], read by k_topo
+                               // by k_knn; topological order: 18 rows, of which k_topo makes the 14
   int ordering;                // PTM_ORDER_EUCLIDEAN or PTM_ORDER_TOPOLOGICAL
   uint64_t *lam;               // k_hulls -> k_match: [3][n] Weinberg labelling of snapshot k = 6, 12, 14
   uint32_t *ents;              // [n] their table entries + 1, 10 bits each (0: no match)

@@ -785,33 +785,31 @@ __device__ __noinline__ void wide_quantise(const FrameDesc &d, typename RT<F64>:
   }
 }
 
-// Vector of list entry e from an atom at hs + ls as FP32 pairs h + l: differences
+// Vector of list entry e from the atom at sorted slot s, hs + ls, as FP32 pairs h + l: differences
 // and shift summed without loss but for the low parts, within about 2^-44 of the
 // positions and the cell.  Float64 input takes the pairs of the positions wrapped
 // into the cell, float32 input the positions themselves.  Returns false for an
 // image beyond the next, whose shift may be larger than that allows for.
 template <bool F64>
-__device__ __forceinline__ bool pair_vector(const FrameDesc &d, float4 hs, float4 ls, int2 e, float (&h)[3],
-                                            float (&l)[3]) {
+__device__ __forceinline__ bool pair_vector(const FrameDesc &d, bool wrapped, int s, float4 hs, float2 ls, int2 e,
+                                            float (&h)[3], float (&l)[3]) {
   const float4 p = __ldg((F64 ? d.hi : (const float4 *)d.sorted) + e.x);
-  float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+  float2 q = make_float2(0.f, 0.f);
   int a, b, c;
   img_unpack(e.y, a, b, c);
   if constexpr (F64) {
     q = __ldg(d.lo + e.x);
-    int a1, b1, c1, a2, b2, c2;
-    img_unpack(__float_as_int(q.w), a1, b1, c1);
-    img_unpack(__float_as_int(ls.w), a2, b2, c2);
-    a += a1 - a2; b += b1 - b2; c += c1 - c2;
+    cell_image(d, wrapped, s, e.x, a, b, c);
   }
-  float s[3] = {0.f, 0.f, 0.f}, r[3] = {0.f, 0.f, 0.f};
-  if (a | b | c) shift_f32(d, a, b, c, s[0], s[1], s[2], r[0], r[1], r[2]);
-  const float pj[3] = {p.x, p.y, p.z}, qj[3] = {q.x, q.y, q.z}, pi[3] = {hs.x, hs.y, hs.z}, qi[3] = {ls.x, ls.y, ls.z};
+  float t0[3] = {0.f, 0.f, 0.f}, r[3] = {0.f, 0.f, 0.f};
+  if (a | b | c) shift_f32(d, a, b, c, t0[0], t0[1], t0[2], r[0], r[1], r[2]);
+  const float pj[3] = {p.x, p.y, p.z}, qj[3] = {F64 ? p.w : 0.f, q.x, q.y}, pi[3] = {hs.x, hs.y, hs.z},
+              qi[3] = {F64 ? hs.w : 0.f, ls.x, ls.y};
 #pragma unroll
   for (int k = 0; k < 3; k++) {
     float d1, e1, d2, e2;
     two_sum(pj[k], -pi[k], d1, e1);
-    two_sum(d1, s[k], d2, e2);
+    two_sum(d1, t0[k], d2, e2);
     const float t = __fadd_rn(e1, __fadd_rn(e2, __fadd_rn(__fsub_rn(qj[k], qi[k]), r[k])));
     h[k] = __fadd_rn(d2, t);
     l[k] = __fsub_rn(t, __fsub_rn(h[k], d2));
@@ -869,7 +867,9 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
     };
     float emaxf = 0.f, m = 0.f;
     uint32_t wide = 0, bad = 0;
-    float4 hs, ls = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 hs;
+    float2 ls = make_float2(0.f, 0.f);
+    const bool wrapped = F64 && d.dstat[0] != 0;
     if constexpr (F64) {
       hs = __ldg(d.hi + s);
       ls = __ldg(d.lo + s);
@@ -880,7 +880,7 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
         cnt++;
         wide |= 1u << t;
         float h[3], l[3];
-        if (!pair_vector<F64>(d, hs, ls, e, h, l)) bad |= 1u << t;
+        if (!pair_vector<F64>(d, wrapped, s, hs, ls, e, h, l)) bad |= 1u << t;
 #pragma unroll
         for (int c = 0; c < 3; c++) { sm.Q(t, c) = h[c]; low(t, c) = __float_as_uint(l[c]); m = fmaxf(m, fabsf(h[c])); }
       }
@@ -906,7 +906,7 @@ __device__ int hull_atom(const FrameDesc &d, int s, const Scratch &sm, unsigned 
         const int t = __ffs(w) - 1;
         const int2 e = __ldg(nb + t * nst);
         float h[3], l[3];
-        if (!pair_vector<F64>(d, hs, ls, e, h, l)) bad |= 1u << t;
+        if (!pair_vector<F64>(d, wrapped, s, hs, ls, e, h, l)) bad |= 1u << t;
 #pragma unroll
         for (int c = 0; c < 3; c++) { sm.Q(t, c) = h[c]; low(t, c) = __float_as_uint(l[c]); }
         const float mt = fmaxf(fabsf(h[0]), fmaxf(fabsf(h[1]), fabsf(h[2])));
@@ -1228,7 +1228,7 @@ __global__ void k_scan_add(int *out, const int *block_sums, int n) {
 // wrapped into the cell as an FP32 pair: the neighbour search then works in FP32
 // and on the 27 images, whatever the input.  An excluded atom's pair is NaN.
 __device__ __forceinline__ void scatter_atom(const BinParams &p, const void *pos, int64_t li, int wrap, bool wrapped,
-                                             int slot, void *sorted, float4 *hi, float4 *lo) {
+                                             int slot, void *sorted, float4 *hi, float2 *lo) {
   double x, y, z;
   if (p.f64) {
     const double *q = (const double *)pos + 3 * li;
@@ -1251,13 +1251,13 @@ __device__ __forceinline__ void scatter_atom(const BinParams &p, const void *pos
     if (wrap == PTM_EXCLUDED) x = y = z = NAN;
   }
   const float hx = (float)x, hy = (float)y, hz = (float)z;
-  hi[slot] = make_float4(hx, hy, hz, 0.f);
-  lo[slot] = make_float4((float)(x - hx), (float)(y - hy), (float)(z - hz), __int_as_float(wrap));
+  hi[slot] = make_float4(hx, hy, hz, (float)(x - hx));
+  lo[slot] = make_float2((float)(y - hy), (float)(z - hz));
 }
 
 __global__ void k_scatter(const void *pos, BinParams p, const int *atom_cell, const int *atom_rank,
                           const int *atom_wrap, const int *cell_start, const int *dstat, void *sorted, float4 *hi,
-                          float4 *lo, int *sbin, int *wrapv) {
+                          float2 *lo, int *sbin, int *wrapv) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= p.n) return;
   const int c = atom_cell[i], wrap = atom_wrap[i];
@@ -1277,7 +1277,7 @@ __global__ void k_scatter(const void *pos, BinParams p, const int *atom_cell, co
 __global__ void __launch_bounds__(PTM_SMALL_BLOCK)
     k_cells_small(const __grid_constant__ ShiftTables t, const void *pos, const __grid_constant__ BinParams p, int ncell,
                   ShiftTables *out, int *cell_start, int *dstat, unsigned long long *counters, void *sorted, float4 *hi,
-                  float4 *lo, int *sbin, int *wrapv) {
+                  float2 *lo, int *sbin, int *wrapv) {
   __shared__ int cells[PTM_SMALL_CELLS];
   __shared__ int sh[32];
   __shared__ int any_wrap, overs, excluded;
@@ -1363,7 +1363,7 @@ __global__ void k_bin_batch(const BinParams *__restrict__ bp, const int64_t *__r
 
 __global__ void k_scatter_batch(const BinParams *__restrict__ bp, const int64_t *__restrict__ atom_off, int nframes,
                                 int64_t ntotal, const int *atom_cell, const int *atom_rank, const int *atom_wrap,
-                                const int *cell_start, void *sorted, float4 *hi, float4 *lo, int *sbin, int *wrapv) {
+                                const int *cell_start, void *sorted, float4 *hi, float2 *lo, int *sbin, int *wrapv) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= ntotal) return;
   const int f = frame_of(atom_off, nframes, i);
@@ -1466,7 +1466,7 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM) k_match(co
 }
 
 // Neighbour lists of one frame, one thread per atom: NK = 14 into d.nbr, NK = 18
-// (topological order) into d.nbr18.  Measured against the insertion network and
+// (topological order), into d.nbr.  Measured against the insertion network and
 // the FP64 arithmetic it replaced (k_knn with k_knn_rest, device time):
 //   2^20-atom polycrystal, float32      1.23  -> 0.64 ms (k_knn 0.46, at 46 % of
 //                                       issue and 47 % of L1; 675 -> 226 warp
@@ -1480,7 +1480,7 @@ __global__ void __launch_bounds__(PTM_KNN_BLOCK, KnnShape<NK>::BLOCKS)
   extern __shared__ __align__(16) unsigned char smem[];
   const int64_t s = spread_slot(d.n, apw);
   if (s < 0) return;
-  knn_atom<F64, NK>(d, (int)s, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18, smem, rest, rest_count);
+  knn_atom<F64, NK>(d, (int)s, d.nbr, smem, rest, rest_count);
 }
 
 template <bool F64, int NK>
@@ -1488,7 +1488,7 @@ __global__ void __launch_bounds__(PTM_KNN_BLOCK)
     k_knn_rest(const __grid_constant__ FrameDesc d, const int *rest, const int *rest_count) {
   const int n = rest ? *rest_count : (int)d.n, stride = gridDim.x * (PTM_KNN_BLOCK / 32);
   for (int i = (blockIdx.x * PTM_KNN_BLOCK + threadIdx.x) >> 5; i < n; i += stride)
-    knn_rest_atom<F64, NK>(d, rest ? rest[i] : i, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18);
+    knn_rest_atom<F64, NK>(d, rest ? rest[i] : i, d.nbr);
 }
 
 // The same over a batch: each slot finds its frame; NK = 14 takes the frames in
@@ -1502,7 +1502,7 @@ __global__ void __launch_bounds__(PTM_KNN_BLOCK, KnnShape<NK>::BLOCKS)
   if (s >= ntotal) return;
   const FrameDesc &d = descs[frame_of(atom_off, nframes, s)];
   if ((d.ordering == PTM_ORDER_EUCLIDEAN) != (NK == PTM_KNN)) return;
-  knn_atom<F64, NK>(d, (int)s, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18, smem, rest, rest_count);
+  knn_atom<F64, NK>(d, (int)s, d.nbr, smem, rest, rest_count);
 }
 
 template <bool F64, int NK>
@@ -1513,7 +1513,7 @@ __global__ void __launch_bounds__(PTM_KNN_BLOCK)
   for (int i = (blockIdx.x * PTM_KNN_BLOCK + threadIdx.x) >> 5; i < n; i += stride) {
     const int s = rest[i];
     const FrameDesc &d = descs[frame_of(atom_off, nframes, s)];
-    knn_rest_atom<F64, NK>(d, s, NK == PTM_KNN ? const_cast<int2 *>(d.nbr) : d.nbr18);
+    knn_rest_atom<F64, NK>(d, s, d.nbr);
   }
 }
 

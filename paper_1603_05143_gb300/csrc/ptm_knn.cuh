@@ -232,6 +232,17 @@ __device__ __forceinline__ float knn_band(const FrameDesc &d, float v) {
   return 2.f * (8.5f * u * vmax + 4.f * (sqrtf(vmax) + d.tau) * d.tau);
 }
 
+// Turns (a, b, c), the image of the atom at slot j as the atom at slot i sees it in the input's
+// positions, into its image in positions wrapped into the cell (slots swapped: back).
+// `wrapped`: whether any atom of the frame is (d.dstat[0]).
+__device__ __forceinline__ void cell_image(const FrameDesc &d, bool wrapped, int i, int j, int &a, int &b, int &c) {
+  if (!wrapped) return;
+  int i0, i1, i2, j0, j1, j2;
+  img_unpack(__ldg(d.wrapv + i), i0, i1, i2);
+  img_unpack(__ldg(d.wrapv + j), j0, j1, j2);
+  a += j0 - i0; b += j1 - i1; c += j2 - i2;
+}
+
 // Position at hs + ls less the shift of a lattice image (s + r, FP32 pair), as a pair h + l.
 __device__ __forceinline__ void shift_pair(float hs, float ls, float s, float r, float &h, float &l) {
   float e;
@@ -251,20 +262,21 @@ __device__ __forceinline__ void shift_pair(float hs, float ls, float s, float r,
 // roundings of the component, whatever the image shift, plus terms in u^2 of
 // the positions (d.tau).
 template <bool SPLIT, int CAP>
-__device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__restrict__ hi, float4 hs, float4 ls,
+__device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__restrict__ hi, float4 hs, float2 ls,
                                           int bx, int by, int bz, float T, const KnnList &list) {
   int cnt = 0;
   for_cells27(d, bx, by, bz, [&](int ca, int cb, int mx, int my, int mz) {
     int j = __ldg(d.cell_start + ca);
     const int j1 = __ldg(d.cell_start + cb + 1);
-    float hx = hs.x, hy = hs.y, hz = hs.z, lx = ls.x, ly = ls.y, lz = ls.z;
+    const float l0 = SPLIT ? hs.w : 0.f;
+    float hx = hs.x, hy = hs.y, hz = hs.z, lx = l0, ly = ls.x, lz = ls.y;
     const bool shifted = (mx | my | mz) != 0;
     if (shifted) {
       const ShiftTables &t = *d.tab;
       const int i = (mx + 2) * 25 + (my + 2) * 5 + (mz + 2);
-      shift_pair(hs.x, ls.x, t.s32[i][0], t.slo[i][0], hx, lx);
-      shift_pair(hs.y, ls.y, t.s32[i][1], t.slo[i][1], hy, ly);
-      shift_pair(hs.z, ls.z, t.s32[i][2], t.slo[i][2], hz, lz);
+      shift_pair(hs.x, l0, t.s32[i][0], t.slo[i][0], hx, lx);
+      shift_pair(hs.y, ls.x, t.s32[i][1], t.slo[i][1], hy, ly);
+      shift_pair(hs.z, ls.y, t.s32[i][2], t.slo[i][2], hz, lz);
     }
     const uint8_t code = (uint8_t)((mx + 1) << 4 | (my + 1) << 2 | (mz + 1));
     auto test = [&](int jj, float x, float y, float z) {
@@ -280,7 +292,8 @@ __device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__re
     constexpr int U = SPLIT ? 3 : 4;
     if (SPLIT || shifted) {
       for (; j < j1; j += U) {
-        float4 p[U], q[U];
+        float4 p[U];
+        float2 q[U];
 #pragma unroll
         for (int k = 0; k < U; k++) {
           p[k] = __ldg(hi + min(j + k, j1 - 1));
@@ -290,7 +303,7 @@ __device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__re
         for (int k = 0; k < U; k++) {
           if (k && j + k >= j1) break;
           if constexpr (SPLIT)
-            test(j + k, (p[k].x - hx) + (q[k].x - lx), (p[k].y - hy) + (q[k].y - ly), (p[k].z - hz) + (q[k].z - lz));
+            test(j + k, (p[k].x - hx) + (p[k].w - lx), (p[k].y - hy) + (q[k].x - ly), (p[k].z - hz) + (q[k].y - lz));
           else
             test(j + k, (p[k].x - hx) - lx, (p[k].y - hy) - ly, (p[k].z - hz) - lz);
         }
@@ -355,8 +368,8 @@ __device__ __noinline__ float crowded_radius(const FrameDesc &d, const float4 *_
 // ordered by the FP64 key (d2, atom id, image); a run across slot NK takes
 // every candidate within the band.
 template <bool F64, bool SPLIT, int NK>
-__device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int by, int bz, int2 *out, int64_t nst,
-                                         const KnnList &list) {
+__device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int by, int bz, bool wrapped, int2 *out,
+                                         int64_t nst, const KnnList &list) {
   typedef typename RT<F64>::T IN;
   constexpr int CAP = KnnShape<NK>::CAP;
   constexpr float AIM = KnnShape<NK>::AIM;
@@ -366,7 +379,7 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
   const float Tmax = rg * rg * (1.f - 1e-3f);
   const float4 *__restrict__ hi = SPLIT ? d.hi : (const float4 *)d.sorted;
   const float4 hs = __ldg(hi + s);
-  float4 ls = make_float4(0.f, 0.f, 0.f, 0.f);
+  float2 ls = make_float2(0.f, 0.f);
   if constexpr (SPLIT) ls = __ldg(d.lo + s);
   int cnt = 0;
   float T;
@@ -393,15 +406,9 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
     T = fminf(Tmax, T * (cnt > CAP ? f : fmaxf(f, 1.2f)));
   }
   // image of list entry i: the cells' image, less the wraps of the two atoms
-  int w0 = 0, w1 = 0, w2 = 0;
-  if constexpr (SPLIT) img_unpack(__float_as_int(ls.w), w0, w1, w2);
   auto image = [&](int j, int code, int &a, int &b, int &c) {
-    a = (code >> 4) - 1 + w0; b = (code >> 2 & 3) - 1 + w1; c = (code & 3) - 1 + w2;
-    if constexpr (SPLIT) {
-      int q0, q1, q2;
-      img_unpack(__float_as_int(__ldg(&d.lo[j].w)), q0, q1, q2);
-      a -= q0; b -= q1; c -= q2;
-    }
+    a = (code >> 4) - 1; b = (code >> 2 & 3) - 1; c = (code & 3) - 1;
+    if constexpr (SPLIT) cell_image(d, wrapped, j, s, a, b, c);
   };
   auto put = [&](int t, int i) {
     const int j = list.J(i);
@@ -519,9 +526,10 @@ __device__ __forceinline__ void knn_atom(const FrameDesc &d, int s, int2 *rows, 
   const int bz = b % d.nb[2], byx = b / d.nb[2];
   const int by = byx % d.nb[1], bx = byx / d.nb[1];
   const KnnList list = knn_list<KnnShape<NK>::CAP>(smem);
+  const bool wrapped = d.dstat[0] != 0;
   bool done;
-  if (F64 || d.dstat[0] != 0) done = knn_fast<F64, true, NK>(d, s, bx, by, bz, out, nst, list);
-  else done = knn_fast<F64, false, NK>(d, s, bx, by, bz, out, nst, list);
+  if (F64 || wrapped) done = knn_fast<F64, true, NK>(d, s, bx, by, bz, wrapped, out, nst, list);
+  else done = knn_fast<F64, false, NK>(d, s, bx, by, bz, wrapped, out, nst, list);
   if (!done) rest[atomicAdd(rest_count, 1)] = s;
 }
 
@@ -670,25 +678,24 @@ __device__ void knn_rest_atom(const FrameDesc &d, int s, int2 *rows) {
     float v = INFINITY;
     if (mine) {
       const float4 p = __ldg(hi + lj);
-      float4 ls = make_float4(0.f, 0.f, 0.f, 0.f), q = ls;
+      float2 ls = make_float2(0.f, 0.f), q = ls;
       int a, b, c;
       img_unpack(limg, a, b, c);
       if (split) {
         ls = __ldg(d.lo + s);
         q = __ldg(d.lo + lj);
-        int q0, q1, q2;
-        img_unpack(__float_as_int(q.w), q0, q1, q2);
-        a += q0 - wi0; b += q1 - wi1; c += q2 - wi2;
+        cell_image(d, true, s, lj, a, b, c);
       }
-      float hx = hs.x, hy = hs.y, hz = hs.z, lx = ls.x, ly = ls.y, lz = ls.z;
+      const float l0 = split ? hs.w : 0.f, q0 = split ? p.w : 0.f;
+      float hx = hs.x, hy = hs.y, hz = hs.z, lx = l0, ly = ls.x, lz = ls.y;
       if (a | b | c) {
         float sx, sy, sz, rx, ry, rz;
         shift_f32(d, a, b, c, sx, sy, sz, rx, ry, rz);
-        shift_pair(hs.x, ls.x, sx, rx, hx, lx);
-        shift_pair(hs.y, ls.y, sy, ry, hy, ly);
-        shift_pair(hs.z, ls.z, sz, rz, hz, lz);
+        shift_pair(hs.x, l0, sx, rx, hx, lx);
+        shift_pair(hs.y, ls.x, sy, ry, hy, ly);
+        shift_pair(hs.z, ls.y, sz, rz, hz, lz);
       }
-      const float x = (p.x - hx) + (q.x - lx), y = (p.y - hy) + (q.y - ly), z = (p.z - hz) + (q.z - lz);
+      const float x = (p.x - hx) + (q0 - lx), y = (p.y - hy) + (q.x - ly), z = (p.z - hz) + (q.y - lz);
       v = fmaf(x, x, fmaf(y, y, z * z));
     }
     const int have = min(NK, __popc(__ballot_sync(ALL, mine)));

@@ -326,15 +326,16 @@ struct TopoSide {
 // polygon larger than the FP32 buffers) is appended to `list` for the FP64 pass
 // instead of being decided here, so that no warp waits on one lane's FP64 work;
 // the first cap_side listed atoms leave their areas and uncertain faces in
-// `side`.  The 18 nearest come from k_knn (d.nbr18; a slot of -1: fewer).
+// `side`.  The 18 nearest come from k_knn (d.nbr; a slot of -1: fewer); their first 14
+// rows take the order, a listed atom's by the FP64 pass.
 template <bool F64>
-__device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict__ out, int *list, int *list_count,
-                          TopoSide *side, int cap_side) {
+__device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int *list, int *list_count, TopoSide *side,
+                          int cap_side) {
   typedef typename RT<F64>::T TI;
   const int t = threadIdx.x;
   auto VF = [&](int k, int c) -> float & { return ((float *)tsm)[(3 * k + c) * PTM_BLOCK + t]; };
   const int64_t n = d.n, sl = s - d.atom_offset;     // frame-local slot
-  const int2 *nb = d.nbr18 + sl;
+  int2 *nb = d.nbr + sl;
   TI xi, yi, zi;
   int idi;
   load_atom<F64>(d, s, xi, yi, zi, idi);
@@ -345,7 +346,7 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict_
   float mean2 = 0.f, dmax2 = 0.f;
 #pragma unroll 2
   for (int k = 0; k < PTM_TOPO_N; k++) {
-    const int2 en = __ldg(nb + (int64_t)k * n);
+    const int2 en = nb[(int64_t)k * n];
     if (en.x < 0) break;                              // the valid entries form a prefix
     m++;
     TI xj, yj, zj;
@@ -389,10 +390,14 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict_
         for (int k = 0; k < PTM_TOPO_N; k++) sd.area[k] = k < m ? area[k] : 0.f;
         sd.faces = over ? ~0u : near;
       }
+      return;
     }
   }
-  for (int k = 0; k < PTM_KNN; k++)
-    out[(int64_t)k * n + sl] = k < m ? __ldg(nb + (int64_t)o[k] * n) : make_int2(-1, 0);
+  int2 e[PTM_KNN];
+#pragma unroll
+  for (int k = 0; k < PTM_KNN; k++) e[k] = k < m ? nb[(int64_t)o[k] * n] : make_int2(-1, 0);
+#pragma unroll
+  for (int k = 0; k < PTM_KNN; k++) nb[(int64_t)k * n] = e[k];
 }
 
 // FP64 pass for listed atom i (= list position), one thread: FP64 neighbour
@@ -408,7 +413,7 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int2 *__restrict_
 // pipe, 2 operations a clock per SM, sees only those.
 template <bool F64>
 __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *side, int cap_side, double *P,
-                            double *Q, float *vf32, int2 *__restrict__ out, unsigned wmask) {
+                            double *Q, float *vf32, unsigned wmask) {
   typedef typename RT<F64>::T TI;
   TI xi, yi, zi;
   int idi;
@@ -417,7 +422,7 @@ __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *si
   int jn[PTM_TOPO_N], im[PTM_TOPO_N], m = 0;
   double a64[PTM_TOPO_N];
   for (int k = 0; k < PTM_TOPO_N; k++) {
-    const int2 e = d.nbr18[(int64_t)k * n + sl];
+    const int2 e = d.nbr[(int64_t)k * n + sl];
     jn[k] = e.x;
     im[k] = e.y;
     m += e.x >= 0;
@@ -455,19 +460,19 @@ __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *si
     a64[k] = topo_face_area64(m, k, lines, R, vd, vf, P, Q, PTM_BLOCK, PTM_TOPO_VMAX);
   }
   if (m > 0) topo_order<double>(m, a64, mean64, o);
-  for (int k = 0; k < PTM_KNN; k++) out[(int64_t)k * n + sl] = k < m ? make_int2(jn[o[k]], im[o[k]]) : make_int2(-1, 0);
+  for (int k = 0; k < PTM_KNN; k++) d.nbr[(int64_t)k * n + sl] = k < m ? make_int2(jn[o[k]], im[o[k]]) : make_int2(-1, 0);
 }
 
 // Bounded by instruction issue (55 %; 624 M warp instructions per 262 k atoms):
 // 1.69 ms with every plane clipping every vertex, 1.35 ms with marks and one copy
 // per cut, 0.99 ms nearest line first and at 8 blocks per SM.
 template <bool F64>
-__global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO_BLOCKS_PER_SM) k_topo(const __grid_constant__ FrameDesc d, int2 *__restrict__ out,
-                                                    int *list, int *list_count, TopoSide *side, int cap_side) {
+__global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO_BLOCKS_PER_SM) k_topo(const __grid_constant__ FrameDesc d, int *list,
+                                                    int *list_count, TopoSide *side, int cap_side) {
   extern __shared__ __align__(16) unsigned char tsm_raw[];
   const int64_t s = (int64_t)blockIdx.x * PTM_BLOCK + threadIdx.x;
   if (s >= d.n) return;
-  topo_atom<F64>(d, (int)s, (int *)tsm_raw, out, list, list_count, side, cap_side);
+  topo_atom<F64>(d, (int)s, (int *)tsm_raw, list, list_count, side, cap_side);
 }
 
 // Second pass over the listed atoms, one thread per atom (grid-stride over the
@@ -485,20 +490,20 @@ __device__ __forceinline__ void topo64_list(int cnt, Fn &&fn) {
 }
 
 template <bool F64>
-__global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO64_BLOCKS_PER_SM) k_topo64(const __grid_constant__ FrameDesc d, int2 *__restrict__ out,
+__global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO64_BLOCKS_PER_SM) k_topo64(const __grid_constant__ FrameDesc d,
                                                       const int *list, const int *list_count, const TopoSide *side,
                                                       int cap_side) {
   extern __shared__ __align__(16) unsigned char tsm_raw[];
   double *P = (double *)tsm_raw + threadIdx.x, *Q = P + 2 * PTM_TOPO_VMAX * PTM_BLOCK;
   float *vf = (float *)((double *)tsm_raw + 4 * PTM_TOPO_VMAX * PTM_BLOCK) + threadIdx.x;
   topo64_list(*list_count, [&](int i, unsigned wmask) {
-    topo_atom64<F64>(d, list[i], i, side, cap_side, P, Q, vf, out, wmask);
+    topo_atom64<F64>(d, list[i], i, side, cap_side, P, Q, vf, wmask);
   });
 }
 
 // The same two passes over a batch: every slot finds its frame (frames in the
-// Euclidean order have no topological buffer and are skipped); each frame's
-// order lands in its own segment of the batch's buffer (FrameDesc::topo).
+// Euclidean order are skipped); each frame's list is its own segment of the batch's
+// (FrameDesc::nbr).
 template <bool F64>
 __global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO_BLOCKS_PER_SM)
     k_topo_batch(const FrameDesc *__restrict__ descs, const int64_t *__restrict__ atom_off, int nframes,
@@ -508,7 +513,7 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO_BLOCKS_PER_SM)
   if (s >= ntotal) return;
   const FrameDesc &d = descs[frame_of(atom_off, nframes, s)];
   if (d.ordering != PTM_ORDER_TOPOLOGICAL) return;
-  topo_atom<F64>(d, (int)s, (int *)tsm_raw, const_cast<int2 *>(d.nbr), list, list_count, side, cap_side);
+  topo_atom<F64>(d, (int)s, (int *)tsm_raw, list, list_count, side, cap_side);
 }
 
 template <bool F64>
@@ -521,7 +526,7 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO64_BLOCKS_PER_SM)
   topo64_list(*list_count, [&](int i, unsigned wmask) {
     const int s = list[i];
     const FrameDesc &d = descs[frame_of(atom_off, nframes, s)];
-    topo_atom64<F64>(d, s, i, side, cap_side, P, Q, vf, const_cast<int2 *>(d.nbr), wmask);
+    topo_atom64<F64>(d, s, i, side, cap_side, P, Q, vf, wmask);
   });
 }
 

@@ -1480,7 +1480,7 @@ __global__ void __launch_bounds__(PTM_KNN_BLOCK, KnnShape<NK>::BLOCKS)
   extern __shared__ __align__(16) unsigned char smem[];
   const int64_t s = spread_slot(d.n, apw);
   if (s < 0) return;
-  knn_atom<F64, NK>(d, (int)s, d.nbr, smem, rest, rest_count);
+  knn_atom<F64, NK>(d, (int)s, d.n, d.nbr, smem, rest, rest_count);
 }
 
 template <bool F64, int NK>
@@ -1502,7 +1502,7 @@ __global__ void __launch_bounds__(PTM_KNN_BLOCK, KnnShape<NK>::BLOCKS)
   if (s >= ntotal) return;
   const FrameDesc &d = descs[frame_of(atom_off, nframes, s)];
   if ((d.ordering == PTM_ORDER_EUCLIDEAN) != (NK == PTM_KNN)) return;
-  knn_atom<F64, NK>(d, (int)s, d.nbr, smem, rest, rest_count);
+  knn_atom<F64, NK>(d, (int)s, ntotal, d.nbr, smem, rest, rest_count);
 }
 
 template <bool F64, int NK>

@@ -5,8 +5,8 @@
 //   k_knn_rest  one warp per atom that k_knn left undecided
 //
 // k_knn reads the 27 cells around the atom once.  A radius chosen from their
-// occupancy admits about NT candidates, appended to a per-thread list in shared
-// memory; a sorting network then orders the list in registers.  What bounds it
+// occupancy admits about 24 candidates (36 for 18 neighbours), appended to a
+// per-thread list in shared memory; a sorting network then orders the list in registers.  What bounds it
 // is instruction issue: an insertion network run at every admitted candidate
 // issued 21 k instructions per warp at 14 of 32 active lanes, because some lane
 // inserts at nearly every candidate; the list costs three predicated stores per
@@ -157,15 +157,23 @@ template <int NK> struct KnnShape {
 constexpr size_t knn_smem_bytes(int nk) { return (size_t)PTM_KNN_BLOCK * (nk == PTM_KNN ? 32 : 64) * 9; }
 
 // Cells hold about 7 atoms (192 in 27) where the frame fills its box.  A cluster in a box of
-// vacuum has hundreds of times as many, in a few cells that are far from evenly filled:
-// the first radius is much too wide, and a thread reads everything three times over.
-// Frames of up to PTM_KNN_CROWDED_FRAME atoms, too few warps to hide that latency, leave
-// atoms with nearly all of the frame in reach to the warp search (8,000 atoms in a box
-// of 10 diameters: 2.95 ms a call without, 0.77 with; 20,000 in 7: 6.4 and 3.1; at 60,000 the
-// warps take 22.8 ms and the threads 19.3).  More atoms than that in the 27 cells, and a
-// sample sets the radius (60,000: 19.3 -> 15.3 ms; 200,000: 57.6 -> 54.6).
-#define PTM_KNN_CROWDED 1024
-#define PTM_KNN_CROWDED_FRAME 24576
+// vacuum has hundreds of times as many, in a few cells that are far from evenly filled: a
+// radius guessed from their filling is much too wide, and two or three gathers read
+// everything again.  With more than PTM_KNN_CROWDED atoms in the 27 cells
+//   - up to PTM_KNN_CROWDED_LAUNCH atoms in the launch (half for float64 input), too few warps
+//     to hide a thread's loads, atoms with nearly all of their frame in reach are left to
+//     the warp search: 3,000 atoms in a box of 7 diameters 0.31 ms a call, 0.60 with knn_crowded;
+//     8,000 0.83 and 1.28, 16,000 2.4 and 2.4; float64 3,000 0.42 and 0.60, 8,000 1.7 and 1.2;
+//   - the radius is guessed from the fullest cell where the cells are filled evenly (the
+//     inside of a cluster of several cells);
+//   - otherwise knn_crowded reads them once, and so it does after a gather that shows the
+//     guess to be far off.
+// ms a call, with guesses and gathers alone and now: 64 frames of 1,500 atoms in boxes of 3
+// diameters 1.09 and 0.80, 20 frames of 20,000 in 10 diameters 23.5 and 13.7, one
+// frame of 24,000 in 10 diameters 7.9 and 3.9, of 60,000 in 10 22.6 and 9.8 (and 2.04,
+// 59.9, 10.9 and 17.3 with all of them left to the warp search or a sampled radius).
+#define PTM_KNN_CROWDED 512
+#define PTM_KNN_CROWDED_LAUNCH 8192
 
 // Per-thread candidate list in shared memory, entry i at [i][thread]: FP32
 // squared distance, sorted slot, image code (m + 1 in two bits per axis).
@@ -324,52 +332,99 @@ __device__ __forceinline__ int knn_gather(const FrameDesc &d, const float4 *__re
   return cnt;
 }
 
-// Square of the radius of a sphere around the atom that holds about `aim` atoms, from every
-// step-th atom of the 27 cells: the sphere around about 32 of these, scaled down.
-// `T`: that square if the cells were evenly filled.
-__device__ __noinline__ float crowded_radius(const FrameDesc &d, const float4 *__restrict__ hi, float4 hs, int bx, int by,
-                                             int bz, int step, float T, float aim) {
-  const float want = 32.f;
-  float t = T * exp2f(0.6666667f * __log2f(__fdividef(want * (float)step, aim)));
-  int c = 0;
-#pragma unroll 1
-  for (int trip = 0; trip < 4; trip++) {
-    int off = 0;
-    c = 0;
-    for_cells27(d, bx, by, bz, [&](int ca, int cb, int mx, int my, int mz) {
-      const int i = (mx + 2) * 25 + (my + 2) * 5 + (mz + 2);
-      const float hx = hs.x - d.tab->s32[i][0], hy = hs.y - d.tab->s32[i][1], hz = hs.z - d.tab->s32[i][2];
-      const int j1 = __ldg(d.cell_start + cb + 1);
-      int j = __ldg(d.cell_start + ca) + off;
-      for (; j < j1; j += step) {
-        const float4 p = __ldg(hi + j);
-        const float x = p.x - hx, y = p.y - hy, z = p.z - hz;
-        c += fmaf(x, x, fmaf(y, y, z * z)) < t;
+// The same for crowded cells, in one pass from the widest radius: when a lane's list is
+// nearly full, every lane of the warp brings its radius in to the first gap after NK + 1
+// candidates and drops what lies beyond.  T is the radius (squared) in the end: the
+// list holds all candidates within it.  Returns their number: 0 where no gap leaves the
+// list room (more than 24 or 56 atoms, 10 or 38 of them at one distance).
+template <bool SPLIT, int NK>
+__device__ __noinline__ int knn_crowded(const FrameDesc &d, const float4 *__restrict__ hi, float4 hs, float2 ls, int bx,
+                                        int by, int bz, float &T, const KnnList &list) {
+  constexpr int CAP = KnnShape<NK>::CAP, U = 8;        // U loads in flight
+  const unsigned mask = __activemask();                // these lanes stay together
+  const float l0 = SPLIT ? hs.w : 0.f;
+  const int nbx = d.nb[0], nby = d.nb[1], nbz = d.nb[2];
+  float hx = 0.f, hy = 0.f, hz = 0.f, lx = 0.f, ly = 0.f, lz = 0.f;
+  uint8_t code = 0;
+  int cell = 0, j = 0, j1 = 0, cnt = 0;
+  for (;;) {
+    while (j >= j1 && cell < 27) {                     // this lane's next cell, its own first
+      const int ix = cell / 9, iy = cell / 3 % 3, iz = cell % 3;
+      int cx = bx + (ix == 2 ? -1 : ix), cy = by + (iy == 2 ? -1 : iy), cz = bz + (iz == 2 ? -1 : iz), mx = 0, my = 0, mz = 0;
+      cell++;
+      if (cx < 0) { cx += nbx; mx = -1; } else if (cx >= nbx) { cx -= nbx; mx = 1; }
+      if (cy < 0) { cy += nby; my = -1; } else if (cy >= nby) { cy -= nby; my = 1; }
+      if (cz < 0) { cz += nbz; mz = -1; } else if (cz >= nbz) { cz -= nbz; mz = 1; }
+      if ((mx && !d.pbc[0]) || (my && !d.pbc[1]) || (mz && !d.pbc[2])) continue;
+      const int c = (cx * nby + cy) * nbz + cz, i = (mx + 2) * 25 + (my + 2) * 5 + (mz + 2);
+      j = __ldg(d.cell_start + c);
+      j1 = __ldg(d.cell_start + c + 1);
+      const ShiftTables &t = *d.tab;
+      shift_pair(hs.x, l0, t.s32[i][0], t.slo[i][0], hx, lx);
+      shift_pair(hs.y, ls.x, t.s32[i][1], t.slo[i][1], hy, ly);
+      shift_pair(hs.z, ls.y, t.s32[i][2], t.slo[i][2], hz, lz);
+      code = (uint8_t)((mx + 1) << 4 | (my + 1) << 2 | (mz + 1));
+    }
+    if (!__any_sync(mask, j < j1)) break;
+    if (j < j1) {
+      float4 p[U];
+      float2 q[U];
+#pragma unroll
+      for (int k = 0; k < U; k++) {
+        p[k] = __ldg(hi + min(j + k, j1 - 1));
+        if constexpr (SPLIT) q[k] = __ldg(d.lo + min(j + k, j1 - 1));
       }
-      off = j - j1;
-    });
-    if (c >= 16 && c <= 64) break;
-    t *= exp2f(0.6666667f * __log2f(__fdividef(want, fmaxf((float)c, 1.f))));
-    c = (int)want;                                   // what the new radius should hold
+#pragma unroll
+      for (int k = 0; k < U; k++) {
+        float x = (p[k].x - hx) - lx, y = (p[k].y - hy) - ly, z = (p[k].z - hz) - lz;
+        if constexpr (SPLIT) { x = (p[k].x - hx) + (p[k].w - lx); y = (p[k].y - hy) + (q[k].x - ly); z = (p[k].z - hz) + (q[k].y - lz); }
+        const float v = fmaf(x, x, fmaf(y, y, z * z));
+        if (j + k < j1 && v < T) {                     // at most CAP - U entries before: there is room
+          list.V(cnt) = v; list.J(cnt) = j + k; list.M(cnt) = code;
+          cnt++;
+        }
+      }
+      j += U;
+    }
+    if (!__any_sync(mask, cnt > CAP - U)) continue;
+    uint32_t v[CAP];
+#pragma unroll
+    for (int i = 0; i < CAP; i++) v[i] = __float_as_uint(i < cnt ? list.V(i) : T);
+    oe_sort<0, CAP>(v);
+    uint32_t cut = 0;
+#pragma unroll
+    for (int c = CAP - U; c > NK; c--) cut = v[c] > v[c - 1] ? v[c] : cut;
+    if (cut) T = __uint_as_float(cut);                 // (fewer candidates than that: T still)
+    int kept = 0;
+#pragma unroll 4
+    for (int i = 0; i < cnt; i++) {
+      const float x = list.V(i);
+      if (!(x < T)) continue;
+      list.V(kept) = x; list.J(kept) = list.J(i); list.M(kept) = list.M(i);
+      kept++;
+    }
+    cnt = kept;
+    if (cnt > CAP - U) { cnt = 0; cell = 27; j = j1 = 0; }
   }
-  return t * exp2f(0.6666667f * __log2f(__fdividef(aim, (float)step * (float)c)));
+  return cnt;
 }
 
 // NK nearest images of the atom at sorted slot s, written to out[t * n], t = 0 ..
 // NK - 1; false when k_knn_rest must decide (the NK-th neighbour may lie outside
 // the 27 cells, or no radius admits a fitting number of candidates).
 //
-// The radius is that of a sphere holding NT atoms at the density of the 27
+// The radius is that of a sphere holding AIM atoms at the density of the 27
 // cells, at most what they are sure to cover; too many or too few candidates
-// rescale it.  The list is sorted once by its FP32 values with the entry number
-// in the low bits; if the NK + 1 smallest (or the NK in it and the radius) then
-// differ by more than the error band, their order is the FP64 order.  Otherwise the values are sorted again
-// without entry numbers, close ones form runs, and a run's candidates are
+// rescale it, and crowded cells are read another way (PTM_KNN_CROWDED; `launch`: atoms
+// of the launch, all its frames together).  The list is sorted once by its FP32
+// values with the entry number in the low bits; if the NK + 1 smallest (or the NK in
+// it and the radius) then differ by more than the error band, their order is the FP64
+// order.  Otherwise the values are sorted again without entry numbers, close ones form runs, and a run's candidates are
 // ordered by the FP64 key (d2, atom id, image); a run across slot NK takes
 // every candidate within the band.
 template <bool F64, bool SPLIT, int NK>
 __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int by, int bz, bool wrapped, int2 *out,
-                                         int64_t nst, const KnnList &list) {
+                                         int64_t nst, const KnnList &list, int64_t launch) {
   typedef typename RT<F64>::T IN;
   constexpr int CAP = KnnShape<NK>::CAP;
   constexpr float AIM = KnnShape<NK>::AIM;
@@ -381,29 +436,37 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
   const float4 hs = __ldg(hi + s);
   float2 ls = make_float2(0.f, 0.f);
   if constexpr (SPLIT) ls = __ldg(d.lo + s);
-  int cnt = 0;
-  float T;
-  {
-    int atoms = 0, cells = 0;
+  int cnt = 0, atoms = 0, cells = 0;
+  for_cells27(d, bx, by, bz, [&](int ca, int cb, int, int, int) {
+    atoms += __ldg(d.cell_start + cb + 1) - __ldg(d.cell_start + ca);
+    cells += cb - ca + 1;
+  });
+  float filled = (float)atoms;                       // atoms in as many cells filled evenly
+  bool uneven = false;
+  if (atoms > PTM_KNN_CROWDED) {
+    if (launch <= PTM_KNN_CROWDED_LAUNCH >> F64 && atoms > (int)(d.n - d.n / 16)) return false;
+    int most = 0;
     for_cells27(d, bx, by, bz, [&](int ca, int cb, int, int, int) {
-      atoms += __ldg(d.cell_start + cb + 1) - __ldg(d.cell_start + ca);
-      cells += cb - ca + 1;
+      for (int c = ca; c <= cb; c++) most = max(most, __ldg(d.cell_start + c + 1) - __ldg(d.cell_start + c));
     });
-    const float r3 = AIM * 0.2387324f * d.cell_vol * __fdividef((float)cells, (float)atoms);
-    T = exp2f(0.6666667f * __log2f(r3));
-    if (atoms > PTM_KNN_CROWDED) {
-      const int n = (int)d.n;
-      if (n <= PTM_KNN_CROWDED_FRAME && atoms > n - n / 16) return false;
-      if (atoms > PTM_KNN_CROWDED_FRAME) T = crowded_radius(d, hi, hs, bx, by, bz, atoms >> 8, T, AIM);
-    }
-    T = fminf(Tmax, T);
+    // (without the constant, whose weight falls as the atoms in reach grow, the surfaces of
+    // large clusters leave the guess: 32,000 atoms in 2 diameters 0.68 -> 0.75 ms)
+    filled = (float)most * (float)cells;
+    uneven = filled > 3.f * (float)atoms + 1536.f;
   }
-  for (int attempt = 0;; attempt++) {
+  const float r3 = AIM * 0.2387324f * d.cell_vol * __fdividef((float)cells, filled);
+  float T = uneven ? Tmax : fminf(Tmax, exp2f(0.6666667f * __log2f(r3)));
+  for (int attempt = 0; !uneven; attempt++) {
     cnt = knn_gather<SPLIT, CAP>(d, hi, hs, ls, bx, by, bz, T, list);
     if (cnt > NK && cnt <= CAP) break;
-    if (attempt == 3 || (cnt <= NK && T >= Tmax)) return false;
+    if (cnt <= NK && (attempt == 3 || T >= Tmax)) return false;
+    uneven = cnt > CAP && (attempt == 3 || (attempt ? cnt > 4 * CAP : cnt > 16 * CAP && cnt > atoms / 2));
     const float f = exp2f(0.6666667f * __log2f(__fdividef(AIM, (float)cnt)));
-    T = fminf(Tmax, T * (cnt > CAP ? f : fmaxf(f, 1.2f)));
+    if (!uneven) T = fminf(Tmax, T * (cnt > CAP ? f : fmaxf(f, 1.2f)));
+  }
+  if (uneven) {
+    cnt = knn_crowded<SPLIT, NK>(d, hi, hs, ls, bx, by, bz, T, list);
+    if (cnt <= NK) return false;
   }
   // image of list entry i: the cells' image, less the wraps of the two atoms
   auto image = [&](int j, int code, int &a, int &b, int &c) {
@@ -513,8 +576,8 @@ __device__ __forceinline__ bool knn_fast(const FrameDesc &d, int s, int bx, int 
 
 // One atom of k_knn; an undecided one is appended to the list of k_knn_rest.
 template <bool F64, int NK>
-__device__ __forceinline__ void knn_atom(const FrameDesc &d, int s, int2 *rows, unsigned char *smem, int *rest,
-                                         int *rest_count) {
+__device__ __forceinline__ void knn_atom(const FrameDesc &d, int s, int64_t launch, int2 *rows, unsigned char *smem,
+                                         int *rest, int *rest_count) {
   const int64_t nst = d.n;
   int2 *out = rows + (s - d.atom_offset);
   if (__ldg(d.wrapv + s) == PTM_EXCLUDED) {           // excluded by the binning: no neighbours
@@ -528,8 +591,8 @@ __device__ __forceinline__ void knn_atom(const FrameDesc &d, int s, int2 *rows, 
   const KnnList list = knn_list<KnnShape<NK>::CAP>(smem);
   const bool wrapped = d.dstat[0] != 0;
   bool done;
-  if (F64 || wrapped) done = knn_fast<F64, true, NK>(d, s, bx, by, bz, wrapped, out, nst, list);
-  else done = knn_fast<F64, false, NK>(d, s, bx, by, bz, wrapped, out, nst, list);
+  if (F64 || wrapped) done = knn_fast<F64, true, NK>(d, s, bx, by, bz, wrapped, out, nst, list, launch);
+  else done = knn_fast<F64, false, NK>(d, s, bx, by, bz, wrapped, out, nst, list, launch);
   if (!done) rest[atomicAdd(rest_count, 1)] = s;
 }
 

@@ -279,8 +279,8 @@ __device__ __forceinline__ float topo_face32(int m, int j, float R, Vec V, float
 
 // Order o[0..m) of neighbour ranks by (area descending, rank ascending), then
 // group by the band and order each group by rank.  Returns the faces (bit =
-// neighbour rank) on either side of a gap between consecutive areas that lies
-// within the guard of the band edge; 0 when every gap is clear of it.
+// neighbour rank) that may stand on either side of a gap between consecutive areas
+// that lies within the guard of the band edge; 0 when every gap is clear of it.
 template <typename T>
 __device__ uint32_t topo_order(int m, const T *area, T mean2, int *o) {
   for (int k = 0; k < m; k++) o[k] = k;
@@ -297,7 +297,14 @@ __device__ uint32_t topo_order(int m, const T *area, T mean2, int *o) {
     bool split = k == m;
     if (k < m) {
       const T gap = area[o[k - 1]] - area[o[k]];
-      if (fabs(gap - band) <= guard) near |= (1u << o[k - 1]) | (1u << o[k]);
+      if (fabs(gap - band) <= guard) {
+        // the two faces of the gap, and those so near to either in area that rounding may
+        // have put them in its place (an area of exactly 0 is not rounding's)
+        near |= (1u << o[k - 1]) | (1u << o[k]);
+        for (int q = k - 1; q > 0 && area[o[q - 1]] - area[o[q]] <= guard / 2; q--) near |= 1u << o[q - 1];
+        for (int q = k; q + 1 < m && area[o[q]] - area[o[q + 1]] <= guard / 2 && area[o[q + 1]] > (T)0; q++)
+          near |= 1u << o[q + 1];
+      }
       split = gap > band;
     }
     if (split) {                                      // group o[g0..k): order by rank
@@ -314,8 +321,8 @@ __device__ uint32_t topo_order(int m, const T *area, T mean2, int *o) {
 }
 
 // What the FP32 pass leaves for the FP64 pass about a listed atom: its FP32 face
-// areas and the faces to recompute in FP64 (bit = neighbour rank: the two faces
-// of every gap at the band edge, or all).
+// areas and the faces to recompute in FP64 (bit = neighbour rank: those beside
+// every gap at the band edge, or all).
 struct TopoSide {
   float area[PTM_TOPO_N];
   uint32_t faces;
@@ -402,7 +409,7 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int *list, int *l
 
 // FP64 pass for listed atom i (= list position), one thread: FP64 neighbour
 // vectors, and in FP64 the areas of the faces the FP32 pass could not decide
-// (the two faces of every gap at the band edge); the others keep their FP32
+// (those beside every gap at the band edge); the others keep their FP32
 // areas, whose error (measured within 3.1e-6 of the mean squared distance) is
 // far below the guard, so every gap decided from them is decided as in FP64.
 // Atoms past the side buffer recompute every face.  Polygon buffers in shared memory, element e at P[e * PTM_BLOCK].  The

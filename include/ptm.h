@@ -6,8 +6,8 @@
  * For every atom of a periodic frame the library
  *   - selects the 14 nearest neighbours, Euclidean order (Sec. 3, Table 1);
  *   - builds the convex hulls of the first 6, 12 and 14 neighbours and labels
- *     each hull graph by a Weinberg walk, looked up among the codes of the
- *     template triangulations (Sec. 4);
+ *     each hull graph with the Weinberg labels of the template triangulation it
+ *     equals, found by a code of its adjacency matrix (Sec. 4);
  *   - matches the labels against the SC, FCC, HCP, ICO and BCC templates and
  *     evaluates the scale-invariant RMSD (Eq. 3-4) of every admissible
  *     correspondence (Algorithm 1);
@@ -68,7 +68,7 @@ enum { PTM_F32 = 0, PTM_F64 = 1 };
 enum { PTM_ORDER_EUCLIDEAN = 0, PTM_ORDER_TOPOLOGICAL = 1 };
 
 /* Arithmetic of the metric steps (QCP, selection, outputs).  The exact hull
-   predicates, Weinberg codes and lookup are the same in both. */
+   predicates, graph codes and lookup are the same in both. */
 enum {
   PTM_PREC_FP32 = 0,         /* FP32, with FP64 where stability needs it (the product path) */
   PTM_PREC_FP64 = 1          /* every candidate and the winner's outputs in FP64: the
@@ -203,8 +203,8 @@ typedef struct {
 
 /* Build a batch of n_frames frames (all PTM_F32 or all PTM_F64; device
    buffers; outs[i] belongs to frames[i]).  Allocates the batch workspace
-   (about 40 B per atom plus 8 B per cell) and copies the frame descriptors to
-   the device.  tuning may be NULL. */
+   (about 180 B per atom, 220 for PTM_F64, 56 more in the topological order, and
+   8 B per cell) and copies the frame descriptors to the device.  tuning may be NULL. */
 ptm_status ptm_batch_create(ptm_context *ctx, int n_frames, const ptm_frame *frames,
                             const ptm_outputs *outs, const ptm_tuning *tuning, ptm_batch **out);
 
@@ -235,10 +235,11 @@ ptm_status ptm_autotune_batch(ptm_context *ctx, int n_frames, const ptm_frame *f
    In-situ analysis of MD frames that arrive at any time.  A server owns one
    scheduler thread and a few non-blocking streams.  Submitted frames (HOST
    buffers, ideally page-locked) wait in a FIFO and are admitted when their
-   device bytes (inputs, outputs and workspace, about 300 B per atom) fit the
-   HBM budget next to the frames already on the device.  Whenever a stream is
-   free, the admitted frames not yet launched (up to max_batch_frames and
-   max_batch_atoms, in arrival order) form one batch: copy in, one persistent launch, copy out.  Frames arriving while
+   device bytes (inputs, outputs and workspace: 359 B per atom, 411 for PTM_F64,
+   56 more in the topological order) fit the HBM budget next to the frames
+   already on the device.  Whenever a stream is free, the admitted frames not yet
+   launched (up to max_batch_frames and max_batch_atoms, in arrival order) form
+   one batch: copy in, one persistent launch, copy out.  Frames arriving while
    batches run join the next batch as memory and streams free up, and batches
    on different streams overlap on the device (continuous batching).  Device
    memory is pooled and reused; nothing is freed while the server runs.  Each
@@ -303,7 +304,7 @@ ptm_status ptm_server_inject(ptm_server *server, int fault);
    needed: the call runs on the current device, on `stream`, with the same
    kernels and results as ptm_classify_frame; positions, species and outputs are
    DEVICE pointers owned by the caller.  Its workspace is one static device
-   array of about 7.0 MiB that every GPU loading this library holds until the
+   array of about 7.8 MiB that every GPU loading this library holds until the
    process exits.  Its device address belongs to the CUDA context current at
    the call: every call outside stream capture looks it up again (so a device
    reset or a caller-made driver context is followed), and a call on a

@@ -137,9 +137,6 @@ constexpr int SCRATCH_WORDS = 42 + 24 + 18;   // 32-bit words per k_hulls thread
 
 // -------------------------------------------------------------- small helpers
 __device__ __forceinline__ int nib(uint64_t x, int i) { return (int)((x >> (4 * i)) & 15); }
-__device__ __forceinline__ uint64_t setnib(uint64_t x, int i, int v) {
-  return (x & ~(15ull << (4 * i))) | ((uint64_t)v << (4 * i));
-}
 
 // Lattice image (a, b, c) in 10 bits a component, in the order of the components: atoms may
 // stand 100 periods outside the cell (PTM_FAR_PERIODS), so the image of a neighbour runs

@@ -10,7 +10,7 @@
 //              (ptm_knn.cuh; for the topological order the 18 nearest, from
 //              which k_topo in ptm_topo.cuh makes the list)
 //   k_knn_rest one warp per atom that k_knn left undecided
-//   k_hulls    one thread per atom: hulls, Weinberg codes, template lookup
+//   k_hulls    one thread per atom: hulls, graph codes, template lookup
 //   k_match    one thread per atom: QCP, selection, outputs
 // The phases run as separate kernels so that the warps of an SM share one
 // phase of the method and its code (the instruction cache held none of the
@@ -22,12 +22,12 @@ namespace ptm {
 
 // ---------------------------------------------------------- per-atom state
 // Per-atom selection state.  Plain scalars (no arrays) so that it stays in
-// registers; snapshot k = 6, 12, 14 keeps its walk labelling and table entry.
+// registers; snapshot k = 6, 12, 14 keeps its Weinberg labelling and table entry.
 struct Best {
   float b1, b2;                 // best and second-best FP32 RMSD^2
   int K, cand;                  // winning snapshot (6, 12, 14) and candidate index
   int fp64;                     // the winner's eigenvalue needed the FP64 solve
-  uint64_t lam6, lam12, lam14;  // walk labelling per snapshot
+  uint64_t lam6, lam12, lam14;  // Weinberg labelling per snapshot
   int ent6, ent12, ent14;       // table entry per snapshot, -1 = none
   __device__ __forceinline__ uint64_t lam(int K) const { return K == 6 ? lam6 : (K == 12 ? lam12 : lam14); }
   __device__ __forceinline__ int ent(int K) const { return K == 6 ? ent6 : (K == 12 ? ent12 : ent14); }
@@ -37,7 +37,7 @@ struct Best {
 struct MatchCounts { int scored, points, matched; };
 
 // Template slots of neighbours 0 .. K - 1 (nibble j) under the correspondence given
-// by the walk labelling and the table candidate.
+// by the Weinberg labelling and the table candidate.
 __device__ __forceinline__ uint64_t slots_of(int K, uint64_t lab, uint64_t cand) {
   uint64_t slots = 0;
 #pragma unroll 2
@@ -1465,15 +1465,14 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_MATCH_BLOCKS_PER_SM) k_match(co
   count_warp(d, C_MATCHED, 0xffffffffu, c.matched);
 }
 
-// Neighbour lists of one frame, one thread per atom: NK = 14 into d.nbr, NK = 18
-// (topological order), into d.nbr.  Measured against the insertion network and
+// Neighbour lists of one frame, one thread per atom: NK = 14, or 18 for the
+// topological order.  Measured against the insertion network and
 // the FP64 arithmetic it replaced (k_knn with k_knn_rest, device time):
-//   2^20-atom polycrystal, float32      1.23  -> 0.64 ms (k_knn 0.46, at 46 % of
-//                                       issue and 47 % of L1; 675 -> 226 warp
-//                                       instructions an atom)
-//   250,000 atoms, float64              6.03  -> 0.23 ms (was FP64-pipe bound)
-//   199,680 atoms, unwrapped float32    4.04  -> 0.16 ms (was the general search)
-//   256 frames, 31.7 M atoms            31.2  -> 16.0 ms
+//   2^20-atom polycrystal, float32      1.23  -> 0.48 ms (k_knn 0.41, at 52 % of
+//                                       issue; 675 -> 232 warp instructions an atom)
+//   250,000 atoms, float64              6.03  -> 0.15 ms (was FP64-pipe bound)
+//   202,500 atoms, unwrapped float32    4.04  -> 0.14 ms (was the general search)
+//   256 frames, 31.7 M atoms            31.2  -> 15.8 ms
 template <bool F64, int NK>
 __global__ void __launch_bounds__(PTM_KNN_BLOCK, KnnShape<NK>::BLOCKS)
     k_knn(const __grid_constant__ FrameDesc d, int apw, int *rest, int *rest_count) {

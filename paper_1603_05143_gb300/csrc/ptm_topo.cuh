@@ -412,11 +412,11 @@ __device__ void topo_atom(const FrameDesc &d, int s, int *tsm, int *list, int *l
 // (those beside every gap at the band edge); the others keep their FP32
 // areas, whose error (measured within 3.1e-6 of the mean squared distance) is
 // far below the guard, so every gap decided from them is decided as in FP64.
-// Atoms past the side buffer recompute every face.  Polygon buffers in shared memory, element e at P[e * PTM_BLOCK].  The
-// lanes of `wmask` call this together and take their faces in step, one face
-// per lane per trip, so a warp makes as many trips as its busiest lane has
-// faces (not one per face index that any lane needs).  A face is first clipped
-// again in FP32, which finds the lines that matter (about 6 of 17), so the FP64
+// Atoms past the side buffer recompute every face.  Polygon buffers in shared
+// memory, element e at P[e * PTM_BLOCK].  The lanes of `wmask` call this
+// together and take their faces in step, one face per lane per trip, so a warp
+// makes as many trips as its busiest lane has faces (not one per face index that
+// any lane needs).  A face is first clipped again in FP32, which finds the lines that matter (about 6 of 17), so the FP64
 // pipe, 2 operations a clock per SM, sees only those.
 template <bool F64>
 __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *side, int cap_side, double *P,
@@ -470,9 +470,9 @@ __device__ void topo_atom64(const FrameDesc &d, int s, int i, const TopoSide *si
   for (int k = 0; k < PTM_KNN; k++) d.nbr[(int64_t)k * n + sl] = k < m ? make_int2(jn[o[k]], im[o[k]]) : make_int2(-1, 0);
 }
 
-// Bounded by instruction issue (55 %; 624 M warp instructions per 262 k atoms):
-// 1.69 ms with every plane clipping every vertex, 1.35 ms with marks and one copy
-// per cut, 0.99 ms nearest line first and at 8 blocks per SM.
+// Bounded by instruction issue (60 % of the slots; 2,000 warp instructions an atom).  262 k
+// atoms: 1.69 ms with every plane clipping every vertex, 1.35 ms with marks and one copy
+// per cut, 1.01 ms nearest line first and at 8 blocks per SM.
 template <bool F64>
 __global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO_BLOCKS_PER_SM) k_topo(const __grid_constant__ FrameDesc d, int *list,
                                                     int *list_count, TopoSide *side, int cap_side) {
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(PTM_BLOCK, PTM_TOPO_BLOCKS_PER_SM) k_topo(cons
 // list: its length is read on the device): fn(position in the list, lanes of the
 // warp that call together).  (Spreading a short list thinner, 8 atoms per warp, made
 // 3 times the FP64 warp instructions: 0.37 -> 0.44 ms for 7,800 atoms; clipping by
-// the lines that matter only: 0.24 ms.)
+// the lines that matter only: 0.24 ms, 0.27 with the lines left out checked in FP32.)
 template <typename Fn>
 __device__ __forceinline__ void topo64_list(int cnt, Fn &&fn) {
   for (int i0 = blockIdx.x * PTM_BLOCK + (threadIdx.x & ~31); i0 < cnt; i0 += gridDim.x * PTM_BLOCK) {

@@ -231,7 +231,7 @@ def edge_key(deg, th, a, b):
 
 def start_codes(facets):
     """Weinberg code -> first-visit labellings, over every start edge with the
-    largest key (definition in the module docstring).  The kernels walk from one
+    largest key (definition in the module docstring).  The kernels take one
     such start, whichever comes first in their facet list, so the tables hold
     the code of each of them; starts related by an automorphism give the same
     code."""
